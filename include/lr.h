@@ -11,7 +11,7 @@
  * Method: sparse ruling set (Section 2.1, Algorithm 1): pick rulers (every
  * head is forced to be one), chase each ruler's packet along succ until the
  * next ruler while recording (ruler, offset) per element, rank the reduced
- * list of rulers recursively (a single-CTA pointer-doubling base case ends the
+ * list of rulers recursively (a pointer-jumping base case ends the
  * recursion), then give every element rank[ruler] - offset.
  *
  * Conventions shared by every entry point below:
@@ -82,12 +82,12 @@ typedef enum lr_dtype { LR_NONE = 0, LR_I32 = 1, LR_I64 = 2 } lr_dtype;
  * element order's L2 prefetch lead in K elements, 0 off, 4 by default).
  */
 typedef struct lr_tuning {
-    uint32_t f0_inv;     /* 1/f at level 0 (default by n: 4 below 2^16, 8 below  */
-                         /* 2^22, 16 below 2^27, 48 below 2^29, 96 from 2^29;   */
-                         /* a batch keeps 16 from 2^22 up)                       */
-    uint32_t f_inv;      /* 1/f at levels >= 1 (default 8)                       */
-    uint32_t cutoff;     /* largest level ranked by the single-CTA base case     */
-                         /* (default and maximum 12288)                          */
+    uint32_t f0_inv;     /* 1/f at level 0 (default by n: 4 to 16 below 2^27,    */
+                         /* 48 below 2^29, 96 from 2^29; a batch keeps 16 from   */
+                         /* 2^22 up)                                             */
+    uint32_t f_inv;      /* 1/f at levels >= 1 (default 4 or 8, by size)         */
+    uint32_t cutoff;     /* largest level ranked by the base case when below     */
+                         /* 12288; 12288 and more, and 0: the built-in bound     */
     uint32_t chase_block;/* threads per CTA of the chase kernel (default 256)    */
     uint32_t chase_ctas; /* CTAs per SM of the chase kernel (default: occupancy; */
                          /* a batch's level 0, chased in element order, 1024    */
@@ -540,8 +540,8 @@ void lr_autotune_clear(void);
  * submission still overlap this ranking), and the engine grows its own
  * buffers to the count.  depth: 2..4 (0 selects 2).  Device memory:
  * depth * max_n * (4 + weight bytes + rank bytes), plus
- * lr_workspace_size(max_n, 0, opts) per ranking stream when max_lists > 0
- * (the engine's own buffers per ranking stream otherwise).
+ * per ranking stream, when max_lists > 0, the most that lr_workspace_size
+ * gives for any size up to max_n (the engine's own buffers otherwise).
  *
  * Host buffers should be pinned (cudaHostAlloc / cudaHostRegister); pageable
  * buffers work but their copies block the submitting thread.  The caller

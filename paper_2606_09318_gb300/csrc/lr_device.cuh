@@ -17,12 +17,11 @@ namespace lr {
 // ---------------------------------------------------------------- constants
 constexpr uint32_t kUnvisited = 0xFFFFFFFFu;   // tag word of a record not yet chased
 constexpr uint32_t kZeroCid = 0xFFFFFFFEu;     // "ruler" of a resolved singleton: R = 0
-constexpr uint32_t kEnd = 0xFFFFFFFFu;         // no successor (pointer doubling)
+constexpr uint32_t kEnd = 0xFFFFFFFFu;         // no successor (pointer jumping, doubling)
 constexpr int kMaxLevels = 12;                 // SRS levels in a static plan
 constexpr int kHeadBlocks = 512;               // CTAs of the head-selection kernels
 constexpr int kHeadThreads = 256;
-constexpr int kBaseThreads = 1024;             // single-CTA base case
-constexpr uint32_t kMaxCutoff = 12288;         // largest base-case level (SMEM bound)
+constexpr uint32_t kMaxCutoff = 12288;         // largest base-case bound a caller can set
 constexpr int kContractTileShift = 12;         // tile-local contraction: tiles of 4096 ids
 
 // error bits recorded on the device (mapped to lr_status by the host)
@@ -48,7 +47,7 @@ constexpr bool kDebugChecks = false;
 #endif
 
 // per-level mode, decided on the device by the previous level
-enum : uint32_t { kModeOff = 0, kModeSrs = 1, kModeBase = 2, kModePd = 3 };
+enum : uint32_t { kModeOff = 0, kModeSrs = 1, kModeBase = 2 };
 
 // Level descriptor (device memory).  n/r/mode of level l+1 are written by the
 // head-selection scan of level l; the host writes level 0 and the static
@@ -63,9 +62,9 @@ struct LevelDesc {
   uint32_t f_inv;    // static: 1/f
   uint32_t cap;      // static: capacity of this level's arrays
   uint64_t seed;     // static: permutation seed
-  uint32_t rounds;   // static: pointer-doubling rounds of the fallback base
   uint32_t hsrc;     // where this level's heads come from: kHeadsBitmap or kHeadsList
   uint32_t nraw;     // with spawning: ruler ids of the next level before compaction (else 0)
+  unsigned long long check;  // base case: nonzero when an element has two predecessors (k_jump)
 };
 
 enum : uint32_t { kHeadsBitmap = 0, kHeadsList = 1 };
@@ -160,6 +159,19 @@ __device__ __forceinline__ bool dbg_fail(bool ok, uint32_t *err) {
     return true;
   }
   return false;
+}
+
+// Two predecessors of an element of a level that the base case ranked: its
+// check sum (k_jump) does not vanish.  A cycle with a single ruler closes the
+// ruler on itself, which upsets the sum too and is already recorded.
+__device__ __forceinline__ uint32_t merge_errors(const LevelDesc &ranked, const uint32_t *err) {
+  return ranked.mode == kModeBase && ranked.check && !(__ldcg(err) & kErrCycle) ? kErrNotList : 0u;
+}
+
+// What the propagation into level d finds wrong with the input: elements that
+// no chase reached, or two predecessors in the level below.
+__device__ __forceinline__ uint32_t level_errors(const LevelDesc &d, const LevelDesc &next, const uint32_t *err) {
+  return (d.visited != d.n ? kErrCycle : 0u) | merge_errors(next, err);
 }
 
 // L2-only loads/stores for data with no reuse in L1.

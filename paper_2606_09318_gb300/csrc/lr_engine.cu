@@ -7,7 +7,7 @@
 // doubling).  The number of levels and every array size are fixed on the host
 // from n and a bound h on the number of lists:
 //   cap_0 = n,  cap_{l+1} = min(cap_l, ceil(cap_l / f_l) + h),
-// until a level fits the single-CTA base case.  The actual sizes are decided
+// until a level is small enough for the base case (k_jump).  The actual sizes are decided
 // on the device (each level's head scan writes the next level's size and
 // mode), so a call never waits for the device unless h has to be counted
 // first, and a call with a known bound can be captured in a CUDA graph.
@@ -44,14 +44,19 @@ static uint32_t env_u32(const char *spec, const char *key, uint32_t dflt) {
 }
 
 // Default ruler fraction at level 0 by size (measured on GB300, random
-// order, f = 1/8 above level 0).  Small lists are bound by the latency of
-// the dependent exchanges along one segment, so they take more rulers and
-// shorter segments; from 2^27 up the chase is bound by the random-access
+// order).  Up to 2^23 elements the rulers' list goes straight to the base
+// case (k_jump), whose time grows with its size, and the chase is bound by
+// the latency of its longest segment, about f ln(n / f) dependent steps: the
+// two balance near 200 to 350 thousand rulers (2^20: 172 us a call at 1/3 to
+// 1/8, 199 at 1/12; 2^21: 189 at 1/8, 207 at 1/4, 211 at 1/16; 2^22: 271 at
+// 1/12, 276 at 1/8).  From 2^27 up the chase is bound by the random-access
 // rate, and fewer rulers shrink the recursion more than their longer
 // segments lengthen the chase's tail (1/48 at 2^28, 1/96 at 2^30).
 static uint32_t default_f0_inv(int64_t n) {
-  if (n < ((int64_t)1 << 16)) return 4;
-  if (n < ((int64_t)1 << 22)) return 8;
+  if (n < 3 * ((int64_t)1 << 18)) return 4;
+  if (n < 5 * ((int64_t)1 << 18)) return 6;
+  if (n < 5 * ((int64_t)1 << 19)) return 8;
+  if (n < 3 * ((int64_t)1 << 21)) return 12;
   if (n < ((int64_t)1 << 27)) return 16;
   if (n < ((int64_t)1 << 29)) return 48;
   return 96;
@@ -65,11 +70,23 @@ static uint32_t default_f0_inv_batch(int64_t n) {
   return n < ((int64_t)1 << 22) ? default_f0_inv(n) : 16;
 }
 
+// Largest level below the first that the base case ranks (k_jump), unless the
+// caller sets a smaller bound: with 262 / 350 / 524 thousand elements it takes
+// 25 / 35 / 65 us, one more level in front of it (chase at 1/4, selection,
+// propagation) about 60 us less the smaller base case's 18.
+constexpr uint32_t kJumpMax = 3u << 17;
+
+// Default ruler fraction below level 0: 1/4 where that already reaches the
+// base case (2^24, 10^6 rulers: 900 us a call at 1/4, 907 at 1/6, 912 at 1/8).
+static uint32_t default_f_inv(int64_t n, uint32_t f0_inv) {
+  return n / f0_inv <= (int64_t)kJumpMax * 4 ? 4 : 8;
+}
+
 Tuning resolve_tuning_builtin(int64_t n, bool weighted, bool batch) {
   (void)weighted;
   Tuning u;
   u.f0_inv = batch ? default_f0_inv_batch(n) : default_f0_inv(n);
-  u.f_inv = 8;
+  u.f_inv = default_f_inv(n, u.f0_inv);
   u.cutoff = kMaxCutoff;
   u.block = 256;
   u.ctas = 0;
@@ -79,12 +96,15 @@ Tuning resolve_tuning_builtin(int64_t n, bool weighted, bool batch) {
   u.contract = LR_CONTRACT_AUTO;
   u.spawn = 0;
   u.ord = 2;              // batches: every level of 2^20 or more in element order
+  u.base0 = kMaxCutoff;
+  u.base = kJumpMax;
   u.pf = 4;               // ... prefetching its records 4K elements ahead of each draw
   return u;
 }
 
 Tuning resolve_tuning(const lr_tuning *t, int64_t n, bool weighted, bool batch) {
   Tuning u = resolve_tuning_builtin(n, weighted, batch);
+  u.f_inv = 0;
   lr_tuning tt;
   if (tuned_lookup(n, weighted, batch, &tt)) {
     if (tt.f0_inv) u.f0_inv = tt.f0_inv;
@@ -119,9 +139,11 @@ Tuning resolve_tuning(const lr_tuning *t, int64_t n, bool weighted, bool batch) 
     if (t->chase_ctas) u.ctas = t->chase_ctas;
   }
   u.f0_inv = std::max<uint32_t>(2, u.f0_inv);
-  u.f_inv = std::max<uint32_t>(2, u.f_inv);
+  u.f_inv = u.f_inv ? std::max<uint32_t>(2, u.f_inv) : default_f_inv(n, u.f0_inv);
   u.cutoff = std::min<uint32_t>(std::max<uint32_t>(u.cutoff, 64), kMaxCutoff);
   if (u.block != 128 && u.block != 256 && u.block != 512) u.block = 256;
+  u.base0 = u.cutoff;
+  u.base = u.cutoff >= kMaxCutoff ? kJumpMax : u.cutoff;
   return u;
 }
 
@@ -131,7 +153,7 @@ Tuning resolve_tuning(const lr_tuning *t, int64_t n, bool weighted, bool batch) 
 // spawning (an exchange-form feature) was asked for.
 constexpr uint64_t kLogAutoMin = 1ull << 25;
 static bool use_log0(const Tuning &u, uint64_t n, bool weighted, int rank_bytes, bool extras, bool multi) {
-  if (weighted || rank_bytes != 4 || extras || multi || n <= u.cutoff || n > (1ull << 30) || !u.xchg)
+  if (weighted || rank_bytes != 4 || extras || multi || n <= u.base0 || n > (1ull << 30) || !u.xchg)
     return false;
   if (u.chase0 == LR_CHASE0_LOG) return true;
   return u.chase0 == LR_CHASE0_AUTO && n >= kLogAutoMin && !u.spawn;
@@ -143,12 +165,6 @@ static bool use_log0(const Tuning &u, uint64_t n, bool weighted, int rank_bytes,
 // pass, the rank gathers within a footprint the L2 holds.
 static bool use_ord0(const Tuning &u, uint64_t n, bool log0, bool spawn0, bool extras, bool multi) {
   return u.ord != 0 && multi && !log0 && !spawn0 && !extras && n <= 0x7FFFFFFFull;
-}
-
-static uint32_t ceil_log2(uint64_t x) {
-  uint32_t b = 0;
-  while ((1ull << b) < x) ++b;
-  return b;
 }
 
 static size_t align_up(size_t x, size_t a = 256) { return (x + a - 1) / a * a; }
@@ -187,16 +203,17 @@ Plan make_plan(uint64_t n, uint64_t h, const Tuning &u, bool rec16_0, int rank_b
   p.rec16_0 = rec16_0;
   p.log0 = log0;
   p.rank_bytes = rank_bytes;
-  p.cutoff = u.cutoff;
+  p.base = u.base;
   p.chase_grid = chase_grid;
   p.chase_block = (int)u.block;
   p.hcap = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(h, std::max<uint64_t>(n, 1)));
   p.cap[0] = (uint32_t)n;
   p.f_inv[0] = u.f0_inv;
   int L = 0;
-  const bool sp = spawn0 && (n > u.cutoff || force_srs);
+  p.low[0] = n;
+  const bool sp = spawn0 && (n > u.base0 || force_srs);
   p.spawn_cap = sp ? spawn_capacity(n, (uint64_t)chase_grid * u.block) : 0;
-  if (n > u.cutoff || force_srs) {
+  if (n > u.base0 || force_srs) {
     for (;;) {
       const uint64_t r = (p.cap[L] + p.f_inv[L] - 1) / p.f_inv[L];
       uint64_t nc = std::min<uint64_t>(p.cap[L], r + p.hcap);
@@ -206,16 +223,14 @@ Plan make_plan(uint64_t n, uint64_t h, const Tuning &u, bool rec16_0, int rank_b
       }
       ++L;
       p.cap[L] = (uint32_t)nc;
+      p.low[L] = (p.low[L - 1] + p.f_inv[L - 1] - 1) / p.f_inv[L - 1];   // the sampled rulers alone
       p.f_inv[L] = u.f_inv;
-      if (nc <= u.cutoff) break;
+      if (nc <= u.base) break;
       if (L == kMaxLevels) break;
-      if (L == 1 && p.cap[0] <= u.cutoff) break;
       if (L >= 3 && (uint64_t)p.cap[L] * 4 > (uint64_t)p.cap[L - 1] * 3) break;  // stalled
     }
   }
   p.nlev = L + 1;
-  p.has_pd = p.cap[L] > u.cutoff;
-  p.pd_rounds = p.has_pd ? ceil_log2(p.cap[L]) + 1 : 0;
   for (int l = 0; l <= L; ++l) p.seed[l] = splitmix64(seed + 0x9E37ull * (uint64_t)(l + 1));
 
   // fixed part: independent of h
@@ -264,12 +279,6 @@ Plan make_plan(uint64_t n, uint64_t h, const Tuning &u, bool rec16_0, int rank_b
   p.off_hA = o; o = align_up(o + 4 * (size_t)p.hcap);
   p.off_hB = o; o = align_up(o + 4 * (size_t)p.hcap);
   p.off_ns = o; o = align_up(o + 4 * (size_t)p.hcap);
-  if (p.has_pd) {
-    p.off_pd[0] = o; o = align_up(o + 4 * (size_t)p.cap[L]);
-    p.off_pd[1] = o; o = align_up(o + 4 * (size_t)p.cap[L]);
-    p.off_pd[2] = o; o = align_up(o + 8 * (size_t)p.cap[L]);
-    p.off_pd[3] = o; o = align_up(o + 8 * (size_t)p.cap[L]);
-  }
   if (p.spawn_cap) {
     const size_t words = (p.spawn_cap + 31) / 32;
     p.off_sraw = o; o = align_up(o + 16 * (size_t)p.raw_cap);
@@ -296,10 +305,6 @@ Plan make_plan(uint64_t n, uint64_t h, const Tuning &u, bool rec16_0, int rank_b
       p.off_tid[l] = o; o = align_up(o + 4 * (size_t)p.cap[l]);
     }
     p.off_hC = o; o = align_up(o + 4 * (size_t)p.hcap);   // keeps level 0's head list intact
-    if (p.has_pd) {
-      p.off_pdt[0] = o; o = align_up(o + 4 * (size_t)p.cap[L]);
-      p.off_pdt[1] = o; o = align_up(o + 4 * (size_t)p.cap[L]);
-    }
     if (t0ws) { p.off_T0 = o; o = align_up(o + 4 * (size_t)n); }
   }
   p.var_bytes = std::max<size_t>(o, 256);
@@ -325,8 +330,7 @@ lr_status setup_device_once() {
   if (e != cudaSuccess) return from_cuda(e);
   std::lock_guard<std::mutex> g(g_mu);
   if (dev >= 0 && dev < 64 && !g_setup_done[dev]) {
-    e = kernels_setup();
-    if (e == cudaSuccess) e = log_setup();
+    e = log_setup();
     if (e == cudaSuccess) e = lc_setup();
     if (e != cudaSuccess) return from_cuda(e);
     // Place lr_rank_noalloc's scratch array on this device now, while the
@@ -585,7 +589,7 @@ static lr_status run_wyllie(const Inputs &in, Ctx *c, cudaStream_t s) {
   LR_TRY(cudaMemsetAsync(base, 0, in.validate ? q.off_a : q.zero_bytes, s));
   // without validation the scratch sums stand in for the bitmap, so the
   // pass issues no per-element atomics
-  LR_TRY(launch_prep0(in.succ, in.weight, in.wtype, (uint32_t)in.n, A, bitmap, err, in.validate,
+  LR_TRY(launch_prep0(in.succ, in.weight, in.wtype, (uint32_t)in.n, A, w16, bitmap, err, in.validate,
                       in.offsets, in.k, in.validate ? nullptr : sums, nullptr, s));
   prof.mark(PH_PREP);
   LR_TRY(launch_wyllie(A, B, w16, (uint32_t)in.n, in.rank, in.rank_bytes, err, s));
@@ -692,8 +696,9 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
     return run_wyllie(in, c, s);
   }
   if (u.algo != LR_ALGO_SRS && u.algo != LR_ALGO_WYLLIE) return LR_ERR_INVALID_ARGUMENT;
-  const bool rec16_0 = in.wtype != 0;
   const bool extras = in.term != nullptr || in.prefix != nullptr || in.incl != 0;
+  // 16-byte level-0 records: weighted, or ranked at level 0 with terminal ids
+  const bool rec16_0 = in.wtype != 0 || (extras && in.n <= u.base0);
   if (extras && ptrs) return LR_ERR_INVALID_ARGUMENT;
   const bool log0 = use_log0(u, in.n, in.wtype != 0, in.rank_bytes, extras, ptrs || in.offsets != nullptr);
   const bool t0ws = extras && in.term == nullptr;
@@ -715,7 +720,7 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
   const bool count_local = contractible && u.contract == LR_CONTRACT_AUTO;
   const int grid = chase_grid_for(u, rec16_0, log0, ord0);
   const bool need_count = in.max_lists <= 0 && (in.ws == nullptr || in.count_in_ws) &&
-                          (in.n > u.cutoff || ptrs);
+                          (in.n > u.base0 || ptrs);
   if (need_count && capturing) return LR_ERR_CAPTURE;
   uint64_t hb = in.max_lists > 0 ? (uint64_t)in.max_lists : in.n;
   Plan p = make_plan(in.n, hb, u, rec16_0, in.rank_bytes, in.seed, grid, ptrs, log0, extras, t0ws, spawn0,
@@ -743,13 +748,13 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
 
   // Single instance, no validation: heads from the streaming sums (one list)
   // with the bitmap as the fallback, instead of atomics for every element.
-  const bool sums0 = !log0 && !ptrs && in.offsets == nullptr && !in.validate && in.n > u.cutoff;
+  const bool sums0 = !log0 && !ptrs && in.offsets == nullptr && !in.validate && in.n > u.base0;
   // A batch (contiguous or one pointer per instance): per-instance sums (kept
   // at the start of the bitmap's memory, which must hold 16 bytes per
   // instance) give one head per instance and the number of lists, with the
   // bitmap as the fallback for the heads.
   const bool sums0b = !log0 && in.offsets != nullptr && !in.validate && !extras && !spawn0 &&
-                      in.n > u.cutoff && in.k > 0 && (uint64_t)in.k * 16 <= 4 * ((in.n + 31) / 32);
+                      in.n > u.base0 && in.k > 0 && (uint64_t)in.k * 16 <= 4 * ((in.n + 31) / 32);
   Profiler prof;
   if (!in.ctx) prof.begin(s, (int64_t)in.n);
   unsigned long long *acc = (unsigned long long *)(fixed + p.off_acc);
@@ -785,7 +790,7 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
     LR_TRY(launch_prep0_sums(in.succ, in.weight, in.wtype, (uint32_t)in.n, work0, err, in.offsets, in.k,
                              reinterpret_cast<unsigned long long *>(bitmap), s));
   else
-    LR_TRY(launch_prep0(in.succ, in.weight, in.wtype, (uint32_t)in.n, work0, bitmap, err,
+    LR_TRY(launch_prep0(in.succ, in.weight, in.wtype, (uint32_t)in.n, work0, rec16_0, bitmap, err,
                         in.validate, in.offsets, in.k, sums0 ? acc : nullptr, nullptr, s));
   if (need_count) {
     // count the lists (one wait), then size the recursion for exactly that many:
@@ -833,14 +838,11 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
   ip.nlev = p.nlev;
   ip.n0 = (uint32_t)in.n;
   ip.mode0 = p.nlev == 1 ? kModeBase : kModeSrs;
-  ip.cutoff = p.cutoff;
   for (int l = 0; l < p.nlev; ++l) {
     ip.f_inv[l] = p.f_inv[l];
     ip.cap[l] = p.cap[l];
     ip.seed[l] = p.seed[l];
   }
-  ip.pd_rounds = p.pd_rounds;
-  ip.has_pd = p.has_pd;
   ip.hcap = p.hcap;
   LR_TRY(launch_init(desc, ip, s));
   if (!in.ctx) { c->last_desc = desc; c->last_nlev = p.nlev; }
@@ -880,21 +882,23 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
   uint32_t *hB = (uint32_t *)(var + p.off_hB);
   uint32_t *hC = extras ? (uint32_t *)(var + p.off_hC) : hA;
   uint32_t *ns = (uint32_t *)(var + p.off_ns);
+  // head lists alternate between buffers; with extra outputs level 0's list
+  // (hA) stays intact for the prefix pass
+  auto head_list = [&](int l) -> uint32_t * { return l == 0 ? hA : ((l & 1) ? hB : hC); };
   const int L = p.nlev - 1;
   for (int l = 0; l < L; ++l) {
     const bool r16 = l > 0 || rec16_0;
-    // head lists alternate between buffers; with extra outputs level 0's
-    // list (hA) stays intact for the prefix pass
-    uint32_t *hin = l == 0 ? hA : ((l & 1) ? hB : hC);
-    uint32_t *hout = l == 0 ? hB : ((l & 1) ? hC : hB);
+    uint32_t *hin = head_list(l), *hout = head_list(l + 1);
     if (l > 0) {
-      LR_TRY(launch_base(desc, l, work_of(l), r16, R_of(l), p.rank_bytes, p.cutoff, err, tid_of(l),
-                         T_of(l), s));
-      prof.mark(PH_BASE);
+      if (p.low[l] <= p.base) {
+        LR_TRY(launch_jump(desc, l, work_of(l), r16, R_of(l), p.rank_bytes, p.cap[l], err, hin, tid_of(l),
+                           T_of(l), s));
+        prof.mark(PH_BASE);
+      }
     }
     const int kind = (l == 0 && log0) ? kRecKindSucc : (r16 ? kRecKind16 : kRecKind8);
     LR_TRY(launch_heads(desc, l, p.nlev, bitmap, hin, (l == 0 && log0) ? (void *)in.succ : work_of(l),
-                        kind, ns, hout, bcnt, err, p.cutoff, p.hcap, p.has_pd ? 1u : 0u, s));
+                        kind, ns, hout, bcnt, err, p.base, p.hcap, s));
     prof.mark(PH_SELECT);
     if (l == 0 && log0)
       LR_TRY(launch_chase_log(desc, in.succ, work_of(1), ns, qctr, p.chase_grid, p.chase_block, err,
@@ -905,8 +909,7 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
       LR_TRY(launch_chase(desc, 0, work0, r16, var + p.off_sraw, ns, qctr, p.chase_grid, p.chase_block,
                           err, (int)u.xchg, nullptr, nullptr, &spa, nullptr, s));
       LR_TRY(launch_spawn_compact(desc, 0, p.nlev, spa.ctr, spa.cap, spa.used, (uint32_t *)(var + p.off_supre),
-                                  var + p.off_sraw, work_of(1), p.raw_cap, p.cutoff, p.has_pd ? 1u : 0u,
-                                  err, s));
+                                  var + p.off_sraw, work_of(1), p.raw_cap, p.base, err, s));
     } else {
       OrdArgs oa;
       memset(&oa, 0, sizeof(oa));
@@ -924,16 +927,8 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
     if (l == 0) prof.call.log0 = log0;
     prof.mark(l == 0 ? PH_CHASE0 : PH_CHASE);
   }
-  LR_TRY(launch_base(desc, L, work_of(L), L > 0 || rec16_0, R_of(L), p.rank_bytes, p.cutoff, err,
-                     tid_of(L), T_of(L), s));
-  if (p.has_pd) {
-    uint32_t *pt0 = extras ? (uint32_t *)(var + p.off_pdt[0]) : nullptr;
-    uint32_t *pt1 = extras ? (uint32_t *)(var + p.off_pdt[1]) : nullptr;
-    LR_TRY(launch_pd(desc, L, work_of(L), p.cap[L], p.pd_rounds, (uint32_t *)(var + p.off_pd[0]),
-                     (uint32_t *)(var + p.off_pd[1]), (uint64_t *)(var + p.off_pd[2]),
-                     (uint64_t *)(var + p.off_pd[3]), R_of(L), p.rank_bytes, err, tid_of(L), pt0, pt1,
-                     T_of(L), s));
-  }
+  LR_TRY(launch_jump(desc, L, work_of(L), L > 0 || rec16_0, R_of(L), p.rank_bytes, p.cap[L], err,
+                     L > 0 ? head_list(L) : nullptr, tid_of(L), T_of(L), s));
   prof.mark(PH_BASE);
   for (int l = L - 1; l >= 0; --l) {
     if (l == 0 && log0)
@@ -1297,6 +1292,24 @@ static lr_status rank_host_impl(const uint32_t *succ_host, const void *weight_ho
   return sync ? device_status(s) : LR_OK;
 }
 
+}  // extern "C"
+
+namespace lr {
+// The plan's size is not monotone in n: the default ruler fraction falls as n
+// grows.  Each fraction's largest size counts, and each power of two (tuned
+// entries are kept per power of two).
+size_t workspace_upto(int64_t n, const lr_opts *opts) {
+  size_t w = lr_workspace_size(n, 0, opts);
+  auto consider = [&](int64_t m) { if (m > 0 && m < n) w = std::max(w, lr_workspace_size(m, 0, opts)); };
+  for (int64_t m = 1; m < n; m *= 2) { consider(m - 1); consider(m); }
+  for (int64_t m = 1; m < n; m *= 2)
+    for (int64_t q : {3 * m, 5 * m}) consider(q - 1);
+  return w;
+}
+}  // namespace lr
+
+extern "C" {
+
 size_t lr_workspace_size(int64_t n_total, int32_t k, const lr_opts *opts) {
   return lr_workspace_size_outputs(n_total, k, nullptr, opts);
 }
@@ -1322,7 +1335,8 @@ size_t lr_workspace_size_outputs(int64_t n_total, int32_t k, const lr_outputs *o
                              extras, k != 0);
   const bool spawn0 = u.spawn != 0 && u.xchg != 0 && !log0 && !extras;
   const bool ord0 = use_ord0(u, (uint64_t)n_total, log0, spawn0, extras, k != 0);
-  Plan p = make_plan((uint64_t)n_total, h, u, opts->wtype != LR_NONE,
+  Plan p = make_plan((uint64_t)n_total, h, u,
+                     opts->wtype != LR_NONE || (extras && (uint64_t)n_total <= u.base0),
                      opts->rtype == LR_I64 ? 8 : 4, opts->seed, 256 * 16, false, log0, extras,
                      extras && !outs->term, spawn0, ord0);
   return p.fixed_bytes + p.var_bytes;

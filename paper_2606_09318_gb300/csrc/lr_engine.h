@@ -12,6 +12,7 @@ namespace lr {
 
 struct Tuning {
   uint32_t f0_inv, f_inv, cutoff, block, ctas, xchg, chase0, algo, contract, spawn, ord, pf;
+  uint32_t base0, base;             // largest level 0 / deeper level that the base case ranks
 };
 
 struct Plan {
@@ -20,10 +21,9 @@ struct Plan {
   uint32_t cap[kMaxLevels + 1];
   uint32_t f_inv[kMaxLevels + 1];
   uint64_t seed[kMaxLevels + 1];
-  bool has_pd;
-  uint32_t pd_rounds;
+  uint64_t low[kMaxLevels + 1];     // least size of each level: its sampled rulers
   uint32_t hcap;                    // head-list capacity (bound on lists)
-  uint32_t cutoff;
+  uint32_t base;                    // largest level >= 1 that the base case ranks
   bool rec16_0;
   bool log0;                        // level 0 on the log path (lr_log.cu)
   int rank_bytes;
@@ -34,14 +34,14 @@ struct Plan {
   size_t fixed_bytes;
   // variable part
   size_t off_work[kMaxLevels + 1], off_R[kMaxLevels + 1];
-  size_t off_hA, off_hB, off_ns, off_pd[4];
+  size_t off_hA, off_hB, off_ns;
   uint32_t spawn_cap;               // ruler spawning at level 0: most spawned rulers (0: off)
   uint32_t raw_cap;                 //   ids of level 1 before compaction
   size_t off_sraw, off_sused, off_supre, off_sctr, off_srraw, spawn_zero;
   bool ord0;                        // level 0 chased in element order (a batch)
   size_t off_ord, off_cum;          // its ruler positions, rulers before every 256 positions
   bool term;                        // terminal ids carried through the levels
-  size_t off_T[kMaxLevels + 1], off_tid[kMaxLevels + 1], off_T0, off_hC, off_pdt[2];
+  size_t off_T[kMaxLevels + 1], off_tid[kMaxLevels + 1], off_T0, off_hC;
   size_t off_log, off_hdr, off_pairs, off_pairsB, off_cur;   // log path
   uint32_t total_chunks, shift;
   size_t cur_bytes;
@@ -82,6 +82,9 @@ bool tuned_lookup(int64_t n, bool weighted, bool batch, lr_tuning *out);
 Plan make_plan(uint64_t n, uint64_t h, const Tuning &u, bool rec16_0, int rank_bytes,
                uint64_t seed, int chase_grid, bool force_srs, bool log0, bool term = false,
                bool t0ws = false, bool spawn0 = false, bool ord0 = false);
+// Workspace that serves a single instance of any size up to n (lr_workspace_size
+// is for one size).
+size_t workspace_upto(int64_t n, const lr_opts *opts);
 int chase_grid_for(const Tuning &u, bool rec16, bool log0, bool ord0 = false);
 Ctx *get_ctx(cudaStream_t stream, lr_status *st);
 // Forget the context of a stream that is about to be destroyed (waits for

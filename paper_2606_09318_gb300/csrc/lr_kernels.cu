@@ -10,15 +10,15 @@
 //   chase      per level: one thread per ruler walks succ to the next ruler,
 //              rewriting each visited record as (ruler id, offset) and
 //              emitting one record of the reduced list (ruler chasing);
-//   base       single-CTA pointer doubling (Wyllie) once a level is small
-//              enough (the base case), or a grid-wide pointer-doubling
-//              fallback for a large last level;
+//   jump       pointer jumping over a whole level in one launch, once a level
+//              is small enough (the base case) or stops shrinking;
 //   finalize   per level, deepest first: R_l[i] = R_{l+1}[ruler(i)] - offset(i)
 //              (ruler propagation).
 // The chase records the *next* ruler, so ranks come out relative to the
 // terminal directly and the list never has to be reversed (Section 2.1 notes
 // that the distributed algorithm needs a reversal or the post-processing of
 // Section 2.5; walking succ forward from each ruler makes both unnecessary).
+#include <algorithm>
 #include <atomic>
 #include <cstdio>
 #include <cstring>
@@ -60,9 +60,9 @@ __global__ void k_init(LevelDesc *desc, InitParams p) {
     x.visited = 0;
     x.cap = p.cap[l];
     x.seed = p.seed[l];
-    x.rounds = p.pd_rounds;
     x.hsrc = l == 0 ? (uint32_t)kHeadsBitmap : (uint32_t)kHeadsList;
     x.nraw = 0;
+    x.check = 0;
     desc[l] = x;
   }
 }
@@ -88,7 +88,9 @@ __device__ __forceinline__ uint64_t load_weight(const void *w, uint32_t i) {
 // inclusively.
 // sums != nullptr: instead of the bitmap, accumulate the number of terminals
 // and the sum of the other successors (single-list head, see k_heads_single).
-template <int WT>
+// WIDE: 16-byte records (always when weighted; unweighted, weight 1, when the
+// level's records are to carry terminal ids).
+template <int WT, bool WIDE>
 __global__ void __launch_bounds__(256)
 k_prep0(const uint32_t *__restrict__ succ, const void *__restrict__ weight, uint32_t n,
         void *__restrict__ work, uint32_t *__restrict__ bitmap, uint32_t *__restrict__ err,
@@ -164,7 +166,7 @@ k_prep0(const uint32_t *__restrict__ succ, const void *__restrict__ weight, uint
         sT += 1;
       }
     }
-    if constexpr (WT == 0) {
+    if constexpr (!WIDE) {
       uint2 *out = reinterpret_cast<uint2 *>(work) + i0;
       if (cnt == 4u) {
         st_sector(out, s[0], kUnvisited, s[1], kUnvisited, s[2], kUnvisited, s[3], kUnvisited);
@@ -202,7 +204,7 @@ k_prep0(const uint32_t *__restrict__ succ, const void *__restrict__ weight, uint
 }
 
 cudaError_t launch_prep0(const uint32_t *succ, const void *weight, int wtype, uint32_t n,
-                         void *work, uint32_t *bitmap, uint32_t *err, int validate,
+                         void *work, bool rec16, uint32_t *bitmap, uint32_t *err, int validate,
                          const int64_t *offsets, int32_t k, unsigned long long *sums,
                          unsigned long long *local, cudaStream_t s) {
   if (n == 0) return cudaSuccess;
@@ -211,11 +213,14 @@ cudaError_t launch_prep0(const uint32_t *succ, const void *weight, int wtype, ui
   int vec = ((uintptr_t)succ & 15u) == 0;
   if (wtype == 1) vec = vec && ((uintptr_t)weight & 15u) == 0;
   if (wtype == 2) vec = vec && ((uintptr_t)weight & 15u) == 0;
+#define LR_PREP0(WT, WIDE) \
+  k_prep0<WT, WIDE><<<grid, block, 0, s>>>(succ, weight, n, work, bitmap, err, validate, vec, offsets, k, sums, local)
   switch (wtype) {
-    case 0: k_prep0<0><<<grid, block, 0, s>>>(succ, weight, n, work, bitmap, err, validate, vec, offsets, k, sums, local); break;
-    case 1: k_prep0<1><<<grid, block, 0, s>>>(succ, weight, n, work, bitmap, err, validate, vec, offsets, k, sums, local); break;
-    default: k_prep0<2><<<grid, block, 0, s>>>(succ, weight, n, work, bitmap, err, validate, vec, offsets, k, sums, local); break;
+    case 0: if (rec16) LR_PREP0(0, true); else LR_PREP0(0, false); break;
+    case 1: LR_PREP0(1, true); break;
+    default: LR_PREP0(2, true); break;
   }
+#undef LR_PREP0
   count_launch();
   return cudaGetLastError();
 }
@@ -758,7 +763,7 @@ k_heads_count(const LevelDesc *__restrict__ desc, int lev, const uint32_t *__res
 // Exclusive scan of the per-CTA counts; sizes of the next level; its mode.
 __global__ void __launch_bounds__(kHeadBlocks)
 k_heads_scan(LevelDesc *desc, int lev, int nlev, uint64_t *blockcnt, uint32_t *err,
-             uint32_t cutoff, uint32_t hcap, uint32_t has_pd) {
+             uint32_t cutoff, uint32_t hcap) {
   __shared__ uint64_t sm[33];
   if (desc[lev].mode != kModeSrs) return;
   uint64_t total;
@@ -772,10 +777,8 @@ k_heads_scan(LevelDesc *desc, int lev, int nlev, uint64_t *blockcnt, uint32_t *e
     const uint32_t hNext = (uint32_t)(total >> 32);
     const uint64_t n1 = (uint64_t)d.r + kNew;
     d.k = kNew;
-    bool bad = hNext > hcap || n1 > e.cap;
-    uint32_t mode = kModeSrs;
-    if (n1 <= cutoff) mode = kModeBase;
-    else if (lev + 1 >= nlev - 1) { if (has_pd) mode = kModePd; else bad = true; }
+    const bool bad = hNext > hcap || n1 > e.cap;
+    const uint32_t mode = n1 <= cutoff || lev + 1 >= nlev - 1 ? kModeBase : kModeSrs;
     if (bad) {
       record_error(err, kErrCapacity);
       d.mode = kModeOff;      // nothing more runs at this level or below
@@ -832,7 +835,7 @@ k_heads_write(LevelDesc *__restrict__ desc, int lev, const uint32_t *__restrict_
 cudaError_t launch_heads(LevelDesc *desc, int lev, int nlev, const uint32_t *bitmap,
                          const uint32_t *hlist, void *work, int rec_kind, uint32_t *ns,
                          uint32_t *hnext, uint64_t *blockcnt, uint32_t *err, uint32_t cutoff,
-                         uint32_t hcap, uint32_t has_pd, cudaStream_t s) {
+                         uint32_t hcap, cudaStream_t s) {
 #define LR_HEADS(KERNEL, REC, RES)                                                                \
   KERNEL<REC, RES><<<kHeadBlocks, kHeadThreads, 0, s>>>
   switch (rec_kind) {
@@ -846,7 +849,7 @@ cudaError_t launch_heads(LevelDesc *desc, int lev, int nlev, const uint32_t *bit
       LR_HEADS(k_heads_count, Succ4, false)(desc, lev, bitmap, hlist, reinterpret_cast<const Succ4 *>(work), blockcnt);
       break;
   }
-  k_heads_scan<<<1, kHeadBlocks, 0, s>>>(desc, lev, nlev, blockcnt, err, cutoff, hcap, has_pd);
+  k_heads_scan<<<1, kHeadBlocks, 0, s>>>(desc, lev, nlev, blockcnt, err, cutoff, hcap);
   switch (rec_kind) {
     case kRecKind8:
       LR_HEADS(k_heads_write, Rec8, true)(desc, lev, bitmap, hlist, reinterpret_cast<Rec8 *>(work), ns, hnext, blockcnt);
@@ -1309,7 +1312,7 @@ k_finalize(const LevelDesc *__restrict__ desc, int lev, const Rec *__restrict__ 
   if (d.mode != kModeSrs) return;
   const uint32_t n = d.n, nn = d.nraw ? d.nraw : desc[lev + 1].n;
   uint32_t bad = 0;
-  if (blockIdx.x == 0 && threadIdx.x == 0 && d.visited != n) bad |= kErrCycle;
+  if (blockIdx.x == 0 && threadIdx.x == 0) bad |= level_errors(d, desc[lev + 1], err);
   // each warp takes 128 consecutive elements at a time and lane l the
   // elements base + l + 32 j: every record load and rank store of the warp
   // is one contiguous run, and a lane's four gathers are in flight together
@@ -1346,7 +1349,7 @@ k_finalize_ptrs(const LevelDesc *__restrict__ desc, const Rec *__restrict__ work
   if (d.mode != kModeSrs) return;
   const uint32_t n = d.n, nn = desc[1].n;
   uint32_t bad = 0;
-  if (blockIdx.x == 0 && threadIdx.x == 0 && d.visited != n) bad |= kErrCycle;
+  if (blockIdx.x == 0 && threadIdx.x == 0) bad |= level_errors(d, desc[1], err);
   // each warp takes 128 consecutive elements (lane l: l + 32 j, coalesced
   // record loads and rank stores); the four records, then the four gathers
   // of the next level's ranks are in flight together, and the instances are
@@ -1438,7 +1441,7 @@ __device__ __forceinline__ uint32_t spawn_map(uint32_t c, uint32_t R, const uint
 __global__ void __launch_bounds__(1024)
 k_spawn_scan(LevelDesc *desc, int lev, int nlev, const uint32_t *__restrict__ ctr, uint32_t cap,
              const uint32_t *__restrict__ used, uint32_t *__restrict__ upre, uint32_t cutoff,
-             uint32_t has_pd, uint32_t *__restrict__ err) {
+             uint32_t *__restrict__ err) {
   __shared__ uint64_t sm[33];
   LevelDesc &d = desc[lev];
   if (d.mode != kModeSrs) return;
@@ -1457,12 +1460,9 @@ k_spawn_scan(LevelDesc *desc, int lev, int nlev, const uint32_t *__restrict__ ct
     const uint64_t n1 = R + total;
     d.nraw = (uint32_t)(R + handed);
     if (n1 > e.cap) { record_error(err, kErrCapacity); d.mode = kModeOff; return; }
-    uint32_t mode = kModeSrs;
-    if (n1 <= cutoff) mode = kModeBase;
-    else if (lev + 1 >= nlev - 1) { if (has_pd) mode = kModePd; else { record_error(err, kErrCapacity); d.mode = kModeOff; return; } }
     e.n = (uint32_t)n1;
     e.r = (uint32_t)((n1 + e.f_inv - 1) / e.f_inv);
-    e.mode = mode;
+    e.mode = n1 <= cutoff || lev + 1 >= nlev - 1 ? kModeBase : kModeSrs;
   }
 }
 
@@ -1497,9 +1497,8 @@ __global__ void k_spawn_scatter(const LevelDesc *__restrict__ desc, int lev, con
 
 cudaError_t launch_spawn_compact(LevelDesc *desc, int lev, int nlev, const uint32_t *ctr, uint32_t cap,
                                  const uint32_t *used, uint32_t *upre, const void *raw, void *out,
-                                 uint32_t raw_cap, uint32_t cutoff, uint32_t has_pd, uint32_t *err,
-                                 cudaStream_t s) {
-  k_spawn_scan<<<1, 1024, 0, s>>>(desc, lev, nlev, ctr, cap, used, upre, cutoff, has_pd, err);
+                                 uint32_t raw_cap, uint32_t cutoff, uint32_t *err, cudaStream_t s) {
+  k_spawn_scan<<<1, 1024, 0, s>>>(desc, lev, nlev, ctr, cap, used, upre, cutoff, err);
   k_spawn_compact<<<stream_grid(raw_cap, 256), 256, 0, s>>>(desc, lev, reinterpret_cast<const Rec16 *>(raw),
                                                            reinterpret_cast<Rec16 *>(out), used, upre);
   count_launch(2);
@@ -1596,191 +1595,203 @@ cudaError_t launch_outputs(const LevelDesc *desc, const uint32_t *bitmap, const 
 }
 
 // ---------------------------------------------------------------- base case
-// Pointer doubling (Wyllie) inside one CTA: nxt/val live in shared memory;
-// every round each element adds its successor's value and jumps to its
-// successor's successor, reading the old values before anyone writes.
-// Values are inclusive (a terminal starts with its own weight), so after
-// ceil(log2 n) rounds val[i] is the rank of i at this level.
-// With tout, term[] follows the same rounds: a terminal starts with its
-// original id (tid, or its own index at level 0) and every other element
-// with kEnd; an element takes its successor's entry, which is known exactly
-// when that successor has reached the end, i.e. when the element does.
-template <class Rec, class RT>
-__global__ void __launch_bounds__(kBaseThreads)
-k_base(LevelDesc *__restrict__ desc, int lev, const Rec *__restrict__ work, RT *__restrict__ rout,
-       uint32_t *__restrict__ err, const uint32_t *__restrict__ tid, uint32_t *__restrict__ tout) {
-  extern __shared__ unsigned char smem_raw[];
-  LevelDesc &d = desc[lev];
+// Ranks a whole level by pointer jumping over the level's own records, in one
+// launch and without barriers.  A record is the state of its element j:
+//   untouched  {succ, kUnvisited, w}     as the prep or the chase wrote it
+//              (succ == j marks a terminal, which weighs w);
+//   moved      {nxt, links, sum}         nxt lies `links` links further on and
+//              sum adds up the weights on the way;
+//   settled    {kEnd, terminal, rank}.
+// Each thread owns up to kJumpElems elements, holds their state in registers
+// and repeats: read the record of nxt, append it, publish the result.  Every
+// state of a record is a true statement about the list, and one access reads
+// or writes a whole record (8 or 16 bytes), so it does not matter how far the
+// others have come: where all advance together the pointers double, as in
+// rounds with a barrier after each, and where they have not run yet the walk
+// is slower but right.  Nobody waits for anybody.  An element appends at
+// least one link each time, so one that has gathered more links than the
+// level has elements is on a cycle (its links double too: some log2 n steps);
+// 8-byte records carry no count and need none, their sum being the count.
+//
+// What bounds it: the latency of log2 n dependent L2 reads below some 2^17
+// elements, the L2's rate of random reads above (n log2 n of them; the
+// stores are warp-contiguous).
+constexpr int kJumpThreads = 256;
+constexpr int kJumpElems = 4;
+constexpr int kJumpCtasPerSm = 4;
+
+template <class Rec>
+struct JumpState;
+
+template <>
+struct JumpState<Rec8> {
+  uint32_t nxt, sum;
+  __device__ __forceinline__ void load(const Rec8 *p) {
+    unsigned long long v;
+    asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    nxt = (uint32_t)v;
+    sum = (uint32_t)(v >> 32);
+  }
+  __device__ __forceinline__ void store(Rec8 *p) const {
+    const unsigned long long v = ((unsigned long long)sum << 32) | nxt;
+    asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" :: "l"(p), "l"(v) : "memory");
+  }
+  // own record: false when the element is a terminal (then settled)
+  __device__ __forceinline__ bool open(uint32_t self) {
+    sum = nxt == self ? 0u : 1u;
+    return nxt != self;
+  }
+  // append record q, read at a = nxt; true once the end of the list is reached
+  __device__ __forceinline__ bool append(const JumpState &q, uint32_t a, uint32_t n, uint32_t &bad) {
+    if (q.nxt == kEnd) { sum += q.sum; return true; }
+    if (q.nxt == a) return true;
+    sum += q.sum == kUnvisited ? 1u : q.sum;
+    nxt = q.nxt;
+    if (sum > n) { bad |= kErrCycle; return true; }
+    return false;
+  }
+  __device__ __forceinline__ void settle() { nxt = kEnd; }
+  __device__ __forceinline__ uint64_t rank() const { return sum; }
+  __device__ __forceinline__ uint32_t term() const { return kEnd; }
+};
+
+template <>
+struct JumpState<Rec16> {
+  uint32_t nxt, links;
+  uint64_t sum;
+  __device__ __forceinline__ void load(const Rec16 *p) {
+    unsigned long long lo, hi;
+    asm volatile("{\n\t.reg .b128 d;\n\tld.relaxed.gpu.global.b128 d, [%2];\n\tmov.b128 {%0, %1}, d;\n\t}"
+                 : "=l"(lo), "=l"(hi) : "l"(p) : "memory");
+    nxt = (uint32_t)lo;
+    links = (uint32_t)(lo >> 32);
+    sum = hi;
+  }
+  __device__ __forceinline__ void store(Rec16 *p) const {
+    const unsigned long long lo = ((unsigned long long)links << 32) | nxt, hi = sum;
+    asm volatile("{\n\t.reg .b128 d;\n\tmov.b128 d, {%1, %2};\n\tst.relaxed.gpu.global.b128 [%0], d;\n\t}"
+                 :: "l"(p), "l"(lo), "l"(hi) : "memory");
+  }
+  __device__ __forceinline__ bool open(uint32_t self) {
+    const bool inner = nxt != self;
+    links = inner ? 1u : self;                 // settled: the terminal
+    return inner;
+  }
+  __device__ __forceinline__ bool append(const JumpState &q, uint32_t a, uint32_t n, uint32_t &bad) {
+    sum += q.sum;
+    if (q.nxt == kEnd) { links = q.links; return true; }
+    if (q.nxt == a) { links = a; return true; }
+    const uint64_t l = (uint64_t)links + (q.links == kUnvisited ? 1u : q.links);
+    nxt = q.nxt;
+    links = (uint32_t)l;
+    if (l > n) { bad |= kErrCycle; links = kEnd; return true; }
+    return false;
+  }
+  __device__ __forceinline__ void settle() { nxt = kEnd; }
+  __device__ __forceinline__ uint64_t rank() const { return sum; }
+  __device__ __forceinline__ uint32_t term() const { return links; }
+};
+
+// A level below the first holds every element once among the successors of
+// its non-terminals and its heads, or some element has two predecessors.
+// Both sides are compared as sums of this hash (jump_check in LevelDesc,
+// examined by the propagation that reads the level's ranks).
+__device__ __forceinline__ uint64_t jump_hash(uint32_t x, uint64_t seed) {
+  return splitmix64(seed ^ ((uint64_t)x * 0xD1342543DE82EF95ull));
+}
+
+template <class Rec, class RT, bool TERM>
+__global__ void __launch_bounds__(kJumpThreads, kJumpCtasPerSm)
+k_jump(LevelDesc *__restrict__ desc, int lev, Rec *work, RT *__restrict__ rout, uint32_t *__restrict__ err,
+       const uint32_t *__restrict__ heads, const uint32_t *__restrict__ tid, uint32_t *__restrict__ tout) {
+  const LevelDesc d = desc[lev];
   if (d.mode != kModeBase) return;
   const uint32_t n = d.n;
-  const bool with_term = tout != nullptr;
-  uint32_t *nxt = reinterpret_cast<uint32_t *>(smem_raw);
-  RT *val = reinterpret_cast<RT *>(smem_raw + ((kMaxCutoff * 4 + 15) & ~15));
-  uint32_t *term = reinterpret_cast<uint32_t *>(reinterpret_cast<unsigned char *>(val) + (size_t)kMaxCutoff * sizeof(RT));
-  constexpr int PER = (kMaxCutoff + kBaseThreads - 1) / kBaseThreads;
-  for (uint32_t j = threadIdx.x; j < n; j += blockDim.x) {
-    Rec v = ld_rec(work + j);
-    const uint32_t s = rec_succ(v);
-    nxt[j] = (s == j || s >= n) ? kEnd : s;
-    val[j] = (RT)rec_weight(v, j);
-    if (with_term) term[j] = s == j ? (tid ? __ldcg(tid + j) : j) : kEnd;
-    if (s >= n) record_error(err, kErrInternal);
-  }
-  __syncthreads();
-  uint32_t rounds = 0;
-  while ((1ull << rounds) < n) ++rounds;
-  for (uint32_t it = 0; it < rounds; ++it) {
-    uint32_t tn[PER], tt[PER];
-    RT tv[PER];
-#pragma unroll
-    for (int e = 0; e < PER; ++e) {
-      const uint32_t j = threadIdx.x + e * kBaseThreads;
-      if (j < n) {
-        const uint32_t a = nxt[j];
-        if (a != kEnd) {
-          tv[e] = val[j] + val[a];
-          tn[e] = nxt[a];
-          tt[e] = with_term ? term[a] : 0u;
-        } else {
-          tv[e] = val[j];
-          tn[e] = kEnd;
-          tt[e] = with_term ? term[j] : 0u;
-        }
-      }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int e = 0; e < PER; ++e) {
-      const uint32_t j = threadIdx.x + e * kBaseThreads;
-      if (j < n) {
-        nxt[j] = tn[e];
-        val[j] = tv[e];
-        if (with_term) term[j] = tt[e];
-      }
-    }
-    __syncthreads();
-  }
+  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+  const uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
   uint32_t bad = 0;
-  for (uint32_t j = threadIdx.x; j < n; j += blockDim.x) {
-    if (nxt[j] != kEnd) bad = 1;
-    rout[j] = val[j];
-    if (with_term) tout[j] = term[j];
+  uint64_t chk = 0;
+  if (heads)
+    for (uint64_t e = t; e < d.h; e += stride) chk += jump_hash(__ldcg(heads + e), d.seed);
+  for (uint64_t base = t; base < n; base += stride * kJumpElems) {
+    JumpState<Rec> x[kJumpElems];
+    uint32_t pend = 0;                         // bit e: element e is not settled yet
+#pragma unroll
+    for (int e = 0; e < kJumpElems; ++e) {
+      const uint64_t i = base + stride * e;
+      if (i < n) x[e].load(work + i);
+    }
+#pragma unroll
+    for (int e = 0; e < kJumpElems; ++e) {
+      const uint64_t i = base + stride * e;
+      if (i >= n) continue;
+      const uint32_t s = x[e].nxt;
+      if (x[e].open((uint32_t)i)) {
+        if (s < n) pend |= 1u << e;
+        else bad |= kErrInternal;              // never written by a prep or a chase
+        if (heads) chk += jump_hash(s, d.seed);
+      }
+      if (heads) chk -= jump_hash((uint32_t)i, d.seed);
+    }
+    while (pend) {
+      JumpState<Rec> q[kJumpElems];
+#pragma unroll
+      for (int e = 0; e < kJumpElems; ++e)
+        if (pend >> e & 1u) q[e].load(work + x[e].nxt);
+#pragma unroll
+      for (int e = 0; e < kJumpElems; ++e) {
+        if (!(pend >> e & 1u)) continue;
+        const uint32_t self = (uint32_t)(base + stride * e);
+        bool done = x[e].append(q[e], x[e].nxt, n, bad);
+        if (!done && x[e].nxt >= n) { bad |= kErrInternal; done = true; }
+        // back at itself: a cycle (published, it would read as a terminal)
+        if (!done && x[e].nxt == self) { bad |= kErrCycle; done = true; }
+        if (done) {
+          x[e].settle();
+          pend &= ~(1u << e);
+        }
+        x[e].store(work + self);
+      }
+    }
+#pragma unroll
+    for (int e = 0; e < kJumpElems; ++e) {
+      const uint64_t i = base + stride * e;
+      if (i >= n) continue;
+      rout[i] = (RT)x[e].rank();
+      if constexpr (TERM) {
+        const uint32_t z = x[e].term();
+        tout[i] = z >= n ? kEnd : (tid ? __ldcg(tid + z) : z);
+      }
+    }
   }
-  if (bad) record_error(err, kErrCycle);
-  if (threadIdx.x == 0) d.visited = n;
+  if (bad) record_error(err, bad);
+  if (heads) {
+    for (int dd = 16; dd > 0; dd >>= 1) chk += __shfl_down_sync(0xFFFFFFFFu, chk, dd);
+    if ((threadIdx.x & 31) == 0 && chk) atomicAdd(&desc[lev].check, (unsigned long long)chk);
+  }
+  if (t == 0) desc[lev].visited = n;
 }
 
-static size_t base_smem(int rank_bytes) {
-  // nxt, val and the terminal ids of up to kMaxCutoff elements
-  return ((kMaxCutoff * 4 + 15) & ~15) + (size_t)kMaxCutoff * rank_bytes + (size_t)kMaxCutoff * 4;
-}
-
-cudaError_t launch_base(LevelDesc *desc, int lev, const void *work, bool rec16, void *rout,
-                        int rank_bytes, uint32_t cutoff, uint32_t *err, const uint32_t *tid,
+cudaError_t launch_jump(LevelDesc *desc, int lev, void *work, bool rec16, void *rout, int rank_bytes,
+                        uint32_t cap, uint32_t *err, const uint32_t *heads, const uint32_t *tid,
                         uint32_t *tout, cudaStream_t s) {
-  (void)cutoff;
-  const size_t sm = base_smem(rank_bytes);
-#define LR_BASE(REC, RT)                                                                         \
-  k_base<REC, RT><<<1, kBaseThreads, sm, s>>>(desc, lev, reinterpret_cast<const REC *>(work), \
-                                              reinterpret_cast<RT *>(rout), err, tid, tout)
-  if (rec16) { if (rank_bytes == 4) LR_BASE(Rec16, uint32_t); else LR_BASE(Rec16, unsigned long long); }
-  else { if (rank_bytes == 4) LR_BASE(Rec8, uint32_t); else LR_BASE(Rec8, unsigned long long); }
-#undef LR_BASE
+  const uint64_t ctas = ((uint64_t)cap + kJumpThreads - 1) / kJumpThreads;
+  const uint64_t full = (uint64_t)device_sm_count() * kJumpCtasPerSm;
+  const int grid = (int)std::max<uint64_t>(1, std::min(ctas, full));
+#define LR_JUMP(REC, RT, T)                                                                        \
+  k_jump<REC, RT, T><<<grid, kJumpThreads, 0, s>>>(desc, lev, reinterpret_cast<REC *>(work),       \
+                                                   reinterpret_cast<RT *>(rout), err, heads, tid, tout)
+  if (tout) {
+    if (!rec16) return cudaErrorInvalidValue;   // an 8-byte record has no room for the terminal
+    if (rank_bytes == 4) LR_JUMP(Rec16, uint32_t, true); else LR_JUMP(Rec16, unsigned long long, true);
+  } else if (rec16) {
+    if (rank_bytes == 4) LR_JUMP(Rec16, uint32_t, false); else LR_JUMP(Rec16, unsigned long long, false);
+  } else {
+    if (rank_bytes == 4) LR_JUMP(Rec8, uint32_t, false); else LR_JUMP(Rec8, unsigned long long, false);
+  }
+#undef LR_JUMP
   count_launch();
   return cudaGetLastError();
-}
-
-// ---------------------------------------------------------------- grid-wide pointer doubling
-// Fallback base case for a last level larger than one CTA can hold (many
-// lists whose heads keep the levels from shrinking).  Same rounds as the
-// single-CTA version, one kernel per round, ping-pong buffers.
-// With term arrays (t0/t1 non-null) the terminal ids follow the rounds as in
-// the single-CTA base case.
-__global__ void k_pd_init(const LevelDesc *__restrict__ desc, int lev, const Rec16 *__restrict__ work,
-                          uint32_t *__restrict__ nxt, uint64_t *__restrict__ val,
-                          const uint32_t *__restrict__ tid, uint32_t *__restrict__ term) {
-  const LevelDesc d = desc[lev];
-  if (d.mode != kModePd) return;
-  for (uint32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < d.n; j += gridDim.x * blockDim.x) {
-    Rec16 v = ld_rec(work + j);
-    nxt[j] = (v.succ == j || v.succ >= d.n) ? kEnd : v.succ;
-    val[j] = v.w;
-    if (term) term[j] = v.succ == j ? (tid ? __ldcg(tid + j) : j) : kEnd;
-  }
-}
-
-__global__ void k_pd_round(const LevelDesc *__restrict__ desc, int lev, const uint32_t *__restrict__ nin,
-                           const uint64_t *__restrict__ vin, uint32_t *__restrict__ nout,
-                           uint64_t *__restrict__ vout, const uint32_t *__restrict__ tin,
-                           uint32_t *__restrict__ tout) {
-  const LevelDesc d = desc[lev];
-  if (d.mode != kModePd) return;
-  for (uint32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < d.n; j += gridDim.x * blockDim.x) {
-    const uint32_t a = nin[j];
-    if (a != kEnd) {
-      vout[j] = vin[j] + vin[a];
-      nout[j] = nin[a];
-      if (tout) tout[j] = tin[a];
-    } else {
-      vout[j] = vin[j];
-      nout[j] = kEnd;
-      if (tout) tout[j] = tin[j];
-    }
-  }
-}
-
-template <class RT>
-__global__ void k_pd_out(LevelDesc *__restrict__ desc, int lev, const uint32_t *__restrict__ nxt,
-                         const uint64_t *__restrict__ val, RT *__restrict__ rout, uint32_t *__restrict__ err,
-                         const uint32_t *__restrict__ term, uint32_t *__restrict__ tout) {
-  const LevelDesc d = desc[lev];
-  if (d.mode != kModePd) return;
-  uint32_t bad = 0;
-  for (uint32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < d.n; j += gridDim.x * blockDim.x) {
-    bad |= nxt[j] != kEnd;
-    rout[j] = (RT)val[j];
-    if (tout) tout[j] = term[j];
-  }
-  if (bad) record_error(err, kErrCycle);
-  if (blockIdx.x == 0 && threadIdx.x == 0) desc[lev].visited = d.n;
-}
-
-cudaError_t launch_pd(LevelDesc *desc, int lev, const void *work, uint32_t cap, uint32_t rounds,
-                      uint32_t *nxt0, uint32_t *nxt1, uint64_t *val0, uint64_t *val1, void *rout,
-                      int rank_bytes, uint32_t *err, const uint32_t *tid, uint32_t *t0, uint32_t *t1,
-                      uint32_t *tout, cudaStream_t s) {
-  const int block = 256;
-  const int grid = stream_grid(cap, block);
-  if (!tout) t0 = t1 = nullptr;
-  k_pd_init<<<grid, block, 0, s>>>(desc, lev, reinterpret_cast<const Rec16 *>(work), nxt0, val0, tid, t0);
-  uint32_t *na = nxt0, *nb = nxt1, *ta = t0, *tb = t1;
-  uint64_t *va = val0, *vb = val1;
-  for (uint32_t it = 0; it < rounds; ++it) {
-    k_pd_round<<<grid, block, 0, s>>>(desc, lev, na, va, nb, vb, ta, tb);
-    uint32_t *tn = na; na = nb; nb = tn;
-    uint64_t *tv = va; va = vb; vb = tv;
-    uint32_t *tt = ta; ta = tb; tb = tt;
-  }
-  if (rank_bytes == 4)
-    k_pd_out<uint32_t><<<grid, block, 0, s>>>(desc, lev, na, va, reinterpret_cast<uint32_t *>(rout), err,
-                                              ta, tout);
-  else
-    k_pd_out<unsigned long long><<<grid, block, 0, s>>>(desc, lev, na, va,
-                                                        reinterpret_cast<unsigned long long *>(rout), err,
-                                                        ta, tout);
-  count_launch(2 + (int)rounds);
-  return cudaGetLastError();
-}
-
-cudaError_t kernels_setup() {
-  cudaError_t e;
-  e = cudaFuncSetAttribute(k_base<Rec8, uint32_t>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)base_smem(4));
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_base<Rec8, unsigned long long>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)base_smem(8));
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_base<Rec16, uint32_t>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)base_smem(4));
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(k_base<Rec16, unsigned long long>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)base_smem(8));
 }
 
 }  // namespace lr

@@ -15,12 +15,9 @@ struct InitParams {
   int32_t nlev;                       // levels in the plan (0..nlev-1)
   uint32_t n0;                        // elements at level 0
   uint32_t mode0;                     // kModeSrs or kModeBase
-  uint32_t cutoff;                    // base-case bound
   uint32_t f_inv[kMaxLevels + 1];
   uint32_t cap[kMaxLevels + 1];
   uint64_t seed[kMaxLevels + 1];
-  uint32_t pd_rounds;                 // rounds of the pointer-doubling fallback
-  uint32_t has_pd;                    // the last level may fall back to pointer doubling
   uint32_t hcap;                      // capacity of the head lists
 };
 
@@ -35,9 +32,10 @@ cudaError_t launch_init(LevelDesc *desc, const InitParams &p, cudaStream_t s);
 
 // Level-0 pass.  wtype 0/1/2 (none/i32/i64).  offsets != nullptr: batched
 // input with local successor ids (k instances).
+// rec16: 16-byte records (weighted input always has them).
 // local (optional): counts the links that stay inside their contraction tile.
 cudaError_t launch_prep0(const uint32_t *succ, const void *weight, int wtype, uint32_t n,
-                         void *work, uint32_t *bitmap, uint32_t *err, int validate,
+                         void *work, bool rec16, uint32_t *bitmap, uint32_t *err, int validate,
                          const int64_t *offsets, int32_t k, unsigned long long *sums,
                          unsigned long long *local, cudaStream_t s);
 
@@ -75,7 +73,7 @@ cudaError_t launch_local_sample(const uint32_t *succ, uint32_t n, unsigned long 
 cudaError_t launch_heads(LevelDesc *desc, int lev, int nlev, const uint32_t *bitmap,
                          const uint32_t *hlist, void *work, int rec_kind, uint32_t *ns,
                          uint32_t *hnext, uint64_t *blockcnt, uint32_t *err, uint32_t cutoff,
-                         uint32_t hcap, uint32_t has_pd, cudaStream_t s);
+                         uint32_t hcap, cudaStream_t s);
 
 // Terminal ids (all optional; null when the call does not ask for them):
 // tid_cur/tid_next hold the original id of each terminal of this/the next
@@ -105,8 +103,7 @@ struct OrdArgs {
 // ranked, scatter its ranks back to the original ids.
 cudaError_t launch_spawn_compact(LevelDesc *desc, int lev, int nlev, const uint32_t *ctr, uint32_t cap,
                                  const uint32_t *used, uint32_t *upre, const void *raw, void *out,
-                                 uint32_t raw_cap, uint32_t cutoff, uint32_t has_pd, uint32_t *err,
-                                 cudaStream_t s);
+                                 uint32_t raw_cap, uint32_t cutoff, uint32_t *err, cudaStream_t s);
 cudaError_t launch_spawn_scatter(LevelDesc *desc, int lev, const void *rc, void *rraw, int rank_bytes,
                                  const uint32_t *used, const uint32_t *upre, uint32_t raw_cap,
                                  cudaStream_t s);
@@ -127,14 +124,13 @@ cudaError_t launch_chase(LevelDesc *desc, int lev, void *work, bool rec16, void 
                          int xchg, const uint32_t *tid_cur, uint32_t *tid_next, const SpawnArgs *spawn,
                          const OrdArgs *ord, cudaStream_t s);
 
-cudaError_t launch_base(LevelDesc *desc, int lev, const void *work, bool rec16, void *rout,
-                        int rank_bytes, uint32_t cutoff, uint32_t *err, const uint32_t *tid,
+// Base case: rank level lev (at most cap elements) by pointer jumping in its
+// own records.  heads: the level's head list (levels >= 1), to detect two
+// predecessors; null at level 0.  tid / tout: terminal ids, 16-byte records
+// only.
+cudaError_t launch_jump(LevelDesc *desc, int lev, void *work, bool rec16, void *rout, int rank_bytes,
+                        uint32_t cap, uint32_t *err, const uint32_t *heads, const uint32_t *tid,
                         uint32_t *tout, cudaStream_t s);
-
-cudaError_t launch_pd(LevelDesc *desc, int lev, const void *work, uint32_t cap, uint32_t rounds,
-                      uint32_t *nxt0, uint32_t *nxt1, uint64_t *val0, uint64_t *val1, void *rout,
-                      int rank_bytes, uint32_t *err, const uint32_t *tid, uint32_t *t0, uint32_t *t1,
-                      uint32_t *tout, cudaStream_t s);
 
 // Level-0 extra outputs after the ranks and terminal ids are written:
 // prefix (head-relative) ranks, the inclusive-tail form, local terminal ids.
@@ -182,7 +178,6 @@ cudaError_t log_setup();
 int chase_log_occupancy(int block);
 
 int chase_occupancy(bool rec16, int block);
-cudaError_t kernels_setup();
 
 // Tile-local contraction (lr_contract.cu).
 uint32_t lc_tiles(uint64_t n);

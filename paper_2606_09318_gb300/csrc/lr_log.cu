@@ -642,7 +642,10 @@ k_win_scatter(const LevelDesc *__restrict__ desc, const uint2 *__restrict__ in, 
   if (threadIdx.x == 0) *s_count = 0;
   __syncthreads();
   uint32_t bad = 0, got = 0;
-  if (blockIdx.x == 0 && threadIdx.x == 0 && d.visited != n) bad |= d.visited > n ? kErrNotList : kErrCycle;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    if (d.visited != n) bad |= d.visited > n ? kErrNotList : kErrCycle;
+    bad |= merge_errors(desc[1], err);
+  }
   // a region holds whole quads of pairs (claims are multiples of four), 32-byte aligned
   const uint32_t nq = min(__ldcg(cur + blockIdx.x), cap) / 4;
   const uint4 *src = reinterpret_cast<const uint4 *>(in + (size_t)blockIdx.x * cap);
