@@ -76,6 +76,15 @@ static uint32_t default_f0_inv_batch(int64_t n) {
 // propagation) about 60 us less the smaller base case's 18.
 constexpr uint32_t kJumpMax = 3u << 17;
 
+// Largest level 0 that the base case ranks (k_jump needs no heads, no count of
+// the lists and so no wait, and no further launches, but reads n log2 n
+// records where the ruling set's chase reads n).  Random order, a whole call,
+// base case / ruling set: 131 thousand elements 70 / 145 us, 2^19 108 / 165,
+// 2^20 177 / 197, 1.5 million 226 / 211.  Beyond some 620 thousand elements
+// not all of them are held by running threads, which costs lists in memory
+// order most (1.5 million in locality order 467 / 143 us).
+constexpr uint32_t kBase0Max = 1u << 19;
+
 // Default ruler fraction below level 0: 1/4 where that already reaches the
 // base case (2^24, 10^6 rulers: 900 us a call at 1/4, 907 at 1/6, 912 at 1/8).
 static uint32_t default_f_inv(int64_t n, uint32_t f0_inv) {
@@ -96,7 +105,7 @@ Tuning resolve_tuning_builtin(int64_t n, bool weighted, bool batch) {
   u.contract = LR_CONTRACT_AUTO;
   u.spawn = 0;
   u.ord = 2;              // batches: every level of 2^20 or more in element order
-  u.base0 = kMaxCutoff;
+  u.base0 = kBase0Max;
   u.base = kJumpMax;
   u.pf = 4;               // ... prefetching its records 4K elements ahead of each draw
   return u;
@@ -142,7 +151,10 @@ Tuning resolve_tuning(const lr_tuning *t, int64_t n, bool weighted, bool batch) 
   u.f_inv = u.f_inv ? std::max<uint32_t>(2, u.f_inv) : default_f_inv(n, u.f0_inv);
   u.cutoff = std::min<uint32_t>(std::max<uint32_t>(u.cutoff, 64), kMaxCutoff);
   if (u.block != 128 && u.block != 256 && u.block != 512) u.block = 256;
-  u.base0 = u.cutoff;
+  // what asks for the ruling set itself keeps level 0 to it
+  const bool srs = u.cutoff < kMaxCutoff || u.spawn || u.chase0 != LR_CHASE0_AUTO || env_u32(env, "f0", 0) ||
+                   (t && t->f0_inv);
+  u.base0 = srs ? u.cutoff : kBase0Max;
   u.base = u.cutoff >= kMaxCutoff ? kJumpMax : u.cutoff;
   return u;
 }
@@ -195,8 +207,7 @@ static uint32_t spawn_capacity(uint64_t n, uint64_t threads) {
 }
 
 Plan make_plan(uint64_t n, uint64_t h, const Tuning &u, bool rec16_0, int rank_bytes,
-               uint64_t seed, int chase_grid, bool force_srs, bool log0, bool term, bool t0ws,
-               bool spawn0, bool ord0) {
+               uint64_t seed, int chase_grid, bool log0, bool term, bool t0ws, bool spawn0, bool ord0) {
   Plan p;
   memset(&p, 0, sizeof(p));
   p.n = n;
@@ -211,9 +222,9 @@ Plan make_plan(uint64_t n, uint64_t h, const Tuning &u, bool rec16_0, int rank_b
   p.f_inv[0] = u.f0_inv;
   int L = 0;
   p.low[0] = n;
-  const bool sp = spawn0 && (n > u.base0 || force_srs);
+  const bool sp = spawn0 && (n > u.base0);
   p.spawn_cap = sp ? spawn_capacity(n, (uint64_t)chase_grid * u.block) : 0;
-  if (n > u.base0 || force_srs) {
+  if (n > u.base0) {
     for (;;) {
       const uint64_t r = (p.cap[L] + p.f_inv[L] - 1) / p.f_inv[L];
       uint64_t nc = std::min<uint64_t>(p.cap[L], r + p.hcap);
@@ -590,7 +601,7 @@ static lr_status run_wyllie(const Inputs &in, Ctx *c, cudaStream_t s) {
   // without validation the scratch sums stand in for the bitmap, so the
   // pass issues no per-element atomics
   LR_TRY(launch_prep0(in.succ, in.weight, in.wtype, (uint32_t)in.n, A, w16, bitmap, err, in.validate,
-                      in.offsets, in.k, in.validate ? nullptr : sums, nullptr, s));
+                      in.offsets, in.k, in.validate ? nullptr : sums, nullptr, nullptr, nullptr, s));
   prof.mark(PH_PREP);
   LR_TRY(launch_wyllie(A, B, w16, (uint32_t)in.n, in.rank, in.rank_bytes, err, s));
   prof.mark(PH_BASE);
@@ -599,6 +610,69 @@ static lr_status run_wyllie(const Inputs &in, Ctx *c, cudaStream_t s) {
 }
 
 lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s);
+
+static InitParams init_params(const Plan &p) {
+  InitParams ip;
+  memset(&ip, 0, sizeof(ip));
+  ip.nlev = p.nlev;
+  ip.n0 = (uint32_t)p.n;
+  ip.mode0 = p.nlev == 1 ? kModeBase : kModeSrs;
+  for (int l = 0; l < p.nlev; ++l) {
+    ip.f_inv[l] = p.f_inv[l];
+    ip.cap[l] = p.cap[l];
+    ip.seed[l] = p.seed[l];
+  }
+  ip.hcap = p.hcap;
+  return ip;
+}
+
+// An input that the base case ranks as it is: one pass that packs the records,
+// then k_jump, which needs no heads.  From `checked` elements on (and for a
+// batch of separate buffers) two predecessors and a broken promise of
+// max_lists are looked for, as the ruling set notices them there.
+static lr_status run_base(const Inputs &in, const Plan &p, bool checked, char *fixed, char *var, Ctx *c,
+                          cudaStream_t s) {
+  const uint32_t n = (uint32_t)in.n;
+  const bool extras = p.term, marks = checked || in.validate || in.prefix != nullptr;
+  LevelDesc *desc = (LevelDesc *)(fixed + p.off_desc);
+  uint32_t *err = in.err_ext ? in.err_ext : (uint32_t *)(fixed + p.off_err);
+  uint32_t *bitmap = (uint32_t *)(fixed + p.off_bitmap);
+  void *work = fixed + p.off_work[0];
+  uint32_t *T0 = extras ? (in.term ? in.term : (uint32_t *)(var + p.off_T0)) : nullptr;
+  Profiler prof;
+  if (!in.ctx) prof.begin(s, (int64_t)in.n);
+  // the bitmap follows the words that start at zero
+  LR_TRY(cudaMemsetAsync(fixed + p.off_zero, 0,
+                         p.off_bitmap - p.off_zero + (marks ? 4 * (((size_t)n + 31) / 32) : 0), s));
+  const InitParams ip = init_params(p);
+  if (in.sptr) {
+    LR_TRY(launch_init(desc, ip, s));
+    LR_TRY(launch_prep0_ptrs(in.sptr, in.wptr, in.wtype, n, work, bitmap, err, 1, in.offsets, in.k, s));
+  } else {
+    LR_TRY(launch_prep0(in.succ, in.weight, in.wtype, n, work, p.rec16_0, marks ? bitmap : nullptr, err,
+                        checked || in.validate, in.offsets, in.k, nullptr, nullptr, desc, &ip, s));
+  }
+  if (!in.ctx) { c->last_desc = desc; c->last_nlev = 1; }
+  prof.mark(PH_PREP);
+  JumpInput ji;
+  memset(&ji, 0, sizeof(ji));
+  if (checked && in.max_lists > 0) {
+    ji.max_lists = (uint64_t)in.max_lists;
+    ji.bitmap = bitmap;
+    ji.count = (uint32_t *)(fixed + p.off_hcount);
+  }
+  ji.rptr = in.rptr;
+  ji.offsets = in.offsets;
+  ji.k = in.k;
+  LR_TRY(launch_jump(desc, 0, work, p.rec16_0, in.rank, p.rank_bytes, n, err, nullptr, nullptr, T0, &ji, s));
+  prof.mark(PH_BASE);
+  if (extras)
+    LR_TRY(launch_outputs(desc, bitmap, nullptr, n, T0, in.rank, in.prefix, p.rank_bytes, in.incl, in.weight,
+                          in.wtype, in.offsets, in.k, in.offsets != nullptr && in.term != nullptr, s));
+  prof.mark(PH_FINAL);
+  prof.end();
+  return finish_call(c, err, in.sync, s);
+}
 
 // Tile-local contraction (lr_contract.cu) around the ruling set: count the
 // local heads of every tile, build the contracted list, rank it (inclusive
@@ -717,14 +791,17 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
     const lr_status cs = run_contracted(in, tuning, c, true, s);
     if (cs != LR_ERR_NOT_FOUND) return cs;
   }
-  const bool count_local = contractible && u.contract == LR_CONTRACT_AUTO;
+  const bool count_local = contractible && u.contract == LR_CONTRACT_AUTO && in.n > u.base0;
   const int grid = chase_grid_for(u, rec16_0, log0, ord0);
-  const bool need_count = in.max_lists <= 0 && (in.ws == nullptr || in.count_in_ws) &&
-                          (in.n > u.base0 || ptrs);
-  if (need_count && capturing) return LR_ERR_CAPTURE;
+  // Counting the lists needs a wait.  The base case ranks level 0 without a
+  // count, but a call above the smallest sizes is not capturable without a
+  // promise of max_lists whichever way it is ranked.
+  const bool checked = in.n > u.cutoff || ptrs;
+  const bool may_count = in.max_lists <= 0 && (in.ws == nullptr || in.count_in_ws);
+  if (may_count && checked && capturing) return LR_ERR_CAPTURE;
+  const bool need_count = may_count && in.n > u.base0;
   uint64_t hb = in.max_lists > 0 ? (uint64_t)in.max_lists : in.n;
-  Plan p = make_plan(in.n, hb, u, rec16_0, in.rank_bytes, in.seed, grid, ptrs, log0, extras, t0ws, spawn0,
-                     ord0);
+  Plan p = make_plan(in.n, hb, u, rec16_0, in.rank_bytes, in.seed, grid, log0, extras, t0ws, spawn0, ord0);
 
   // fixed part (level 0)
   char *fixed = nullptr;
@@ -738,6 +815,14 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
     if (st != LR_OK) return st;
     fixed = (char *)c->fixed;
   }
+  if (p.nlev == 1) {
+    if (!in.ws) {
+      st = ensure_buffer(&c->var, &c->var_bytes, p.var_bytes, s);
+      if (st != LR_OK) return st;
+      var = (char *)c->var;
+    }
+    return run_base(in, p, checked, fixed, var, c, s);
+  }
   LevelDesc *desc = (LevelDesc *)(fixed + p.off_desc);
   uint32_t *err = in.err_ext ? in.err_ext : (uint32_t *)(fixed + p.off_err);
   uint32_t *hcount = (uint32_t *)(fixed + p.off_hcount);
@@ -748,13 +833,13 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
 
   // Single instance, no validation: heads from the streaming sums (one list)
   // with the bitmap as the fallback, instead of atomics for every element.
-  const bool sums0 = !log0 && !ptrs && in.offsets == nullptr && !in.validate && in.n > u.base0;
+  const bool sums0 = !log0 && !ptrs && in.offsets == nullptr && !in.validate;
   // A batch (contiguous or one pointer per instance): per-instance sums (kept
   // at the start of the bitmap's memory, which must hold 16 bytes per
   // instance) give one head per instance and the number of lists, with the
   // bitmap as the fallback for the heads.
   const bool sums0b = !log0 && in.offsets != nullptr && !in.validate && !extras && !spawn0 &&
-                      in.n > u.base0 && in.k > 0 && (uint64_t)in.k * 16 <= 4 * ((in.n + 31) / 32);
+                      in.k > 0 && (uint64_t)in.k * 16 <= 4 * ((in.n + 31) / 32);
   Profiler prof;
   if (!in.ctx) prof.begin(s, (int64_t)in.n);
   unsigned long long *acc = (unsigned long long *)(fixed + p.off_acc);
@@ -791,7 +876,7 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
                              reinterpret_cast<unsigned long long *>(bitmap), s));
   else
     LR_TRY(launch_prep0(in.succ, in.weight, in.wtype, (uint32_t)in.n, work0, rec16_0, bitmap, err,
-                        in.validate, in.offsets, in.k, sums0 ? acc : nullptr, nullptr, s));
+                        in.validate, in.offsets, in.k, sums0 ? acc : nullptr, nullptr, nullptr, nullptr, s));
   if (need_count) {
     // count the lists (one wait), then size the recursion for exactly that many:
     // a single-instance pass counts terminals in its reduction, a batch adds
@@ -820,8 +905,7 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
       }
     }
     hb = std::max<uint64_t>(1, c->host_words[1]);
-    p = make_plan(in.n, hb, u, rec16_0, in.rank_bytes, in.seed, grid, ptrs, log0, extras, t0ws, spawn0,
-                  ord0);
+    p = make_plan(in.n, hb, u, rec16_0, in.rank_bytes, in.seed, grid, log0, extras, t0ws, spawn0, ord0);
   }
   if (!in.ws) {
     st = ensure_buffer(&c->var, &c->var_bytes, p.var_bytes, s);
@@ -833,17 +917,7 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
   }
   prof.mark(PH_PREP);
 
-  InitParams ip;
-  memset(&ip, 0, sizeof(ip));
-  ip.nlev = p.nlev;
-  ip.n0 = (uint32_t)in.n;
-  ip.mode0 = p.nlev == 1 ? kModeBase : kModeSrs;
-  for (int l = 0; l < p.nlev; ++l) {
-    ip.f_inv[l] = p.f_inv[l];
-    ip.cap[l] = p.cap[l];
-    ip.seed[l] = p.seed[l];
-  }
-  ip.hcap = p.hcap;
+  const InitParams ip = init_params(p);
   LR_TRY(launch_init(desc, ip, s));
   if (!in.ctx) { c->last_desc = desc; c->last_nlev = p.nlev; }
   if (p.spawn_cap) LR_TRY(cudaMemsetAsync(var + p.off_sctr, 0, p.spawn_zero, s));
@@ -892,7 +966,7 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
     if (l > 0) {
       if (p.low[l] <= p.base) {
         LR_TRY(launch_jump(desc, l, work_of(l), r16, R_of(l), p.rank_bytes, p.cap[l], err, hin, tid_of(l),
-                           T_of(l), s));
+                           T_of(l), nullptr, s));
         prof.mark(PH_BASE);
       }
     }
@@ -927,8 +1001,8 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
     if (l == 0) prof.call.log0 = log0;
     prof.mark(l == 0 ? PH_CHASE0 : PH_CHASE);
   }
-  LR_TRY(launch_jump(desc, L, work_of(L), L > 0 || rec16_0, R_of(L), p.rank_bytes, p.cap[L], err,
-                     L > 0 ? head_list(L) : nullptr, tid_of(L), T_of(L), s));
+  LR_TRY(launch_jump(desc, L, work_of(L), true, R_of(L), p.rank_bytes, p.cap[L], err, head_list(L),
+                     tid_of(L), T_of(L), nullptr, s));
   prof.mark(PH_BASE);
   for (int l = L - 1; l >= 0; --l) {
     if (l == 0 && log0)
@@ -1337,7 +1411,7 @@ size_t lr_workspace_size_outputs(int64_t n_total, int32_t k, const lr_outputs *o
   const bool ord0 = use_ord0(u, (uint64_t)n_total, log0, spawn0, extras, k != 0);
   Plan p = make_plan((uint64_t)n_total, h, u,
                      opts->wtype != LR_NONE || (extras && (uint64_t)n_total <= u.base0),
-                     opts->rtype == LR_I64 ? 8 : 4, opts->seed, 256 * 16, false, log0, extras,
+                     opts->rtype == LR_I64 ? 8 : 4, opts->seed, 256 * 16, log0, extras,
                      extras && !outs->term, spawn0, ord0);
   return p.fixed_bytes + p.var_bytes;
 }

@@ -47,8 +47,7 @@ int stream_grid(uint64_t work_items, int block) {
 }
 
 // ---------------------------------------------------------------- init
-__global__ void k_init(LevelDesc *desc, InitParams p) {
-  const int l = threadIdx.x;
+__device__ __forceinline__ void init_levels(LevelDesc *desc, const InitParams &p, int l) {
   if (l < p.nlev) {
     LevelDesc x;
     x.mode = l == 0 ? p.mode0 : (uint32_t)kModeOff;
@@ -66,6 +65,8 @@ __global__ void k_init(LevelDesc *desc, InitParams p) {
     desc[l] = x;
   }
 }
+
+__global__ void k_init(LevelDesc *desc, InitParams p) { init_levels(desc, p, (int)threadIdx.x); }
 
 cudaError_t launch_init(LevelDesc *desc, const InitParams &p, cudaStream_t s) {
   k_init<<<1, 32, 0, s>>>(desc, p);
@@ -88,6 +89,8 @@ __device__ __forceinline__ uint64_t load_weight(const void *w, uint32_t i) {
 // inclusively.
 // sums != nullptr: instead of the bitmap, accumulate the number of terminals
 // and the sum of the other successors (single-list head, see k_heads_single).
+// Neither: an input small enough for the base case, which needs no heads.
+// desc != nullptr: also write the level descriptors (saves k_init's launch).
 // WIDE: 16-byte records (always when weighted; unweighted, weight 1, when the
 // level's records are to carry terminal ids).
 template <int WT, bool WIDE>
@@ -95,7 +98,9 @@ __global__ void __launch_bounds__(256)
 k_prep0(const uint32_t *__restrict__ succ, const void *__restrict__ weight, uint32_t n,
         void *__restrict__ work, uint32_t *__restrict__ bitmap, uint32_t *__restrict__ err,
         int validate, int vec, const int64_t *__restrict__ offsets, int32_t k,
-        unsigned long long *__restrict__ sums, unsigned long long *__restrict__ local) {
+        unsigned long long *__restrict__ sums, unsigned long long *__restrict__ local,
+        LevelDesc *__restrict__ desc, InitParams ip) {
+  if (desc && blockIdx.x == 0) init_levels(desc, ip, (int)threadIdx.x);
   unsigned long long sT = 0, sS = 0, sL = 0;
   const uint32_t ngroups = (uint32_t)(((uint64_t)n + 3u) / 4u);
   const uint32_t stride = gridDim.x * blockDim.x;
@@ -153,7 +158,7 @@ k_prep0(const uint32_t *__restrict__ succ, const void *__restrict__ weight, uint
       if (s[j] != i) {
         if (sums) {
           sS += s[j];
-        } else {
+        } else if (bitmap) {
           const uint32_t bit = 1u << (s[j] & 31u);
           if (validate) {
             if (atomicOr(bitmap + (s[j] >> 5), bit) & bit) record_error(err, kErrNotList);
@@ -206,15 +211,19 @@ k_prep0(const uint32_t *__restrict__ succ, const void *__restrict__ weight, uint
 cudaError_t launch_prep0(const uint32_t *succ, const void *weight, int wtype, uint32_t n,
                          void *work, bool rec16, uint32_t *bitmap, uint32_t *err, int validate,
                          const int64_t *offsets, int32_t k, unsigned long long *sums,
-                         unsigned long long *local, cudaStream_t s) {
+                         unsigned long long *local, LevelDesc *desc, const InitParams *init, cudaStream_t s) {
   if (n == 0) return cudaSuccess;
+  InitParams ip;
+  memset(&ip, 0, sizeof(ip));
+  if (desc) ip = *init;
   const int block = 256;
   const int grid = stream_grid(((uint64_t)n + 3) / 4, block);
   int vec = ((uintptr_t)succ & 15u) == 0;
   if (wtype == 1) vec = vec && ((uintptr_t)weight & 15u) == 0;
   if (wtype == 2) vec = vec && ((uintptr_t)weight & 15u) == 0;
 #define LR_PREP0(WT, WIDE) \
-  k_prep0<WT, WIDE><<<grid, block, 0, s>>>(succ, weight, n, work, bitmap, err, validate, vec, offsets, k, sums, local)
+  k_prep0<WT, WIDE><<<grid, block, 0, s>>>(succ, weight, n, work, bitmap, err, validate, vec, offsets, k, sums, local, \
+                                           desc, ip)
   switch (wtype) {
     case 0: if (rec16) LR_PREP0(0, true); else LR_PREP0(0, false); break;
     case 1: LR_PREP0(1, true); break;
@@ -1613,6 +1622,12 @@ cudaError_t launch_outputs(const LevelDesc *desc, const uint32_t *bitmap, const 
 // level has elements is on a cycle (its links double too: some log2 n steps);
 // 8-byte records carry no count and need none, their sum being the count.
 //
+// Warps take chunks of 32 consecutive elements in a random order.  In element
+// order, a list that follows memory would have the first threads walk link by
+// link through everything that does not run yet: 51 ms for 700 thousand
+// elements in locality order, where the grid holds 623 thousand at once (and
+// the same could happen when other kernels keep part of this grid waiting).
+//
 // What bounds it: the latency of log2 n dependent L2 reads below some 2^17
 // elements, the L2's rate of random reads above (n log2 n of them; the
 // stores are warp-contiguous).
@@ -1700,38 +1715,50 @@ __device__ __forceinline__ uint64_t jump_hash(uint32_t x, uint64_t seed) {
   return splitmix64(seed ^ ((uint64_t)x * 0xD1342543DE82EF95ull));
 }
 
-template <class Rec, class RT, bool TERM>
+// Level 0 (JumpInput): heads are not needed; with a bound on the lists, those
+// of two or more elements are counted from the has-predecessor bitmap.  PTRS:
+// ranks go to one buffer per instance.
+template <class Rec, class RT, bool TERM, bool PTRS>
 __global__ void __launch_bounds__(kJumpThreads, kJumpCtasPerSm)
 k_jump(LevelDesc *__restrict__ desc, int lev, Rec *work, RT *__restrict__ rout, uint32_t *__restrict__ err,
-       const uint32_t *__restrict__ heads, const uint32_t *__restrict__ tid, uint32_t *__restrict__ tout) {
+       const uint32_t *__restrict__ heads, const uint32_t *__restrict__ tid, uint32_t *__restrict__ tout,
+       JumpInput in) {
   const LevelDesc d = desc[lev];
   if (d.mode != kModeBase) return;
   const uint32_t n = d.n;
+  const uint32_t lane = threadIdx.x & 31u;
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   const uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  uint32_t bad = 0;
+  uint32_t bad = 0, lists = 0;
   uint64_t chk = 0;
   if (heads)
     for (uint64_t e = t; e < d.h; e += stride) chk += jump_hash(__ldcg(heads + e), d.seed);
-  for (uint64_t base = t; base < n; base += stride * kJumpElems) {
+  const uint32_t chunks = (uint32_t)(((uint64_t)n + 31u) / 32u), warps = (uint32_t)(stride >> 5);
+  Perm P;
+  P.init(chunks, d.seed);
+  for (uint64_t c0 = t >> 5; c0 < chunks; c0 += (uint64_t)warps * kJumpElems) {   // uniform in the warp
     JumpState<Rec> x[kJumpElems];
+    uint32_t idx[kJumpElems];                  // this lane's element of each chunk, or kEnd
     uint32_t pend = 0;                         // bit e: element e is not settled yet
 #pragma unroll
     for (int e = 0; e < kJumpElems; ++e) {
-      const uint64_t i = base + stride * e;
+      const uint64_t c = c0 + (uint64_t)warps * e;
+      const uint64_t i = c < chunks ? (uint64_t)P.fwd((uint32_t)c) * 32u + lane : n;
+      idx[e] = i < n ? (uint32_t)i : kEnd;
       if (i < n) x[e].load(work + i);
     }
 #pragma unroll
     for (int e = 0; e < kJumpElems; ++e) {
-      const uint64_t i = base + stride * e;
-      if (i >= n) continue;
+      const uint32_t i = idx[e];
+      if (i == kEnd) continue;
       const uint32_t s = x[e].nxt;
-      if (x[e].open((uint32_t)i)) {
+      if (x[e].open(i)) {
         if (s < n) pend |= 1u << e;
         else bad |= kErrInternal;              // never written by a prep or a chase
         if (heads) chk += jump_hash(s, d.seed);
+        if (in.max_lists) lists += !((__ldcg(in.bitmap + (i >> 5)) >> (i & 31u)) & 1u);
       }
-      if (heads) chk -= jump_hash((uint32_t)i, d.seed);
+      if (heads) chk -= jump_hash(i, d.seed);
     }
     while (pend) {
       JumpState<Rec> q[kJumpElems];
@@ -1741,7 +1768,7 @@ k_jump(LevelDesc *__restrict__ desc, int lev, Rec *work, RT *__restrict__ rout, 
 #pragma unroll
       for (int e = 0; e < kJumpElems; ++e) {
         if (!(pend >> e & 1u)) continue;
-        const uint32_t self = (uint32_t)(base + stride * e);
+        const uint32_t self = idx[e];
         bool done = x[e].append(q[e], x[e].nxt, n, bad);
         if (!done && x[e].nxt >= n) { bad |= kErrInternal; done = true; }
         // back at itself: a cycle (published, it would read as a terminal)
@@ -1753,41 +1780,70 @@ k_jump(LevelDesc *__restrict__ desc, int lev, Rec *work, RT *__restrict__ rout, 
         x[e].store(work + self);
       }
     }
+    if constexpr (PTRS) {
 #pragma unroll
-    for (int e = 0; e < kJumpElems; ++e) {
-      const uint64_t i = base + stride * e;
-      if (i >= n) continue;
-      rout[i] = (RT)x[e].rank();
-      if constexpr (TERM) {
-        const uint32_t z = x[e].term();
-        tout[i] = z >= n ? kEnd : (tid ? __ldcg(tid + z) : z);
+      for (int e = 0; e < kJumpElems; ++e) {
+        const uint32_t i = idx[e];
+        const uint32_t first = __shfl_sync(0xFFFFFFFFu, i, 0);
+        if (first == kEnd) continue;           // no such chunk (uniform in the warp)
+        int32_t lo = warp_instance(in.offsets, in.k, first, lane);
+        uint64_t ib = (uint64_t)__ldg(in.offsets + lo), ie = (uint64_t)__ldg(in.offsets + lo + 1);
+        if (i != kEnd) {
+          while (i >= ie && lo + 1 < in.k) { ++lo; ib = ie; ie = (uint64_t)__ldg(in.offsets + lo + 1); }
+          reinterpret_cast<RT *>(in.rptr[lo])[i - ib] = (RT)x[e].rank();
+        }
+      }
+    } else {
+#pragma unroll
+      for (int e = 0; e < kJumpElems; ++e) {
+        const uint32_t i = idx[e];
+        if (i == kEnd) continue;
+        rout[i] = (RT)x[e].rank();
+        if constexpr (TERM) {
+          const uint32_t z = x[e].term();
+          tout[i] = z >= n ? kEnd : (tid ? __ldcg(tid + z) : z);
+        }
       }
     }
+  }
+  if (in.max_lists) {
+    lists = __reduce_add_sync(0xFFFFFFFFu, lists);
+    if (lane == 0 && lists && (uint64_t)atomicAdd(in.count, lists) + lists > in.max_lists) bad |= kErrCapacity;
   }
   if (bad) record_error(err, bad);
   if (heads) {
     for (int dd = 16; dd > 0; dd >>= 1) chk += __shfl_down_sync(0xFFFFFFFFu, chk, dd);
-    if ((threadIdx.x & 31) == 0 && chk) atomicAdd(&desc[lev].check, (unsigned long long)chk);
+    if (lane == 0 && chk) atomicAdd(&desc[lev].check, (unsigned long long)chk);
   }
   if (t == 0) desc[lev].visited = n;
 }
 
 cudaError_t launch_jump(LevelDesc *desc, int lev, void *work, bool rec16, void *rout, int rank_bytes,
                         uint32_t cap, uint32_t *err, const uint32_t *heads, const uint32_t *tid,
-                        uint32_t *tout, cudaStream_t s) {
+                        uint32_t *tout, const JumpInput *input, cudaStream_t s) {
+  JumpInput in;
+  memset(&in, 0, sizeof(in));
+  if (input) in = *input;
   const uint64_t ctas = ((uint64_t)cap + kJumpThreads - 1) / kJumpThreads;
   const uint64_t full = (uint64_t)device_sm_count() * kJumpCtasPerSm;
   const int grid = (int)std::max<uint64_t>(1, std::min(ctas, full));
-#define LR_JUMP(REC, RT, T)                                                                        \
-  k_jump<REC, RT, T><<<grid, kJumpThreads, 0, s>>>(desc, lev, reinterpret_cast<REC *>(work),       \
-                                                   reinterpret_cast<RT *>(rout), err, heads, tid, tout)
+#define LR_JUMP(REC, T, P)                                                                             \
+  do {                                                                                                 \
+    if (rank_bytes == 4)                                                                               \
+      k_jump<REC, uint32_t, T, P><<<grid, kJumpThreads, 0, s>>>(                                       \
+          desc, lev, reinterpret_cast<REC *>(work), reinterpret_cast<uint32_t *>(rout), err, heads, tid, tout, in); \
+    else                                                                                               \
+      k_jump<REC, unsigned long long, T, P><<<grid, kJumpThreads, 0, s>>>(                             \
+          desc, lev, reinterpret_cast<REC *>(work), reinterpret_cast<unsigned long long *>(rout), err, heads, tid, \
+          tout, in);                                                                                   \
+  } while (0)
   if (tout) {
     if (!rec16) return cudaErrorInvalidValue;   // an 8-byte record has no room for the terminal
-    if (rank_bytes == 4) LR_JUMP(Rec16, uint32_t, true); else LR_JUMP(Rec16, unsigned long long, true);
-  } else if (rec16) {
-    if (rank_bytes == 4) LR_JUMP(Rec16, uint32_t, false); else LR_JUMP(Rec16, unsigned long long, false);
+    LR_JUMP(Rec16, true, false);
+  } else if (in.rptr) {
+    if (rec16) LR_JUMP(Rec16, false, true); else LR_JUMP(Rec8, false, true);
   } else {
-    if (rank_bytes == 4) LR_JUMP(Rec8, uint32_t, false); else LR_JUMP(Rec8, unsigned long long, false);
+    if (rec16) LR_JUMP(Rec16, false, false); else LR_JUMP(Rec8, false, false);
   }
 #undef LR_JUMP
   count_launch();

@@ -33,11 +33,14 @@ cudaError_t launch_init(LevelDesc *desc, const InitParams &p, cudaStream_t s);
 // Level-0 pass.  wtype 0/1/2 (none/i32/i64).  offsets != nullptr: batched
 // input with local successor ids (k instances).
 // rec16: 16-byte records (weighted input always has them).
+// sums: the number of terminals and the sum of the other successors instead
+// of predecessor marks in bitmap (which may be null then, and when neither is
+// wanted).  desc (optional): also writes the level descriptors from *init.
 // local (optional): counts the links that stay inside their contraction tile.
 cudaError_t launch_prep0(const uint32_t *succ, const void *weight, int wtype, uint32_t n,
                          void *work, bool rec16, uint32_t *bitmap, uint32_t *err, int validate,
                          const int64_t *offsets, int32_t k, unsigned long long *sums,
-                         unsigned long long *local, cudaStream_t s);
+                         unsigned long long *local, LevelDesc *desc, const InitParams *init, cudaStream_t s);
 
 // Batched prep that sums each instance's terminals and local successors
 // (isums[2k], zeroed) instead of marking predecessors; then the level-0 head
@@ -124,13 +127,26 @@ cudaError_t launch_chase(LevelDesc *desc, int lev, void *work, bool rec16, void 
                          int xchg, const uint32_t *tid_cur, uint32_t *tid_next, const SpawnArgs *spawn,
                          const OrdArgs *ord, cudaStream_t s);
 
+// What the base case needs to rank level 0 itself (all optional): the most
+// lists of two or more elements the caller promised (0: any number), counted
+// from the has-predecessor bitmap into *count (zeroed); one rank buffer per
+// instance.
+struct JumpInput {
+  uint64_t max_lists;
+  const uint32_t *bitmap;
+  uint32_t *count;
+  void *const *rptr;
+  const int64_t *offsets;
+  int32_t k;
+};
+
 // Base case: rank level lev (at most cap elements) by pointer jumping in its
 // own records.  heads: the level's head list (levels >= 1), to detect two
 // predecessors; null at level 0.  tid / tout: terminal ids, 16-byte records
 // only.
 cudaError_t launch_jump(LevelDesc *desc, int lev, void *work, bool rec16, void *rout, int rank_bytes,
                         uint32_t cap, uint32_t *err, const uint32_t *heads, const uint32_t *tid,
-                        uint32_t *tout, cudaStream_t s);
+                        uint32_t *tout, const JumpInput *input, cudaStream_t s);
 
 // Level-0 extra outputs after the ranks and terminal ids are written:
 // prefix (head-relative) ranks, the inclusive-tail form, local terminal ids.

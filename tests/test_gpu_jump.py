@@ -83,3 +83,64 @@ def test_two_lists_that_merge(seed):
     for f0 in (2, 8):
         assert status_of(succ, tuning=lr.Tuning(f0_inv=f0)) == "LR_ERR_NOT_A_LIST"
         assert status_of(succ, tuning=lr.Tuning(f0_inv=f0), validate=True) == "LR_ERR_NOT_A_LIST"
+
+
+# ---- level 0 ranked by the base case itself (no ruling set), and its limits
+@pytest.mark.parametrize("n", [12289, 40_001, 1 << 19, (1 << 19) + 1])
+@pytest.mark.parametrize("kind", ["random", "locality", "identity", "forest"])
+def test_level0_equals_the_oracle(n, kind):
+    if kind == "forest":
+        succ, nl = gen.forest(n, 7500 + n, n_long=2, long_len=n // 8, mean_short=9)
+    else:
+        succ, nl = gen.list_of_order_kind(kind, n, 7500 + n), 1
+    w = gen.weights_i32(n, 7501)
+    want, want_t, want_p = oracle.rank_ext(succ, w, np.int64)
+    np.testing.assert_array_equal(lr.rank(dev(succ), validate=True).cpu().numpy(), oracle.rank(succ))
+    np.testing.assert_array_equal(lr.rank(dev(succ), dev(w), max_lists=nl).cpu().numpy(), want)
+    for weight in (None, dev(w)):                     # 8- and 16-byte records, the latter with terminals
+        r, t, p = lr.rank_outputs(dev(succ), weight, term=True, prefix=weight is not None)
+        np.testing.assert_array_equal(t.cpu().numpy().view(np.uint32), want_t)
+    np.testing.assert_array_equal(r.cpu().numpy(), want)
+    np.testing.assert_array_equal(p.cpu().numpy(), want_p)
+
+
+@pytest.mark.parametrize("total_exp", [8.0, 13.0, 15.0])
+@pytest.mark.parametrize("wt", [None, "i64"])
+def test_batches_at_level0(total_exp, wt):
+    k = 24
+    lens = np.floor(2.0 ** gen.rng(int(total_exp)).uniform(0, total_exp, size=k)).astype(np.int64)
+    lens[[0, 7, 23]] = 0
+    offsets = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    lists = [gen.random_list(int(m), 7600 + j) if m else np.zeros(0, np.uint32) for j, m in enumerate(lens)]
+    succ = np.concatenate(lists).astype(np.uint32)
+    w = gen.weights_i64(succ.shape[0], 7601) if wt else None
+    rt = np.int64 if wt else np.int32
+    want = oracle.rank_batch(offsets, succ, w, rt)
+    for ml in (0, k):
+        got = lr.rank_batch(dev(offsets), dev(succ), None if w is None else dev(w), max_lists=ml)
+        np.testing.assert_array_equal(got.cpu().numpy(), want)
+        parts = lr.rank_batch_ptrs([dev(a) for a in lists],
+                                   None if w is None else [dev(w[a:b]) for a, b in zip(offsets, offsets[1:])],
+                                   max_lists=ml)
+        np.testing.assert_array_equal(np.concatenate([q.cpu().numpy() for q in parts]), want)
+
+
+@pytest.mark.parametrize("n", [4097, 12288, 12289, 200_003])
+def test_promised_lists_and_capture(n):
+    succ, nl = gen.forest(n, 7700, n_long=1, long_len=n // 4, mean_short=16)
+    want = oracle.rank(succ)
+    np.testing.assert_array_equal(lr.rank(dev(succ), max_lists=nl).cpu().numpy(), want)
+    if n <= 12288:                                    # the smallest sizes never counted lists
+        np.testing.assert_array_equal(lr.rank(dev(succ), max_lists=1).cpu().numpy(), want)
+    else:
+        assert status_of(succ, max_lists=nl // 4) == "LR_ERR_CAPACITY"
+    s, out, side = dev(succ), torch.empty(n, dtype=torch.int32, device="cuda"), torch.cuda.Stream()
+    lr.rank(s, out=out, max_lists=nl, stream=side)
+    out.zero_()
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=side):
+        lr.rank(s, out=out, max_lists=nl, sync=False)
+    g.replay()
+    torch.cuda.synchronize()
+    np.testing.assert_array_equal(out.cpu().numpy(), want)
