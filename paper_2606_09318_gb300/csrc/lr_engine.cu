@@ -341,7 +341,8 @@ lr_status setup_device_once() {
   if (e != cudaSuccess) return from_cuda(e);
   std::lock_guard<std::mutex> g(g_mu);
   if (dev >= 0 && dev < 64 && !g_setup_done[dev]) {
-    e = log_setup();
+    e = small_setup();
+    if (e == cudaSuccess) e = log_setup();
     if (e == cudaSuccess) e = lc_setup();
     if (e != cudaSuccess) return from_cuda(e);
     // Place lr_rank_noalloc's scratch array on this device now, while the
@@ -541,9 +542,10 @@ static lr_status map_device_bits(uint32_t bits) {
   } while (0)
 
 // Copy the call's device error word to the context's pinned status word;
-// with sync, wait and return the status it encodes.
+// with sync, wait and return the status it encodes.  err == nullptr: a kernel
+// has written the status word itself.
 static lr_status finish_call(Ctx *c, const uint32_t *err, int sync, cudaStream_t s) {
-  LR_TRY(cudaMemcpyAsync(c->host_words, err, 4, cudaMemcpyDeviceToHost, s));
+  if (err) LR_TRY(cudaMemcpyAsync(c->host_words, err, 4, cudaMemcpyDeviceToHost, s));
   c->pending_status = true;
   if (sync) {
     LR_TRY(cudaStreamSynchronize(s));
@@ -641,6 +643,17 @@ static lr_status run_base(const Inputs &in, const Plan &p, bool checked, char *f
   uint32_t *T0 = extras ? (in.term ? in.term : (uint32_t *)(var + p.off_T0)) : nullptr;
   Profiler prof;
   if (!in.ctx) prof.begin(s, (int64_t)in.n);
+  // (a context passed in, or a shared error word, has no status word of its
+  // own that the device can write)
+  if (n <= small_max() && !in.sptr && !in.offsets && !extras && !in.ctx && !in.err_ext) {
+    LR_TRY(launch_small(in.succ, in.weight, in.wtype, n, in.rank, p.rank_bytes, in.validate, desc, init_params(p),
+                        c->host_words, s));
+    c->last_desc = desc;
+    c->last_nlev = 1;
+    prof.mark(PH_BASE);
+    prof.end();
+    return finish_call(c, nullptr, in.sync, s);
+  }
   // the bitmap follows the words that start at zero
   LR_TRY(cudaMemsetAsync(fixed + p.off_zero, 0,
                          p.off_bitmap - p.off_zero + (marks ? 4 * (((size_t)n + 31) / 32) : 0), s));

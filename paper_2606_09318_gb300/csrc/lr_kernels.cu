@@ -1850,4 +1850,125 @@ cudaError_t launch_jump(LevelDesc *desc, int lev, void *work, bool rec16, void *
   return cudaGetLastError();
 }
 
+// ---------------------------------------------------------------- small lists
+// A single list or forest of at most kSmallMax elements, whole call in one
+// launch: one CTA reads the successors, doubles pointers in shared memory and
+// writes the ranks, and the status straight to the host's status word.  At
+// these sizes a call is all latency: as a clear, a packing pass, k_jump and a
+// status copy it took 54 us at n = 1000, of which the kernels were 16.
+//
+// One 32-bit word holds an element's pointer and the links up to it,
+// links << 16 | settled | pointer; the settled bit is set once the pointer is
+// a terminal and travels with it.  A round adds the word (weighted: and the
+// sum) of the element pointed to, from one buffer into the other; a list
+// settles in log2 n rounds, a cycle never does.
+constexpr uint32_t kSmallMax = 4096;
+constexpr int kSmallThreads = 1024;
+constexpr int kSmallElems = (int)kSmallMax / kSmallThreads;
+constexpr uint32_t kSmallSettled = 0x8000u, kSmallPtr = kSmallMax - 1u;
+constexpr int kSmallRounds = 13;               // links double each round: 2^13 fits their 16 bits
+
+template <int WT, class RT>
+__global__ void __launch_bounds__(kSmallThreads)
+k_small(const uint32_t *__restrict__ succ, const void *__restrict__ weight, uint32_t n, RT *__restrict__ rank,
+        int validate, LevelDesc *__restrict__ desc, InitParams ip, uint32_t *__restrict__ status) {
+  extern __shared__ __align__(16) unsigned char small_smem[];
+  __shared__ uint32_t s_bad, s_pred[kSmallMax / 32];
+  init_levels(desc, ip, (int)threadIdx.x);
+  RT *sum = reinterpret_cast<RT *>(small_smem);                                    // [2][n], weighted only
+  uint32_t *word = reinterpret_cast<uint32_t *>(small_smem + (WT ? 2 * n * sizeof(RT) : 0));   // [2][n]
+  if (threadIdx.x == 0) s_bad = 0;
+  for (uint32_t w = threadIdx.x; w < kSmallMax / 32; w += blockDim.x) s_pred[w] = 0;
+  __syncthreads();
+  uint32_t x[kSmallElems], bad = 0;
+  RT v[kSmallElems];
+#pragma unroll
+  for (int e = 0; e < kSmallElems; ++e) {
+    const uint32_t j = threadIdx.x + e * blockDim.x;
+    x[e] = kSmallSettled;
+    v[e] = 0;
+    if (j >= n) continue;
+    const uint32_t s = __ldg(succ + j);
+    const bool inner = s != j && s < n;
+    if (s >= n) bad |= kErrRange;
+    x[e] = inner ? 1u << 16 | s : kSmallSettled | j;
+    word[j] = x[e];
+    if constexpr (WT != 0) {
+      v[e] = inner ? (RT)load_weight<WT>(weight, j) : (RT)0;
+      sum[j] = v[e];
+    }
+    if (validate && inner && (atomicOr(&s_pred[s >> 5], 1u << (s & 31u)) >> (s & 31u) & 1u)) bad |= kErrNotList;
+  }
+  __syncthreads();
+  uint32_t b = 0, all;
+  for (int round = 0; round < kSmallRounds; ++round) {
+    const uint32_t *wcur = word + b * n;
+    const RT *scur = sum + b * n;
+    uint32_t *wnxt = word + (b ^ 1u) * n;
+    RT *snxt = sum + (b ^ 1u) * n;
+    all = kSmallSettled;
+#pragma unroll
+    for (int e = 0; e < kSmallElems; ++e) {
+      const uint32_t j = threadIdx.x + e * blockDim.x;
+      if (j >= n) continue;
+      if (!(x[e] & kSmallSettled)) {
+        const uint32_t a = x[e] & kSmallPtr;
+        x[e] = (x[e] & 0xFFFF0000u) + wcur[a];
+        if constexpr (WT != 0) v[e] += scur[a];
+      }
+      all &= x[e];
+      wnxt[j] = x[e];
+      if constexpr (WT != 0) snxt[j] = v[e];
+    }
+    b ^= 1u;
+    if (__syncthreads_and((all & kSmallSettled) != 0)) break;
+  }
+#pragma unroll
+  for (int e = 0; e < kSmallElems; ++e) {
+    const uint32_t j = threadIdx.x + e * blockDim.x;
+    if (j >= n) continue;
+    if (!(x[e] & kSmallSettled)) bad |= kErrCycle;
+    rank[j] = WT != 0 ? v[e] : (RT)(x[e] >> 16);
+  }
+  if (bad) atomicOr(&s_bad, bad);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    *status = s_bad;
+    desc[0].visited = n;
+  }
+}
+
+uint32_t small_max() { return kSmallMax; }
+
+cudaError_t small_setup() {
+  const int most = 2 * kSmallMax * (8 + 4);
+  cudaError_t e = cudaFuncSetAttribute(k_small<1, uint32_t>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_small<1, unsigned long long>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_small<2, uint32_t>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_small<2, unsigned long long>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  return e;
+}
+
+cudaError_t launch_small(const uint32_t *succ, const void *weight, int wtype, uint32_t n, void *rank, int rank_bytes,
+                         int validate, LevelDesc *desc, const InitParams &ip, uint32_t *status, cudaStream_t s) {
+  if (n == 0 || n > kSmallMax) return cudaErrorInvalidValue;
+  const int block = (int)std::min<uint32_t>(kSmallThreads, (n + 31u) / 32u * 32u);
+  const size_t smem = 2 * (size_t)n * (4 + (wtype ? rank_bytes : 0));
+#define LR_SMALL(W)                                                                                             \
+  do {                                                                                                          \
+    if (rank_bytes == 4)                                                                                        \
+      k_small<W, uint32_t><<<1, block, smem, s>>>(succ, weight, n, reinterpret_cast<uint32_t *>(rank), validate, desc, \
+                                                  ip, status);                                                  \
+    else                                                                                                        \
+      k_small<W, unsigned long long><<<1, block, smem, s>>>(                                                    \
+          succ, weight, n, reinterpret_cast<unsigned long long *>(rank), validate, desc, ip, status);           \
+  } while (0)
+  if (wtype == 0) LR_SMALL(0);
+  else if (wtype == 1) LR_SMALL(1);
+  else LR_SMALL(2);
+#undef LR_SMALL
+  count_launch();
+  return cudaGetLastError();
+}
+
 }  // namespace lr

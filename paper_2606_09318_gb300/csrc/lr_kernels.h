@@ -148,6 +148,13 @@ cudaError_t launch_jump(LevelDesc *desc, int lev, void *work, bool rec16, void *
                         uint32_t cap, uint32_t *err, const uint32_t *heads, const uint32_t *tid,
                         uint32_t *tout, const JumpInput *input, cudaStream_t s);
 
+// A single instance of at most small_max() elements in one launch, ranks and
+// all; the error bits go to *status (host memory the device can write).
+uint32_t small_max();
+cudaError_t small_setup();
+cudaError_t launch_small(const uint32_t *succ, const void *weight, int wtype, uint32_t n, void *rank, int rank_bytes,
+                         int validate, LevelDesc *desc, const InitParams &ip, uint32_t *status, cudaStream_t s);
+
 // Level-0 extra outputs after the ranks and terminal ids are written:
 // prefix (head-relative) ranks, the inclusive-tail form, local terminal ids.
 cudaError_t launch_outputs(const LevelDesc *desc, const uint32_t *bitmap, const uint32_t *hlist0,

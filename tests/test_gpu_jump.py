@@ -144,3 +144,31 @@ def test_promised_lists_and_capture(n):
     g.replay()
     torch.cuda.synchronize()
     np.testing.assert_array_equal(out.cpu().numpy(), want)
+
+
+# ---- the one-launch path of short lists (k_small) and the size above it
+@pytest.mark.parametrize("n", [1, 2, 31, 32, 33, 1023, 1024, 1025, 4095, 4096, 4097])
+@pytest.mark.parametrize("wt,rt", [(None, np.int32), (None, np.int64), (np.int32, np.int64), (np.int64, np.int32)])
+def test_short_lists(n, wt, rt):
+    trt = torch.int32 if rt == np.int32 else torch.int64
+    for succ in (gen.random_list(n, 7800 + n), gen.identity_list(n), np.arange(n, dtype=np.uint32)):
+        w = None
+        if wt is not None:
+            info = np.iinfo(wt)
+            w = gen.rng(n).integers(info.min, info.max, size=n, dtype=wt, endpoint=True)
+        want = oracle.rank(succ, w, rt)
+        dw = None if w is None else dev(w)
+        np.testing.assert_array_equal(lr.rank(dev(succ), dw, rank_dtype=trt, validate=True).cpu().numpy(), want)
+        assert lr.level_sizes() == [n]
+        np.testing.assert_array_equal(lr.rank(dev(succ), dw, rank_dtype=trt, sync=False).cpu().numpy(), want)
+        assert lr.device_status() == 0
+    if n > 1:
+        cyc = np.roll(np.arange(n, dtype=np.uint32), -1)          # one ring
+        assert status_of(cyc) == "LR_ERR_CYCLE"
+        out = gen.random_list(n, 7801)
+        out[0] = n
+        assert status_of(out) == "LR_ERR_OUT_OF_RANGE"
+        star = np.zeros(n, dtype=np.uint32)                       # everybody before element 0
+        assert status_of(star, validate=True) == ("LR_ERR_NOT_A_LIST" if n > 2 else "LR_OK")
+        lr.rank(dev(cyc), sync=False)
+        assert lr.status_string(lr.device_status()) == "LR_ERR_CYCLE"
