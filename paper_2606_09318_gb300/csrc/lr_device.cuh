@@ -63,6 +63,7 @@ struct LevelDesc {
   uint32_t cap;      // static: capacity of this level's arrays
   uint64_t seed;     // static: permutation seed
   uint32_t hsrc;     // where this level's heads come from: kHeadsBitmap or kHeadsList
+  uint32_t picked;   // this level's rulers were chosen with its descriptor (a single head)
   uint32_t nraw;     // with spawning: ruler ids of the next level before compaction (else 0)
   unsigned long long check;  // base case: nonzero when an element has two predecessors (k_jump)
 };

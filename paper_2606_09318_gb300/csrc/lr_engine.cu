@@ -185,6 +185,9 @@ static size_t align_up(size_t x, size_t a = 256) { return (x + a - 1) / a * a; }
 // width (threads x ruler spacing) must stay small enough that the instances
 // it crosses fit in L2; more threads only queue at the memory system.
 constexpr int kOrdCtasPerSm = 4;
+// Below this size the packing pass counts the links that stay in their tiles
+// itself, instead of a sample and a wait of its own before it.
+constexpr uint64_t kPackFirst = 1ull << 22;
 // Deeper levels of a batch keep each instance's rulers together too; from
 // this size on they are chased in order as well (LR_TUNING ord=1: level 0
 // only; ord=0: no level).
@@ -625,6 +628,7 @@ static InitParams init_params(const Plan &p) {
     ip.seed[l] = p.seed[l];
   }
   ip.hcap = p.hcap;
+  ip.base = p.base;
   return ip;
 }
 
@@ -659,7 +663,7 @@ static lr_status run_base(const Inputs &in, const Plan &p, bool checked, char *f
                          p.off_bitmap - p.off_zero + (marks ? 4 * (((size_t)n + 31) / 32) : 0), s));
   const InitParams ip = init_params(p);
   if (in.sptr) {
-    LR_TRY(launch_init(desc, ip, s));
+    LR_TRY(launch_init(desc, ip, nullptr, nullptr, nullptr, nullptr, s));
     LR_TRY(launch_prep0_ptrs(in.sptr, in.wptr, in.wtype, n, work, bitmap, err, 1, in.offsets, in.k, s));
   } else {
     LR_TRY(launch_prep0(in.succ, in.weight, in.wtype, n, work, p.rec16_0, marks ? bitmap : nullptr, err,
@@ -856,13 +860,19 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
   Profiler prof;
   if (!in.ctx) prof.begin(s, (int64_t)in.n);
   unsigned long long *acc = (unsigned long long *)(fixed + p.off_acc);
-  LR_TRY(cudaMemsetAsync(fixed + p.off_zero, 0, p.zero_bytes, s));
+  const size_t bitmap_bytes = sizeof(uint32_t) * ((in.n + 31) / 32);
+  // A single instance needs the bitmap only if it turns out not to be one
+  // list; otherwise it is cleared here with the words that start at zero,
+  // which it follows.
+  const bool late_bitmap = (log0 || sums0) && need_count && !in.validate;
+  LR_TRY(cudaMemsetAsync(fixed + p.off_zero, 0, p.zero_bytes + (late_bitmap ? 0 : bitmap_bytes), s));
   // A first pass that packs records (the exchange form) would pack them in
-  // vain for an input that is then contracted: decide from a sample of the
-  // tiles first.  (The log form's first pass only reads succ, and counts
-  // every tile on the way.)
-  const bool local_exact = count_local && log0;
-  if (count_local && !log0) {
+  // vain for an input that is then contracted: from kPackFirst elements on,
+  // decide from a sample of the tiles first.  (The log form's first pass only
+  // reads succ, and counts every tile on the way; a shorter list is packed
+  // sooner than the wait for the sample takes.)
+  const bool local_exact = count_local && (log0 || (sums0 && in.n < kPackFirst));
+  if (count_local && !local_exact) {
     LR_TRY(launch_local_sample(in.succ, (uint32_t)in.n, acc + 2, s));
     LR_TRY(cudaMemcpyAsync(c->host_words + 4, acc + 2, 16, cudaMemcpyDeviceToHost, s));
     LR_TRY(cudaStreamSynchronize(s));
@@ -875,7 +885,6 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
       prof.begin(s, (int64_t)in.n);            // not contracted after all: carry on
     }
   }
-  LR_TRY(cudaMemsetAsync(bitmap, 0, sizeof(uint32_t) * ((in.n + 31) / 32), s));
   if (log0)
     LR_TRY(launch_sum0(in.succ, (uint32_t)in.n, acc, local_exact ? acc + 2 : nullptr, err, s));
   else if (ptrs && sums0b)
@@ -889,14 +898,17 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
                              reinterpret_cast<unsigned long long *>(bitmap), s));
   else
     LR_TRY(launch_prep0(in.succ, in.weight, in.wtype, (uint32_t)in.n, work0, rec16_0, bitmap, err,
-                        in.validate, in.offsets, in.k, sums0 ? acc : nullptr, nullptr, nullptr, nullptr, s));
+                        in.validate, in.offsets, in.k, sums0 ? acc : nullptr,
+                        sums0 && local_exact ? acc + 2 : nullptr, nullptr, nullptr, s));
+  bool one_list = false;                       // the host has seen that level 0 is one list
   if (need_count) {
     // count the lists (one wait), then size the recursion for exactly that many:
     // a single-instance pass counts terminals in its reduction, a batch adds
     // its instances' terminal counts, the other passes count zero bits of the
     // has-predecessor bitmap
+    uint64_t sums[3];                          // terminals, other successors, local links
     if (log0 || sums0) {
-      LR_TRY(cudaMemcpyAsync(c->host_words + 1, acc, 4, cudaMemcpyDeviceToHost, s));
+      LR_TRY(cudaMemcpyAsync(c->host_words + 4, acc, sizeof(sums), cudaMemcpyDeviceToHost, s));
     } else if (sums0b) {
       LR_TRY(launch_count_batch(reinterpret_cast<const unsigned long long *>(bitmap), in.k, hcount, s));
       LR_TRY(cudaMemcpyAsync(c->host_words + 1, hcount, 4, cudaMemcpyDeviceToHost, s));
@@ -904,13 +916,14 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
       LR_TRY(launch_count_heads(bitmap, (uint32_t)in.n, hcount, s));
       LR_TRY(cudaMemcpyAsync(c->host_words + 1, hcount, 4, cudaMemcpyDeviceToHost, s));
     }
-    if (local_exact)
-      LR_TRY(cudaMemcpyAsync(c->host_words + 2, acc + 2, 8, cudaMemcpyDeviceToHost, s));
     LR_TRY(cudaStreamSynchronize(s));
+    if (log0 || sums0) {
+      memcpy(sums, c->host_words + 4, sizeof(sums));
+      c->host_words[1] = (uint32_t)sums[0];
+      one_list = late_bitmap && sums[0] == 1 && in.n * (in.n - 1) / 2 - sums[1] < in.n;
+    }
     if (local_exact) {
-      uint64_t local_links;
-      memcpy(&local_links, c->host_words + 2, 8);
-      if (local_links * 2 >= in.n) {           // at least half the links stay in their tile
+      if (sums[2] * 2 >= in.n) {           // at least half the links stay in their tile
         prof.cancel();
         const lr_status cs = run_contracted(in, tuning, c, false, s);
         if (cs != LR_ERR_NOT_FOUND) return cs;
@@ -930,8 +943,12 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
   }
   prof.mark(PH_PREP);
 
-  const InitParams ip = init_params(p);
-  LR_TRY(launch_init(desc, ip, s));
+  uint32_t *hA = (uint32_t *)(var + p.off_hA);
+  uint32_t *hB = (uint32_t *)(var + p.off_hB);
+  uint32_t *hC = extras ? (uint32_t *)(var + p.off_hC) : hA;
+  uint32_t *ns = (uint32_t *)(var + p.off_ns);
+  const bool acc_heads = (log0 || sums0) && !in.validate;
+  LR_TRY(launch_init(desc, init_params(p), acc_heads ? acc : nullptr, hA, ns, hB, s));
   if (!in.ctx) { c->last_desc = desc; c->last_nlev = p.nlev; }
   if (p.spawn_cap) LR_TRY(cudaMemsetAsync(var + p.off_sctr, 0, p.spawn_zero, s));
   SpawnArgs spa;
@@ -942,15 +959,15 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
     spa.used = (uint32_t *)(var + p.off_sused);
     spa.cursor = (uint32_t *)(var + p.off_sctr + 16);
   }
-  uint32_t *hA0 = (uint32_t *)(var + p.off_hA);
   if (log0) {
     LR_TRY(cudaMemsetAsync(var + p.off_hdr, 0xFF, (size_t)p.total_chunks * 8, s));
     LR_TRY(cudaMemsetAsync(var + p.off_cur, 0, p.cur_bytes, s));
   }
-  if (log0 || sums0)
-    LR_TRY(launch_heads0_log(desc, acc, hA0, in.succ, (uint32_t)in.n, bitmap, err, in.validate, s));
-  else if (sums0b)
-    LR_TRY(launch_heads0_batch(desc, reinterpret_cast<unsigned long long *>(bitmap), in.offsets, in.k, hA0,
+  if ((log0 || sums0) && !one_list) {
+    if (late_bitmap) LR_TRY(cudaMemsetAsync(bitmap, 0, bitmap_bytes, s));
+    LR_TRY(launch_bitmap0(desc, in.succ, (uint32_t)in.n, bitmap, err, in.validate, s));
+  } else if (sums0b)
+    LR_TRY(launch_heads0_batch(desc, reinterpret_cast<unsigned long long *>(bitmap), in.offsets, in.k, hA,
                                p.hcap, work0, rec16_0, (uint32_t)in.n, bitmap, s));
 
   auto work_of = [&](int l) -> void * { return l == 0 ? work0 : (void *)(var + p.off_work[l]); };
@@ -965,10 +982,6 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
   auto tid_of = [&](int l) -> uint32_t * {
     return (extras && l > 0) ? (uint32_t *)(var + p.off_tid[l]) : nullptr;
   };
-  uint32_t *hA = (uint32_t *)(var + p.off_hA);
-  uint32_t *hB = (uint32_t *)(var + p.off_hB);
-  uint32_t *hC = extras ? (uint32_t *)(var + p.off_hC) : hA;
-  uint32_t *ns = (uint32_t *)(var + p.off_ns);
   // head lists alternate between buffers; with extra outputs level 0's list
   // (hA) stays intact for the prefix pass
   auto head_list = [&](int l) -> uint32_t * { return l == 0 ? hA : ((l & 1) ? hB : hC); };
@@ -984,7 +997,8 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
       }
     }
     const int kind = (l == 0 && log0) ? kRecKindSucc : (r16 ? kRecKind16 : kRecKind8);
-    LR_TRY(launch_heads(desc, l, p.nlev, bitmap, hin, (l == 0 && log0) ? (void *)in.succ : work_of(l),
+    if (l > 0 || !one_list)
+      LR_TRY(launch_heads(desc, l, p.nlev, bitmap, hin, (l == 0 && log0) ? (void *)in.succ : work_of(l),
                         kind, ns, hout, bcnt, err, p.base, p.hcap, s));
     prof.mark(PH_SELECT);
     if (l == 0 && log0)
@@ -1037,7 +1051,7 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
                              p.rank_bytes, p.cap[l], err, T_of(l + 1), T_of(l), tid_of(l), s));
   }
   if (extras)
-    LR_TRY(launch_outputs(desc, bitmap, hA0, (uint32_t)in.n, T0, in.rank, in.prefix, p.rank_bytes,
+    LR_TRY(launch_outputs(desc, bitmap, hA, (uint32_t)in.n, T0, in.rank, in.prefix, p.rank_bytes,
                           in.incl, in.weight, in.wtype, in.offsets, in.k,
                           in.offsets != nullptr && in.term != nullptr, s));
   prof.mark(PH_FINAL);

@@ -60,16 +60,52 @@ __device__ __forceinline__ void init_levels(LevelDesc *desc, const InitParams &p
     x.cap = p.cap[l];
     x.seed = p.seed[l];
     x.hsrc = l == 0 ? (uint32_t)kHeadsBitmap : (uint32_t)kHeadsList;
+    x.picked = 0;
     x.nraw = 0;
     x.check = 0;
     desc[l] = x;
   }
 }
 
-__global__ void k_init(LevelDesc *desc, InitParams p) { init_levels(desc, p, (int)threadIdx.x); }
+// Size, rulers and mode of the level below one with r sampled and k extra
+// rulers, of which `heads` are heads.
+__device__ __forceinline__ void open_level(LevelDesc &e, uint64_t n1, uint32_t heads, bool last, uint32_t base) {
+  e.n = (uint32_t)n1;
+  e.r = (uint32_t)((n1 + e.f_inv - 1) / e.f_inv);
+  e.h = heads;
+  e.mode = n1 <= base || last ? kModeBase : kModeSrs;
+}
 
-cudaError_t launch_init(LevelDesc *desc, const InitParams &p, cudaStream_t s) {
-  k_init<<<1, 32, 0, s>>>(desc, p);
+// One warp: the descriptors; and with a single list (one terminal, and the
+// other successors are every id but the head's) its head and level 0's choice
+// of rulers, which otherwise takes five more launches.
+__global__ void __launch_bounds__(32)
+k_init(LevelDesc *desc, InitParams p, const unsigned long long *__restrict__ acc, uint32_t *__restrict__ hlist0,
+       uint32_t *__restrict__ ns, uint32_t *__restrict__ hnext) {
+  init_levels(desc, p, (int)threadIdx.x);
+  __syncwarp();
+  if (threadIdx.x != 0 || !acc || p.nlev < 2) return;
+  LevelDesc &d = desc[0];
+  const unsigned long long n = p.n0, h = n * (n - 1) / 2 - acc[1];
+  if (acc[0] != 1 || h >= n) return;
+  hlist0[0] = (uint32_t)h;
+  d.h = 1;
+  d.hsrc = kHeadsList;
+  Perm P;
+  P.init(p.n0, p.seed[0]);
+  const uint32_t id = P.fwd((uint32_t)h);
+  const uint32_t r = (uint32_t)((n + p.f_inv[0] - 1) / p.f_inv[0]);
+  const bool sampled = id < r;
+  if (!sampled) ns[0] = (uint32_t)h;
+  hnext[0] = sampled ? id : r;
+  d.k = sampled ? 0u : 1u;
+  d.picked = 1u;
+  open_level(desc[1], (uint64_t)r + d.k, 1u, p.nlev == 2, p.base);
+}
+
+cudaError_t launch_init(LevelDesc *desc, const InitParams &p, const unsigned long long *acc, uint32_t *hlist0,
+                        uint32_t *ns, uint32_t *hnext, cudaStream_t s) {
+  k_init<<<1, 32, 0, s>>>(desc, p, acc, hlist0, ns, hnext);
   count_launch();
   return cudaGetLastError();
 }
@@ -88,7 +124,7 @@ __device__ __forceinline__ uint64_t load_weight(const void *w, uint32_t i) {
 // weight is stored as 0, so every deeper computation can treat weights
 // inclusively.
 // sums != nullptr: instead of the bitmap, accumulate the number of terminals
-// and the sum of the other successors (single-list head, see k_heads_single).
+// and the sum of the other successors (single-list head, see k_init).
 // Neither: an input small enough for the base case, which needs no heads.
 // desc != nullptr: also write the level descriptors (saves k_init's launch).
 // WIDE: 16-byte records (always when weighted; unweighted, weight 1, when the
@@ -753,7 +789,7 @@ k_heads_count(const LevelDesc *__restrict__ desc, int lev, const uint32_t *__res
               uint64_t *__restrict__ blockcnt) {
   __shared__ uint64_t sm[33];
   const LevelDesc d = desc[lev];
-  if (d.mode != kModeSrs) return;
+  if (d.mode != kModeSrs || d.picked) return;
   Perm P;
   P.init(d.n, d.seed);
   uint32_t nS = 0, nN = 0;
@@ -774,7 +810,7 @@ __global__ void __launch_bounds__(kHeadBlocks)
 k_heads_scan(LevelDesc *desc, int lev, int nlev, uint64_t *blockcnt, uint32_t *err,
              uint32_t cutoff, uint32_t hcap) {
   __shared__ uint64_t sm[33];
-  if (desc[lev].mode != kModeSrs) return;
+  if (desc[lev].mode != kModeSrs || desc[lev].picked) return;
   uint64_t total;
   const uint64_t v = blockcnt[threadIdx.x];
   const uint64_t ex = block_exclusive_scan(v, sm, &total);
@@ -786,17 +822,12 @@ k_heads_scan(LevelDesc *desc, int lev, int nlev, uint64_t *blockcnt, uint32_t *e
     const uint32_t hNext = (uint32_t)(total >> 32);
     const uint64_t n1 = (uint64_t)d.r + kNew;
     d.k = kNew;
-    const bool bad = hNext > hcap || n1 > e.cap;
-    const uint32_t mode = n1 <= cutoff || lev + 1 >= nlev - 1 ? kModeBase : kModeSrs;
-    if (bad) {
+    if (hNext > hcap || n1 > e.cap) {
       record_error(err, kErrCapacity);
       d.mode = kModeOff;      // nothing more runs at this level or below
       return;
     }
-    e.n = (uint32_t)n1;
-    e.r = (uint32_t)((n1 + e.f_inv - 1) / e.f_inv);
-    e.h = hNext;
-    e.mode = mode;
+    open_level(e, n1, hNext, lev + 1 >= nlev - 1, cutoff);
   }
 }
 
@@ -808,7 +839,7 @@ k_heads_write(LevelDesc *__restrict__ desc, int lev, const uint32_t *__restrict_
               const uint64_t *__restrict__ blockoff) {
   __shared__ uint64_t sm[33];
   const LevelDesc d = desc[lev];
-  if (d.mode != kModeSrs) return;
+  if (d.mode != kModeSrs || d.picked) return;
   Perm P;
   P.init(d.n, d.seed);
   uint32_t nS = 0, nN = 0;
@@ -841,10 +872,65 @@ k_heads_write(LevelDesc *__restrict__ desc, int lev, const uint32_t *__restrict_
   if ((threadIdx.x & 31) == 0 && nZ) atomicAdd(&desc[lev].visited, nZ);
 }
 
+// The same for a level whose few heads come as a list: one CTA, one launch.
+constexpr uint32_t kFewHeads = 2048;
+template <class Rec>
+__global__ void __launch_bounds__(1024)
+k_heads_few(LevelDesc *desc, int lev, int nlev, const uint32_t *__restrict__ hlist, Rec *__restrict__ work,
+            uint32_t *__restrict__ ns, uint32_t *__restrict__ hnext, uint32_t *__restrict__ err, uint32_t cutoff,
+            uint32_t hcap) {
+  __shared__ uint64_t sm[33];
+  const LevelDesc d = desc[lev];
+  if (d.mode != kModeSrs || d.picked) return;
+  Perm P;
+  P.init(d.n, d.seed);
+  uint32_t nN = 0, nH = 0, nZ = 0;               // extra rulers, heads below, resolved so far
+  for (uint32_t e0 = 0; e0 < d.h; e0 += blockDim.x) {
+    const uint32_t e = e0 + threadIdx.x;
+    uint32_t x = 0, p = 0;
+    uint64_t w = 0;
+    int c = -1;
+    if (e < d.h) {
+      x = __ldcg(hlist + e);
+      c = classify_head<Rec, true>(x, P, d.r, work, &p, &w);
+    }
+    const bool isnew = c == kCatNew, ishead = isnew || c == kCatSampled;
+    uint64_t total;
+    const uint64_t at = block_exclusive_scan(((uint64_t)ishead << 32) | (isnew ? 1u : 0u), sm, &total);
+    const uint32_t posN = nN + (uint32_t)at, posH = nH + (uint32_t)(at >> 32);
+    // (the list itself is no longer than hcap, and so is what it leaves)
+    if (ishead && posH < hcap) hnext[posH] = isnew ? d.r + posN : p;
+    if (isnew && posN < hcap) ns[posN] = x;
+    if (c == kCatSingle) st_rec(work + x, kZeroCid, (uint64_t)0 - w);
+    nZ += __syncthreads_count(c == kCatSingle);
+    nN += (uint32_t)total;
+    nH += (uint32_t)(total >> 32);
+  }
+  if (threadIdx.x == 0) {
+    LevelDesc &m = desc[lev];
+    LevelDesc &e = desc[lev + 1];
+    const uint64_t n1 = (uint64_t)d.r + nN;
+    m.k = nN;
+    m.visited += nZ;
+    if (nH > hcap || n1 > e.cap) {
+      record_error(err, kErrCapacity);
+      m.mode = kModeOff;
+      return;
+    }
+    open_level(e, n1, nH, lev + 1 >= nlev - 1, cutoff);
+  }
+}
+
 cudaError_t launch_heads(LevelDesc *desc, int lev, int nlev, const uint32_t *bitmap,
                          const uint32_t *hlist, void *work, int rec_kind, uint32_t *ns,
                          uint32_t *hnext, uint64_t *blockcnt, uint32_t *err, uint32_t cutoff,
                          uint32_t hcap, cudaStream_t s) {
+  if (lev > 0 && hcap <= kFewHeads) {
+    k_heads_few<Rec16><<<1, 1024, 0, s>>>(desc, lev, nlev, hlist, reinterpret_cast<Rec16 *>(work), ns, hnext, err,
+                                          cutoff, hcap);
+    count_launch();
+    return cudaGetLastError();
+  }
 #define LR_HEADS(KERNEL, REC, RES)                                                                \
   KERNEL<REC, RES><<<kHeadBlocks, kHeadThreads, 0, s>>>
   switch (rec_kind) {

@@ -19,6 +19,7 @@ struct InitParams {
   uint32_t cap[kMaxLevels + 1];
   uint64_t seed[kMaxLevels + 1];
   uint32_t hcap;                      // capacity of the head lists
+  uint32_t base;                      // largest level >= 1 that the base case ranks
 };
 
 // Kernel launch counter (all streams).
@@ -28,7 +29,12 @@ int64_t launch_count();
 int device_sm_count();
 int stream_grid(uint64_t work_items, int block);
 
-cudaError_t launch_init(LevelDesc *desc, const InitParams &p, cudaStream_t s);
+// Level descriptors.  acc (optional): the terminals and the sum of the other
+// successors of a single instance; where they show one list, its head goes to
+// hlist0 and level 0's rulers are chosen on the spot (ns, hnext: see
+// launch_heads, which then does nothing).
+cudaError_t launch_init(LevelDesc *desc, const InitParams &p, const unsigned long long *acc, uint32_t *hlist0,
+                        uint32_t *ns, uint32_t *hnext, cudaStream_t s);
 
 // Level-0 pass.  wtype 0/1/2 (none/i32/i64).  offsets != nullptr: batched
 // input with local successor ids (k instances).
@@ -179,9 +185,9 @@ cudaError_t launch_finalize(LevelDesc *desc, int lev, const void *work, bool rec
 constexpr uint32_t kLogWindow = 32;
 cudaError_t launch_sum0(const uint32_t *succ, uint32_t n, unsigned long long *acc, unsigned long long *local,
                         uint32_t *err, cudaStream_t s);
-cudaError_t launch_heads0_log(LevelDesc *desc, const unsigned long long *acc, uint32_t *hlist0,
-                              const uint32_t *succ, uint32_t n, uint32_t *bitmap, uint32_t *err,
-                              int validate, cudaStream_t s);
+// The has-predecessor bitmap (zeroed), unless launch_init found a single head.
+cudaError_t launch_bitmap0(const LevelDesc *desc, const uint32_t *succ, uint32_t n, uint32_t *bitmap, uint32_t *err,
+                           int validate, cudaStream_t s);
 cudaError_t launch_chase_log(LevelDesc *desc, const uint32_t *succ, void *next_work, const uint32_t *ns,
                              uint32_t *qctr, int grid, int block, uint32_t *err, uint32_t *log,
                              uint2 *hdr, uint32_t total_chunks, uint32_t *ctr, cudaStream_t s);

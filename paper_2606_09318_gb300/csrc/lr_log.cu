@@ -89,22 +89,6 @@ cudaError_t launch_sum0(const uint32_t *succ, uint32_t n, unsigned long long *ac
   return cudaGetLastError();
 }
 
-// One thread: the single head, or a switch to the bitmap.
-__global__ void k_heads_single(LevelDesc *desc, const unsigned long long *acc, uint32_t *hlist0,
-                               int validate) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  LevelDesc &d = desc[0];
-  const unsigned long long n = d.n;
-  const unsigned long long h = n * (n - 1) / 2 - acc[1];
-  if (!validate && acc[0] == 1 && h < n) {
-    hlist0[0] = (uint32_t)h;
-    d.h = 1;
-    d.hsrc = kHeadsList;
-  } else {
-    d.hsrc = kHeadsBitmap;
-  }
-}
-
 // Has-predecessor bitmap, only when the single-head shortcut does not apply.
 __global__ void __launch_bounds__(256)
 k_bitmap0(const LevelDesc *__restrict__ desc, const uint32_t *__restrict__ succ, uint32_t n,
@@ -122,12 +106,10 @@ k_bitmap0(const LevelDesc *__restrict__ desc, const uint32_t *__restrict__ succ,
   }
 }
 
-cudaError_t launch_heads0_log(LevelDesc *desc, const unsigned long long *acc, uint32_t *hlist0,
-                              const uint32_t *succ, uint32_t n, uint32_t *bitmap, uint32_t *err,
-                              int validate, cudaStream_t s) {
-  k_heads_single<<<1, 32, 0, s>>>(desc, acc, hlist0, validate);
+cudaError_t launch_bitmap0(const LevelDesc *desc, const uint32_t *succ, uint32_t n, uint32_t *bitmap, uint32_t *err,
+                           int validate, cudaStream_t s) {
   k_bitmap0<<<stream_grid(n, 256), 256, 0, s>>>(desc, succ, n, bitmap, err, validate);
-  count_launch(2);
+  count_launch();
   return cudaGetLastError();
 }
 
