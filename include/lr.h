@@ -78,13 +78,13 @@ typedef enum lr_dtype { LR_NONE = 0, LR_I32 = 1, LR_I64 = 2 } lr_dtype;
  * (visits by load and store instead of an atomic exchange); log=0 / log=1
  * (force the level-0 form); algo, contract, spawn; ord (batches: 0 chases
  * by per-CTA slices of ruler ids, 1 takes level 0's rulers in element
- * order, 2, the default, every level of 2^20 elements or more); pf (the
+ * order, 2, the default, every level; only levels whose records exceed L2); pf (the
  * element order's L2 prefetch lead in K elements, 0 off, 4 by default).
  */
 typedef struct lr_tuning {
-    uint32_t f0_inv;     /* 1/f at level 0 (default by n: 4 to 16 below 2^27,    */
-                         /* 48 below 2^29, 96 from 2^29; a batch keeps 16 from   */
-                         /* 2^22 up)                                             */
+    uint32_t f0_inv;     /* 1/f at level 0 (default by n: 4 for the smallest     */
+                         /* lists that take it to 96 from 2^29; a batch takes    */
+                         /* 16 from 2^23 and 12 from 2^24)                       */
     uint32_t f_inv;      /* 1/f at levels >= 1 (default 4 or 8, by size)         */
     uint32_t cutoff;     /* largest level ranked by the base case when below     */
                          /* 12288; 12288 and more, and 0: the built-in bound     */

@@ -43,31 +43,40 @@ static uint32_t env_u32(const char *spec, const char *key, uint32_t dflt) {
   return dflt;
 }
 
-// Default ruler fraction at level 0 by size (measured on GB300, random
-// order).  Up to 2^23 elements the rulers' list goes straight to the base
-// case (k_jump), whose time grows with its size, and the chase is bound by
-// the latency of its longest segment, about f ln(n / f) dependent steps: the
-// two balance near 200 to 350 thousand rulers (2^20: 172 us a call at 1/3 to
-// 1/8, 199 at 1/12; 2^21: 189 at 1/8, 207 at 1/4, 211 at 1/16; 2^22: 271 at
-// 1/12, 276 at 1/8).  From 2^27 up the chase is bound by the random-access
-// rate, and fewer rulers shrink the recursion more than their longer
-// segments lengthen the chase's tail (1/48 at 2^28, 1/96 at 2^30).
+// Default ruler fraction at level 0 by size (measured on GB300, random order;
+// a single list, int32 weights / unweighted where both are given).
+//  - Up to 4.7 million elements the rulers' list goes straight to the base
+//    case (k_jump), whose time grows with its size, and the chase is bound by
+//    the latency of its longest segment, about f ln(n / f) dependent steps:
+//    the two balance near 200 to 400 thousand rulers (2^20: 172 us a call at
+//    1/3 to 1/8, 199 at 1/12; 2^21: 189 at 1/8, 207 at 1/4, 211 at 1/16).
+//  - Then one more level stands between them and rulers get cheaper: 7
+//    million 377 / 296 us at 1/8, 393 / 326 at 1/16; 20 million 1033 / 822 at
+//    1/12, 1066 / 849 at 1/16, 1098 / 860 at 1/24.
+//  - Beyond L2 the chase is bound by the random-access rate; fewer rulers
+//    shrink the recursion and the final pass's gathers more than their longer
+//    segments lengthen the chase's tail: 2^26 3.11 / 2.29 ms at 1/24, 3.13 /
+//    2.35 at 1/16; 2^27 4.84 at 1/48, 4.94 at 1/24; 2^28 10.10 at 1/64, 10.20
+//    at 1/48, 11.00 at 1/16; 2^30 43.1 at 1/96, 43.6 at 1/64.
+struct F0Step { int64_t below; uint32_t f0_inv; };
+static const F0Step kF0Steps[] = {
+    {3ll << 18, 4}, {5ll << 18, 6}, {5ll << 19, 8}, {9ll << 19, 12}, {1ll << 23, 8}, {3ll << 23, 12},
+    {5ll << 23, 16}, {3ll << 25, 24}, {1ll << 27, 32}, {3ll << 26, 48}, {1ll << 29, 64}};
+
 static uint32_t default_f0_inv(int64_t n) {
-  if (n < 3 * ((int64_t)1 << 18)) return 4;
-  if (n < 5 * ((int64_t)1 << 18)) return 6;
-  if (n < 5 * ((int64_t)1 << 19)) return 8;
-  if (n < 3 * ((int64_t)1 << 21)) return 12;
-  if (n < ((int64_t)1 << 27)) return 16;
-  if (n < ((int64_t)1 << 29)) return 48;
+  for (const F0Step &t : kF0Steps)
+    if (n < t.below) return t.f0_inv;
   return 96;
 }
 
-// A batch chases level 0 in element order: its records stay in L2 only if
-// the front (threads x ruler spacing) is narrow, so it keeps 1/16 from 2^22
-// up (on the 1024-instance batch of 4.3e8 elements: 17.3 ms at 1/16 and
-// 1/24, 17.8 at 1/32, 18.8 at 1/48).
+// A batch beyond L2 chases level 0 in element order: its records stay in L2
+// only if the front (threads x ruler spacing) is narrow (1024 instances,
+// 4.7e8 elements: 15.9 ms at 1/12, 16.1 at 1/16, 17.4 at 1/8, 17.7 at 1/24;
+// 22 million elements 1.00 / 1.03 / 1.04 / 1.14 ms).
+constexpr int64_t kOrdSpacingFrom = 1ll << 24;
 static uint32_t default_f0_inv_batch(int64_t n) {
-  return n < ((int64_t)1 << 22) ? default_f0_inv(n) : 16;
+  if (n < (1ll << 23)) return default_f0_inv(n);
+  return n < kOrdSpacingFrom ? 16 : 12;
 }
 
 // Largest level below the first that the base case ranks (k_jump), unless the
@@ -175,8 +184,14 @@ static bool use_log0(const Tuning &u, uint64_t n, bool weighted, int rank_bytes,
 // element order: a front that crosses the instances a few at a time keeps
 // the records it touches, the reduced records it writes and, in the final
 // pass, the rank gathers within a footprint the L2 holds.
-static bool use_ord0(const Tuning &u, uint64_t n, bool log0, bool spawn0, bool extras, bool multi) {
-  return u.ord != 0 && multi && !log0 && !spawn0 && !extras && n <= 0x7FFFFFFFull;
+// While the level's records fit L2 anyway, the order only costs: five launches
+// to build it and half the threads (3.8 million weighted elements 249 us
+// without, 306 with it; 15 million unweighted 586 / 663; 22 million weighted,
+// 355 MB of records, 1237 / 1016).
+constexpr uint64_t kOrdMinBytes = 128ull << 20;
+static bool use_ord0(const Tuning &u, uint64_t n, bool rec16, bool log0, bool spawn0, bool extras, bool multi) {
+  return u.ord != 0 && multi && !log0 && !spawn0 && !extras && n <= 0x7FFFFFFFull &&
+         n * (rec16 ? 16 : 8) > kOrdMinBytes;
 }
 
 static size_t align_up(size_t x, size_t a = 256) { return (x + a - 1) / a * a; }
@@ -188,10 +203,9 @@ constexpr int kOrdCtasPerSm = 4;
 // Below this size the packing pass counts the links that stay in their tiles
 // itself, instead of a sample and a wait of its own before it.
 constexpr uint64_t kPackFirst = 1ull << 22;
-// Deeper levels of a batch keep each instance's rulers together too; from
-// this size on they are chased in order as well (LR_TUNING ord=1: level 0
-// only; ord=0: no level).
-constexpr uint32_t kOrdMinLevel = 1u << 20;
+// (Deeper levels of a batch keep each instance's rulers together too, and are
+// chased in order by the same rule; LR_TUNING ord=1: level 0 only; ord=0: no
+// level.)
 
 int chase_grid_for(const Tuning &u, bool rec16, bool log0, bool ord0) {
   int per = u.ctas ? (int)u.ctas : (log0 ? chase_log_occupancy((int)u.block) : chase_occupancy(rec16, (int)u.block));
@@ -797,7 +811,7 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
   // a batch chases its level-0 rulers in element order (the has-predecessor
   // bitmap, free once the heads are chosen, holds the ruler marks; level 1's
   // rank array, written only after the chase, holds the order)
-  const bool ord0 = use_ord0(u, in.n, log0, spawn0, extras, ptrs || in.offsets != nullptr);
+  const bool ord0 = use_ord0(u, in.n, rec16_0, log0, spawn0, extras, ptrs || in.offsets != nullptr);
   // tile-local contraction: forced, or decided from the count of links that
   // stay inside their tile (the log form's first pass counts them and they
   // are read with the list count; otherwise a sample of the tiles decides)
@@ -1014,7 +1028,7 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
     } else {
       OrdArgs oa;
       memset(&oa, 0, sizeof(oa));
-      if (p.ord0 && (l == 0 || (u.ord >= 2 && p.cap[l] >= kOrdMinLevel))) {
+      if (p.ord0 && (l == 0 || (u.ord >= 2 && 16ull * p.cap[l] > kOrdMinBytes))) {
         oa.ord = (uint32_t *)(var + p.off_ord);
         oa.cum = (uint32_t *)(var + p.off_cum);
         oa.bits = bitmap;        // the has-predecessor bitmap is free once level 0's heads are chosen
@@ -1403,8 +1417,7 @@ size_t workspace_upto(int64_t n, const lr_opts *opts) {
   size_t w = lr_workspace_size(n, 0, opts);
   auto consider = [&](int64_t m) { if (m > 0 && m < n) w = std::max(w, lr_workspace_size(m, 0, opts)); };
   for (int64_t m = 1; m < n; m *= 2) { consider(m - 1); consider(m); }
-  for (int64_t m = 1; m < n; m *= 2)
-    for (int64_t q : {3 * m, 5 * m}) consider(q - 1);
+  for (const F0Step &t : kF0Steps) consider(t.below - 1);
   return w;
 }
 }  // namespace lr
@@ -1435,7 +1448,7 @@ size_t lr_workspace_size_outputs(int64_t n_total, int32_t k, const lr_outputs *o
   const bool log0 = use_log0(u, (uint64_t)n_total, opts->wtype != LR_NONE, opts->rtype == LR_I64 ? 8 : 4,
                              extras, k != 0);
   const bool spawn0 = u.spawn != 0 && u.xchg != 0 && !log0 && !extras;
-  const bool ord0 = use_ord0(u, (uint64_t)n_total, log0, spawn0, extras, k != 0);
+  const bool ord0 = use_ord0(u, (uint64_t)n_total, opts->wtype != LR_NONE, log0, spawn0, extras, k != 0);
   Plan p = make_plan((uint64_t)n_total, h, u,
                      opts->wtype != LR_NONE || (extras && (uint64_t)n_total <= u.base0),
                      opts->rtype == LR_I64 ? 8 : 4, opts->seed, 256 * 16, log0, extras,
