@@ -11,6 +11,7 @@ cannot load, importing the ranking functions raises.
     rank = lr.rank_batch(offsets, succ, w)    # many lists, one launch sequence
 """
 import ctypes
+import itertools
 import os
 import threading
 
@@ -192,57 +193,63 @@ def _check(code, what=""):
 
 
 # ---------------------------------------------------------------- torch glue
+# A short call is mostly marshalling, so what does not change is looked up
+# once: the torch module, the accepted dtypes, and the integer handle of the
+# current stream (torch's own accessor where it has one).
+_torch_mod = None
+_SUCC = _INTS = _OFFS = _WCODES = None
+_raw_stream = None
+
+
 def _torch():
-    import torch
-    return torch
+    global _torch_mod, _SUCC, _INTS, _OFFS, _WCODES, _raw_stream
+    if _torch_mod is None:
+        import torch
+        _SUCC = tuple(d for d in (getattr(torch, "uint32", None), torch.int32) if d is not None)
+        _INTS = (torch.int32, torch.int64)
+        _OFFS = (torch.int64,)
+        _WCODES = {torch.int32: LR_I32, torch.int64: LR_I64}
+        _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        _torch_mod = torch
+    return _torch_mod
 
 
 def _stream_handle(stream):
     torch = _torch()
     if stream is None:
+        if _raw_stream is not None:
+            return _raw_stream(torch.cuda.current_device())
         stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+    return stream.cuda_stream
 
 
 def _dev_ptr(t, name, dtypes):
-    torch = _torch()
-    if not isinstance(t, torch.Tensor) or not t.is_cuda:
+    if not isinstance(t, _torch().Tensor) or not t.is_cuda:
         raise TypeError("%s must be a CUDA tensor" % name)
     if t.dtype not in dtypes:
         raise TypeError("%s has dtype %s, expected one of %s" % (name, t.dtype, dtypes))
     if not t.is_contiguous():
         raise ValueError("%s must be contiguous" % name)
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _succ_dtypes():
-    torch = _torch()
-    return tuple(d for d in (getattr(torch, "uint32", None), torch.int32) if d is not None)
+    _torch()
+    return _SUCC
 
 
 def _wcode(weight):
-    torch = _torch()
-    if weight is None:
-        return LR_NONE
-    return {torch.int32: LR_I32, torch.int64: LR_I64}[weight.dtype]
+    _torch()
+    return LR_NONE if weight is None else _WCODES[weight.dtype]
 
 
 def _opts(wtype, rtype, validate=False, seed=0x5EED, max_lists=0, tuning=None, sync=False,
           n_total=0, workspace=None):
-    o = _Opts()
-    load().lr_opts_default(ctypes.byref(o))
-    o.wtype, o.rtype = wtype, rtype
-    o.validate = 1 if validate else 0
-    o.sync = 1 if sync else 0
-    o.seed = int(seed) & (2**64 - 1)
-    o.max_lists = int(max_lists)
-    o.n_total = int(n_total)
-    if tuning is not None:
-        o.tuning = ctypes.pointer(tuning)
-    if workspace is not None:
-        o.workspace = ctypes.c_void_p(workspace.data_ptr())
-        o.ws_bytes = workspace.numel() * workspace.element_size()
-    return o
+    """lr_opts with every field given (the defaults here are lr_opts_default's)."""
+    return _Opts(wtype, rtype, None if tuning is None else ctypes.pointer(tuning),
+                 None if workspace is None else workspace.data_ptr(),
+                 0 if workspace is None else workspace.numel() * workspace.element_size(),
+                 1 if validate else 0, 1 if sync else 0, int(seed) & (2**64 - 1), int(max_lists), int(n_total))
 
 
 def _rank_dtype(weight, rank_dtype):
@@ -333,38 +340,45 @@ def rank_batch_ptrs(succs, weights=None, outs=None, rank_dtype=None, validate=Fa
     device = succs[0].device
     wdt = None if weights is None else weights[0].dtype
     rdt = _rank_dtype(None if weights is None else weights[0], rank_dtype)
-    sizes, sp, wp, rp = [], [], [], []
-    if outs is None:
-        outs = [torch.empty(t.numel(), dtype=rdt, device=device) for t in succs]
-    for j, t in enumerate(succs):
-        if t.device != device:
-            raise ValueError("every tensor must be on the same device")
-        sp.append(_dev_ptr(t, "succs[%d]" % j, _succ_dtypes()).value or 0)
-        sizes.append(t.numel())
-        if weights is not None:
-            w = weights[j]
-            if w.dtype != wdt or w.numel() != t.numel():
-                raise ValueError("weights[%d] has another dtype or length" % j)
-            wp.append(_dev_ptr(w, "weights[%d]" % j, (torch.int32, torch.int64)).value or 0)
-        o = outs[j]
-        if o.dtype != outs[0].dtype or o.numel() != t.numel():
-            raise ValueError("outs[%d] has another dtype or length" % j)
-        rp.append(_dev_ptr(o, "outs[%d]" % j, (torch.int32, torch.int64)).value or 0)
-    offsets = torch.zeros(k + 1, dtype=torch.int64)
-    offsets[1:] = torch.cumsum(torch.tensor(sizes, dtype=torch.int64), 0)
+    sizes = [t.numel() for t in succs]
+    fresh = outs is None
+    if fresh:
+        outs = [torch.empty(m, dtype=rdt, device=device) for m in sizes]
+
+    def pointers(what, ts, dtypes, one_dtype):
+        """Data pointers of CUDA tensors that match the instances."""
+        got = []
+        for j, (t, m) in enumerate(zip(ts, sizes)):
+            if one_dtype is not None and (t.dtype != one_dtype or t.numel() != m):
+                raise ValueError("%s[%d] has another dtype or length" % (what, j))
+            if not (isinstance(t, torch.Tensor) and t.is_cuda and t.dtype in dtypes and t.is_contiguous()):
+                _dev_ptr(t, "%s[%d]" % (what, j), dtypes)      # raises, naming the fault
+            got.append(t.data_ptr())
+        return got
+
+    if any(t.device != device for t in succs):
+        raise ValueError("every tensor must be on the same device")
+    sp = pointers("succs", succs, _succ_dtypes(), None)
+    wp = [] if weights is None else pointers("weights", weights, _INTS, wdt)
+    rp = [t.data_ptr() for t in outs] if fresh and rdt in _INTS else pointers("outs", outs, _INTS, outs[0].dtype)
+    # one table of all offsets and pointers, copied at once on the stream that
+    # reads it (from pinned memory that torch keeps until the copy is done)
+    table = [0]
+    table.extend(itertools.accumulate(sizes))
+    n_total = table[k]
+    table += sp
+    table += rp
+    table += wp
     if stream is None:
         stream = torch.cuda.current_stream(device)
-    with torch.cuda.stream(stream):          # the tables are copied on the stream that reads them
-        d_off = offsets.to(device)
-        d_sp = torch.tensor(sp, dtype=torch.int64).to(device)
-        d_rp = torch.tensor(rp, dtype=torch.int64).to(device)
-        d_wp = None if weights is None else torch.tensor(wp, dtype=torch.int64).to(device)
-    wcode = LR_NONE if weights is None else {torch.int32: LR_I32, torch.int64: LR_I64}[wdt]
+    with torch.cuda.stream(stream):
+        d_tab = torch.tensor(table, dtype=torch.int64, pin_memory=True).to(device, non_blocking=True)
+    at = d_tab.data_ptr()
+    wcode = LR_NONE if weights is None else _WCODES[wdt]
     o = _opts(wcode, LR_I32 if outs[0].dtype == torch.int32 else LR_I64, validate, seed,
-              max_lists, tuning, sync, n_total=int(offsets[-1]))
-    code = lib.lr_rank_batch_ptrs(ctypes.c_void_p(d_off.data_ptr()), ctypes.c_void_p(d_sp.data_ptr()),
-                                  None if d_wp is None else ctypes.c_void_p(d_wp.data_ptr()),
-                                  ctypes.c_void_p(d_rp.data_ptr()), k, ctypes.byref(o), _stream_handle(stream))
+              max_lists, tuning, sync, n_total=n_total)
+    code = lib.lr_rank_batch_ptrs(at, at + 8 * (k + 1), at + 8 * (3 * k + 1) if wp else None,
+                                  at + 8 * (2 * k + 1), k, ctypes.byref(o), _stream_handle(stream))
     _check(code, "lr_rank_batch_ptrs")
     return outs
 

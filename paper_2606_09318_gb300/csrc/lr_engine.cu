@@ -352,11 +352,9 @@ static lr_status from_cuda(cudaError_t e) {
   return LR_ERR_CUDA;
 }
 
-lr_status setup_device_once() {
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return from_cuda(e);
-  std::lock_guard<std::mutex> g(g_mu);
+// (with g_mu held)
+static lr_status setup_device_locked(int dev) {
+  cudaError_t e = cudaSuccess;
   if (dev >= 0 && dev < 64 && !g_setup_done[dev]) {
     e = small_setup();
     if (e == cudaSuccess) e = log_setup();
@@ -373,13 +371,21 @@ lr_status setup_device_once() {
   return LR_OK;
 }
 
+lr_status setup_device_once() {
+  int dev = 0;
+  const cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return from_cuda(e);
+  std::lock_guard<std::mutex> g(g_mu);
+  return setup_device_locked(dev);
+}
+
 Ctx *get_ctx(cudaStream_t stream, lr_status *st) {
-  *st = setup_device_once();
-  if (*st != LR_OK) return nullptr;
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) { *st = from_cuda(e); return nullptr; }
   std::lock_guard<std::mutex> g(g_mu);
+  *st = setup_device_locked(dev);
+  if (*st != LR_OK) return nullptr;
   auto key = std::make_pair(dev, (uintptr_t)stream);
   auto it = g_ctx.find(key);
   if (it != g_ctx.end()) { *st = LR_OK; return it->second; }

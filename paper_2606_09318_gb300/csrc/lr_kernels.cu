@@ -31,11 +31,26 @@ static std::atomic<int64_t> g_launches{0};
 void count_launch(int k) { g_launches.fetch_add(k, std::memory_order_relaxed); }
 int64_t launch_count() { return g_launches.load(std::memory_order_relaxed); }
 
-int device_sm_count() {
-  int dev = 0, sms = 0;
+// A device attribute that never changes, asked for once (every launch sizes
+// its grid by it).  Threads that ask at the same time store the same value.
+int cached_per_device(CachedInt &c, int (*ask)(int dev, int arg), int arg) {
+  int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return 1;
-  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 1;
-  return sms > 0 ? sms : 1;
+  if (dev < 0 || dev >= CachedInt::kDevices) return ask(dev, arg);
+  int v = c.value[dev].load(std::memory_order_relaxed);
+  if (v == 0) {
+    v = ask(dev, arg);
+    if (v > 0) c.value[dev].store(v, std::memory_order_relaxed);
+  }
+  return v > 0 ? v : 1;
+}
+
+int device_sm_count() {
+  static CachedInt cache;
+  return cached_per_device(cache, [](int dev, int) {
+    int sms = 0;
+    return cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess ? sms : 0;
+  }, 0);
 }
 
 int stream_grid(uint64_t work_items, int block) {
@@ -1367,10 +1382,13 @@ cudaError_t launch_chase(LevelDesc *desc, int lev, void *work, bool rec16, void 
 }
 
 int chase_occupancy(bool rec16, int block) {
-  int nb = 0;
-  if (rec16) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_chase<Rec16, false, false, false>, block, 0);
-  else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_chase<Rec8, false, false, false>, block, 0);
-  return nb > 0 ? nb : 1;
+  static CachedInt cache[2][3];                // per record size and block (128, 256, 512)
+  return cached_per_device(cache[rec16][block == 128 ? 0 : block == 256 ? 1 : 2], [](int, int arg) {
+    int nb = 0;
+    if (arg < 0) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_chase<Rec16, false, false, false>, -arg, 0);
+    else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_chase<Rec8, false, false, false>, arg, 0);
+    return nb;
+  }, rec16 ? -block : block);
 }
 
 // ---------------------------------------------------------------- finalize

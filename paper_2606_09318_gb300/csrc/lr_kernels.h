@@ -1,6 +1,7 @@
 // lr_kernels.h -- host-side launchers of the list-ranking kernels (C++ linkage,
 // internal to liblr.so).
 #pragma once
+#include <atomic>
 #include <cstddef>
 #include <cstdint>
 #include <cuda_runtime.h>
@@ -26,6 +27,13 @@ struct InitParams {
 void count_launch(int k = 1);
 int64_t launch_count();
 
+// A positive number per device, found by ask(device, arg) when first needed
+// (1 if it cannot be found).
+struct CachedInt {
+  static constexpr int kDevices = 64;
+  std::atomic<int> value[kDevices] = {};
+};
+int cached_per_device(CachedInt &c, int (*ask)(int dev, int arg), int arg);
 int device_sm_count();
 int stream_grid(uint64_t work_items, int block);
 

@@ -270,9 +270,12 @@ cudaError_t launch_chase_log(LevelDesc *desc, const uint32_t *succ, void *next_w
 }
 
 int chase_log_occupancy(int block) {
-  int nb = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_chase_log, block, 0);
-  return nb > 0 ? nb : 1;
+  static CachedInt cache[3];                   // per block (128, 256, 512)
+  return cached_per_device(cache[block == 128 ? 0 : block == 256 ? 1 : 2], [](int, int b) {
+    int nb = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_chase_log, b, 0);
+    return nb;
+  }, block);
 }
 
 // ---------------------------------------------------------------- propagation
