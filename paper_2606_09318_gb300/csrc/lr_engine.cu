@@ -198,8 +198,9 @@ static size_t align_up(size_t x, size_t a = 256) { return (x + a - 1) / a * a; }
 
 // CTAs of 256 threads per SM for the chase in element order: the front's
 // width (threads x ruler spacing) must stay small enough that the instances
-// it crosses fit in L2; more threads only queue at the memory system.
-constexpr int kOrdCtasPerSm = 4;
+// it crosses fit in L2 (7.5e7 elements at 1/12, 4 / 6 / 8 CTAs: weighted 1.21 /
+// 1.31 / 1.55 ms, unweighted 1.37 / 1.06 / 1.06; 4.7e8 weighted 6.7 / 7.7 / 9.4).
+constexpr int kOrdCtasWeighted = 4, kOrdCtasUnweighted = 6;
 // Below this size the packing pass counts the links that stay in their tiles
 // itself, instead of a sample and a wait of its own before it.
 constexpr uint64_t kPackFirst = 1ull << 22;
@@ -207,9 +208,9 @@ constexpr uint64_t kPackFirst = 1ull << 22;
 // chased in order by the same rule; LR_TUNING ord=1: level 0 only; ord=0: no
 // level.)
 
-int chase_grid_for(const Tuning &u, bool rec16, bool log0, bool ord0) {
+int chase_grid_for(const Tuning &u, bool rec16, bool log0, bool ord0, bool weighted) {
   int per = u.ctas ? (int)u.ctas : (log0 ? chase_log_occupancy((int)u.block) : chase_occupancy(rec16, (int)u.block));
-  if (ord0 && !u.ctas) per = std::min(per, kOrdCtasPerSm * 256 / (int)u.block);
+  if (ord0 && !u.ctas) per = std::min(per, (weighted ? kOrdCtasWeighted : kOrdCtasUnweighted) * 256 / (int)u.block);
   return device_sm_count() * std::max(1, per);
 }
 
@@ -829,7 +830,7 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
     if (cs != LR_ERR_NOT_FOUND) return cs;
   }
   const bool count_local = contractible && u.contract == LR_CONTRACT_AUTO && in.n > u.base0;
-  const int grid = chase_grid_for(u, rec16_0, log0, ord0);
+  const int grid = chase_grid_for(u, rec16_0, log0, ord0, in.wtype != 0);
   // Counting the lists needs a wait.  The base case ranks level 0 without a
   // count, but a call above the smallest sizes is not capturable without a
   // promise of max_lists whichever way it is ranked.

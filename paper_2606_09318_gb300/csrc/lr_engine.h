@@ -85,7 +85,7 @@ Plan make_plan(uint64_t n, uint64_t h, const Tuning &u, bool rec16_0, int rank_b
 // Workspace that serves a single instance of any size up to n (lr_workspace_size
 // is for one size).
 size_t workspace_upto(int64_t n, const lr_opts *opts);
-int chase_grid_for(const Tuning &u, bool rec16, bool log0, bool ord0 = false);
+int chase_grid_for(const Tuning &u, bool rec16, bool log0, bool ord0, bool weighted);
 Ctx *get_ctx(cudaStream_t stream, lr_status *st);
 // Forget the context of a stream that is about to be destroyed (waits for
 // the stream, frees the context's buffers).

@@ -1111,38 +1111,92 @@ cudaError_t launch_order(LevelDesc *desc, int lev, uint32_t cap, uint64_t *cnt, 
 
 
 // Ordered queue: CTAs draw positions of the ruler sequence from one global
-// counter, kOrdChunk at a time, and hand them to their threads one by one
-// through a shared-memory window (end << 32) | next.  The thread that draws
-// next == end refills the window; threads that draw past its end meanwhile
-// take single positions from the global counter.  Nobody waits.
-constexpr uint32_t kOrdChunk = 32;
+// counter, kOrdChunk at a time, and hand them to their threads through a
+// shared-memory window, (end << 32) | next.  The lanes of a warp that ask
+// together take theirs with one atomic.  The group that brings the window
+// down to kOrdLow positions draws the next chunk, which waits in s_next; the
+// first group that runs past the window's end and finds it there makes it the
+// window.  A group that does not find it draws just what it lacks from the
+// global counter.  Nobody waits.
+//
+// The counter is one address, which serves one atomic in some 1.5 ns, so how
+// often it is asked can bound the chase.  With 32 positions a draw, fetched
+// only when the window had run out, and single draws until they came, a batch
+// of 7.5e7 unweighted elements took 1.51 ms, however many threads chased; now
+// 1.37 ms, and 1.06 with half as many threads again.  A CTA that starts with
+// one draw for all its threads saves 0.23 ms at any size, and once the
+// sequence has run out, nobody asks.
+constexpr uint32_t kOrdChunk = 128, kOrdLow = kOrdChunk / 2;
+static_assert(kOrdLow >= 32, "a chunk serves a warp and stays above the low mark");
 
-// The counter is one address, which serves about one atomic in 1.5 ns: a CTA
-// starts with two positions per thread from a single draw (all threads drawing
-// at once cost 0.23 ms, at any size), and once the sequence has run out no
-// thread asks it again.
-__device__ __forceinline__ uint64_t ord_take(unsigned long long *s_win, uint32_t *s_out, uint32_t *gq, uint64_t total,
-                                             bool *refilled = nullptr) {
-  const unsigned long long w = atomicAdd(s_win, 1ull);
-  const uint32_t next = (uint32_t)w, end = (uint32_t)(w >> 32);
-  if (next < end) return next;
-  if (*(volatile uint32_t *)s_out) return total;
-  if (next == end) {
-    if (refilled) *refilled = true;
-    // the chunk is this CTA's whatever its length: every position of it
-    // must be handed out, up to the end of the sequence
-    const uint32_t j = atomicAdd(gq, kOrdChunk);
-    if (j < total) {
-      const uint64_t e = (uint64_t)j + kOrdChunk < total ? (uint64_t)j + kOrdChunk : total;
-      atomicExch(s_win, (e << 32) | (j + 1u));
-    } else {
-      *(volatile uint32_t *)s_out = 1u;
-    }
-    return j;
+struct OrdQueue {
+  unsigned long long win, next;    // the window; the chunk after it (0: not there)
+  uint32_t out;                    // the sequence has run out
+};
+
+__device__ __forceinline__ unsigned long long ord_window(uint64_t from, uint64_t to) {
+  return ((unsigned long long)to << 32) | from;
+}
+
+// Draw a chunk from the global counter; 0 when there is none.
+__device__ __forceinline__ unsigned long long ord_draw(OrdQueue &q, uint32_t *gq, uint64_t total, uint32_t *fresh) {
+  const uint32_t j = atomicAdd(gq, kOrdChunk);
+  if (j >= total) {
+    *(volatile uint32_t *)&q.out = 1u;
+    return 0ull;
   }
-  const uint32_t j = atomicAdd(gq, 1u);
-  if (j >= total) *(volatile uint32_t *)s_out = 1u;
-  return j;
+  *fresh = j;
+  // the chunk is this CTA's whatever its length: every position of it must be
+  // handed out, up to the end of the sequence
+  return ord_window(j, (uint64_t)j + kOrdChunk < total ? (uint64_t)j + kOrdChunk : total);
+}
+
+// Position for this lane (total or more: none left).  *fresh: set on the lane
+// that drew a chunk, to the chunk's first position.
+__device__ __forceinline__ uint64_t ord_take(OrdQueue &q, uint32_t *gq, uint64_t total, uint32_t *fresh) {
+  const uint32_t mask = __activemask();
+  const uint32_t lane = threadIdx.x & 31u, leader = __ffs(mask) - 1;
+  const uint32_t cnt = __popc(mask), mine = __popc(mask & ((1u << lane) - 1u));
+  unsigned long long w = 0;
+  if (lane == leader) w = atomicAdd(&q.win, (unsigned long long)cnt);
+  w = __shfl_sync(mask, w, leader);
+  const uint32_t next = (uint32_t)w, end = (uint32_t)(w >> 32);
+  const uint32_t have = next < end ? min(end - next, cnt) : 0u, lack = cnt - have;
+  uint64_t more = total;                       // where the lacking positions start
+  if (lane == leader) {
+    bool draw = next + kOrdLow < end && next + cnt + kOrdLow >= end;     // brings the window down to the mark
+    if (lack) {
+      const unsigned long long c = atomicExch(&q.next, 0ull);
+      if (c) {
+        const uint32_t from = (uint32_t)c, to = (uint32_t)(c >> 32), left = to - from;
+        more = from;
+        draw = left <= lack + kOrdLow;         // a short chunk starts below the mark
+        if (left > lack) {
+          // the window, unless another group has opened one since this one
+          // asked: then it goes back (whoever holds the chunk is the only one
+          // who could open a window)
+          const unsigned long long now = *(volatile unsigned long long *)&q.win;
+          const bool spent = (uint32_t)now >= (uint32_t)(now >> 32);
+          atomicExch(spent ? &q.win : &q.next, ord_window(from + lack, to));
+          draw = draw && spent;
+        }
+        if (left < lack) {                     // only the sequence's last chunk: the rest is past its end
+          *(volatile uint32_t *)&q.out = 1u;
+          draw = false;
+        }
+      } else if (!*(volatile uint32_t *)&q.out) {
+        const uint32_t j = atomicAdd(gq, lack);
+        more = j;
+        if (j >= total) *(volatile uint32_t *)&q.out = 1u;
+      }
+    }
+    if (draw && !*(volatile uint32_t *)&q.out) {
+      const unsigned long long c = ord_draw(q, gq, total, fresh);
+      if (c) atomicExch(&q.next, c);
+    }
+  }
+  more = __shfl_sync(mask, more, leader);
+  return mine < have ? (uint64_t)next + mine : more + (mine - have);
 }
 
 // ---------------------------------------------------------------- chase
@@ -1193,17 +1247,16 @@ k_chase(LevelDesc *__restrict__ desc, int lev, Rec *__restrict__ work, Rec16 *__
         const uint32_t *__restrict__ tid_cur, uint32_t *__restrict__ tid_next, SpawnArgs sp,
         OrdArgs oa) {
   const uint32_t *__restrict__ ord = oa.ord;
-  __shared__ unsigned long long s_win;
-  __shared__ uint32_t s_out;
+  __shared__ OrdQueue s_q;
   const LevelDesc d = desc[lev];
   if (d.mode != kModeSrs) return;
   const uint32_t n = d.n, r = d.r;
   const uint64_t R = (uint64_t)r + d.k;
-  if (ord && threadIdx.x == 0) {               // the CTA's first window of the ordered queue
-    const uint32_t j = atomicAdd(qctr, 2u * blockDim.x);
-    const uint64_t e = min((uint64_t)j + 2u * blockDim.x, R);
-    s_win = j < R ? (e << 32) | j : 0ull;
-    s_out = j >= R;
+  if (ord && threadIdx.x == 0) {               // the CTA's first window and chunk
+    const uint32_t first = 2u * blockDim.x, j = atomicAdd(qctr, first);
+    s_q.win = j < R ? ord_window(j, min((uint64_t)j + first, R)) : 0ull;
+    s_q.next = 0ull;
+    s_q.out = j >= R;
   }
   __syncthreads();
   Perm P;
@@ -1215,9 +1268,9 @@ k_chase(LevelDesc *__restrict__ desc, int lev, Rec *__restrict__ work, Rec16 *__
   // an index of the ordered sequence
   auto take = [&]() -> uint64_t {
     if (ord) {
-      bool refilled = false;
-      const uint64_t j = ord_take(&s_win, &s_out, qctr, R, &refilled);
-      if (refilled && oa.pf_lead && j >= d.k && j < R) {
+      uint32_t fresh = 0xFFFFFFFFu;              // first position of a chunk this thread drew
+      const uint64_t got = ord_take(s_q, qctr, R, &fresh);
+      if (const uint64_t j = fresh; fresh != 0xFFFFFFFFu && oa.pf_lead && j >= d.k) {
         // the CTA took the rulers from j on: bring the records of the
         // elements up to its next draw's first ruler, pf_lead elements ahead,
         // into L2 before the front reaches them
@@ -1231,7 +1284,7 @@ k_chase(LevelDesc *__restrict__ desc, int lev, Rec *__restrict__ work, Rec16 *__
             asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" :: "l"(pa), "r"((uint32_t)(pb - pa)) : "memory");
         }
       }
-      return j;
+      return got;
     }
     return (uint64_t)lo + atomicAdd(q, 1u);
   };
