@@ -63,6 +63,7 @@ struct LevelDesc {
   uint32_t cap;      // static: capacity of this level's arrays
   uint64_t seed;     // static: permutation seed
   uint32_t hsrc;     // where this level's heads come from: kHeadsBitmap or kHeadsList
+  uint32_t narrow;   // level 0: weights and offsets in 32 bits (kNarrow*), else 16-byte records
   uint32_t picked;   // this level's rulers were chosen with its descriptor (a single head)
   uint32_t nraw;     // with spawning: ruler ids of the next level before compaction (else 0)
   unsigned long long check;  // base case: nonzero when an element has two predecessors (k_jump)
@@ -149,6 +150,33 @@ struct __align__(16) Rec16 {
   uint64_t w;    // weight (wrapping), then offset
 };
 
+// Level-0 weighted record, 8 bytes: before {succ, weight}, after
+// {ruler id | kSeen, offset}, both halves of what Rec16 holds in half the
+// room, for ids below 2^31 and inputs whose weights and offsets fit 32 bits:
+//  - int32 ranks: everything is taken modulo 2^32 anyway;
+//  - else all weights in [-2^19, 2^19) or all in [0, 2^20), with a ruler's
+//    segment cut after kNarrowSteps elements (k_chase).
+struct __align__(8) Rec8w {
+  uint32_t lo;   // succ, then kSeen | ruler id
+  uint32_t hi;   // weight, then offset
+};
+constexpr uint32_t kSeen = 0x80000000u;
+constexpr uint32_t kNarrowSteps = 4096;
+
+enum : uint32_t { kNarrowNone = 0, kNarrowSigned = 1, kNarrowUnsigned = 2 };
+// What a pass over the weights finds: some outside [-2^19, 2^19); some below
+// 0 or from 2^20 on.
+constexpr uint32_t kWideSigned = 1u, kWideUnsigned = 2u;
+__host__ __device__ __forceinline__ uint32_t wide_flags(uint64_t w) {
+  return (w + (1u << 19) >= (1u << 20) ? kWideSigned : 0u) | (w >= (1u << 20) ? kWideUnsigned : 0u);
+}
+__host__ __device__ __forceinline__ uint32_t narrow_mode(uint32_t flags) {
+  return !(flags & kWideSigned) ? kNarrowSigned : !(flags & kWideUnsigned) ? kNarrowUnsigned : kNarrowNone;
+}
+__device__ __forceinline__ uint64_t widen(uint32_t v, uint32_t mode) {
+  return mode == kNarrowUnsigned ? (uint64_t)v : (uint64_t)(int64_t)(int32_t)v;
+}
+
 __device__ __forceinline__ void record_error(uint32_t *err, uint32_t bits) {
   atomicOr(err, bits);
 }
@@ -224,6 +252,19 @@ __device__ __forceinline__ Rec16 xchg_rec(Rec16 *p, uint32_t cid, uint64_t off) 
   return r;
 }
 
+__device__ __forceinline__ Rec8w ld_rec(const Rec8w *p) {
+  uint2 v = __ldcg(reinterpret_cast<const uint2 *>(p));
+  return Rec8w{v.x, v.y};
+}
+__device__ __forceinline__ void st_rec(Rec8w *p, uint32_t cid, uint64_t off) {
+  __stcg(reinterpret_cast<uint2 *>(p), make_uint2(cid | kSeen, (uint32_t)off));
+}
+__device__ __forceinline__ Rec8w xchg_rec(Rec8w *p, uint32_t cid, uint64_t off) {
+  const unsigned long long nv = ((unsigned long long)(uint32_t)off << 32) | (cid | kSeen);
+  const unsigned long long ov = atomicExch(reinterpret_cast<unsigned long long *>(p), nv);
+  return Rec8w{(uint32_t)ov, (uint32_t)(ov >> 32)};
+}
+
 // Ruler spawning (Section 2.2).  A spawner claims an unvisited element as a
 // new ruler c by exchanging in a claim mark, which no visited record can
 // equal: an 8-byte record {offset, id} never carries offset 0xFFFFFFFF (an
@@ -278,11 +319,23 @@ __device__ __forceinline__ uint32_t rec_succ(const Rec8 &r) { return r.lo; }
 __device__ __forceinline__ uint32_t rec_succ(const Rec16 &r) { return r.succ; }
 __device__ __forceinline__ uint32_t rec_tag(const Rec8 &r) { return r.hi; }
 __device__ __forceinline__ uint32_t rec_tag(const Rec16 &r) { return r.tag; }
+__device__ __forceinline__ uint32_t rec_succ(const Rec8w &r) { return r.lo; }
+__device__ __forceinline__ uint32_t rec_tag(const Rec8w &r) { return r.lo & kSeen ? r.lo & ~kSeen : kUnvisited; }
+// Link weight of a record in a level of the given narrow mode.
+template <class Rec>
+__device__ __forceinline__ uint64_t rec_weight(const Rec &r, uint32_t self, uint32_t) { return rec_weight(r, self); }
+__device__ __forceinline__ uint64_t rec_weight(const Rec8w &r, uint32_t, uint32_t mode) { return widen(r.hi, mode); }
 // After the chase: (ruler id, offset)
+__device__ __forceinline__ uint32_t done_cid(const Rec8w &r) {
+  return !(r.lo & kSeen) ? kUnvisited : r.lo == kZeroCid ? kZeroCid : r.lo & ~kSeen;
+}
 __device__ __forceinline__ uint32_t done_cid(const Rec8 &r) { return r.hi; }
 __device__ __forceinline__ uint32_t done_cid(const Rec16 &r) { return r.tag; }
 __device__ __forceinline__ uint64_t done_off(const Rec8 &r) { return r.lo; }
 __device__ __forceinline__ uint64_t done_off(const Rec16 &r) { return r.w; }
+template <class Rec>
+__device__ __forceinline__ uint64_t done_off(const Rec &r, uint32_t) { return done_off(r); }
+__device__ __forceinline__ uint64_t done_off(const Rec8w &r, uint32_t mode) { return widen(r.hi, mode); }
 
 // ---------------------------------------------------------------- block scan
 // Exclusive scan of one 64-bit value per thread across a CTA (warp shuffles,

@@ -214,6 +214,19 @@ int chase_grid_for(const Tuning &u, bool rec16, bool log0, bool ord0, bool weigh
   return device_sm_count() * std::max(1, per);
 }
 
+// Level 0 of a weighted call tries 8-byte records (Rec8w): half the bytes of
+// every pass over them, and of the footprint that sets the rate of the chase's
+// random exchanges (2^24 elements: 128 MiB and 61 G/s against 256 MiB and 35).
+// The packing pass finds out whether the weights allow it.  A call that waits
+// for its list count learns the answer there; another launches the kernels of
+// both kinds, of which those of the wrong one return at once, so it tries from
+// a size on where their 10 us do not count.
+constexpr uint64_t kNarrowAsyncMin = 1ull << 22;
+static bool use_narrow(const Tuning &u, uint64_t n, bool weighted, bool spawn0, bool extras, bool waits) {
+  return weighted && !extras && !spawn0 && u.xchg && n > u.base0 && n <= 0x7FFFFF00ull &&
+         (waits || n >= kNarrowAsyncMin);
+}
+
 // Static plan for n elements and at most h lists.
 // Spawned rulers provided for at level 0: t waves leave about t ln(n/t)
 // rulers in all (Section 2.5 cites this for spawning); a few t more as slack.
@@ -225,7 +238,8 @@ static uint32_t spawn_capacity(uint64_t n, uint64_t threads) {
 }
 
 Plan make_plan(uint64_t n, uint64_t h, const Tuning &u, bool rec16_0, int rank_bytes,
-               uint64_t seed, int chase_grid, bool log0, bool term, bool t0ws, bool spawn0, bool ord0) {
+               uint64_t seed, int chase_grid, bool log0, bool term, bool t0ws, bool spawn0, bool ord0,
+               bool narrow) {
   Plan p;
   memset(&p, 0, sizeof(p));
   p.n = n;
@@ -250,6 +264,7 @@ Plan make_plan(uint64_t n, uint64_t h, const Tuning &u, bool rec16_0, int rank_b
         p.raw_cap = (uint32_t)std::min<uint64_t>(0xFFFFFFF0ull, nc + p.spawn_cap);
         nc = std::min<uint64_t>(p.cap[0], nc + p.spawn_cap);
       }
+      if (L == 0 && narrow) nc += n / kNarrowSteps + 1;
       ++L;
       p.cap[L] = (uint32_t)nc;
       p.low[L] = (p.low[L - 1] + p.f_inv[L - 1] - 1) / p.f_inv[L - 1];   // the sampled rulers alone
@@ -268,7 +283,7 @@ Plan make_plan(uint64_t n, uint64_t h, const Tuning &u, bool rec16_0, int rank_b
   p.off_zero = o;
   p.off_err = o; o = align_up(o + 16);
   p.off_hcount = o; o = align_up(o + 16);
-  p.off_acc = o; o = align_up(o + 32);        // sums of terminals, successors; local links
+  p.off_acc = o; o = align_up(o + 40);        // sums of terminals, successors; local links, sample; flags
   p.off_logctr = o; o = align_up(o + 16);
   p.off_bctr = o; o = align_up(o + sizeof(uint32_t) * 256);
   p.off_q = o; o = align_up(o + sizeof(uint32_t) * (size_t)chase_grid * kMaxLevels);
@@ -626,8 +641,9 @@ static lr_status run_wyllie(const Inputs &in, Ctx *c, cudaStream_t s) {
   LR_TRY(cudaMemsetAsync(base, 0, in.validate ? q.off_a : q.zero_bytes, s));
   // without validation the scratch sums stand in for the bitmap, so the
   // pass issues no per-element atomics
-  LR_TRY(launch_prep0(in.succ, in.weight, in.wtype, (uint32_t)in.n, A, w16, bitmap, err, in.validate,
-                      in.offsets, in.k, in.validate ? nullptr : sums, nullptr, nullptr, nullptr, s));
+  LR_TRY(launch_prep0(in.succ, in.weight, in.wtype, (uint32_t)in.n, A, w16 ? kRecKind16 : kRecKind8, bitmap, err,
+                      in.validate, in.offsets, in.k, in.validate ? nullptr : sums, nullptr, WeightScan{}, nullptr,
+                      nullptr, s));
   prof.mark(PH_PREP);
   LR_TRY(launch_wyllie(A, B, w16, (uint32_t)in.n, in.rank, in.rank_bytes, err, s));
   prof.mark(PH_BASE);
@@ -683,12 +699,14 @@ static lr_status run_base(const Inputs &in, const Plan &p, bool checked, char *f
   LR_TRY(cudaMemsetAsync(fixed + p.off_zero, 0,
                          p.off_bitmap - p.off_zero + (marks ? 4 * (((size_t)n + 31) / 32) : 0), s));
   const InitParams ip = init_params(p);
+  const int kind = p.rec16_0 ? kRecKind16 : kRecKind8;
   if (in.sptr) {
-    LR_TRY(launch_init(desc, ip, nullptr, nullptr, nullptr, nullptr, s));
-    LR_TRY(launch_prep0_ptrs(in.sptr, in.wptr, in.wtype, n, work, bitmap, err, 1, in.offsets, in.k, s));
+    LR_TRY(launch_init(desc, ip, nullptr, nullptr, nullptr, nullptr, nullptr, s));
+    LR_TRY(launch_prep0_ptrs(in.sptr, in.wptr, in.wtype, n, work, kind, WeightScan{}, bitmap, err, 1, in.offsets,
+                             in.k, s));
   } else {
-    LR_TRY(launch_prep0(in.succ, in.weight, in.wtype, n, work, p.rec16_0, marks ? bitmap : nullptr, err,
-                        checked || in.validate, in.offsets, in.k, nullptr, nullptr, desc, &ip, s));
+    LR_TRY(launch_prep0(in.succ, in.weight, in.wtype, n, work, kind, marks ? bitmap : nullptr, err,
+                        checked || in.validate, in.offsets, in.k, nullptr, nullptr, WeightScan{}, desc, &ip, s));
   }
   if (!in.ctx) { c->last_desc = desc; c->last_nlev = 1; }
   prof.mark(PH_PREP);
@@ -830,7 +848,6 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
     if (cs != LR_ERR_NOT_FOUND) return cs;
   }
   const bool count_local = contractible && u.contract == LR_CONTRACT_AUTO && in.n > u.base0;
-  const int grid = chase_grid_for(u, rec16_0, log0, ord0, in.wtype != 0);
   // Counting the lists needs a wait.  The base case ranks level 0 without a
   // count, but a call above the smallest sizes is not capturable without a
   // promise of max_lists whichever way it is ranked.
@@ -838,8 +855,13 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
   const bool may_count = in.max_lists <= 0 && (in.ws == nullptr || in.count_in_ws);
   if (may_count && checked && capturing) return LR_ERR_CAPTURE;
   const bool need_count = may_count && in.n > u.base0;
+  const bool narrow = use_narrow(u, in.n, in.wtype != 0, spawn0, extras, need_count);
+  // the element order, where the records that level 0 really has call for it
+  const bool rec16_used = rec16_0 && !narrow;
+  const bool ord_used = ord0 && in.n * (rec16_used ? 16 : 8) > kOrdMinBytes;
+  const int grid = chase_grid_for(u, rec16_used, log0, ord_used, in.wtype != 0);
   uint64_t hb = in.max_lists > 0 ? (uint64_t)in.max_lists : in.n;
-  Plan p = make_plan(in.n, hb, u, rec16_0, in.rank_bytes, in.seed, grid, log0, extras, t0ws, spawn0, ord0);
+  Plan p = make_plan(in.n, hb, u, rec16_0, in.rank_bytes, in.seed, grid, log0, extras, t0ws, spawn0, ord0, narrow);
 
   // fixed part (level 0)
   char *fixed = nullptr;
@@ -906,28 +928,42 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
       prof.begin(s, (int64_t)in.n);            // not contracted after all: carry on
     }
   }
+  // flags of weights too wide for 8-byte records (int32 ranks: none is)
+  uint32_t *wflags = narrow ? reinterpret_cast<uint32_t *>(acc + 4) : nullptr;
+  // The pass that packs level 0's records.  `again`: only the records, in 16
+  // bytes, after a pass whose flags forbid 8-byte ones (unless_narrow: if they do).
+  auto pack = [&](int kind, bool again, const uint32_t *unless_narrow) -> cudaError_t {
+    const uint32_t n = (uint32_t)in.n;
+    WeightScan scan;
+    scan.flags = kind == kRecKind8w && in.rank_bytes == 8 ? wflags : nullptr;
+    scan.unless_narrow = unless_narrow;
+    unsigned long long *isums = again ? nullptr : reinterpret_cast<unsigned long long *>(bitmap);
+    uint32_t *marks = again ? nullptr : bitmap;
+    if (ptrs && sums0b)
+      return launch_prep0_ptrs_sums(in.sptr, in.wptr, in.wtype, n, work0, kind, scan, err, in.offsets, in.k, isums, s);
+    if (ptrs)
+      return launch_prep0_ptrs(in.sptr, in.wptr, in.wtype, n, work0, kind, scan, marks, err, in.validate, in.offsets,
+                               in.k, s);
+    if (sums0b)
+      return launch_prep0_sums(in.succ, in.weight, in.wtype, n, work0, kind, scan, err, in.offsets, in.k, isums, s);
+    return launch_prep0(in.succ, in.weight, in.wtype, n, work0, kind, marks, err, in.validate, in.offsets, in.k,
+                        sums0 && !again ? acc : nullptr, sums0 && local_exact && !again ? acc + 2 : nullptr, scan,
+                        nullptr, nullptr, s);
+  };
+  int kind0 = narrow ? kRecKind8w : rec16_0 ? kRecKind16 : kRecKind8;
+  bool both = narrow && !need_count;           // 8- or 16-byte records: the device decides
   if (log0)
     LR_TRY(launch_sum0(in.succ, (uint32_t)in.n, acc, local_exact ? acc + 2 : nullptr, err, s));
-  else if (ptrs && sums0b)
-    LR_TRY(launch_prep0_ptrs_sums(in.sptr, in.wptr, in.wtype, (uint32_t)in.n, work0, err, in.offsets, in.k,
-                                  reinterpret_cast<unsigned long long *>(bitmap), s));
-  else if (ptrs)
-    LR_TRY(launch_prep0_ptrs(in.sptr, in.wptr, in.wtype, (uint32_t)in.n, work0, bitmap, err,
-                             in.validate, in.offsets, in.k, s));
-  else if (sums0b)
-    LR_TRY(launch_prep0_sums(in.succ, in.weight, in.wtype, (uint32_t)in.n, work0, err, in.offsets, in.k,
-                             reinterpret_cast<unsigned long long *>(bitmap), s));
   else
-    LR_TRY(launch_prep0(in.succ, in.weight, in.wtype, (uint32_t)in.n, work0, rec16_0, bitmap, err,
-                        in.validate, in.offsets, in.k, sums0 ? acc : nullptr,
-                        sums0 && local_exact ? acc + 2 : nullptr, nullptr, nullptr, s));
+    LR_TRY(pack(kind0, false, nullptr));
+  if (both) LR_TRY(pack(kRecKind16, true, wflags));
   bool one_list = false;                       // the host has seen that level 0 is one list
   if (need_count) {
     // count the lists (one wait), then size the recursion for exactly that many:
     // a single-instance pass counts terminals in its reduction, a batch adds
     // its instances' terminal counts, the other passes count zero bits of the
     // has-predecessor bitmap
-    uint64_t sums[3];                          // terminals, other successors, local links
+    uint64_t sums[5];                          // terminals, other successors, local links, (sample), flags
     if (log0 || sums0) {
       LR_TRY(cudaMemcpyAsync(c->host_words + 4, acc, sizeof(sums), cudaMemcpyDeviceToHost, s));
     } else if (sums0b) {
@@ -937,6 +973,7 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
       LR_TRY(launch_count_heads(bitmap, (uint32_t)in.n, hcount, s));
       LR_TRY(cudaMemcpyAsync(c->host_words + 1, hcount, 4, cudaMemcpyDeviceToHost, s));
     }
+    if (narrow && !sums0) LR_TRY(cudaMemcpyAsync(c->host_words + 12, wflags, 4, cudaMemcpyDeviceToHost, s));
     LR_TRY(cudaStreamSynchronize(s));
     if (log0 || sums0) {
       memcpy(sums, c->host_words + 4, sizeof(sums));
@@ -951,8 +988,12 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
         prof.begin(s, (int64_t)in.n);          // not contracted after all: carry on
       }
     }
+    if (narrow && narrow_mode(c->host_words[12]) == kNarrowNone) {      // (the flags, either way)
+      kind0 = kRecKind16;
+      LR_TRY(pack(kind0, true, nullptr));
+    }
     hb = std::max<uint64_t>(1, c->host_words[1]);
-    p = make_plan(in.n, hb, u, rec16_0, in.rank_bytes, in.seed, grid, log0, extras, t0ws, spawn0, ord0);
+    p = make_plan(in.n, hb, u, rec16_0, in.rank_bytes, in.seed, grid, log0, extras, t0ws, spawn0, ord0, narrow);
   }
   if (!in.ws) {
     st = ensure_buffer(&c->var, &c->var_bytes, p.var_bytes, s);
@@ -969,7 +1010,8 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
   uint32_t *hC = extras ? (uint32_t *)(var + p.off_hC) : hA;
   uint32_t *ns = (uint32_t *)(var + p.off_ns);
   const bool acc_heads = (log0 || sums0) && !in.validate;
-  LR_TRY(launch_init(desc, init_params(p), acc_heads ? acc : nullptr, hA, ns, hB, s));
+  LR_TRY(launch_init(desc, init_params(p), acc_heads ? acc : nullptr, kind0 == kRecKind8w ? wflags : nullptr, hA, ns,
+                     hB, s));
   if (!in.ctx) { c->last_desc = desc; c->last_nlev = p.nlev; }
   if (p.spawn_cap) LR_TRY(cudaMemsetAsync(var + p.off_sctr, 0, p.spawn_zero, s));
   SpawnArgs spa;
@@ -989,7 +1031,7 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
     LR_TRY(launch_bitmap0(desc, in.succ, (uint32_t)in.n, bitmap, err, in.validate, s));
   } else if (sums0b)
     LR_TRY(launch_heads0_batch(desc, reinterpret_cast<unsigned long long *>(bitmap), in.offsets, in.k, hA,
-                               p.hcap, work0, rec16_0, (uint32_t)in.n, bitmap, s));
+                               p.hcap, work0, kind0, (uint32_t)in.n, bitmap, s));
 
   auto work_of = [&](int l) -> void * { return l == 0 ? work0 : (void *)(var + p.off_work[l]); };
   auto R_of = [&](int l) -> void * { return l == 0 ? in.rank : (void *)(var + p.off_R[l]); };
@@ -1017,7 +1059,7 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
         prof.mark(PH_BASE);
       }
     }
-    const int kind = (l == 0 && log0) ? kRecKindSucc : (r16 ? kRecKind16 : kRecKind8);
+    const int kind = (l == 0 && log0) ? kRecKindSucc : l == 0 ? kind0 : kRecKind16;
     if (l > 0 || !one_list)
       LR_TRY(launch_heads(desc, l, p.nlev, bitmap, hin, (l == 0 && log0) ? (void *)in.succ : work_of(l),
                         kind, ns, hout, bcnt, err, p.base, p.hcap, s));
@@ -1028,23 +1070,26 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
                               p.total_chunks, (uint32_t *)(fixed + p.off_logctr), s));
     else if (l == 0 && p.spawn_cap) {
       // spawning: reduced records at uncompacted ids, then compacted into level 1
-      LR_TRY(launch_chase(desc, 0, work0, r16, var + p.off_sraw, ns, qctr, p.chase_grid, p.chase_block,
+      LR_TRY(launch_chase(desc, 0, work0, kind, var + p.off_sraw, ns, qctr, p.chase_grid, p.chase_block,
                           err, (int)u.xchg, nullptr, nullptr, &spa, nullptr, s));
       LR_TRY(launch_spawn_compact(desc, 0, p.nlev, spa.ctr, spa.cap, spa.used, (uint32_t *)(var + p.off_supre),
                                   var + p.off_sraw, work_of(1), p.raw_cap, p.base, err, s));
     } else {
       OrdArgs oa;
       memset(&oa, 0, sizeof(oa));
-      if (p.ord0 && (l == 0 || (u.ord >= 2 && 16ull * p.cap[l] > kOrdMinBytes))) {
+      if (p.ord0 && ord_used && (l == 0 || (u.ord >= 2 && 16ull * p.cap[l] > kOrdMinBytes))) {
         oa.ord = (uint32_t *)(var + p.off_ord);
         oa.cum = (uint32_t *)(var + p.off_cum);
         oa.bits = bitmap;        // the has-predecessor bitmap is free once level 0's heads are chosen
         oa.pf_lead = u.pf << 10;
         LR_TRY(launch_order(desc, l, p.cap[l], bcnt, &oa, hout, p.hcap, err, s));
       }
-      LR_TRY(launch_chase(desc, l, work_of(l), r16, work_of(l + 1), ns,
+      LR_TRY(launch_chase(desc, l, work_of(l), kind, work_of(l + 1), ns,
                           qctr + (size_t)l * p.chase_grid, p.chase_grid, p.chase_block, err,
                           (int)u.xchg, tid_of(l), tid_of(l + 1), nullptr, oa.ord ? &oa : nullptr, s));
+      if (l == 0 && both)
+        LR_TRY(launch_chase(desc, 0, work0, kRecKind16, work_of(1), ns, qctr, p.chase_grid, p.chase_block, err,
+                            (int)u.xchg, nullptr, nullptr, nullptr, oa.ord ? &oa : nullptr, s));
     }
     if (l == 0) prof.call.log0 = log0;
     prof.mark(l == 0 ? PH_CHASE0 : PH_CHASE);
@@ -1060,16 +1105,24 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
                                  (uint2 *)(var + p.off_pairsB), (uint32_t *)(var + p.off_cur),
                                  (uint32_t *)(var + p.off_cur) + p.lg.na, p.lg, (uint32_t *)in.rank, err, s));
     else if (l == 0 && ptrs)
-      LR_TRY(launch_finalize_ptrs(desc, work0, rec16_0, R_of(1), in.rptr, p.rank_bytes, p.cap[0],
+      LR_TRY(launch_finalize_ptrs(desc, work0, kind0, R_of(1), in.rptr, p.rank_bytes, p.cap[0],
                                   in.offsets, in.k, err, s));
     else if (l == 0 && p.spawn_cap) {
       LR_TRY(launch_spawn_scatter(desc, 0, R_of(1), var + p.off_srraw, p.rank_bytes, spa.used,
                                   (uint32_t *)(var + p.off_supre), p.raw_cap, s));
-      LR_TRY(launch_finalize(desc, 0, work0, rec16_0, var + p.off_srraw, R_of(0), p.rank_bytes, p.cap[0],
+      LR_TRY(launch_finalize(desc, 0, work0, kind0, var + p.off_srraw, R_of(0), p.rank_bytes, p.cap[0],
                              err, nullptr, nullptr, nullptr, s));
     } else
-      LR_TRY(launch_finalize(desc, l, work_of(l), l > 0 || rec16_0, R_of(l + 1), R_of(l),
+      LR_TRY(launch_finalize(desc, l, work_of(l), l > 0 ? (int)kRecKind16 : kind0, R_of(l + 1), R_of(l),
                              p.rank_bytes, p.cap[l], err, T_of(l + 1), T_of(l), tid_of(l), s));
+    if (l == 0 && both) {
+      if (ptrs)
+        LR_TRY(launch_finalize_ptrs(desc, work0, kRecKind16, R_of(1), in.rptr, p.rank_bytes, p.cap[0], in.offsets,
+                                    in.k, err, s));
+      else
+        LR_TRY(launch_finalize(desc, 0, work0, kRecKind16, R_of(1), R_of(0), p.rank_bytes, p.cap[0], err, nullptr,
+                               nullptr, nullptr, s));
+    }
   }
   if (extras)
     LR_TRY(launch_outputs(desc, bitmap, hA, (uint32_t)in.n, T0, in.rank, in.prefix, p.rank_bytes,
@@ -1459,7 +1512,8 @@ size_t lr_workspace_size_outputs(int64_t n_total, int32_t k, const lr_outputs *o
   Plan p = make_plan((uint64_t)n_total, h, u,
                      opts->wtype != LR_NONE || (extras && (uint64_t)n_total <= u.base0),
                      opts->rtype == LR_I64 ? 8 : 4, opts->seed, 256 * 16, log0, extras,
-                     extras && !outs->term, spawn0, ord0);
+                     extras && !outs->term, spawn0, ord0,
+                     use_narrow(u, (uint64_t)n_total, opts->wtype != LR_NONE, spawn0, extras, true));
   return p.fixed_bytes + p.var_bytes;
 }
 

@@ -77,11 +77,13 @@ Tuning resolve_tuning(const lr_tuning *t, int64_t n, bool weighted, bool batch);
 Tuning resolve_tuning_builtin(int64_t n, bool weighted, bool batch = false);
 // Autotuned entry for a call of this shape (lr_tune.cu).
 bool tuned_lookup(int64_t n, bool weighted, bool batch, lr_tuning *out);
+// narrow: level 0 may hold 8-byte weighted records (room for 16-byte ones is
+// kept, and for the rulers that long segments add).
 // term: also lay out the terminal-id arrays of every level; t0ws: and the
 // level-0 terminal ids (when the caller does not receive them).
 Plan make_plan(uint64_t n, uint64_t h, const Tuning &u, bool rec16_0, int rank_bytes,
                uint64_t seed, int chase_grid, bool log0, bool term = false, bool t0ws = false,
-               bool spawn0 = false, bool ord0 = false);
+               bool spawn0 = false, bool ord0 = false, bool narrow = false);
 // Workspace that serves a single instance of any size up to n (lr_workspace_size
 // is for one size).
 size_t workspace_upto(int64_t n, const lr_opts *opts);

@@ -22,6 +22,7 @@
 #include <atomic>
 #include <cstdio>
 #include <cstring>
+#include <type_traits>
 
 #include "lr_kernels.h"
 
@@ -75,6 +76,7 @@ __device__ __forceinline__ void init_levels(LevelDesc *desc, const InitParams &p
     x.cap = p.cap[l];
     x.seed = p.seed[l];
     x.hsrc = l == 0 ? (uint32_t)kHeadsBitmap : (uint32_t)kHeadsList;
+    x.narrow = kNarrowNone;
     x.picked = 0;
     x.nraw = 0;
     x.check = 0;
@@ -95,12 +97,14 @@ __device__ __forceinline__ void open_level(LevelDesc &e, uint64_t n1, uint32_t h
 // other successors are every id but the head's) its head and level 0's choice
 // of rulers, which otherwise takes five more launches.
 __global__ void __launch_bounds__(32)
-k_init(LevelDesc *desc, InitParams p, const unsigned long long *__restrict__ acc, uint32_t *__restrict__ hlist0,
-       uint32_t *__restrict__ ns, uint32_t *__restrict__ hnext) {
+k_init(LevelDesc *desc, InitParams p, const unsigned long long *__restrict__ acc, const uint32_t *__restrict__ wflags,
+       uint32_t *__restrict__ hlist0, uint32_t *__restrict__ ns, uint32_t *__restrict__ hnext) {
   init_levels(desc, p, (int)threadIdx.x);
   __syncwarp();
-  if (threadIdx.x != 0 || !acc || p.nlev < 2) return;
+  if (threadIdx.x != 0) return;
   LevelDesc &d = desc[0];
+  if (wflags) d.narrow = narrow_mode(*wflags);
+  if (!acc || p.nlev < 2) return;
   const unsigned long long n = p.n0, h = n * (n - 1) / 2 - acc[1];
   if (acc[0] != 1 || h >= n) return;
   hlist0[0] = (uint32_t)h;
@@ -118,9 +122,9 @@ k_init(LevelDesc *desc, InitParams p, const unsigned long long *__restrict__ acc
   open_level(desc[1], (uint64_t)r + d.k, 1u, p.nlev == 2, p.base);
 }
 
-cudaError_t launch_init(LevelDesc *desc, const InitParams &p, const unsigned long long *acc, uint32_t *hlist0,
-                        uint32_t *ns, uint32_t *hnext, cudaStream_t s) {
-  k_init<<<1, 32, 0, s>>>(desc, p, acc, hlist0, ns, hnext);
+cudaError_t launch_init(LevelDesc *desc, const InitParams &p, const unsigned long long *acc, const uint32_t *wflags,
+                        uint32_t *hlist0, uint32_t *ns, uint32_t *hnext, cudaStream_t s) {
+  k_init<<<1, 32, 0, s>>>(desc, p, acc, wflags, hlist0, ns, hnext);
   count_launch();
   return cudaGetLastError();
 }
@@ -133,6 +137,50 @@ __device__ __forceinline__ uint64_t load_weight(const void *w, uint32_t i) {
   else return 1u;
 }
 
+// Write the records of elements i0 .. i0 + cnt - 1 (cnt <= 4; i0 a multiple of
+// 4), whole sectors at a time.
+template <int KIND>
+__device__ __forceinline__ void store_records(void *work, uint32_t i0, uint32_t cnt, const uint32_t (&s)[4],
+                                              const uint64_t (&w)[4]) {
+  if constexpr (KIND == kRecKind16) {
+    uint4 *out = reinterpret_cast<uint4 *>(work) + i0;
+    if (cnt == 4u) {
+      st_sector(out, s[0], kUnvisited, (uint32_t)w[0], (uint32_t)(w[0] >> 32),
+                s[1], kUnvisited, (uint32_t)w[1], (uint32_t)(w[1] >> 32));
+      st_sector(out + 2, s[2], kUnvisited, (uint32_t)w[2], (uint32_t)(w[2] >> 32),
+                s[3], kUnvisited, (uint32_t)w[3], (uint32_t)(w[3] >> 32));
+    } else {
+      for (uint32_t j = 0; j < cnt; ++j)
+        __stcs(out + j, make_uint4(s[j], kUnvisited, (uint32_t)w[j], (uint32_t)(w[j] >> 32)));
+    }
+  } else {
+    uint32_t hi[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) hi[j] = KIND == kRecKind8w ? (uint32_t)w[j] : kUnvisited;
+    uint2 *out = reinterpret_cast<uint2 *>(work) + i0;
+    if (cnt == 4u) {
+      st_sector(out, s[0], hi[0], s[1], hi[1], s[2], hi[2], s[3], hi[3]);
+    } else {
+      for (uint32_t j = 0; j < cnt; ++j) out[j] = make_uint2(s[j], hi[j]);
+    }
+  }
+}
+
+// One record of a coalesced run.
+template <int KIND>
+__device__ __forceinline__ void store_record(void *work, size_t i, uint32_t s, uint64_t w) {
+  if constexpr (KIND == kRecKind16)
+    __stcs(reinterpret_cast<uint4 *>(work) + i, make_uint4(s, kUnvisited, (uint32_t)w, (uint32_t)(w >> 32)));
+  else
+    reinterpret_cast<uint2 *>(work)[i] = make_uint2(s, KIND == kRecKind8w ? (uint32_t)w : kUnvisited);
+}
+
+// Add a thread's flags to the call's (whole warps).
+__device__ __forceinline__ void add_flags(uint32_t *flags, uint32_t mine) {
+  mine = __reduce_or_sync(0xFFFFFFFFu, mine);
+  if (mine && (threadIdx.x & 31u) == 0) atomicOr(flags, mine);
+}
+
 // One pass over the input: check every successor, mark the has-predecessor
 // bit of every successor (the complement gives the heads, Algorithm 1's
 // findInit), and pack {succ, kUnvisited[, link weight]} records.  A terminal's
@@ -142,15 +190,17 @@ __device__ __forceinline__ uint64_t load_weight(const void *w, uint32_t i) {
 // and the sum of the other successors (single-list head, see k_init).
 // Neither: an input small enough for the base case, which needs no heads.
 // desc != nullptr: also write the level descriptors (saves k_init's launch).
-// WIDE: 16-byte records (always when weighted; unweighted, weight 1, when the
-// level's records are to carry terminal ids).
-template <int WT, bool WIDE>
+// KIND: the records (unweighted input may have 16-byte ones too, weight 1, when
+// they are to carry terminal ids).
+template <int WT, int KIND>
 __global__ void __launch_bounds__(256)
 k_prep0(const uint32_t *__restrict__ succ, const void *__restrict__ weight, uint32_t n,
         void *__restrict__ work, uint32_t *__restrict__ bitmap, uint32_t *__restrict__ err,
         int validate, int vec, const int64_t *__restrict__ offsets, int32_t k,
         unsigned long long *__restrict__ sums, unsigned long long *__restrict__ local,
-        LevelDesc *__restrict__ desc, InitParams ip) {
+        WeightScan scan, LevelDesc *__restrict__ desc, InitParams ip) {
+  if (scan.unless_narrow && narrow_mode(*scan.unless_narrow)) return;
+  uint32_t wide = 0;
   if (desc && blockIdx.x == 0) init_levels(desc, ip, (int)threadIdx.x);
   unsigned long long sT = 0, sS = 0, sL = 0;
   const uint32_t ngroups = (uint32_t)(((uint64_t)n + 3u) / 4u);
@@ -222,26 +272,11 @@ k_prep0(const uint32_t *__restrict__ succ, const void *__restrict__ weight, uint
         sT += 1;
       }
     }
-    if constexpr (!WIDE) {
-      uint2 *out = reinterpret_cast<uint2 *>(work) + i0;
-      if (cnt == 4u) {
-        st_sector(out, s[0], kUnvisited, s[1], kUnvisited, s[2], kUnvisited, s[3], kUnvisited);
-      } else {
-        for (uint32_t j = 0; j < cnt; ++j) out[j] = make_uint2(s[j], kUnvisited);
-      }
-    } else {
-      uint4 *out = reinterpret_cast<uint4 *>(work) + i0;
-      if (cnt == 4u) {
-        st_sector(out, s[0], kUnvisited, (uint32_t)w[0], (uint32_t)(w[0] >> 32),
-                  s[1], kUnvisited, (uint32_t)w[1], (uint32_t)(w[1] >> 32));
-        st_sector(out + 2, s[2], kUnvisited, (uint32_t)w[2], (uint32_t)(w[2] >> 32),
-                  s[3], kUnvisited, (uint32_t)w[3], (uint32_t)(w[3] >> 32));
-      } else {
-        for (uint32_t j = 0; j < cnt; ++j)
-          __stcs(out + j, make_uint4(s[j], kUnvisited, (uint32_t)w[j], (uint32_t)(w[j] >> 32)));
-      }
-    }
+    store_records<KIND>(work, i0, cnt, s, w);
+    if constexpr (KIND == kRecKind8w)
+      for (uint32_t j = 0; j < cnt; ++j) wide |= wide_flags(w[j]);
   }
+  if (KIND == kRecKind8w && scan.flags) add_flags(scan.flags, wide);
   if (sums) {
     for (int d = 16; d > 0; d >>= 1) {
       sS += __shfl_down_sync(0xFFFFFFFFu, sS, d);
@@ -260,9 +295,10 @@ k_prep0(const uint32_t *__restrict__ succ, const void *__restrict__ weight, uint
 }
 
 cudaError_t launch_prep0(const uint32_t *succ, const void *weight, int wtype, uint32_t n,
-                         void *work, bool rec16, uint32_t *bitmap, uint32_t *err, int validate,
+                         void *work, int kind, uint32_t *bitmap, uint32_t *err, int validate,
                          const int64_t *offsets, int32_t k, unsigned long long *sums,
-                         unsigned long long *local, LevelDesc *desc, const InitParams *init, cudaStream_t s) {
+                         unsigned long long *local, const WeightScan &ws, LevelDesc *desc, const InitParams *init,
+                         cudaStream_t s) {
   if (n == 0) return cudaSuccess;
   InitParams ip;
   memset(&ip, 0, sizeof(ip));
@@ -272,13 +308,14 @@ cudaError_t launch_prep0(const uint32_t *succ, const void *weight, int wtype, ui
   int vec = ((uintptr_t)succ & 15u) == 0;
   if (wtype == 1) vec = vec && ((uintptr_t)weight & 15u) == 0;
   if (wtype == 2) vec = vec && ((uintptr_t)weight & 15u) == 0;
-#define LR_PREP0(WT, WIDE) \
-  k_prep0<WT, WIDE><<<grid, block, 0, s>>>(succ, weight, n, work, bitmap, err, validate, vec, offsets, k, sums, local, \
-                                           desc, ip)
+#define LR_PREP0(WT, KIND)                                                                                        \
+  k_prep0<WT, KIND><<<grid, block, 0, s>>>(succ, weight, n, work, bitmap, err, validate, vec, offsets, k, sums,    \
+                                           local, ws, desc, ip)
+  const bool w8 = kind == kRecKind8w;
   switch (wtype) {
-    case 0: if (rec16) LR_PREP0(0, true); else LR_PREP0(0, false); break;
-    case 1: LR_PREP0(1, true); break;
-    default: LR_PREP0(2, true); break;
+    case 0: if (kind == kRecKind16) LR_PREP0(0, kRecKind16); else LR_PREP0(0, kRecKind8); break;
+    case 1: if (w8) LR_PREP0(1, kRecKind8w); else LR_PREP0(1, kRecKind16); break;
+    default: if (w8) LR_PREP0(2, kRecKind8w); else LR_PREP0(2, kRecKind16); break;
   }
 #undef LR_PREP0
   count_launch();
@@ -330,11 +367,13 @@ cudaError_t launch_local_sample(const uint32_t *succ, uint32_t n, unsigned long 
 // j's terminals and isums[2 j + 1] sums its local successors; a warp whose
 // 128 elements lie in one instance adds its sums with two atomics.  Records
 // as in k_prep0.  The loop runs warp-uniformly so that the warp can combine.
-template <int WT>
+template <int WT, int KIND>
 __global__ void __launch_bounds__(256)
 k_prep0_sums(const uint32_t *__restrict__ succ, const void *__restrict__ weight, uint32_t n,
-             void *__restrict__ work, uint32_t *__restrict__ err, int vec, const int64_t *__restrict__ offsets,
+             void *__restrict__ work, WeightScan scan, uint32_t *__restrict__ err, int vec, const int64_t *__restrict__ offsets,
              int32_t k, unsigned long long *__restrict__ isums) {
+  if (scan.unless_narrow && narrow_mode(*scan.unless_narrow)) return;
+  uint32_t wide = 0;
   const uint32_t ngroups = (uint32_t)(((uint64_t)n + 3u) / 4u);
   const uint32_t stride = gridDim.x * blockDim.x;
   const uint32_t lane = threadIdx.x & 31u;
@@ -401,7 +440,7 @@ k_prep0_sums(const uint32_t *__restrict__ succ, const void *__restrict__ weight,
       }
       if (first >= 0) {
         inst = first;
-      } else if (first == -1) {            // rare: add each element's share alone
+      } else if (first == -1 && isums) {   // rare: add each element's share alone
         sT = 0; sS = 0;
         uint64_t b2 = (uint64_t)__ldg(offsets + lo);
         int32_t l2 = lo;
@@ -412,26 +451,11 @@ k_prep0_sums(const uint32_t *__restrict__ succ, const void *__restrict__ weight,
           else atomicAdd(isums + 2 * (size_t)l2 + 1, (unsigned long long)(s[jj] - b2));
         }
       }
-      if constexpr (WT == 0) {
-        uint2 *out = reinterpret_cast<uint2 *>(work) + i0;
-        if (cnt == 4u) {
-          st_sector(out, s[0], kUnvisited, s[1], kUnvisited, s[2], kUnvisited, s[3], kUnvisited);
-        } else {
-          for (uint32_t j = 0; j < cnt; ++j) out[j] = make_uint2(s[j], kUnvisited);
-        }
-      } else {
-        uint4 *out = reinterpret_cast<uint4 *>(work) + i0;
-        if (cnt == 4u) {
-          st_sector(out, s[0], kUnvisited, (uint32_t)w[0], (uint32_t)(w[0] >> 32),
-                    s[1], kUnvisited, (uint32_t)w[1], (uint32_t)(w[1] >> 32));
-          st_sector(out + 2, s[2], kUnvisited, (uint32_t)w[2], (uint32_t)(w[2] >> 32),
-                    s[3], kUnvisited, (uint32_t)w[3], (uint32_t)(w[3] >> 32));
-        } else {
-          for (uint32_t j = 0; j < cnt; ++j)
-            __stcs(out + j, make_uint4(s[j], kUnvisited, (uint32_t)w[j], (uint32_t)(w[j] >> 32)));
-        }
-      }
+      store_records<KIND>(work, i0, cnt, s, w);
+      if constexpr (KIND == kRecKind8w)
+        for (uint32_t j = 0; j < cnt; ++j) wide |= wide_flags(w[j]);
     }
+    if (!isums) continue;
     // combine: one pair of atomics per warp when all its lanes share an instance
     const int32_t inst0 = __shfl_sync(0xFFFFFFFFu, inst, 0);
     if (__all_sync(0xFFFFFFFFu, inst == inst0 || (inst == -1 && sT == 0 && sS == 0)) && inst0 >= 0) {
@@ -448,21 +472,26 @@ k_prep0_sums(const uint32_t *__restrict__ succ, const void *__restrict__ weight,
       if (sS) atomicAdd(isums + 2 * (size_t)inst + 1, sS);
     }
   }
+  if (KIND == kRecKind8w && scan.flags) add_flags(scan.flags, wide);
 }
 
-cudaError_t launch_prep0_sums(const uint32_t *succ, const void *weight, int wtype, uint32_t n, void *work,
-                              uint32_t *err, const int64_t *offsets, int32_t k, unsigned long long *isums,
+cudaError_t launch_prep0_sums(const uint32_t *succ, const void *weight, int wtype, uint32_t n, void *work, int kind,
+                              const WeightScan &ws, uint32_t *err, const int64_t *offsets, int32_t k, unsigned long long *isums,
                               cudaStream_t s) {
   if (n == 0) return cudaSuccess;
   const int block = 256;
   const int grid = stream_grid(((uint64_t)n + 3) / 4, block);
   int vec = ((uintptr_t)succ & 15u) == 0;
   if (wtype != 0) vec = vec && ((uintptr_t)weight & 15u) == 0;
+#define LR_SUMS(WT, KIND) \
+  k_prep0_sums<WT, KIND><<<grid, block, 0, s>>>(succ, weight, n, work, ws, err, vec, offsets, k, isums)
+  const bool w8 = kind == kRecKind8w;
   switch (wtype) {
-    case 0: k_prep0_sums<0><<<grid, block, 0, s>>>(succ, weight, n, work, err, vec, offsets, k, isums); break;
-    case 1: k_prep0_sums<1><<<grid, block, 0, s>>>(succ, weight, n, work, err, vec, offsets, k, isums); break;
-    default: k_prep0_sums<2><<<grid, block, 0, s>>>(succ, weight, n, work, err, vec, offsets, k, isums); break;
+    case 0: LR_SUMS(0, kRecKind8); break;
+    case 1: if (w8) LR_SUMS(1, kRecKind8w); else LR_SUMS(1, kRecKind16); break;
+    default: if (w8) LR_SUMS(2, kRecKind8w); else LR_SUMS(2, kRecKind16); break;
   }
+#undef LR_SUMS
   count_launch();
   return cudaGetLastError();
 }
@@ -520,6 +549,7 @@ __global__ void __launch_bounds__(256)
 k_bitmap0_recs(const LevelDesc *__restrict__ desc, const uint32_t *__restrict__ recs, uint32_t words_per_rec,
                uint32_t n, uint32_t *__restrict__ bitmap) {
   if (desc[0].hsrc != kHeadsBitmap) return;
+  if (words_per_rec == 0) words_per_rec = desc[0].narrow ? 2u : 4u;      // kind 8w: as the level decided
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const uint32_t s = __ldcs(recs + (size_t)i * words_per_rec);
     if (s != i) atomicOr(bitmap + (s >> 5), 1u << (s & 31u));
@@ -544,22 +574,25 @@ cudaError_t launch_count_batch(const unsigned long long *isums, int32_t k, uint3
 }
 
 cudaError_t launch_heads0_batch(LevelDesc *desc, unsigned long long *isums, const int64_t *offsets, int32_t k,
-                                uint32_t *hlist0, uint32_t hcap, const void *work, bool rec16, uint32_t n,
+                                uint32_t *hlist0, uint32_t hcap, const void *work, int kind, uint32_t n,
                                 uint32_t *bitmap, cudaStream_t s) {
   k_heads0_batch<<<1, 1024, 0, s>>>(desc, isums, offsets, k, hlist0, hcap, n);
   k_bitmap0_recs<<<stream_grid(n, 256), 256, 0, s>>>(desc, reinterpret_cast<const uint32_t *>(work),
-                                                      rec16 ? 4u : 2u, n, bitmap);
+                                                      kind == kRecKind8w ? 0u : kind == kRecKind16 ? 4u : 2u, n,
+                                                      bitmap);
   count_launch(2);
   return cudaGetLastError();
 }
 
 // Batched input given as one device pointer per instance (the serving path
 // ranks requests where they already live, without gathering them first).
-template <int WT>
+template <int WT, int KIND>
 __global__ void __launch_bounds__(256)
 k_prep0_ptrs(const uint32_t *const *__restrict__ sptr, const void *const *__restrict__ wptr,
-             uint32_t n, void *__restrict__ work, uint32_t *__restrict__ bitmap,
+             uint32_t n, void *__restrict__ work, WeightScan scan, uint32_t *__restrict__ bitmap,
              uint32_t *__restrict__ err, int validate, const int64_t *__restrict__ offsets, int32_t k) {
+  if (scan.unless_narrow && narrow_mode(*scan.unless_narrow)) return;
+  uint32_t wide = 0;
   const uint32_t stride = gridDim.x * blockDim.x;
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
     int32_t lo = 0, hi = k;
@@ -577,7 +610,8 @@ k_prep0_ptrs(const uint32_t *const *__restrict__ sptr, const void *const *__rest
     else s = (uint32_t)(base + s);
     if (s != i) {
       const uint32_t bit = 1u << (s & 31u);
-      if (validate) {
+      if (!bitmap) {
+      } else if (validate) {
         if (atomicOr(bitmap + (s >> 5), bit) & bit) record_error(err, kErrNotList);
       } else {
         atomicOr(bitmap + (s >> 5), bit);
@@ -585,22 +619,27 @@ k_prep0_ptrs(const uint32_t *const *__restrict__ sptr, const void *const *__rest
     } else {
       w = 0u;
     }
-    if constexpr (WT == 0) reinterpret_cast<uint2 *>(work)[i] = make_uint2(s, kUnvisited);
-    else __stcs(reinterpret_cast<uint4 *>(work) + i, make_uint4(s, kUnvisited, (uint32_t)w, (uint32_t)(w >> 32)));
+    store_record<KIND>(work, i, s, w);
+    if constexpr (KIND == kRecKind8w) wide |= wide_flags(w);
   }
+  if (KIND == kRecKind8w && scan.flags) add_flags(scan.flags, wide);
 }
 
 cudaError_t launch_prep0_ptrs(const uint32_t *const *sptr, const void *const *wptr, int wtype,
-                              uint32_t n, void *work, uint32_t *bitmap, uint32_t *err, int validate,
-                              const int64_t *offsets, int32_t k, cudaStream_t s) {
+                              uint32_t n, void *work, int kind, const WeightScan &ws, uint32_t *bitmap, uint32_t *err,
+                              int validate, const int64_t *offsets, int32_t k, cudaStream_t s) {
   if (n == 0) return cudaSuccess;
   const int block = 256;
   const int grid = stream_grid(n, block);
+#define LR_PTRS(WT, KIND) \
+  k_prep0_ptrs<WT, KIND><<<grid, block, 0, s>>>(sptr, wptr, n, work, ws, bitmap, err, validate, offsets, k)
+  const bool w8 = kind == kRecKind8w;
   switch (wtype) {
-    case 0: k_prep0_ptrs<0><<<grid, block, 0, s>>>(sptr, wptr, n, work, bitmap, err, validate, offsets, k); break;
-    case 1: k_prep0_ptrs<1><<<grid, block, 0, s>>>(sptr, wptr, n, work, bitmap, err, validate, offsets, k); break;
-    default: k_prep0_ptrs<2><<<grid, block, 0, s>>>(sptr, wptr, n, work, bitmap, err, validate, offsets, k); break;
+    case 0: LR_PTRS(0, kRecKind8); break;
+    case 1: if (w8) LR_PTRS(1, kRecKind8w); else LR_PTRS(1, kRecKind16); break;
+    default: if (w8) LR_PTRS(2, kRecKind8w); else LR_PTRS(2, kRecKind16); break;
   }
+#undef LR_PTRS
   count_launch();
   return cudaGetLastError();
 }
@@ -632,11 +671,13 @@ __device__ __forceinline__ int32_t warp_instance(const int64_t *__restrict__ off
 // loads and record stores are coalesced); the warp finds the instance of
 // the first (warp_instance) and every lane walks forward from it.  A warp
 // whose elements all lie in one instance adds its sums with two atomics.
-template <int WT>
+template <int WT, int KIND>
 __global__ void __launch_bounds__(256)
 k_prep0_ptrs_sums(const uint32_t *const *__restrict__ sptr, const void *const *__restrict__ wptr,
-                  uint32_t n, void *__restrict__ work, uint32_t *__restrict__ err,
+                  uint32_t n, void *__restrict__ work, WeightScan scan, uint32_t *__restrict__ err,
                   const int64_t *__restrict__ offsets, int32_t k, unsigned long long *__restrict__ isums) {
+  if (scan.unless_narrow && narrow_mode(*scan.unless_narrow)) return;
+  uint32_t wide = 0;
   const uint32_t lane = threadIdx.x & 31u;
   const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const uint64_t step = ((uint64_t)gridDim.x * blockDim.x >> 5) * 128u;
@@ -692,19 +733,19 @@ k_prep0_ptrs_sums(const uint32_t *const *__restrict__ sptr, const void *const *_
         term = (uint64_t)s == i - ib;
         if (!term) {
           if (one) sS += s;
-          else atomicAdd(isums + 2 * (size_t)inst[j] + 1, (unsigned long long)s);
+          else if (isums) atomicAdd(isums + 2 * (size_t)inst[j] + 1, (unsigned long long)s);
         }
         s = (uint32_t)(ib + s);
       }
       if (term) {
         w = 0u;
         if (one) sT += 1;
-        else atomicAdd(isums + 2 * (size_t)inst[j], 1ull);
+        else if (isums) atomicAdd(isums + 2 * (size_t)inst[j], 1ull);
       }
-      if constexpr (WT == 0) reinterpret_cast<uint2 *>(work)[i] = make_uint2(s, kUnvisited);
-      else __stcs(reinterpret_cast<uint4 *>(work) + i, make_uint4(s, kUnvisited, (uint32_t)w, (uint32_t)(w >> 32)));
+      store_record<KIND>(work, i, s, w);
+      if constexpr (KIND == kRecKind8w) wide |= wide_flags(w);
     }
-    if (one) {
+    if (one && isums) {
       for (int d = 16; d > 0; d >>= 1) {
         sT += __shfl_down_sync(0xFFFFFFFFu, sT, d);
         sS += __shfl_down_sync(0xFFFFFFFFu, sS, d);
@@ -715,19 +756,24 @@ k_prep0_ptrs_sums(const uint32_t *const *__restrict__ sptr, const void *const *_
       }
     }
   }
+  if (KIND == kRecKind8w && scan.flags) add_flags(scan.flags, wide);
 }
 
 cudaError_t launch_prep0_ptrs_sums(const uint32_t *const *sptr, const void *const *wptr, int wtype, uint32_t n,
-                                   void *work, uint32_t *err, const int64_t *offsets, int32_t k,
-                                   unsigned long long *isums, cudaStream_t s) {
+                                   void *work, int kind, const WeightScan &ws, uint32_t *err, const int64_t *offsets,
+                                   int32_t k, unsigned long long *isums, cudaStream_t s) {
   if (n == 0) return cudaSuccess;
   const int block = 256;
   const int grid = stream_grid(((uint64_t)n + 3) / 4, block);
+#define LR_PTRS_SUMS(WT, KIND) \
+  k_prep0_ptrs_sums<WT, KIND><<<grid, block, 0, s>>>(sptr, wptr, n, work, ws, err, offsets, k, isums)
+  const bool w8 = kind == kRecKind8w;
   switch (wtype) {
-    case 0: k_prep0_ptrs_sums<0><<<grid, block, 0, s>>>(sptr, wptr, n, work, err, offsets, k, isums); break;
-    case 1: k_prep0_ptrs_sums<1><<<grid, block, 0, s>>>(sptr, wptr, n, work, err, offsets, k, isums); break;
-    default: k_prep0_ptrs_sums<2><<<grid, block, 0, s>>>(sptr, wptr, n, work, err, offsets, k, isums); break;
+    case 0: LR_PTRS_SUMS(0, kRecKind8); break;
+    case 1: if (w8) LR_PTRS_SUMS(1, kRecKind8w); else LR_PTRS_SUMS(1, kRecKind16); break;
+    default: if (w8) LR_PTRS_SUMS(2, kRecKind8w); else LR_PTRS_SUMS(2, kRecKind16); break;
   }
+#undef LR_PTRS_SUMS
   count_launch();
   return cudaGetLastError();
 }
@@ -759,13 +805,17 @@ enum : int { kCatSampled = 0, kCatNew = 1, kCatSingle = 2 };
 // Classify head x of a level: a sampled ruler keeps id pi(x); a head that is
 // also a terminal is a one-element list whose rank is its own weight
 // (resolved here, never chased); any other head becomes an extra ruler.
+// (A level of 8-byte weighted records: `narrow` says whether it has them.)
 template <class Rec, bool RESOLVE>
-__device__ __forceinline__ int classify_head(uint32_t x, const Perm &P, uint32_t r,
+__device__ __forceinline__ int classify_head(uint32_t x, const Perm &P, uint32_t r, uint32_t narrow,
                                              const Rec *work, uint32_t *pid, uint64_t *wself) {
   const uint32_t p = P.fwd(x);
   *pid = p;
   if (p < r) return kCatSampled;
-  if constexpr (RESOLVE) {
+  if constexpr (RESOLVE && std::is_same<Rec, Rec8w>::value) {
+    const uint32_t s = narrow ? ld_rec(work + x).lo : ld_rec(reinterpret_cast<const Rec16 *>(work) + x).succ;
+    if (s == x) { *wself = 0; return kCatSingle; }     // level 0: a terminal weighs 0
+  } else if constexpr (RESOLVE) {
     Rec v = ld_rec(work + x);
     if (rec_succ(v) == x) { *wself = rec_weight(v, x); return kCatSingle; }
   }
@@ -811,7 +861,7 @@ k_heads_count(const LevelDesc *__restrict__ desc, int lev, const uint32_t *__res
   for_each_head(d, bitmap, hlist, [&](uint32_t x) {
     uint32_t p;
     uint64_t w;
-    const int c = classify_head<Rec, RESOLVE>(x, P, d.r, work, &p, &w);
+    const int c = classify_head<Rec, RESOLVE>(x, P, d.r, d.narrow, work, &p, &w);
     nS += c == kCatSampled;
     nN += c == kCatNew;
   });
@@ -861,7 +911,7 @@ k_heads_write(LevelDesc *__restrict__ desc, int lev, const uint32_t *__restrict_
   for_each_head(d, bitmap, hlist, [&](uint32_t x) {
     uint32_t p;
     uint64_t w;
-    const int c = classify_head<Rec, RESOLVE>(x, P, d.r, work, &p, &w);
+    const int c = classify_head<Rec, RESOLVE>(x, P, d.r, d.narrow, work, &p, &w);
     nS += c == kCatSampled;
     nN += c == kCatNew;
   });
@@ -871,7 +921,7 @@ k_heads_write(LevelDesc *__restrict__ desc, int lev, const uint32_t *__restrict_
   for_each_head(d, bitmap, hlist, [&](uint32_t x) {
     uint32_t p;
     uint64_t w;
-    const int c = classify_head<Rec, RESOLVE>(x, P, d.r, work, &p, &w);
+    const int c = classify_head<Rec, RESOLVE>(x, P, d.r, d.narrow, work, &p, &w);
     if (c == kCatSampled) {
       hnext[posH++] = p;
     } else if (c == kCatNew) {
@@ -879,7 +929,10 @@ k_heads_write(LevelDesc *__restrict__ desc, int lev, const uint32_t *__restrict_
       hnext[posH++] = d.r + posN;
       ++posN;
     } else {
-      st_rec(work + x, kZeroCid, (uint64_t)0 - w);   // R(x) = 0 - (-w) = w
+      if (std::is_same<Rec, Rec8w>::value && !d.narrow)
+        st_rec(reinterpret_cast<Rec16 *>(work) + x, kZeroCid, 0);
+      else
+        st_rec(work + x, kZeroCid, (uint64_t)0 - w);   // R(x) = 0 - (-w) = w
       ++nZ;
     }
   });
@@ -907,7 +960,7 @@ k_heads_few(LevelDesc *desc, int lev, int nlev, const uint32_t *__restrict__ hli
     int c = -1;
     if (e < d.h) {
       x = __ldcg(hlist + e);
-      c = classify_head<Rec, true>(x, P, d.r, work, &p, &w);
+      c = classify_head<Rec, true>(x, P, d.r, d.narrow, work, &p, &w);
     }
     const bool isnew = c == kCatNew, ishead = isnew || c == kCatSampled;
     uint64_t total;
@@ -955,6 +1008,9 @@ cudaError_t launch_heads(LevelDesc *desc, int lev, int nlev, const uint32_t *bit
     case kRecKind16:
       LR_HEADS(k_heads_count, Rec16, true)(desc, lev, bitmap, hlist, reinterpret_cast<const Rec16 *>(work), blockcnt);
       break;
+    case kRecKind8w:
+      LR_HEADS(k_heads_count, Rec8w, true)(desc, lev, bitmap, hlist, reinterpret_cast<const Rec8w *>(work), blockcnt);
+      break;
     default:
       LR_HEADS(k_heads_count, Succ4, false)(desc, lev, bitmap, hlist, reinterpret_cast<const Succ4 *>(work), blockcnt);
       break;
@@ -966,6 +1022,9 @@ cudaError_t launch_heads(LevelDesc *desc, int lev, int nlev, const uint32_t *bit
       break;
     case kRecKind16:
       LR_HEADS(k_heads_write, Rec16, true)(desc, lev, bitmap, hlist, reinterpret_cast<Rec16 *>(work), ns, hnext, blockcnt);
+      break;
+    case kRecKind8w:
+      LR_HEADS(k_heads_write, Rec8w, true)(desc, lev, bitmap, hlist, reinterpret_cast<Rec8w *>(work), ns, hnext, blockcnt);
       break;
     default:
       LR_HEADS(k_heads_write, Succ4, false)(desc, lev, bitmap, hlist, reinterpret_cast<Succ4 *>(work), ns, hnext, blockcnt);
@@ -1220,6 +1279,17 @@ __device__ __forceinline__ Rec visit(Rec *p, uint32_t cid, uint64_t off) {
   }
 }
 
+// A level of one kind of weighted records is none of the other kind's business.
+template <class Rec>
+__device__ __forceinline__ bool wrong_kind(const LevelDesc &d) {
+  return std::is_same<Rec, Rec8w>::value ? !d.narrow : std::is_same<Rec, Rec16>::value && d.narrow;
+}
+
+// 8-byte weighted records: a segment of kNarrowSteps elements is cut there,
+// so that its offsets fit 32 bits; the walk goes on as a further ruler with
+// an id past all others (the next level's size counts them).  With 1/f rulers
+// drawn at random this happens once in e^(4096 / f) segments.
+//
 // TERM: a ruler whose segment ends at a terminal y becomes a terminal of the
 // next level; it records y's original id (y itself at level 0, tid_cur[y]
 // deeper) in tid_next, so the terminal of every element can be carried back.
@@ -1249,7 +1319,7 @@ k_chase(LevelDesc *__restrict__ desc, int lev, Rec *__restrict__ work, Rec16 *__
   const uint32_t *__restrict__ ord = oa.ord;
   __shared__ OrdQueue s_q;
   const LevelDesc d = desc[lev];
-  if (d.mode != kModeSrs) return;
+  if (d.mode != kModeSrs || wrong_kind<Rec>(d)) return;
   const uint32_t n = d.n, r = d.r;
   const uint64_t R = (uint64_t)r + d.k;
   if (ord && threadIdx.x == 0) {               // the CTA's first window and chunk
@@ -1353,8 +1423,8 @@ k_chase(LevelDesc *__restrict__ desc, int lev, Rec *__restrict__ work, Rec16 *__
     } else {
       break;
     }
-    uint64_t o = rec_weight(v, rho);
-    uint32_t steps = 1, nxt = c;
+    uint64_t o = rec_weight(v, rho, d.narrow);
+    uint32_t steps = 1, nxt = c, cut = kNarrowSteps;
     bad |= rec_tag(v) != kUnvisited;
     uint32_t y = rec_succ(v);
     uint32_t tend = (TERM && y == rho && rec_tag(v) == kUnvisited) ? rho : kEnd;
@@ -1368,6 +1438,15 @@ k_chase(LevelDesc *__restrict__ desc, int lev, Rec *__restrict__ work, Rec16 *__
           if (nxt == c) bad |= 2u;   // came back to itself: a cycle
           break;
         }
+        if (std::is_same<Rec, Rec8w>::value && steps == cut) {
+          const uint32_t more = atomicAdd(&desc[lev + 1].n, 1u);
+          if (more >= ncap) { bad |= 8u; break; }
+          __stcg(reinterpret_cast<uint4 *>(next + c),
+                 make_uint4(more, kUnvisited, (uint32_t)o, (uint32_t)(o >> 32)));
+          nxt = c = more;
+          o = 0;
+          cut = steps + kNarrowSteps;
+        }
         v = visit<XCHG>(work + y, c, o);
         if constexpr (SPAWN) {
           if (rec_is_claim(v)) {     // reached a spawned ruler
@@ -1380,7 +1459,7 @@ k_chase(LevelDesc *__restrict__ desc, int lev, Rec *__restrict__ work, Rec16 *__
         }
         ++steps;
         if (rec_tag(v) != kUnvisited) { bad |= 1u; break; }   // second predecessor
-        o += rec_weight(v, y);
+        o += rec_weight(v, y, d.narrow);
         const uint32_t s = rec_succ(v);
         if (s == y) {                // terminal: the reduced element is terminal too
           if constexpr (TERM) tend = y;
@@ -1400,11 +1479,12 @@ k_chase(LevelDesc *__restrict__ desc, int lev, Rec *__restrict__ work, Rec16 *__
   if (bad & 1u) record_error(err, kErrNotList);
   if (bad & 2u) record_error(err, kErrCycle);
   if (bad & 4u) record_error(err, kErrInternal);
+  if (bad & 8u) record_error(err, kErrCapacity);
   for (int dd = 16; dd > 0; dd >>= 1) visited += __shfl_down_sync(0xFFFFFFFFu, visited, dd);
   if ((threadIdx.x & 31) == 0 && visited) atomicAdd(&desc[lev].visited, visited);
 }
 
-cudaError_t launch_chase(LevelDesc *desc, int lev, void *work, bool rec16, void *next_work,
+cudaError_t launch_chase(LevelDesc *desc, int lev, void *work, int kind, void *next_work,
                          const uint32_t *ns, uint32_t *qctr, int grid, int block, uint32_t *err,
                          int xchg, const uint32_t *tid_cur, uint32_t *tid_next, const SpawnArgs *spawn,
                          const OrdArgs *ord, cudaStream_t s) {
@@ -1419,7 +1499,11 @@ cudaError_t launch_chase(LevelDesc *desc, int lev, void *work, bool rec16, void 
 #define LR_CHASE(REC, X, T, SP) \
   k_chase<REC, X, T, SP><<<grid, block, 0, s>>>(desc, lev, reinterpret_cast<REC *>(work), nx, ns, qctr, err, \
                                                 tid_cur, tid_next, sp, oa)
-  if (spawn) {
+  const bool rec16 = kind == kRecKind16;
+  if (kind == kRecKind8w) {
+    if (spawn || tid_next || !xchg) return cudaErrorInvalidValue;
+    LR_CHASE(Rec8w, true, false, false);
+  } else if (spawn) {
     if (rec16) LR_CHASE(Rec16, true, false, true);
     else LR_CHASE(Rec8, true, false, true);
   } else if (tid_next) {
@@ -1490,7 +1574,7 @@ k_finalize(const LevelDesc *__restrict__ desc, int lev, const Rec *__restrict__ 
            const uint32_t *__restrict__ tnext, uint32_t *__restrict__ tout,
            const uint32_t *__restrict__ tid_cur) {
   const LevelDesc d = desc[lev];
-  if (d.mode != kModeSrs) return;
+  if (d.mode != kModeSrs || wrong_kind<Rec>(d)) return;
   const uint32_t n = d.n, nn = d.nraw ? d.nraw : desc[lev + 1].n;
   uint32_t bad = 0;
   if (blockIdx.x == 0 && threadIdx.x == 0) bad |= level_errors(d, desc[lev + 1], err);
@@ -1511,7 +1595,7 @@ k_finalize(const LevelDesc *__restrict__ desc, int lev, const Rec *__restrict__ 
     for (int j = 0; j < 4; ++j) {
       const uint64_t i = base + lane + 32u * j;
       if (i < n) {
-        const RT r = propagate<RT>(done_cid(v[j]), done_off(v[j]), nn, rnext, bad);
+        const RT r = propagate<RT>(done_cid(v[j]), done_off(v[j], d.narrow), nn, rnext, bad);
         if constexpr (TERM) __stcs(tout + i, propagate_term(done_cid(v[j]), (uint32_t)i, nn, tnext, tid_cur));
         __stcs(rout + i, r);
       }
@@ -1527,7 +1611,7 @@ k_finalize_ptrs(const LevelDesc *__restrict__ desc, const Rec *__restrict__ work
                 const RT *__restrict__ rnext, RT *const *__restrict__ rptr,
                 const int64_t *__restrict__ offsets, int32_t k, uint32_t *__restrict__ err) {
   const LevelDesc d = desc[0];
-  if (d.mode != kModeSrs) return;
+  if (d.mode != kModeSrs || wrong_kind<Rec>(d)) return;
   const uint32_t n = d.n, nn = desc[1].n;
   uint32_t bad = 0;
   if (blockIdx.x == 0 && threadIdx.x == 0) bad |= level_errors(d, desc[1], err);
@@ -1550,7 +1634,7 @@ k_finalize_ptrs(const LevelDesc *__restrict__ desc, const Rec *__restrict__ work
     RT val[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      if (lane + 32u * j < rem) val[j] = propagate<RT>(done_cid(v[j]), done_off(v[j]), nn, rnext, bad);
+      if (lane + 32u * j < rem) val[j] = propagate<RT>(done_cid(v[j]), done_off(v[j], d.narrow), nn, rnext, bad);
     }
     int32_t lo = warp_instance(offsets, k, base, lane);
     uint32_t ib = (uint32_t)__ldg(offsets + lo), ie = (uint32_t)__ldg(offsets + lo + 1);
@@ -1567,7 +1651,7 @@ k_finalize_ptrs(const LevelDesc *__restrict__ desc, const Rec *__restrict__ work
   if (bad) record_error(err, bad);
 }
 
-cudaError_t launch_finalize_ptrs(LevelDesc *desc, const void *work, bool rec16, const void *rnext,
+cudaError_t launch_finalize_ptrs(LevelDesc *desc, const void *work, int kind, const void *rnext,
                                  void *const *rptr, int rank_bytes, uint32_t cap,
                                  const int64_t *offsets, int32_t k, uint32_t *err, cudaStream_t s) {
   const int block = 256;
@@ -1576,14 +1660,15 @@ cudaError_t launch_finalize_ptrs(LevelDesc *desc, const void *work, bool rec16, 
   k_finalize_ptrs<REC, RT><<<grid, block, 0, s>>>(desc, reinterpret_cast<const REC *>(work),      \
                                                   reinterpret_cast<const RT *>(rnext),            \
                                                   reinterpret_cast<RT *const *>(rptr), offsets, k, err)
-  if (rec16) { if (rank_bytes == 4) LR_FINP(Rec16, uint32_t); else LR_FINP(Rec16, unsigned long long); }
+  if (kind == kRecKind8w) { if (rank_bytes == 4) LR_FINP(Rec8w, uint32_t); else LR_FINP(Rec8w, unsigned long long); }
+  else if (kind == kRecKind16) { if (rank_bytes == 4) LR_FINP(Rec16, uint32_t); else LR_FINP(Rec16, unsigned long long); }
   else { if (rank_bytes == 4) LR_FINP(Rec8, uint32_t); else LR_FINP(Rec8, unsigned long long); }
 #undef LR_FINP
   count_launch();
   return cudaGetLastError();
 }
 
-cudaError_t launch_finalize(LevelDesc *desc, int lev, const void *work, bool rec16,
+cudaError_t launch_finalize(LevelDesc *desc, int lev, const void *work, int kind,
                             const void *rnext, void *rout, int rank_bytes, uint32_t cap,
                             uint32_t *err, const uint32_t *tnext, uint32_t *tout,
                             const uint32_t *tid_cur, cudaStream_t s) {
@@ -1594,7 +1679,11 @@ cudaError_t launch_finalize(LevelDesc *desc, int lev, const void *work, bool rec
                                                 reinterpret_cast<const RT *>(rnext),            \
                                                 reinterpret_cast<RT *>(rout), err, tnext,       \
                                                 tout, tid_cur)
-  if (tout) {
+  const bool rec16 = kind == kRecKind16;
+  if (kind == kRecKind8w) {
+    if (tout) return cudaErrorInvalidValue;
+    if (rank_bytes == 4) LR_FIN(Rec8w, uint32_t, false); else LR_FIN(Rec8w, unsigned long long, false);
+  } else if (tout) {
     if (rec16) { if (rank_bytes == 4) LR_FIN(Rec16, uint32_t, true); else LR_FIN(Rec16, unsigned long long, true); }
     else { if (rank_bytes == 4) LR_FIN(Rec8, uint32_t, true); else LR_FIN(Rec8, unsigned long long, true); }
   } else {

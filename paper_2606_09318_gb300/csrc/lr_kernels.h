@@ -10,7 +10,11 @@
 
 namespace lr {
 
-enum : int { kRecKind8 = 0, kRecKind16 = 1, kRecKindSucc = 2 };
+// Level records: unweighted, 16-byte, the raw successors (log form), or 8-byte
+// weighted.  A level 0 of kind 8w has its narrow mode in its descriptor, where
+// kNarrowNone says that it holds 16-byte records after all; launches for one
+// of the two kinds do nothing when the level is of the other.
+enum : int { kRecKind8 = 0, kRecKind16 = 1, kRecKindSucc = 2, kRecKind8w = 3 };
 
 struct InitParams {
   int32_t nlev;                       // levels in the plan (0..nlev-1)
@@ -41,42 +45,53 @@ int stream_grid(uint64_t work_items, int block);
 // successors of a single instance; where they show one list, its head goes to
 // hlist0 and level 0's rulers are chosen on the spot (ns, hnext: see
 // launch_heads, which then does nothing).
-cudaError_t launch_init(LevelDesc *desc, const InitParams &p, const unsigned long long *acc, uint32_t *hlist0,
-                        uint32_t *ns, uint32_t *hnext, cudaStream_t s);
+// wflags (optional): level 0 holds records of kind 8w, as the flags allow.
+cudaError_t launch_init(LevelDesc *desc, const InitParams &p, const unsigned long long *acc, const uint32_t *wflags,
+                        uint32_t *hlist0, uint32_t *ns, uint32_t *hnext, cudaStream_t s);
+
+// Weighted first passes: where to collect what the weights exceed (wide_flags;
+// zeroed; null when nobody asks), and for a second pass that packs 16-byte
+// records the flags of the first, which it runs by only if they are too wide.
+struct WeightScan {
+  uint32_t *flags;
+  const uint32_t *unless_narrow;
+};
 
 // Level-0 pass.  wtype 0/1/2 (none/i32/i64).  offsets != nullptr: batched
 // input with local successor ids (k instances).
-// rec16: 16-byte records (weighted input always has them).
+// kind: kRecKind8 (unweighted), kRecKind16 or kRecKind8w (weighted).
 // sums: the number of terminals and the sum of the other successors instead
 // of predecessor marks in bitmap (which may be null then, and when neither is
 // wanted).  desc (optional): also writes the level descriptors from *init.
 // local (optional): counts the links that stay inside their contraction tile.
 cudaError_t launch_prep0(const uint32_t *succ, const void *weight, int wtype, uint32_t n,
-                         void *work, bool rec16, uint32_t *bitmap, uint32_t *err, int validate,
+                         void *work, int kind, uint32_t *bitmap, uint32_t *err, int validate,
                          const int64_t *offsets, int32_t k, unsigned long long *sums,
-                         unsigned long long *local, LevelDesc *desc, const InitParams *init, cudaStream_t s);
+                         unsigned long long *local, const WeightScan &ws, LevelDesc *desc, const InitParams *init,
+                         cudaStream_t s);
 
 // Batched prep that sums each instance's terminals and local successors
 // (isums[2k], zeroed) instead of marking predecessors; then the level-0 head
 // list from those sums, or the bitmap from the records when some instance is
 // not one list.
-cudaError_t launch_prep0_sums(const uint32_t *succ, const void *weight, int wtype, uint32_t n, void *work,
-                              uint32_t *err, const int64_t *offsets, int32_t k, unsigned long long *isums,
+// (isums null: only the records.)
+cudaError_t launch_prep0_sums(const uint32_t *succ, const void *weight, int wtype, uint32_t n, void *work, int kind,
+                              const WeightScan &ws, uint32_t *err, const int64_t *offsets, int32_t k, unsigned long long *isums,
                               cudaStream_t s);
 cudaError_t launch_count_batch(const unsigned long long *isums, int32_t k, uint32_t *out, cudaStream_t s);
 cudaError_t launch_heads0_batch(LevelDesc *desc, unsigned long long *isums, const int64_t *offsets, int32_t k,
-                                uint32_t *hlist0, uint32_t hcap, const void *work, bool rec16, uint32_t n,
+                                uint32_t *hlist0, uint32_t hcap, const void *work, int kind, uint32_t n,
                                 uint32_t *bitmap, cudaStream_t s);
 cudaError_t launch_prep0_ptrs(const uint32_t *const *sptr, const void *const *wptr, int wtype,
-                              uint32_t n, void *work, uint32_t *bitmap, uint32_t *err, int validate,
+                              uint32_t n, void *work, int kind, const WeightScan &ws, uint32_t *bitmap, uint32_t *err, int validate,
                               const int64_t *offsets, int32_t k, cudaStream_t s);
 
 // The same sums for a batch given as one pointer per instance.
 cudaError_t launch_prep0_ptrs_sums(const uint32_t *const *sptr, const void *const *wptr, int wtype, uint32_t n,
-                                   void *work, uint32_t *err, const int64_t *offsets, int32_t k,
+                                   void *work, int kind, const WeightScan &ws, uint32_t *err, const int64_t *offsets, int32_t k,
                                    unsigned long long *isums, cudaStream_t s);
 
-cudaError_t launch_finalize_ptrs(LevelDesc *desc, const void *work, bool rec16, const void *rnext,
+cudaError_t launch_finalize_ptrs(LevelDesc *desc, const void *work, int kind, const void *rnext,
                                  void *const *rptr, int rank_bytes, uint32_t cap,
                                  const int64_t *offsets, int32_t k, uint32_t *err, cudaStream_t s);
 
@@ -136,7 +151,7 @@ cudaError_t launch_order(LevelDesc *desc, int lev, uint32_t cap, uint64_t *cnt, 
 // ord: nullptr (per-CTA slices of ruler ids, sampled ids pi(x)) or
 // launch_order's arrays: the chase takes its rulers in element order and
 // gives the sampled ones their ids in that order (no spawning).
-cudaError_t launch_chase(LevelDesc *desc, int lev, void *work, bool rec16, void *next_work,
+cudaError_t launch_chase(LevelDesc *desc, int lev, void *work, int kind, void *next_work,
                          const uint32_t *ns, uint32_t *qctr, int grid, int block, uint32_t *err,
                          int xchg, const uint32_t *tid_cur, uint32_t *tid_next, const SpawnArgs *spawn,
                          const OrdArgs *ord, cudaStream_t s);
@@ -183,7 +198,7 @@ uint32_t wyllie_rounds(uint64_t n);
 cudaError_t launch_wyllie(void *bufA, void *bufB, bool w16, uint32_t n, void *rank, int rank_bytes,
                           uint32_t *err, cudaStream_t s);
 
-cudaError_t launch_finalize(LevelDesc *desc, int lev, const void *work, bool rec16,
+cudaError_t launch_finalize(LevelDesc *desc, int lev, const void *work, int kind,
                             const void *rnext, void *rout, int rank_bytes, uint32_t cap,
                             uint32_t *err, const uint32_t *tnext, uint32_t *tout,
                             const uint32_t *tid_cur, cudaStream_t s);
