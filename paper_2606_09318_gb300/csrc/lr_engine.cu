@@ -432,6 +432,7 @@ void release_ctx(cudaStream_t stream) {
   if (c->hostpath) cudaFree(c->hostpath);
   if (c->contract) cudaFree(c->contract);
   if (c->contract2) cudaFree(c->contract2);
+  if (c->direct) cudaFree(c->direct);
   cudaFreeHost(c->host_words);
   delete c;
 }
@@ -695,9 +696,32 @@ static lr_status run_base(const Inputs &in, const Plan &p, bool checked, char *f
     prof.end();
     return finish_call(c, nullptr, in.sync, s);
   }
-  // the bitmap follows the words that start at zero
-  LR_TRY(cudaMemsetAsync(fixed + p.off_zero, 0,
-                         p.off_bitmap - p.off_zero + (marks ? 4 * (((size_t)n + 31) / 32) : 0), s));
+  // The error word, the list count and the marks start at zero.  The stream's
+  // own ones are left so by k_jump, which also reports the status: a call is
+  // two launches, where a clear before and a copy after them took another 9
+  // us.  Memory that is not the stream's own (or cannot be had now) is cleared.
+  JumpInput ji;
+  memset(&ji, 0, sizeof(ji));
+  bool own = !in.ws && !in.ctx && !in.err_ext && !extras && n <= kBase0Max;
+  const size_t own_bytes = 256 + kBase0Max / 8;
+  if (own && !c->direct) own = !stream_capturing(s) && ensure_buffer(&c->direct, &c->direct_bytes, own_bytes, s) == LR_OK;
+  if (own) {
+    // new, or a call that failed on the way left them as they were
+    if (!c->direct_clean) LR_TRY(cudaMemsetAsync(c->direct, 0, own_bytes, s));
+    c->direct_clean = false;
+    uint32_t *words = (uint32_t *)c->direct;
+    err = words;
+    ji.count = words + 16;
+    ji.ticket = words + 32;
+    ji.status = c->host_words;
+    bitmap = words + 64;
+    if (marks || in.sptr) ji.clear = bitmap;
+  } else {
+    // the bitmap follows the words that start at zero
+    LR_TRY(cudaMemsetAsync(fixed + p.off_zero, 0,
+                           p.off_bitmap - p.off_zero + (marks ? 4 * (((size_t)n + 31) / 32) : 0), s));
+    ji.count = (uint32_t *)(fixed + p.off_hcount);
+  }
   const InitParams ip = init_params(p);
   const int kind = p.rec16_0 ? kRecKind16 : kRecKind8;
   if (in.sptr) {
@@ -710,24 +734,22 @@ static lr_status run_base(const Inputs &in, const Plan &p, bool checked, char *f
   }
   if (!in.ctx) { c->last_desc = desc; c->last_nlev = 1; }
   prof.mark(PH_PREP);
-  JumpInput ji;
-  memset(&ji, 0, sizeof(ji));
   if (checked && in.max_lists > 0) {
     ji.max_lists = (uint64_t)in.max_lists;
     ji.bitmap = bitmap;
-    ji.count = (uint32_t *)(fixed + p.off_hcount);
   }
   ji.rptr = in.rptr;
   ji.offsets = in.offsets;
   ji.k = in.k;
   LR_TRY(launch_jump(desc, 0, work, p.rec16_0, in.rank, p.rank_bytes, n, err, nullptr, nullptr, T0, &ji, s));
+  if (own) c->direct_clean = true;
   prof.mark(PH_BASE);
   if (extras)
     LR_TRY(launch_outputs(desc, bitmap, nullptr, n, T0, in.rank, in.prefix, p.rank_bytes, in.incl, in.weight,
                           in.wtype, in.offsets, in.k, in.offsets != nullptr && in.term != nullptr, s));
   prof.mark(PH_FINAL);
   prof.end();
-  return finish_call(c, err, in.sync, s);
+  return finish_call(c, own ? nullptr : err, in.sync, s);
 }
 
 // Tile-local contraction (lr_contract.cu) around the ruling set: count the

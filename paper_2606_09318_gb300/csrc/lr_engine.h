@@ -62,6 +62,9 @@ struct Ctx {
   size_t contract_bytes = 0;
   void *contract2 = nullptr;        // and the contracted list
   size_t contract2_bytes = 0;
+  void *direct = nullptr;           // run_base's words and predecessor marks: zero between calls
+  size_t direct_bytes = 0;
+  bool direct_clean = false;
   uint32_t *host_words = nullptr;   // [0] device error bits, [1] head count, [2..3] tile-local
                                     // links, [4..7] sampled tile-local links and elements,
                                     // [8..9] int64 scratch

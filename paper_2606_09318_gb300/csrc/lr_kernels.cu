@@ -2021,6 +2021,14 @@ k_jump(LevelDesc *__restrict__ desc, int lev, Rec *work, RT *__restrict__ rout, 
       }
       if (heads) chk -= jump_hash(i, d.seed);
     }
+    if (in.clear) {                            // this warp was its chunks' marks' last reader
+      __syncwarp();
+#pragma unroll
+      for (int e = 0; e < kJumpElems; ++e) {
+        const uint32_t first = __shfl_sync(0xFFFFFFFFu, idx[e], 0);
+        if (lane == 0 && first != kEnd) in.clear[first >> 5] = 0u;
+      }
+    }
     while (pend) {
       JumpState<Rec> q[kJumpElems];
 #pragma unroll
@@ -2077,6 +2085,19 @@ k_jump(LevelDesc *__restrict__ desc, int lev, Rec *work, RT *__restrict__ rout, 
     if (lane == 0 && chk) atomicAdd(&desc[lev].check, (unsigned long long)chk);
   }
   if (t == 0) desc[lev].visited = n;
+  if (in.ticket) {
+    // the last CTA reports the call's error bits and leaves the words at zero
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      __threadfence();
+      if (atomicAdd(in.ticket, 1u) == gridDim.x - 1u) {
+        __threadfence();
+        *in.status = atomicExch(err, 0u);
+        *in.count = 0u;
+        *in.ticket = 0u;
+      }
+    }
+  }
 }
 
 cudaError_t launch_jump(LevelDesc *desc, int lev, void *work, bool rec16, void *rout, int rank_bytes,

@@ -159,7 +159,9 @@ cudaError_t launch_chase(LevelDesc *desc, int lev, void *work, int kind, void *n
 // What the base case needs to rank level 0 itself (all optional): the most
 // lists of two or more elements the caller promised (0: any number), counted
 // from the has-predecessor bitmap into *count (zeroed); one rank buffer per
-// instance.
+// instance.  With ticket (zeroed), the kernel ends the call: it copies the
+// error bits to *status (host memory the device can write) and leaves the
+// error word, *count, *ticket and the bitmap (clear) at zero.
 struct JumpInput {
   uint64_t max_lists;
   const uint32_t *bitmap;
@@ -167,6 +169,7 @@ struct JumpInput {
   void *const *rptr;
   const int64_t *offsets;
   int32_t k;
+  uint32_t *ticket, *status, *clear;
 };
 
 // Base case: rank level lev (at most cap elements) by pointer jumping in its

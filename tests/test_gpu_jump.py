@@ -172,3 +172,44 @@ def test_short_lists(n, wt, rt):
         assert status_of(star, validate=True) == ("LR_ERR_NOT_A_LIST" if n > 2 else "LR_OK")
         lr.rank(dev(cyc), sync=False)
         assert lr.status_string(lr.device_status()) == "LR_ERR_CYCLE"
+
+
+def test_calls_leave_their_words_at_zero():
+    # the error word, the list count and the predecessor marks of the two-launch
+    # path are cleared by the call that used them: whatever came before on the
+    # stream, the next call starts clean, in a captured graph as well
+    st = torch.cuda.Stream()
+    good = {n: gen.random_list(n, 9900 + n) for n in (5000, 20_000, 300_007, 1 << 19)}
+    ring = np.roll(np.arange(20_000, dtype=np.uint32), -1)
+    merged = good[300_007].copy()
+    merged[int(np.flatnonzero(merged == np.arange(300_007))[0])] = merged[5]
+    forest, nl = gen.forest(100_000, 9901, n_long=1, long_len=10, mean_short=5)
+    want = {n: oracle.rank(s) for n, s in good.items()}
+    # torch's streams come from a pool: graph and stream are the library's st
+    s19, out = dev(good[1 << 19]), torch.empty(1 << 19, dtype=torch.int32, device="cuda")
+    lr.rank(s19, out=out, max_lists=1, stream=st)
+    g = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(g, stream=st):
+        lr.rank(s19, out=out, max_lists=1, sync=False)
+
+    def status(succ, **kw):
+        lr.rank(dev(succ), sync=False, stream=st, **kw)
+        return lr.status_string(lr.device_status(st))
+
+    bad = [(ring, {}, "LR_ERR_CYCLE"), (merged, {}, "LR_ERR_NOT_A_LIST"),
+           (forest, {"max_lists": nl // 8}, "LR_ERR_CAPACITY")]
+    for _ in range(2):
+        for succ, kw, name in bad:
+            torch.cuda.synchronize()
+            assert status(succ, **kw) == name
+            for n in good:
+                got = lr.rank(dev(good[n]), validate=n == 5000, max_lists=1, stream=st)
+                np.testing.assert_array_equal(got.cpu().numpy(), want[n])
+            assert status(forest, max_lists=nl) == "LR_OK"
+            out.zero_()
+            torch.cuda.synchronize()
+            with torch.cuda.stream(st):
+                g.replay()
+            assert lr.device_status(st) == 0
+            np.testing.assert_array_equal(out.cpu().numpy(), want[1 << 19])
