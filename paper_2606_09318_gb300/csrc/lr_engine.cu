@@ -283,7 +283,8 @@ Plan make_plan(uint64_t n, uint64_t h, const Tuning &u, bool rec16_0, int rank_b
   p.off_zero = o;
   p.off_err = o; o = align_up(o + 16);
   p.off_hcount = o; o = align_up(o + 16);
-  p.off_acc = o; o = align_up(o + 40);        // sums of terminals, successors; local links, sample; flags
+  p.off_acc = o; o = align_up(o + 48);        // sums of terminals, successors; local links, sample; flags;
+                                              // a terminal
   p.off_logctr = o; o = align_up(o + 16);
   p.off_bctr = o; o = align_up(o + sizeof(uint32_t) * 256);
   p.off_q = o; o = align_up(o + sizeof(uint32_t) * (size_t)chase_grid * kMaxLevels);
@@ -607,7 +608,7 @@ static WyPlan wyllie_plan(uint64_t n, bool w16) {
   WyPlan q;
   size_t o = 0;
   q.off_err = o; o = align_up(o + 16);
-  q.off_sums = o; o = align_up(o + 16);
+  q.off_sums = o; o = align_up(o + 48);
   q.zero_bytes = o;
   q.off_bitmap = o; o = align_up(o + sizeof(uint32_t) * ((n + 31) / 32));
   q.off_a = o; o = align_up(o + (w16 ? 16 : 8) * n);
@@ -848,12 +849,13 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
     return run_wyllie(in, c, s);
   }
   if (u.algo != LR_ALGO_SRS && u.algo != LR_ALGO_WYLLIE) return LR_ERR_INVALID_ARGUMENT;
-  const bool extras = in.term != nullptr || in.prefix != nullptr || in.incl != 0;
+  const bool outputs = in.term != nullptr || in.prefix != nullptr || in.incl != 0;
+  bool extras = outputs;                       // to be carried through the levels
   // 16-byte level-0 records: weighted, or ranked at level 0 with terminal ids
   const bool rec16_0 = in.wtype != 0 || (extras && in.n <= u.base0);
   if (extras && ptrs) return LR_ERR_INVALID_ARGUMENT;
   const bool log0 = use_log0(u, in.n, in.wtype != 0, in.rank_bytes, extras, ptrs || in.offsets != nullptr);
-  const bool t0ws = extras && in.term == nullptr;
+  bool t0ws = extras && in.term == nullptr;
   const bool spawn0 = u.spawn != 0 && u.xchg != 0 && !log0 && !extras && !ptrs;
   // a batch chases its level-0 rulers in element order (the has-predecessor
   // bitmap, free once the heads are chosen, holds the ruler marks; level 1's
@@ -979,13 +981,16 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
   else
     LR_TRY(pack(kind0, false, nullptr));
   if (both) LR_TRY(pack(kRecKind16, true, wflags));
+  uint64_t one_head = 0;
+  uint32_t one_term = 0;
   bool one_list = false;                       // the host has seen that level 0 is one list
   if (need_count) {
     // count the lists (one wait), then size the recursion for exactly that many:
     // a single-instance pass counts terminals in its reduction, a batch adds
     // its instances' terminal counts, the other passes count zero bits of the
     // has-predecessor bitmap
-    uint64_t sums[5];                          // terminals, other successors, local links, (sample), flags
+    uint64_t sums[6];                          // terminals, other successors, local links, (sample), flags,
+                                               // a terminal
     if (log0 || sums0) {
       LR_TRY(cudaMemcpyAsync(c->host_words + 4, acc, sizeof(sums), cudaMemcpyDeviceToHost, s));
     } else if (sums0b) {
@@ -1000,7 +1005,10 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
     if (log0 || sums0) {
       memcpy(sums, c->host_words + 4, sizeof(sums));
       c->host_words[1] = (uint32_t)sums[0];
-      one_list = late_bitmap && sums[0] == 1 && in.n * (in.n - 1) / 2 - sums[1] < in.n;
+      one_head = in.n * (in.n - 1) / 2 - sums[1];
+      one_list = late_bitmap && sums[0] == 1 && one_head < in.n;
+      one_term = (uint32_t)sums[5];
+      if (one_list && sums0) extras = t0ws = false;    // one terminal, one total: added at the end
     }
     if (local_exact) {
       if (sums[2] * 2 >= in.n) {           // at least half the links stay in their tile
@@ -1145,6 +1153,14 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
         LR_TRY(launch_finalize(desc, 0, work0, kRecKind16, R_of(1), R_of(0), p.rank_bytes, p.cap[0], err, nullptr,
                                nullptr, nullptr, s));
     }
+  }
+  if (outputs && !extras) {
+    Perm P;                                    // the head is a ruler: its rank at level 1
+    P.init((uint32_t)in.n, p.seed[0]);
+    const uint32_t id = P.fwd((uint32_t)one_head);
+    const uint32_t r = (uint32_t)((in.n + p.f_inv[0] - 1) / p.f_inv[0]);
+    LR_TRY(launch_out_one((uint32_t)in.n, one_term, (const char *)R_of(1) + (size_t)p.rank_bytes * std::min(id, r),
+                          in.term, in.rank, in.prefix, p.rank_bytes, in.incl, in.weight, in.wtype, s));
   }
   if (extras)
     LR_TRY(launch_outputs(desc, bitmap, hA, (uint32_t)in.n, T0, in.rank, in.prefix, p.rank_bytes,

@@ -57,11 +57,13 @@ struct WeightScan {
   const uint32_t *unless_narrow;
 };
 
+constexpr int kSumTerminal = 5;
+
 // Level-0 pass.  wtype 0/1/2 (none/i32/i64).  offsets != nullptr: batched
 // input with local successor ids (k instances).
 // kind: kRecKind8 (unweighted), kRecKind16 or kRecKind8w (weighted).
-// sums: the number of terminals and the sum of the other successors instead
-// of predecessor marks in bitmap (which may be null then, and when neither is
+// sums: the number of terminals and the sum of the other successors (and some
+// terminal at kSumTerminal) instead of predecessor marks in bitmap (which may be null then, and when neither is
 // wanted).  desc (optional): also writes the level descriptors from *init.
 // local (optional): counts the links that stay inside their contraction tile.
 cudaError_t launch_prep0(const uint32_t *succ, const void *weight, int wtype, uint32_t n,
@@ -193,6 +195,10 @@ cudaError_t launch_outputs(const LevelDesc *desc, const uint32_t *bitmap, const 
                            uint32_t n, uint32_t *term, void *rank, void *prefix, int rank_bytes,
                            int incl, const void *weight, int wtype, const int64_t *offsets, int32_t k,
                            int local, cudaStream_t s);
+
+// The same for one list with terminal t: total holds the rank of its head.
+cudaError_t launch_out_one(uint32_t n, uint32_t t, const void *total, uint32_t *term, void *rank, void *prefix,
+                           int rank_bytes, int incl, const void *weight, int wtype, cudaStream_t s);
 
 // Whole-list Wyllie pointer doubling (lr_wyllie.cu).  bufA holds k_prep0's
 // records (8 B, or 16 B when weighted: w16), bufB the same size; ranks go
