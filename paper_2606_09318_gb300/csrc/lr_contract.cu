@@ -20,9 +20,11 @@
 //
 // Inside a tile, t and the link count to it come from pointer doubling over
 // all of the tile's elements in shared memory, each thread holding the
-// words of its eight elements in registers: at most log2(tile) rounds of
-// one shared-memory gather per unsettled element, with no divergence, until
-// every pointer has reached a local tail.  Weighted distances then follow
+// words of its eight elements in registers.  One element in eight is a stop:
+// everybody doubles up to the next stop or local tail (some six rounds of one
+// shared-memory gather per unsettled element, most of them settled after
+// three), then the 512 stops double among themselves, and who stopped takes
+// the rest from the stop.  Weighted distances then follow
 // from one prefix sum of the weights in list order.  (A ruling set inside
 // the tile does less work, but its walks diverge and its phases need more
 // barriers; on GB300 the doubling was the faster of the two.)
@@ -94,6 +96,7 @@ struct LcMarks {
   uint8_t mark[kTile];       // 1: the element has a local predecessor
   uint32_t pred[kTileWords]; // has-local-predecessor bitmap
   uint32_t tail[kTileWords]; // local-tail bitmap (wide int64 tiles only)
+  uint32_t stop[kLcThreads]; // the stops' words
   uint32_t nlinks, nmarked;  // local links; marked elements
   uint32_t wflags;           // over the tile's local links: kWBig19 | kWNeg | kWBig20
 };
@@ -148,11 +151,22 @@ __device__ __forceinline__ uint32_t *lc_words(LcTile<WT> &S, int b) {
 constexpr uint32_t kLcRuns = kTile / (4 * kLcThreads);
 static_assert(kLcRuns * 4 * kLcThreads == kTile, "a tile is kLcRuns runs of four per thread");
 constexpr uint32_t kLcRunStride = kTile / kLcRuns;
-// Low half of a packed word: the pointer, and a bit set once the pointer is
-// a local tail (the pointer's own word has it then).
+// Low half of a packed word: the pointer as a byte offset into the words (bits
+// 2 to 13), and a bit set once the pointer is a local tail, or in the first
+// stage a stop (the pointer's own word has it then).
 constexpr uint32_t kLcPtrMask = kTile - 1u;
+constexpr uint32_t kLcOffset = 4u * kLcPtrMask;
 constexpr uint32_t kLcSettled = 0x8000u;
-static_assert(kTile <= kLcSettled, "pointers stay below the settled bit");
+static_assert(4u * kTile <= kLcSettled, "offsets stay below the settled bit");
+// Stops: of thread t's elements the first one of run t mod 2, number t.
+static_assert(kLcRuns == 2 && kLcRunStride == 2048 && kTile == 4096, "the stop test below is for these");
+__device__ __forceinline__ bool lc_at_stop(uint32_t w) {      // settled, and on a stop
+  return (w & 0x800Cu) == kLcSettled && !((w ^ (w >> 9)) & 16u);
+}
+__device__ __forceinline__ uint32_t lc_stop_offset(uint32_t w) { return (w >> 2) & (4u * (kLcThreads - 1u)); }
+__device__ __forceinline__ uint32_t lc_word_at(const uint32_t *words, uint32_t w) {
+  return *reinterpret_cast<const uint32_t *>(reinterpret_cast<const unsigned char *>(words) + w);
+}
 // Weighted: the prefix sums are taken by each thread over 8 consecutive
 // positions, then across the threads.
 static_assert(kLcThreads * 8 == kTile, "one thread per 8 positions");
@@ -169,7 +183,8 @@ __device__ void lc_tile_solve(LcTile<WT> &S, uint32_t t, uint32_t len, const uin
   __shared__ uint64_t scan_sm[33];
   const uint32_t base = t << kTileShift;
   const uint32_t tid = threadIdx.x;
-  uint32_t x[kLcRuns][4];      // d << 16 | settled | p
+  uint32_t x[kLcRuns][4];      // d << 16 | settled | 4 p
+  const uint32_t hide = kLcSettled | 4u * ((tid & 1u) * kLcRunStride + 4u * tid);   // this thread's stop as an end
   uint32_t links = 0;
   uint32_t wfl = 0;            // weighted: this thread's kWBig19 | kWNeg | kWBig20
   // int64 weights: does any weight of the tile leave the int32 range?
@@ -222,7 +237,7 @@ __device__ void lc_tile_solve(LcTile<WT> &S, uint32_t t, uint32_t len, const uin
       if (j < len && s[e] >= n) bad |= kErrRange;
       const bool local = j < len && s[e] < n && s[e] != i && (s[e] >> kTileShift) == t;
       p[r][e] = local ? s[e] - base : j;
-      x[r][e] = (local ? 1u << 16 : kLcSettled) | p[r][e];
+      x[r][e] = (local ? 1u << 16 : kLcSettled) | p[r][e] << 2;
       if constexpr (WT != 0) {
         d[r][e] = local ? w[e] : 0u;   // exact in int32 unless the tile is wide
         const int64_t wv = (int64_t)d[r][e];
@@ -237,7 +252,8 @@ __device__ void lc_tile_solve(LcTile<WT> &S, uint32_t t, uint32_t len, const uin
       }
     }
     if (!wide) {
-      *reinterpret_cast<uint4 *>(&lc_words(S, 0)[j0]) = make_uint4(x[r][0], x[r][1], x[r][2], x[r][3]);
+      *reinterpret_cast<uint4 *>(&lc_words(S, 0)[j0]) =
+          make_uint4((tid & 1u) == r ? hide : x[r][0], x[r][1], x[r][2], x[r][3]);
       if constexpr (WT != 0)
         *reinterpret_cast<int4 *>(&S.q.w[j0]) =
             make_int4((int32_t)d[r][0], (int32_t)d[r][1], (int32_t)d[r][2], (int32_t)d[r][3]);
@@ -270,38 +286,56 @@ __device__ void lc_tile_solve(LcTile<WT> &S, uint32_t t, uint32_t len, const uin
     if ((tid & 31u) == 0 && c) atomicAdd(&S.m.nmarked, c);
   }
   if (!wide) {
-    // Pointer doubling on the packed words.  A word whose pointer has
-    // reached a local tail is final: it is not gathered again, and the
-    // rounds end when every word is final (a valid tile needs at most
-    // kTileShift rounds; a cycle never settles).
-    int b = 0;
-    for (int round = 0; round <= kTileShift; ++round) {
+    // Pointer doubling on the packed words, first up to the next stop or
+    // local tail, where the stops show an end instead of their own word.  A
+    // settled word is not gathered again, and the rounds end when every word
+    // is (a cycle without a stop never is).
+    auto round1 = [&](const uint32_t *cur, uint32_t *nxt) -> bool {
       uint32_t all = kLcSettled;
-      const uint32_t *cur = lc_words(S, b);
-      uint32_t *nxt = lc_words(S, b ^ 1);
 #pragma unroll
       for (uint32_t r = 0; r < kLcRuns; ++r) {
 #pragma unroll
         for (uint32_t e = 0; e < 4; ++e) {
           if (!(x[r][e] & kLcSettled)) {
-            const uint32_t v = cur[x[r][e] & kLcPtrMask];
+            const uint32_t v = lc_word_at(cur, x[r][e] & kLcOffset);
             x[r][e] = (x[r][e] & 0xFFFF0000u) + v;
           }
           all &= x[r][e];
         }
         *reinterpret_cast<uint4 *>(&nxt[r * kLcRunStride + 4 * tid]) =
-            make_uint4(x[r][0], x[r][1], x[r][2], x[r][3]);
+            make_uint4((tid & 1u) == r ? hide : x[r][0], x[r][1], x[r][2], x[r][3]);
       }
-      b ^= 1;
-      if (__syncthreads_and(all & kLcSettled)) break;
+      return __syncthreads_and(all & kLcSettled) != 0;
+    };
+    for (int round = 0; round <= kTileShift; round += 2)
+      if (round1(lc_words(S, 0), lc_words(S, 1)) || round1(lc_words(S, 1), lc_words(S, 0))) break;
+    // Then the stops among themselves, in place and without waiting for each
+    // other: a word states a true fact whenever it is read.  A count beyond
+    // the tile is a cycle, and the word is left as it is, unsettled.
+    uint32_t sx = (tid & 1u) ? x[1][0] : x[0][0];
+    if (!(sx & kLcSettled)) sx = 1u << 16 | 4u * tid;                      // into a cycle without a stop
+    else if (lc_at_stop(sx) && sx != hide) sx = (sx & 0xFFFF0000u) | lc_stop_offset(sx);
+    volatile uint32_t *mine = &S.m.stop[tid];
+    *mine = sx;
+    __syncthreads();
+    while (!(sx & kLcSettled)) {
+      const uint32_t nx = (sx & 0xFFFF0000u) +
+          *reinterpret_cast<volatile uint32_t *>(reinterpret_cast<unsigned char *>(S.m.stop) + (sx & 0x7FCu));
+      if ((nx >> 16) > kTile) break;
+      sx = nx;
+      *mine = sx;
     }
-    // unpack; a word that never settled is on, or leads into, a cycle (also
-    // one whose length is a power of two: its pointer comes back to itself)
+    __syncthreads();
+    // Who stopped takes the rest from the stop.  A word that never settled is
+    // on, or leads into, a cycle (also one whose length is a power of two:
+    // its pointer comes back to itself).
 #pragma unroll
     for (uint32_t r = 0; r < kLcRuns; ++r)
 #pragma unroll
       for (uint32_t e = 0; e < 4; ++e) {
-        p[r][e] = (x[r][e] & kLcSettled) ? (x[r][e] & kLcPtrMask) : kEnd16;
+        if (e == 0 && (tid & 1u) == r) x[r][e] = sx;
+        else if (lc_at_stop(x[r][e])) x[r][e] = (x[r][e] & 0xFFFF0000u) + lc_word_at(S.m.stop, lc_stop_offset(x[r][e]));
+        p[r][e] = (x[r][e] & kLcSettled) ? (x[r][e] & kLcOffset) >> 2 : kEnd16;
         if constexpr (WT == 0) d[r][e] = x[r][e] >> 16;
       }
     if constexpr (WT != 0) {
