@@ -171,6 +171,30 @@ __device__ __forceinline__ uint32_t lc_word_at(const uint32_t *words, uint32_t w
 // positions, then across the threads.
 static_assert(kLcThreads * 8 == kTile, "one thread per 8 positions");
 
+// Bulk prefetch of [p, p + bytes) into L2, shrunk inward to 16-byte boundaries.
+__device__ __forceinline__ void lc_prefetch(const void *p, size_t bytes) {
+  const uintptr_t a = ((uintptr_t)p + 15u) & ~(uintptr_t)15u, e = ((uintptr_t)p + bytes) & ~(uintptr_t)15u;
+  if (e > a)
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" :: "l"(a), "r"((uint32_t)(e - a)) : "memory");
+}
+
+// Exclusive scan of v over the CTA with one barrier: every warp adds up the
+// warps' totals itself.  ws may be written again after the next barrier.
+__device__ __forceinline__ uint32_t lc_scan(uint32_t v, uint32_t *ws, uint32_t &total) {
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+  uint32_t x = v;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, d);
+    if ((int)lane >= d) x += y;
+  }
+  if (lane == 31) ws[warp] = x;
+  __syncthreads();
+  const uint32_t w = lane < kLcThreads / 32 ? ws[lane] : 0u;
+  total = __reduce_add_sync(0xFFFFFFFFu, w);
+  return __reduce_add_sync(0xFFFFFFFFu, lane < warp ? w : 0u) + x - v;
+}
+
 // Load tile `t` (len elements) and give every element its local tail p and
 // distance d to it (in the rank's arithmetic, modulo 2^64); p = kEnd16 for
 // an element on, or leading into, a cycle inside the tile.  Two local links
@@ -181,6 +205,7 @@ __device__ void lc_tile_solve(LcTile<WT> &S, uint32_t t, uint32_t len, const uin
                               const void *weight, uint32_t n, bool vec, uint32_t (&p)[kLcRuns][4],
                               uint64_t (&d)[kLcRuns][4], uint32_t &bad) {
   __shared__ uint64_t scan_sm[33];
+  __shared__ uint32_t scan32[2][kLcThreads / 32];
   const uint32_t base = t << kTileShift;
   const uint32_t tid = threadIdx.x;
   uint32_t x[kLcRuns][4];      // d << 16 | settled | 4 p
@@ -341,17 +366,20 @@ __device__ void lc_tile_solve(LcTile<WT> &S, uint32_t t, uint32_t len, const uin
     if constexpr (WT != 0) {
       // positions: every settled local head opens a range of its sublist's
       // length; its tail gets the range's last position
-      uint32_t cnt = 0;
+      uint32_t cnt = 0, heads = 0;             // bit 4 r + e: a head
 #pragma unroll
-      for (uint32_t r = 0; r < kLcRuns; ++r)
+      for (uint32_t r = 0; r < kLcRuns; ++r) {
+        const uint32_t j0 = r * kLcRunStride + 4 * tid;
+        const uint32_t pm = S.m.pred[j0 >> 5] >> (j0 & 31u);
 #pragma unroll
-        for (uint32_t e = 0; e < 4; ++e) {
-          const uint32_t j = r * kLcRunStride + 4 * tid + e;
-          const bool head = j < len && p[r][e] != kEnd16 && !((S.m.pred[j >> 5] >> (j & 31u)) & 1u);
-          if (head) cnt += (x[r][e] >> 16) + 1u;
-        }
-      uint64_t total;
-      uint32_t at = (uint32_t)block_exclusive_scan((uint64_t)cnt, scan_sm, &total);
+        for (uint32_t e = 0; e < 4; ++e)
+          if (j0 + e < len && p[r][e] != kEnd16 && !(pm >> e & 1u)) {
+            heads |= 1u << (4 * r + e);
+            cnt += (x[r][e] >> 16) + 1u;
+          }
+      }
+      uint32_t total;
+      uint32_t at = lc_scan(cnt, scan32[0], total);
       // more positions than elements: merged sublists (two predecessors,
       // reported by the marks); no weighted distances for this tile
       const bool fits = total <= kTile;
@@ -359,14 +387,11 @@ __device__ void lc_tile_solve(LcTile<WT> &S, uint32_t t, uint32_t len, const uin
 #pragma unroll
         for (uint32_t r = 0; r < kLcRuns; ++r)
 #pragma unroll
-          for (uint32_t e = 0; e < 4; ++e) {
-            const uint32_t j = r * kLcRunStride + 4 * tid + e;
-            const bool head = j < len && p[r][e] != kEnd16 && !((S.m.pred[j >> 5] >> (j & 31u)) & 1u);
-            if (head) {
+          for (uint32_t e = 0; e < 4; ++e)
+            if (heads >> (4 * r + e) & 1u) {
               at += (x[r][e] >> 16) + 1u;
               S.q.E[p[r][e]] = (uint16_t)(at - 1u);
             }
-          }
       }
       __syncthreads();                       // E is written; the doubling's buffers are free
       const uint32_t wf = S.m.wflags;
@@ -376,16 +401,19 @@ __device__ void lc_tile_solve(LcTile<WT> &S, uint32_t t, uint32_t len, const uin
         // weights by position (a tail's own link does not count); ids past
         // the end of the last tile are lone tails of no sublist
 #pragma unroll
-        for (uint32_t r = 0; r < kLcRuns; ++r)
+        for (uint32_t r = 0; r < kLcRuns; ++r) {
+          const uint32_t j0 = r * kLcRunStride + 4 * tid;
+          const int4 q = *reinterpret_cast<const int4 *>(&S.q.w[j0]);
+          const int32_t wv[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
           for (uint32_t e = 0; e < 4; ++e) {
-            const uint32_t j = r * kLcRunStride + 4 * tid + e;
-            if (j < len && p[r][e] != kEnd16) {
+            if (j0 + e < len && p[r][e] != kEnd16) {
               const uint32_t pos = ((uint32_t)S.q.E[p[r][e]] - (x[r][e] >> 16)) & kLcPtrMask;
-              if (narrow) S.q.P32[pos] = (uint32_t)S.q.w[j];
-              else S.q.P[pos] = (uint64_t)(int64_t)S.q.w[j];
+              if (narrow) S.q.P32[pos] = (uint32_t)wv[e];
+              else S.q.P[pos] = (uint64_t)(int64_t)wv[e];
             }
           }
+        }
       }
       __syncthreads();
       if (fits && narrow) {
@@ -397,7 +425,8 @@ __device__ void lc_tile_solve(LcTile<WT> &S, uint32_t t, uint32_t len, const uin
         v[4] = u1.x; v[5] = u1.y; v[6] = u1.z; v[7] = u1.w;
 #pragma unroll
         for (int q = 1; q < 8; ++q) v[q] += v[q - 1];
-        const uint32_t off = (uint32_t)block_exclusive_scan((uint64_t)v[7], scan_sm, nullptr);
+        uint32_t all;
+        const uint32_t off = lc_scan(v[7], scan32[1], all);
         uint4 *dst = reinterpret_cast<uint4 *>(&S.q.P32[8 * tid]);
         dst[0] = make_uint4(v[0] + off, v[1] + off, v[2] + off, v[3] + off);
         dst[1] = make_uint4(v[4] + off, v[5] + off, v[6] + off, v[7] + off);
@@ -492,7 +521,7 @@ k_lc_scan(const uint32_t *__restrict__ tcnt, uint32_t ntiles, uint32_t *__restri
 // heads per tile go to hb, wpre and tcnt.  vec: bit 0 = succ and weight
 // 16-byte aligned, bit 1 = rank 16-byte and tail16 8-byte aligned.
 template <int WT, class RT>
-__global__ void __launch_bounds__(kLcThreads, WT == 2 ? 2 : 3)
+__global__ void __launch_bounds__(kLcThreads, WT ? 2 : 3)
 k_lc_solve(const uint32_t *__restrict__ succ, const void *__restrict__ weight, uint32_t n,
            RT *__restrict__ rank, uint16_t *__restrict__ tail16, uint32_t *__restrict__ hb,
            uint16_t *__restrict__ wpre, uint32_t *__restrict__ tcnt, uint32_t *__restrict__ err, int vec) {
@@ -509,6 +538,13 @@ k_lc_solve(const uint32_t *__restrict__ succ, const void *__restrict__ weight, u
     uint32_t p[kLcRuns][4];
     uint64_t d[kLcRuns][4];
     uint32_t bad = 0;
+    if (threadIdx.x == 0 && t + gridDim.x < ntiles) {     // the next tile's input, while this one is solved
+      const uint64_t nb = (uint64_t)(t + gridDim.x) << kTileShift;
+      const size_t m = (size_t)min((uint64_t)kTile, n - nb);
+      lc_prefetch(succ + nb, 4 * m);
+      if constexpr (WT == 1) lc_prefetch(reinterpret_cast<const int *>(weight) + nb, 4 * m);
+      if constexpr (WT == 2) lc_prefetch(reinterpret_cast<const long long *>(weight) + nb, 8 * m);
+    }
     lc_tile_solve<WT>(S, t, len, succ, weight, n, (vec & 1) != 0, p, d, bad);
     bool cyc = false;
 #pragma unroll
@@ -706,7 +742,7 @@ cudaError_t launch_lc_solve(const uint32_t *succ, const void *weight, int wtype,
                             uint32_t *tpre, uint32_t *err, cudaStream_t s) {
   const uint32_t nt = lc_tiles(n);
   const size_t sm = lc_smem_bytes(wtype);
-  const int per_sm = wtype == 2 ? 2 : 3;
+  const int per_sm = wtype ? 2 : 3;
   const int grid = (int)std::min<uint32_t>(nt, (uint32_t)device_sm_count() * per_sm);
   const int vec = (((uintptr_t)succ & 15u) == 0 && ((uintptr_t)weight & 15u) == 0 ? 1 : 0) |
                   (((uintptr_t)rank & 15u) == 0 && ((uintptr_t)tail16 & 7u) == 0 ? 2 : 0);
