@@ -368,4 +368,27 @@ __device__ inline uint64_t block_exclusive_scan(uint64_t v, uint64_t *smem, uint
   return r;
 }
 
+// Add each v[k], summed over the CTA, to *out[k] (null: not wanted), with one
+// atomic per CTA and sum: one address serves an atomic in some 1.5 ns, so a
+// sum from every warp of a full grid would cost 15 us.  All threads call it.
+template <int N>
+__device__ __forceinline__ void block_add(unsigned long long (&v)[N], unsigned long long *const (&out)[N]) {
+  __shared__ unsigned long long part[N][32];
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+#pragma unroll
+  for (int k = 0; k < N; ++k) {
+    for (int d = 16; d > 0; d >>= 1) v[k] += __shfl_down_sync(0xFFFFFFFFu, v[k], d);
+    if (lane == 0) part[k][warp] = v[k];
+  }
+  __syncthreads();
+  if (warp == 0) {
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+      unsigned long long t = lane < warps ? part[k][lane] : 0ull;
+      for (int d = 16; d > 0; d >>= 1) t += __shfl_down_sync(0xFFFFFFFFu, t, d);
+      if (lane == 0 && t && out[k]) atomicAdd(out[k], t);
+    }
+  }
+}
+
 }  // namespace lr

@@ -104,6 +104,7 @@ k_init(LevelDesc *desc, InitParams p, const unsigned long long *__restrict__ acc
   if (threadIdx.x != 0) return;
   LevelDesc &d = desc[0];
   if (wflags) d.narrow = narrow_mode(*wflags);
+  if (p.err_bits) record_error(p.err, p.err_bits);
   if (!acc || p.nlev < 2) return;
   const unsigned long long n = p.n0, h = n * (n - 1) / 2 - acc[1];
   if (acc[0] != 1 || h >= n) return;
@@ -186,9 +187,9 @@ __device__ __forceinline__ void add_flags(uint32_t *flags, uint32_t mine) {
 // findInit), and pack {succ, kUnvisited[, link weight]} records.  A terminal's
 // weight is stored as 0, so every deeper computation can treat weights
 // inclusively.
-// sums != nullptr: instead of the bitmap, accumulate the number of terminals
-// and the sum of the other successors (single-list head, see k_init).
-// Neither: an input small enough for the base case, which needs no heads.
+// sums != nullptr: accumulate the number of terminals and the sum of the other
+// successors (single-list head, see k_init).  Neither: an input small enough
+// for the base case, which needs no heads.
 // desc != nullptr: also write the level descriptors (saves k_init's launch).
 // KIND: the records (unweighted input may have 16-byte ones too, weight 1, when
 // they are to carry terminal ids).
@@ -203,6 +204,7 @@ k_prep0(const uint32_t *__restrict__ succ, const void *__restrict__ weight, uint
   uint32_t wide = 0;
   if (desc && blockIdx.x == 0) init_levels(desc, ip, (int)threadIdx.x);
   unsigned long long sT = 0, sS = 0, sL = 0;
+  uint32_t term = kEnd;
   const uint32_t ngroups = (uint32_t)(((uint64_t)n + 3u) / 4u);
   const uint32_t stride = gridDim.x * blockDim.x;
   for (uint32_t g = blockIdx.x * blockDim.x + threadIdx.x; g < ngroups; g += stride) {
@@ -257,9 +259,8 @@ k_prep0(const uint32_t *__restrict__ succ, const void *__restrict__ weight, uint
       const uint32_t i = i0 + j;
       if (local) sL += s[j] != i && (s[j] >> kContractTileShift) == (i >> kContractTileShift);
       if (s[j] != i) {
-        if (sums) {
-          sS += s[j];
-        } else if (bitmap) {
+        if (sums) sS += s[j];
+        if (bitmap) {
           const uint32_t bit = 1u << (s[j] & 31u);
           if (validate) {
             if (atomicOr(bitmap + (s[j] >> 5), bit) & bit) record_error(err, kErrNotList);
@@ -270,7 +271,7 @@ k_prep0(const uint32_t *__restrict__ succ, const void *__restrict__ weight, uint
       } else {
         w[j] = 0u;   // a terminal has no outgoing link
         sT += 1;
-        if (sums) sums[kSumTerminal] = i;      // (of use when it is the only one)
+        term = i;                              // (of use when it is the only one)
       }
     }
     store_records<KIND>(work, i0, cnt, s, w);
@@ -278,20 +279,12 @@ k_prep0(const uint32_t *__restrict__ succ, const void *__restrict__ weight, uint
       for (uint32_t j = 0; j < cnt; ++j) wide |= wide_flags(w[j]);
   }
   if (KIND == kRecKind8w && scan.flags) add_flags(scan.flags, wide);
-  if (sums) {
-    for (int d = 16; d > 0; d >>= 1) {
-      sS += __shfl_down_sync(0xFFFFFFFFu, sS, d);
-      sT += __shfl_down_sync(0xFFFFFFFFu, sT, d);
-    }
-    if ((threadIdx.x & 31) == 0) {
-      if (sT) atomicAdd(sums + 0, sT);
-      if (sS) atomicAdd(sums + 1, sS);
-    }
-  }
-  if (local) {
-    // links that stay inside their contraction tile (decides whether to contract)
-    for (int d = 16; d > 0; d >>= 1) sL += __shfl_down_sync(0xFFFFFFFFu, sL, d);
-    if ((threadIdx.x & 31) == 0 && sL) atomicAdd(local, sL);
+  if (sums || local) {
+    unsigned long long v[3] = {sT, sS, sL};
+    unsigned long long *const to[3] = {sums, sums ? sums + 1 : nullptr, local};   // local: decides whether to contract
+    block_add(v, to);
+    // only a terminal that its CTA has no second of can be the only one
+    if (sums && __syncthreads_count(term != kEnd) == 1 && term != kEnd) sums[kSumTerminal] = term;
   }
 }
 
@@ -343,14 +336,9 @@ k_local_sample(const uint32_t *__restrict__ succ, uint32_t n, unsigned long long
     cnt += 1;
     loc += sx != (uint32_t)i && (sx >> kContractTileShift) == (uint32_t)(i >> kContractTileShift);
   }
-  for (int d = 16; d > 0; d >>= 1) {
-    loc += __shfl_down_sync(0xFFFFFFFFu, loc, d);
-    cnt += __shfl_down_sync(0xFFFFFFFFu, cnt, d);
-  }
-  if ((threadIdx.x & 31) == 0 && cnt) {
-    atomicAdd(out, loc);
-    atomicAdd(out + 1, cnt);
-  }
+  unsigned long long v[2] = {loc, cnt};
+  unsigned long long *const to[2] = {out, out + 1};
+  block_add(v, to);
 }
 
 cudaError_t launch_local_sample(const uint32_t *succ, uint32_t n, unsigned long long *out, cudaStream_t s) {
@@ -788,8 +776,13 @@ __global__ void k_count_heads(const uint32_t *__restrict__ bitmap, uint32_t n, u
     if (w == words - 1u && (n & 31u)) bits &= (1u << (n & 31u)) - 1u;
     c += __popc(bits);
   }
-  for (int d = 16; d > 0; d >>= 1) c += __shfl_down_sync(0xFFFFFFFFu, c, d);
-  if ((threadIdx.x & 31) == 0 && c) atomicAdd(out, c);
+  __shared__ uint32_t heads;
+  if (threadIdx.x == 0) heads = 0;
+  __syncthreads();
+  c = __reduce_add_sync(0xFFFFFFFFu, c);
+  if ((threadIdx.x & 31) == 0 && c) atomicAdd(&heads, c);
+  __syncthreads();
+  if (threadIdx.x == 0 && heads) atomicAdd(out, heads);
 }
 
 cudaError_t launch_count_heads(const uint32_t *bitmap, uint32_t n, uint32_t *out, cudaStream_t s) {

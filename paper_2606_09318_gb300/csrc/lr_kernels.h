@@ -25,6 +25,8 @@ struct InitParams {
   uint64_t seed[kMaxLevels + 1];
   uint32_t hcap;                      // capacity of the head lists
   uint32_t base;                      // largest level >= 1 that the base case ranks
+  uint32_t err_bits;                  // errors the host has found, recorded in *err
+  uint32_t *err;
 };
 
 // Kernel launch counter (all streams).
@@ -62,9 +64,9 @@ constexpr int kSumTerminal = 5;
 // Level-0 pass.  wtype 0/1/2 (none/i32/i64).  offsets != nullptr: batched
 // input with local successor ids (k instances).
 // kind: kRecKind8 (unweighted), kRecKind16 or kRecKind8w (weighted).
-// sums: the number of terminals and the sum of the other successors (and some
-// terminal at kSumTerminal) instead of predecessor marks in bitmap (which may be null then, and when neither is
-// wanted).  desc (optional): also writes the level descriptors from *init.
+// bitmap: predecessor marks, or null.  sums: the number of terminals and the
+// sum of the other successors (and some terminal at kSumTerminal), or null.
+// desc (optional): also writes the level descriptors from *init.
 // local (optional): counts the links that stay inside their contraction tile.
 cudaError_t launch_prep0(const uint32_t *succ, const void *weight, int wtype, uint32_t n,
                          void *work, int kind, uint32_t *bitmap, uint32_t *err, int validate,

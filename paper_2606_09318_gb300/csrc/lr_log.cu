@@ -67,16 +67,9 @@ k_sum0(const uint32_t *__restrict__ succ, uint32_t n, unsigned long long *__rest
       for (uint32_t j = 0; j < cnt; ++j) take(i0 + j, __ldcs(succ + i0 + j));
     }
   }
-  for (int d = 16; d > 0; d >>= 1) {
-    S += __shfl_down_sync(0xFFFFFFFFu, S, d);
-    T += __shfl_down_sync(0xFFFFFFFFu, T, d);
-    loc += __shfl_down_sync(0xFFFFFFFFu, loc, d);
-  }
-  if ((threadIdx.x & 31) == 0) {
-    if (T) atomicAdd(acc + 0, T);
-    if (S) atomicAdd(acc + 1, S);
-    if (local && loc) atomicAdd(local, (unsigned long long)loc);
-  }
+  unsigned long long v[3] = {T, S, loc};
+  unsigned long long *const to[3] = {acc, acc + 1, local};
+  block_add(v, to);
   if (bad) record_error(err, kErrRange);
 }
 

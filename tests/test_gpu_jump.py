@@ -213,3 +213,35 @@ def test_calls_leave_their_words_at_zero():
                 g.replay()
             assert lr.device_status(st) == 0
             np.testing.assert_array_equal(out.cpu().numpy(), want[1 << 19])
+
+
+@pytest.mark.parametrize("n", [(1 << 19) + 1, (1 << 22) + 9])
+@pytest.mark.parametrize("wt", [None, "i32"])
+def test_validation_by_counts(n, wt):
+    # two predecessors are told from one by as many heads as terminals
+    w = None if wt is None else dev(gen.weights_i32(n, 9950))
+    host_w = None if wt is None else gen.weights_i32(n, 9950)
+    rt = np.int32 if wt is None else np.int64
+    one = gen.random_list(n, 9951)
+    forest, _ = gen.forest(n, 9952, n_long=2, long_len=n // 8, mean_short=7)
+    for succ in (one, forest):
+        np.testing.assert_array_equal(lr.rank(dev(succ), w, validate=True).cpu().numpy(), oracle.rank(succ, host_w, rt))
+        bad = succ.copy()
+        inner = np.flatnonzero(bad != np.arange(n))
+        a, b = int(inner[5]), int(inner[len(inner) // 2])
+        bad[a] = bad[b]                                   # b's successor has two predecessors
+        assert oracle.rank_status(bad)[0] != oracle.OK
+        with pytest.raises(lr.LRError) as e:
+            lr.rank(dev(bad), w, validate=True)
+        assert e.value.name == "LR_ERR_NOT_A_LIST"
+        lr.rank(dev(bad), w, validate=True, sync=False)
+        assert lr.status_string(lr.device_status()) == "LR_ERR_NOT_A_LIST"
+        bad[a] = n + 5
+        with pytest.raises(lr.LRError) as e:
+            lr.rank(dev(bad), w, validate=True)
+        assert e.value.name == "LR_ERR_OUT_OF_RANGE"
+    r, t, p = lr.rank_outputs(dev(one), w, term=True, prefix=True, validate=True)
+    want_r, want_t, want_p = oracle.rank_ext(one, host_w, rt)
+    np.testing.assert_array_equal(r.cpu().numpy(), want_r)
+    np.testing.assert_array_equal(t.cpu().numpy().view(np.uint32), want_t)
+    np.testing.assert_array_equal(p.cpu().numpy(), want_p)
