@@ -349,44 +349,86 @@ cudaError_t launch_local_sample(const uint32_t *succ, uint32_t n, unsigned long 
   return cudaGetLastError();
 }
 
+// The instance of element `base` in a table of k nondecreasing offsets with
+// offsets[0] = 0 <= base < offsets[k]: the largest j < k with offsets[j] <=
+// base, found by the whole warp at once (every lane probes one of 32 points
+// spread over the remaining range, the ballot keeps the last probe at or
+// below base), in at most 3 rounds for up to 32768 instances.  Warp-uniform.
+__device__ __forceinline__ int32_t warp_instance(const int64_t *__restrict__ offsets, int32_t k, uint64_t base,
+                                                 uint32_t lane) {
+  int32_t lo = 0, hi = k;
+  while (hi - lo > 1) {
+    const int64_t span = hi - lo;
+    const int32_t q = lo + (int32_t)(((int64_t)(lane + 1) * span) / 33);
+    const uint32_t le = __ballot_sync(0xFFFFFFFFu, (uint64_t)__ldg(offsets + q) <= base);
+    const int t = __popc(le);
+    const int32_t nlo = __shfl_sync(0xFFFFFFFFu, q, t > 0 ? t - 1 : 0);
+    const int32_t nhi = __shfl_sync(0xFFFFFFFFu, q, t < 32 ? t : 31);
+    if (t > 0) lo = max(lo, nlo);
+    if (t < 32) hi = nhi;
+  }
+  return lo;
+}
+
+// The per-instance sums of a warp that walks consecutive elements: what its
+// lanes have added for the instance `inst` and not yet passed on.
+struct InstSums {
+  int32_t inst = -1;
+  unsigned long long t = 0, s = 0;
+};
+
+// Pass them on (whole warps).
+__device__ __forceinline__ void flush_sums(InstSums &a, unsigned long long *isums, uint32_t lane) {
+  if (!isums || a.inst < 0) return;
+  for (int d = 16; d > 0; d >>= 1) {
+    a.t += __shfl_down_sync(0xFFFFFFFFu, a.t, d);
+    a.s += __shfl_down_sync(0xFFFFFFFFu, a.s, d);
+  }
+  if (lane == 0) {
+    if (a.t) atomicAdd(isums + 2 * (size_t)a.inst, a.t);
+    if (a.s) atomicAdd(isums + 2 * (size_t)a.inst + 1, a.s);
+  }
+  a.t = a.s = 0;
+}
+
+// Groups of 128 consecutive elements that a warp takes at a time.
+constexpr uint32_t kMaxRun = 16;
+static uint32_t run_groups(uint32_t n, int grid, int block) {
+  const uint64_t groups = ((uint64_t)n + 127) / 128, warps = (uint64_t)grid * (block / 32);
+  return (uint32_t)std::min<uint64_t>(kMaxRun, std::max<uint64_t>(1, (groups + warps - 1) / warps));
+}
+
 // Batched prep without per-element atomics.  Each instance j of a batch that
 // is one list has exactly one terminal, and its successors are every local id
 // but the head's, so head_j = n_j (n_j - 1) / 2 - sum of its non-terminal
 // successors (Section 1.1's findInit, by sums).  isums[2 j] counts instance
-// j's terminals and isums[2 j + 1] sums its local successors; a warp whose
-// 128 elements lie in one instance adds its sums with two atomics.  Records
-// as in k_prep0.  The loop runs warp-uniformly so that the warp can combine.
+// j's terminals and isums[2 j + 1] sums its local successors.  Records as in
+// k_prep0.
+// A warp takes runs of `run` consecutive groups of 128 elements and passes an
+// instance's sums on when it leaves the instance: the warps of a grid are
+// mostly in one or two large instances, and the atomics of one address come
+// one after another (0.6 ns each: with a pair of them for every group they
+// bounded the pass, 2.16 ms for 4.6e8 elements with int64 weights; 1.48 ms, 6.3 TB/s, now).
 template <int WT, int KIND>
 __global__ void __launch_bounds__(256)
 k_prep0_sums(const uint32_t *__restrict__ succ, const void *__restrict__ weight, uint32_t n,
              void *__restrict__ work, WeightScan scan, uint32_t *__restrict__ err, int vec, const int64_t *__restrict__ offsets,
-             int32_t k, unsigned long long *__restrict__ isums) {
+             int32_t k, unsigned long long *__restrict__ isums, uint32_t run) {
   if (scan.unless_narrow && narrow_mode(*scan.unless_narrow)) return;
   uint32_t wide = 0;
-  const uint32_t ngroups = (uint32_t)(((uint64_t)n + 3u) / 4u);
-  const uint32_t stride = gridDim.x * blockDim.x;
+  const uint32_t ngroups = (uint32_t)(((uint64_t)n + 127u) / 128u);
+  const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, warps = gridDim.x * blockDim.x >> 5;
   const uint32_t lane = threadIdx.x & 31u;
-  for (uint32_t gw = blockIdx.x * blockDim.x + (threadIdx.x & ~31u); gw < ngroups; gw += stride) {
-    const uint32_t g = gw + lane;
-    const bool active = g < ngroups;
-    const uint32_t i0 = g * 4u;
-    // instance of the warp's first element by binary search (lane 0), then
-    // each lane walks forward to its own
-    int32_t lo = 0;
-    if (lane == 0) {
-      int32_t hi = k;
-      while (hi - lo > 1) {
-        const int32_t mid = (lo + hi) >> 1;
-        if ((uint64_t)__ldg(offsets + mid) <= (uint64_t)gw * 4u) lo = mid; else hi = mid;
-      }
-    }
-    lo = __shfl_sync(0xFFFFFFFFu, lo, 0);
-    int32_t inst = -1;                 // the one instance of this lane's elements, or -1
-    unsigned long long sT = 0, sS = 0;
-    if (active) {
-      const uint32_t cnt = min(4u, n - i0);
-      uint32_t s[4];
-      uint64_t w[4];
+  InstSums acc;
+  for (uint64_t r0 = (uint64_t)warp * run; r0 < ngroups; r0 += (uint64_t)warps * run) {
+    const uint32_t r1 = (uint32_t)min((uint64_t)ngroups, r0 + run);
+    int32_t lo0 = -1;                    // instance of the group's first element (warp-uniform)
+    uint64_t ib0 = 0, ie0 = 0;
+    for (uint32_t g = (uint32_t)r0; g < r1; ++g) {
+      const uint32_t base = g * 128u, i0 = base + lane * 4u;
+      const uint32_t cnt = i0 < n ? min(4u, n - i0) : 0u;
+      uint32_t s[4] = {0, 0, 0, 0};
+      uint64_t w[4] = {1, 1, 1, 1};
       if (vec && cnt == 4u) {
         const uint4 v = __ldcs(reinterpret_cast<const uint4 *>(succ + i0));
         s[0] = v.x; s[1] = v.y; s[2] = v.z; s[3] = v.w;
@@ -398,69 +440,77 @@ k_prep0_sums(const uint32_t *__restrict__ succ, const void *__restrict__ weight,
           const longlong2 *wp = reinterpret_cast<const longlong2 *>(reinterpret_cast<const long long *>(weight) + i0);
           const longlong2 a = __ldcs(wp), b = __ldcs(wp + 1);
           w[0] = (uint64_t)a.x; w[1] = (uint64_t)a.y; w[2] = (uint64_t)b.x; w[3] = (uint64_t)b.y;
-        } else {
-          w[0] = w[1] = w[2] = w[3] = 1u;
         }
       } else {
+#pragma unroll
+        for (uint32_t j = 0; j < 4u; ++j)
+          if (j < cnt) {
+            s[j] = __ldcs(succ + i0 + j);
+            w[j] = load_weight<WT>(weight, i0 + j);
+          }
+      }
+      if (base >= ie0) {
+        lo0 = warp_instance(offsets, k, base, lane);
+        ib0 = (uint64_t)__ldg(offsets + lo0);
+        ie0 = (uint64_t)__ldg(offsets + lo0 + 1);
+      }
+      if (base >= ib0 && (uint64_t)base + 128u <= ie0 && ie0 <= n) {      // the whole group in one instance
+        if (acc.inst != lo0) {
+          flush_sums(acc, isums, lane);
+          acc.inst = lo0;
+        }
+        const uint32_t ib = (uint32_t)ib0, len = (uint32_t)(ie0 - ib0);
+#pragma unroll
         for (uint32_t j = 0; j < 4u; ++j) {
-          s[j] = j < cnt ? __ldcs(succ + i0 + j) : 0u;
-          w[j] = j < cnt ? load_weight<WT>(weight, i0 + j) : 0u;
+          const uint32_t l = i0 + j - ib;
+          bool term = s[j] == l;
+          if (s[j] >= len) {
+            record_error(err, kErrRange);     // successor outside its instance
+            term = true;
+          }
+          if (term) { w[j] = 0u; acc.t += 1; s[j] = l; } else acc.s += s[j];
+          s[j] += ib;
         }
-      }
-      uint64_t base = (uint64_t)__ldg(offsets + lo), end = (uint64_t)__ldg(offsets + lo + 1);
-      int32_t first = -2;
-      for (uint32_t j = 0; j < cnt; ++j) {
-        const uint32_t i = i0 + j;
-        while (i >= end && lo + 1 < k) { ++lo; base = end; end = (uint64_t)__ldg(offsets + lo + 1); }
-        const uint64_t gl = base + s[j];
-        bool term;
-        if (i < base || i >= end || (uint64_t)s[j] >= end - base || gl >= n) {
-          record_error(err, kErrRange);   // successor outside its instance (or a bad table)
-          s[j] = i;
-          term = true;
-        } else {
-          term = gl == i;
-          if (!term) sS += s[j];          // local id
-          s[j] = (uint32_t)gl;
+      } else {
+        // each lane walks forward to its own elements' instances, and passes
+        // its sums on when it leaves one
+        int32_t lo = lo0;
+        uint64_t ib = ib0, ie = ie0;
+        unsigned long long sT = 0, sS = 0;
+        auto pass_on = [&] {
+          if (isums && sT) atomicAdd(isums + 2 * (size_t)lo, sT);
+          if (isums && sS) atomicAdd(isums + 2 * (size_t)lo + 1, sS);
+          sT = sS = 0;
+        };
+#pragma unroll
+        for (uint32_t j = 0; j < 4u; ++j) {
+          if (j >= cnt) continue;
+          const uint32_t i = i0 + j;
+          while (i >= ie && lo + 1 < k) { pass_on(); ++lo; ib = ie; ie = (uint64_t)__ldg(offsets + lo + 1); }
+          const uint64_t gl = ib + s[j];
+          bool term;
+          if (i < ib || i >= ie || (uint64_t)s[j] >= ie - ib || gl >= n) {
+            record_error(err, kErrRange);   // successor outside its instance (or a bad table)
+            s[j] = i;
+            term = true;
+          } else {
+            term = gl == i;
+            if (!term) sS += s[j];          // local id
+            s[j] = (uint32_t)gl;
+          }
+          if (term) { w[j] = 0u; sT += 1; }
         }
-        if (term) { w[j] = 0u; sT += 1; }
-        if (first == -2) first = lo;
-        else if (first != lo) first = -1;  // the group straddles two instances
+        pass_on();
       }
-      if (first >= 0) {
-        inst = first;
-      } else if (first == -1 && isums) {   // rare: add each element's share alone
-        sT = 0; sS = 0;
-        uint64_t b2 = (uint64_t)__ldg(offsets + lo);
-        int32_t l2 = lo;
-        for (int32_t jj = (int32_t)cnt - 1; jj >= 0; --jj) {
-          const uint32_t i = i0 + (uint32_t)jj;
-          while (i < b2 && l2 > 0) { --l2; b2 = (uint64_t)__ldg(offsets + l2); }
-          if (s[jj] == i) atomicAdd(isums + 2 * (size_t)l2, 1ull);
-          else atomicAdd(isums + 2 * (size_t)l2 + 1, (unsigned long long)(s[jj] - b2));
-        }
+      if (cnt) store_records<KIND>(work, i0, cnt, s, w);
+      if constexpr (KIND == kRecKind8w) {
+#pragma unroll
+        for (uint32_t j = 0; j < 4u; ++j)
+          if (j < cnt) wide |= wide_flags(w[j]);
       }
-      store_records<KIND>(work, i0, cnt, s, w);
-      if constexpr (KIND == kRecKind8w)
-        for (uint32_t j = 0; j < cnt; ++j) wide |= wide_flags(w[j]);
-    }
-    if (!isums) continue;
-    // combine: one pair of atomics per warp when all its lanes share an instance
-    const int32_t inst0 = __shfl_sync(0xFFFFFFFFu, inst, 0);
-    if (__all_sync(0xFFFFFFFFu, inst == inst0 || (inst == -1 && sT == 0 && sS == 0)) && inst0 >= 0) {
-      for (int d = 16; d > 0; d >>= 1) {
-        sT += __shfl_down_sync(0xFFFFFFFFu, sT, d);
-        sS += __shfl_down_sync(0xFFFFFFFFu, sS, d);
-      }
-      if (lane == 0) {
-        if (sT) atomicAdd(isums + 2 * (size_t)inst0, sT);
-        if (sS) atomicAdd(isums + 2 * (size_t)inst0 + 1, sS);
-      }
-    } else if (inst >= 0) {
-      if (sT) atomicAdd(isums + 2 * (size_t)inst, sT);
-      if (sS) atomicAdd(isums + 2 * (size_t)inst + 1, sS);
     }
   }
+  flush_sums(acc, isums, lane);
   if (KIND == kRecKind8w && scan.flags) add_flags(scan.flags, wide);
 }
 
@@ -470,10 +520,11 @@ cudaError_t launch_prep0_sums(const uint32_t *succ, const void *weight, int wtyp
   if (n == 0) return cudaSuccess;
   const int block = 256;
   const int grid = stream_grid(((uint64_t)n + 3) / 4, block);
+  const uint32_t run = run_groups(n, grid, block);
   int vec = ((uintptr_t)succ & 15u) == 0;
   if (wtype != 0) vec = vec && ((uintptr_t)weight & 15u) == 0;
 #define LR_SUMS(WT, KIND) \
-  k_prep0_sums<WT, KIND><<<grid, block, 0, s>>>(succ, weight, n, work, ws, err, vec, offsets, k, isums)
+  k_prep0_sums<WT, KIND><<<grid, block, 0, s>>>(succ, weight, n, work, ws, err, vec, offsets, k, isums, run)
   const bool w8 = kind == kRecKind8w;
   switch (wtype) {
     case 0: LR_SUMS(0, kRecKind8); break;
@@ -633,118 +684,102 @@ cudaError_t launch_prep0_ptrs(const uint32_t *const *sptr, const void *const *wp
   return cudaGetLastError();
 }
 
-// The instance of element `base` in a table of k nondecreasing offsets with
-// offsets[0] = 0 <= base < offsets[k]: the largest j < k with offsets[j] <=
-// base, found by the whole warp at once (every lane probes one of 32 points
-// spread over the remaining range, the ballot keeps the last probe at or
-// below base), in at most 3 rounds for up to 32768 instances.  Warp-uniform.
-__device__ __forceinline__ int32_t warp_instance(const int64_t *__restrict__ offsets, int32_t k, uint64_t base,
-                                                 uint32_t lane) {
-  int32_t lo = 0, hi = k;
-  while (hi - lo > 1) {
-    const int64_t span = hi - lo;
-    const int32_t q = lo + (int32_t)(((int64_t)(lane + 1) * span) / 33);
-    const uint32_t le = __ballot_sync(0xFFFFFFFFu, (uint64_t)__ldg(offsets + q) <= base);
-    const int t = __popc(le);
-    const int32_t nlo = __shfl_sync(0xFFFFFFFFu, q, t > 0 ? t - 1 : 0);
-    const int32_t nhi = __shfl_sync(0xFFFFFFFFu, q, t < 32 ? t : 31);
-    if (t > 0) lo = max(lo, nlo);
-    if (t < 32) hi = nhi;
-  }
-  return lo;
-}
-
 // Pointer batches without per-element atomics: the per-instance sums of
-// k_prep0_sums (terminals, local successors), read through one pointer per
-// instance.  A warp takes 128 consecutive elements (lane l: l + 32 j, so that
-// loads and record stores are coalesced); the warp finds the instance of
-// the first (warp_instance) and every lane walks forward from it.  A warp
-// whose elements all lie in one instance adds its sums with two atomics.
+// k_prep0_sums, with the same runs, read through one pointer per instance.
+// Lane l of a warp takes elements l + 32 j of a group, so that loads and
+// record stores are coalesced at any alignment.
 template <int WT, int KIND>
 __global__ void __launch_bounds__(256)
 k_prep0_ptrs_sums(const uint32_t *const *__restrict__ sptr, const void *const *__restrict__ wptr,
                   uint32_t n, void *__restrict__ work, WeightScan scan, uint32_t *__restrict__ err,
-                  const int64_t *__restrict__ offsets, int32_t k, unsigned long long *__restrict__ isums) {
+                  const int64_t *__restrict__ offsets, int32_t k, unsigned long long *__restrict__ isums,
+                  uint32_t run) {
   if (scan.unless_narrow && narrow_mode(*scan.unless_narrow)) return;
   uint32_t wide = 0;
   const uint32_t lane = threadIdx.x & 31u;
-  const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const uint64_t step = ((uint64_t)gridDim.x * blockDim.x >> 5) * 128u;
-  for (uint64_t base = warp * 128u; base < n; base += step) {
-    const int32_t lo0 = warp_instance(offsets, k, base, lane);
-    // each of the lane's four elements: its instance, then all four loads
-    // in flight together
-    int32_t inst[4];
-    uint64_t ibv[4], iev[4];
-    int32_t lo = lo0;
-    uint64_t ib = (uint64_t)__ldg(offsets + lo), ie = (uint64_t)__ldg(offsets + lo + 1);
-    const bool one = ie >= min(base + 128u, (uint64_t)n);   // warp-uniform
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const uint64_t i = base + lane + 32u * j;
-      while (i < n && i >= ie && lo + 1 < k) { ++lo; ib = ie; ie = (uint64_t)__ldg(offsets + lo + 1); }
-      inst[j] = lo;
-      ibv[j] = ib;
-      iev[j] = ie;
-    }
-    uint32_t sv[4];
-    uint64_t wv[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const uint64_t i = base + lane + 32u * j;
-      sv[j] = 0u;
-      wv[j] = 1u;
-      if (i < n && i >= ibv[j] && i < iev[j]) {
-        const uint64_t loc = i - ibv[j];
-        sv[j] = __ldcs(sptr[inst[j]] + loc);
-        if constexpr (WT == 1) wv[j] = (uint64_t)(int64_t)__ldcs(reinterpret_cast<const int *>(wptr[inst[j]]) + loc);
-        if constexpr (WT == 2) wv[j] = (uint64_t)__ldcs(reinterpret_cast<const long long *>(wptr[inst[j]]) + loc);
+  const uint32_t ngroups = (uint32_t)(((uint64_t)n + 127u) / 128u);
+  const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, warps = gridDim.x * blockDim.x >> 5;
+  InstSums acc;
+  for (uint64_t r0 = (uint64_t)warp * run; r0 < ngroups; r0 += (uint64_t)warps * run) {
+    const uint32_t r1 = (uint32_t)min((uint64_t)ngroups, r0 + run);
+    int32_t lo0 = -1;                    // instance of the group's first element (warp-uniform)
+    uint64_t ib0 = 0, ie0 = 0;
+    for (uint32_t g = (uint32_t)r0; g < r1; ++g) {
+      const uint64_t base = (uint64_t)g * 128u;
+      if (base >= ie0) {
+        lo0 = warp_instance(offsets, k, base, lane);
+        ib0 = (uint64_t)__ldg(offsets + lo0);
+        ie0 = (uint64_t)__ldg(offsets + lo0 + 1);
       }
-    }
-    unsigned long long sT = 0, sS = 0;
+      // each of the lane's four elements: its instance, then all four loads
+      // in flight together
+      const bool one = base >= ib0 && ie0 >= min(base + 128u, (uint64_t)n);   // warp-uniform
+      int32_t inst[4];
+      uint64_t ibv[4], iev[4];
+      int32_t lo = lo0;
+      uint64_t ib = ib0, ie = ie0;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const uint64_t i = base + lane + 32u * j;
-      if (i >= n) continue;
-      uint32_t s = sv[j];
-      uint64_t w = wv[j];
-      const uint64_t ib = ibv[j], ie = iev[j];
-      bool term;
-      if (i < ib || i >= ie) {
-        record_error(err, kErrRange);     // a bad offset table
-        s = (uint32_t)i;
-        term = true;
-      } else if ((uint64_t)s >= ie - ib || ib + s >= n) {
-        record_error(err, kErrRange);     // successor outside its instance
-        s = (uint32_t)i;
-        term = true;
-      } else {
-        term = (uint64_t)s == i - ib;
-        if (!term) {
-          if (one) sS += s;
-          else if (isums) atomicAdd(isums + 2 * (size_t)inst[j] + 1, (unsigned long long)s);
+      for (int j = 0; j < 4; ++j) {
+        const uint64_t i = base + lane + 32u * j;
+        if (!one)
+          while (i < n && i >= ie && lo + 1 < k) { ++lo; ib = ie; ie = (uint64_t)__ldg(offsets + lo + 1); }
+        inst[j] = lo;
+        ibv[j] = ib;
+        iev[j] = ie;
+      }
+      uint32_t sv[4];
+      uint64_t wv[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const uint64_t i = base + lane + 32u * j;
+        sv[j] = 0u;
+        wv[j] = 1u;
+        if (i < n && i >= ibv[j] && i < iev[j]) {
+          const uint64_t loc = i - ibv[j];
+          sv[j] = __ldcs(sptr[inst[j]] + loc);
+          if constexpr (WT == 1) wv[j] = (uint64_t)(int64_t)__ldcs(reinterpret_cast<const int *>(wptr[inst[j]]) + loc);
+          if constexpr (WT == 2) wv[j] = (uint64_t)__ldcs(reinterpret_cast<const long long *>(wptr[inst[j]]) + loc);
         }
-        s = (uint32_t)(ib + s);
       }
-      if (term) {
-        w = 0u;
-        if (one) sT += 1;
-        else if (isums) atomicAdd(isums + 2 * (size_t)inst[j], 1ull);
+      if (one && acc.inst != lo0) {
+        flush_sums(acc, isums, lane);
+        acc.inst = lo0;
       }
-      store_record<KIND>(work, i, s, w);
-      if constexpr (KIND == kRecKind8w) wide |= wide_flags(w);
-    }
-    if (one && isums) {
-      for (int d = 16; d > 0; d >>= 1) {
-        sT += __shfl_down_sync(0xFFFFFFFFu, sT, d);
-        sS += __shfl_down_sync(0xFFFFFFFFu, sS, d);
-      }
-      if (lane == 0) {
-        if (sT) atomicAdd(isums + 2 * (size_t)lo0, sT);
-        if (sS) atomicAdd(isums + 2 * (size_t)lo0 + 1, sS);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const uint64_t i = base + lane + 32u * j;
+        if (i >= n) continue;
+        uint32_t s = sv[j];
+        uint64_t w = wv[j];
+        const uint64_t ib = ibv[j], ie = iev[j];
+        bool term;
+        if (i < ib || i >= ie) {
+          record_error(err, kErrRange);     // a bad offset table
+          s = (uint32_t)i;
+          term = true;
+        } else if ((uint64_t)s >= ie - ib || ib + s >= n) {
+          record_error(err, kErrRange);     // successor outside its instance
+          s = (uint32_t)i;
+          term = true;
+        } else {
+          term = (uint64_t)s == i - ib;
+          if (!term) {
+            if (one) acc.s += s;
+            else if (isums) atomicAdd(isums + 2 * (size_t)inst[j] + 1, (unsigned long long)s);
+          }
+          s = (uint32_t)(ib + s);
+        }
+        if (term) {
+          w = 0u;
+          if (one) acc.t += 1;
+          else if (isums) atomicAdd(isums + 2 * (size_t)inst[j], 1ull);
+        }
+        store_record<KIND>(work, i, s, w);
+        if constexpr (KIND == kRecKind8w) wide |= wide_flags(w);
       }
     }
   }
+  flush_sums(acc, isums, lane);
   if (KIND == kRecKind8w && scan.flags) add_flags(scan.flags, wide);
 }
 
@@ -754,8 +789,9 @@ cudaError_t launch_prep0_ptrs_sums(const uint32_t *const *sptr, const void *cons
   if (n == 0) return cudaSuccess;
   const int block = 256;
   const int grid = stream_grid(((uint64_t)n + 3) / 4, block);
+  const uint32_t run = run_groups(n, grid, block);
 #define LR_PTRS_SUMS(WT, KIND) \
-  k_prep0_ptrs_sums<WT, KIND><<<grid, block, 0, s>>>(sptr, wptr, n, work, ws, err, offsets, k, isums)
+  k_prep0_ptrs_sums<WT, KIND><<<grid, block, 0, s>>>(sptr, wptr, n, work, ws, err, offsets, k, isums, run)
   const bool w8 = kind == kRecKind8w;
   switch (wtype) {
     case 0: LR_PTRS_SUMS(0, kRecKind8); break;

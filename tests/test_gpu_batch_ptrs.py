@@ -137,3 +137,32 @@ def test_ptrs_errors():
     outs = lr.rank_batch_ptrs([dev(s) for s in succ])
     for s, o2 in zip(succ, outs):
         np.testing.assert_array_equal(o2.cpu().numpy(), oracle.rank(s))
+
+
+# instance ends at and beside the ends of groups of 128 elements and of the
+# runs of groups that a warp takes (two groups at this total, on 152 SMs)
+EDGES = [128, 1, 127, 256, 257, 0, 255, 3, 1 << 20, 64, 64, 130, 5, (1 << 20) + 128 * 7 - 1, 0, 1, 129, 700_003, 126]
+
+
+@pytest.mark.parametrize("wt", [None, "i32", "i64"])
+@pytest.mark.parametrize("shift", [0, 1])
+def test_instances_across_runs(wt, shift):
+    succs, ws = _instances(9960, EDGES), _weights(wt, EDGES, 9961)
+    rt = np.int32 if wt is None else np.int64
+    want = [oracle.rank(s, None if ws is None else ws[j], rt) if len(s) else np.zeros(0, rt)
+            for j, s in enumerate(succs)]
+    offs = np.concatenate([[0], np.cumsum(EDGES)]).astype(np.int64)
+    # shift: the arrays start one element after a 16-byte boundary
+    pad = lambda a: dev(np.concatenate([a[:1]] * shift + [a]))[shift:]
+    succ, w = np.concatenate(succs), None if ws is None else np.concatenate(ws)
+    args = (dev(offs), pad(succ), None if w is None else pad(w))
+    np.testing.assert_array_equal(lr.rank_batch(*args).cpu().numpy(), np.concatenate(want))
+    got = lr.rank_batch_ptrs([dev(s) for s in succs], None if ws is None else [dev(x) for x in ws])
+    for g, x in zip(got, want):
+        np.testing.assert_array_equal(g.cpu().numpy(), x)
+    for j in (0, 8, 10, 16):                              # a successor just outside its instance
+        bad = succ.copy()
+        bad[offs[j + 1] - 1] = EDGES[j]
+        with pytest.raises(lr.LRError) as e:
+            lr.rank_batch(args[0], pad(bad), args[2])
+        assert e.value.name == "LR_ERR_OUT_OF_RANGE"
