@@ -62,6 +62,22 @@ int stream_grid(uint64_t work_items, int block) {
   return (int)(want < full ? want : full);
 }
 
+// The same for a kernel whose registers keep 2048 threads off an SM: the CTAs
+// that are resident together, so that the equal shares of a grid-stride loop
+// end together (at 40 registers 912 CTAs of 256 run first and the other 304 of
+// 1216 after them, on a third of the threads).
+template <auto Kernel>
+static int fit_grid(uint64_t work_items, int block) {
+  static CachedInt cache;
+  const int per = cached_per_device(cache, [](int, int b) {
+    int nb = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, Kernel, b, 0);
+    return nb;
+  }, block);
+  const uint64_t want = std::max<uint64_t>(1, (work_items + block - 1) / block);
+  return (int)std::min<uint64_t>(want, (uint64_t)device_sm_count() * per);
+}
+
 // ---------------------------------------------------------------- init
 __device__ __forceinline__ void init_levels(LevelDesc *desc, const InitParams &p, int l) {
   if (l < p.nlev) {
@@ -298,13 +314,12 @@ cudaError_t launch_prep0(const uint32_t *succ, const void *weight, int wtype, ui
   memset(&ip, 0, sizeof(ip));
   if (desc) ip = *init;
   const int block = 256;
-  const int grid = stream_grid(((uint64_t)n + 3) / 4, block);
   int vec = ((uintptr_t)succ & 15u) == 0;
   if (wtype == 1) vec = vec && ((uintptr_t)weight & 15u) == 0;
   if (wtype == 2) vec = vec && ((uintptr_t)weight & 15u) == 0;
 #define LR_PREP0(WT, KIND)                                                                                        \
-  k_prep0<WT, KIND><<<grid, block, 0, s>>>(succ, weight, n, work, bitmap, err, validate, vec, offsets, k, sums,    \
-                                           local, ws, desc, ip)
+  k_prep0<WT, KIND><<<fit_grid<k_prep0<WT, KIND>>(((uint64_t)n + 3) / 4, block), block, 0, s>>>(                   \
+      succ, weight, n, work, bitmap, err, validate, vec, offsets, k, sums, local, ws, desc, ip)
   const bool w8 = kind == kRecKind8w;
   switch (wtype) {
     case 0: if (kind == kRecKind16) LR_PREP0(0, kRecKind16); else LR_PREP0(0, kRecKind8); break;
@@ -519,12 +534,14 @@ cudaError_t launch_prep0_sums(const uint32_t *succ, const void *weight, int wtyp
                               cudaStream_t s) {
   if (n == 0) return cudaSuccess;
   const int block = 256;
-  const int grid = stream_grid(((uint64_t)n + 3) / 4, block);
-  const uint32_t run = run_groups(n, grid, block);
   int vec = ((uintptr_t)succ & 15u) == 0;
   if (wtype != 0) vec = vec && ((uintptr_t)weight & 15u) == 0;
-#define LR_SUMS(WT, KIND) \
-  k_prep0_sums<WT, KIND><<<grid, block, 0, s>>>(succ, weight, n, work, ws, err, vec, offsets, k, isums, run)
+#define LR_SUMS(WT, KIND)                                                                                \
+  do {                                                                                                  \
+    const int grid = fit_grid<k_prep0_sums<WT, KIND>>(((uint64_t)n + 3) / 4, block);                    \
+    k_prep0_sums<WT, KIND><<<grid, block, 0, s>>>(succ, weight, n, work, ws, err, vec, offsets, k, isums, \
+                                                  run_groups(n, grid, block));                          \
+  } while (0)
   const bool w8 = kind == kRecKind8w;
   switch (wtype) {
     case 0: LR_SUMS(0, kRecKind8); break;
@@ -788,10 +805,12 @@ cudaError_t launch_prep0_ptrs_sums(const uint32_t *const *sptr, const void *cons
                                    int32_t k, unsigned long long *isums, cudaStream_t s) {
   if (n == 0) return cudaSuccess;
   const int block = 256;
-  const int grid = stream_grid(((uint64_t)n + 3) / 4, block);
-  const uint32_t run = run_groups(n, grid, block);
-#define LR_PTRS_SUMS(WT, KIND) \
-  k_prep0_ptrs_sums<WT, KIND><<<grid, block, 0, s>>>(sptr, wptr, n, work, ws, err, offsets, k, isums, run)
+#define LR_PTRS_SUMS(WT, KIND)                                                                           \
+  do {                                                                                                  \
+    const int grid = fit_grid<k_prep0_ptrs_sums<WT, KIND>>(((uint64_t)n + 3) / 4, block);               \
+    k_prep0_ptrs_sums<WT, KIND><<<grid, block, 0, s>>>(sptr, wptr, n, work, ws, err, offsets, k, isums, \
+                                                       run_groups(n, grid, block));                     \
+  } while (0)
   const bool w8 = kind == kRecKind8w;
   switch (wtype) {
     case 0: LR_PTRS_SUMS(0, kRecKind8); break;
@@ -1685,11 +1704,11 @@ cudaError_t launch_finalize_ptrs(LevelDesc *desc, const void *work, int kind, co
                                  void *const *rptr, int rank_bytes, uint32_t cap,
                                  const int64_t *offsets, int32_t k, uint32_t *err, cudaStream_t s) {
   const int block = 256;
-  const int grid = stream_grid(((uint64_t)cap + 3) / 4, block);
 #define LR_FINP(REC, RT)                                                                          \
-  k_finalize_ptrs<REC, RT><<<grid, block, 0, s>>>(desc, reinterpret_cast<const REC *>(work),      \
-                                                  reinterpret_cast<const RT *>(rnext),            \
-                                                  reinterpret_cast<RT *const *>(rptr), offsets, k, err)
+  k_finalize_ptrs<REC, RT><<<fit_grid<k_finalize_ptrs<REC, RT>>(((uint64_t)cap + 3) / 4, block),  \
+                             block, 0, s>>>(desc, reinterpret_cast<const REC *>(work),            \
+                                            reinterpret_cast<const RT *>(rnext),                  \
+                                            reinterpret_cast<RT *const *>(rptr), offsets, k, err)
   if (kind == kRecKind8w) { if (rank_bytes == 4) LR_FINP(Rec8w, uint32_t); else LR_FINP(Rec8w, unsigned long long); }
   else if (kind == kRecKind16) { if (rank_bytes == 4) LR_FINP(Rec16, uint32_t); else LR_FINP(Rec16, unsigned long long); }
   else { if (rank_bytes == 4) LR_FINP(Rec8, uint32_t); else LR_FINP(Rec8, unsigned long long); }
@@ -1703,12 +1722,11 @@ cudaError_t launch_finalize(LevelDesc *desc, int lev, const void *work, int kind
                             uint32_t *err, const uint32_t *tnext, uint32_t *tout,
                             const uint32_t *tid_cur, cudaStream_t s) {
   const int block = 256;
-  const int grid = stream_grid(((uint64_t)cap + 3) / 4, block);
 #define LR_FIN(REC, RT, T)                                                                      \
-  k_finalize<REC, RT, T><<<grid, block, 0, s>>>(desc, lev, reinterpret_cast<const REC *>(work), \
-                                                reinterpret_cast<const RT *>(rnext),            \
-                                                reinterpret_cast<RT *>(rout), err, tnext,       \
-                                                tout, tid_cur)
+  k_finalize<REC, RT, T><<<fit_grid<k_finalize<REC, RT, T>>(((uint64_t)cap + 3) / 4, block),    \
+                           block, 0, s>>>(desc, lev, reinterpret_cast<const REC *>(work),       \
+                                          reinterpret_cast<const RT *>(rnext),                  \
+                                          reinterpret_cast<RT *>(rout), err, tnext, tout, tid_cur)
   const bool rec16 = kind == kRecKind16;
   if (kind == kRecKind8w) {
     if (tout) return cudaErrorInvalidValue;
