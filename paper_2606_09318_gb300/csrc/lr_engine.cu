@@ -408,9 +408,9 @@ Ctx *get_ctx(cudaStream_t stream, lr_status *st) {
   if (it != g_ctx.end()) { *st = LR_OK; return it->second; }
   Ctx *c = new Ctx();
   c->device = dev;
-  e = cudaMallocHost((void **)&c->host_words, 64);
+  e = cudaMallocHost((void **)&c->host_words, kHostWordsBytes);
   if (e != cudaSuccess) { delete c; *st = LR_ERR_OUT_OF_MEMORY; return nullptr; }
-  memset(c->host_words, 0, 64);
+  memset(c->host_words, 0, kHostWordsBytes);
   g_ctx[key] = c;
   *st = LR_OK;
   return c;
@@ -585,6 +585,20 @@ static lr_status map_device_bits(uint32_t bits) {
 // Copy the call's device error word to the context's pinned status word;
 // with sync, wait and return the status it encodes.  err == nullptr: a kernel
 // has written the status word itself.
+// Wait for a kernel on stream s to write `token` to the pinned word *w.  The
+// stream's state is looked at now and then, so that the wait ends whatever
+// becomes of the kernel.
+static lr_status wait_word(const uint32_t *w, uint32_t token, cudaStream_t s) {
+  for (uint32_t spin = 1; __atomic_load_n(w, __ATOMIC_ACQUIRE) != token; ++spin) {
+    if (spin % 4096 != 0) continue;
+    const cudaError_t e = cudaStreamQuery(s);
+    if (e == cudaErrorNotReady) continue;
+    LR_TRY(e);
+    return __atomic_load_n(w, __ATOMIC_ACQUIRE) == token ? LR_OK : LR_ERR_INTERNAL;
+  }
+  return LR_OK;
+}
+
 static lr_status finish_call(Ctx *c, const uint32_t *err, int sync, cudaStream_t s) {
   if (err) LR_TRY(cudaMemcpyAsync(c->host_words, err, 4, cudaMemcpyDeviceToHost, s));
   c->pending_status = true;
@@ -991,6 +1005,29 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
   uint64_t one_head = 0;
   uint32_t one_term = 0;
   bool one_list = false;                       // the host has seen that level 0 is one list
+  // Most single instances are one list: its descriptors and level-0 chase are
+  // queued before the sums are read, and do nothing if the device finds it is
+  // not one.  The sums come by a pinned word that the host watches, while the
+  // chase runs (2^20 elements: the device sat idle for 13 of the call's 131 us).
+  const bool guess = need_count && sums0 && !in.ws && !spawn0 && !ord0 && !prof.on;
+  bool chased = false;                         // and it was one
+  if (guess) {
+    const Plan g = make_plan(in.n, 1, u, rec16_0, in.rank_bytes, in.seed, grid, log0, false, false, spawn0, ord0, narrow);
+    st = ensure_buffer(&c->var, &c->var_bytes, g.var_bytes, s);
+    if (st != LR_OK) return st;
+    char *v = (char *)c->var;
+    InitParams ip = init_params(g);
+    ip.publish = c->host_words;
+    ip.token = ++c->token;
+    ip.check_local = local_exact;
+    uint32_t *ns = (uint32_t *)(v + g.off_ns);
+    LR_TRY(launch_init(desc, ip, acc, kind0 == kRecKind8w ? wflags : nullptr, (uint32_t *)(v + g.off_hA), ns,
+                       (uint32_t *)(v + g.off_hB), s));
+    LR_TRY(launch_chase(desc, 0, work0, kind0, v + g.off_work[1], ns, qctr, g.chase_grid, g.chase_block, err,
+                        (int)u.xchg, nullptr, nullptr, nullptr, nullptr, s));
+    st = wait_word(c->host_words + kHostToken, ip.token, s);
+    if (st != LR_OK) return st;
+  }
   if (need_count) {
     // count the lists (one wait), then size the recursion for exactly that many:
     // a single-instance pass counts terminals in its reduction, a batch adds
@@ -999,7 +1036,8 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
     uint64_t sums[6];                          // terminals, other successors, local links, (sample), flags,
                                                // a terminal
     const bool acc_read = log0 || sums0 || sumsv;
-    if (acc_read) LR_TRY(cudaMemcpyAsync(c->host_words + 4, acc, sizeof(sums), cudaMemcpyDeviceToHost, s));
+    if (acc_read && !guess)
+      LR_TRY(cudaMemcpyAsync(c->host_words + 4, acc, sizeof(sums), cudaMemcpyDeviceToHost, s));
     if (log0 || sums0) {
     } else if (sums0b) {
       LR_TRY(launch_count_batch(reinterpret_cast<const unsigned long long *>(bitmap), in.k, hcount, s));
@@ -1009,7 +1047,7 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
       LR_TRY(cudaMemcpyAsync(c->host_words + 1, hcount, 4, cudaMemcpyDeviceToHost, s));
     }
     if (narrow && !acc_read) LR_TRY(cudaMemcpyAsync(c->host_words + 12, wflags, 4, cudaMemcpyDeviceToHost, s));
-    LR_TRY(cudaStreamSynchronize(s));
+    if (!guess) LR_TRY(cudaStreamSynchronize(s));
     if (acc_read) {
       memcpy(sums, c->host_words + 4, sizeof(sums));
       if (!sumsv) c->host_words[1] = (uint32_t)sums[0];
@@ -1018,9 +1056,11 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
       one_list = (late_bitmap || sumsv) && sums[0] == 1 && c->host_words[1] == 1 && one_head < in.n;
       one_term = (uint32_t)sums[5];
       if (one_list && !log0) extras = t0ws = false;    // one terminal, one total: added at the end
+      chased = guess && one_list;
     }
     if (local_exact) {
       if (sums[2] * 2 >= in.n) {           // at least half the links stay in their tile
+        chased = false;
         prof.cancel();
         const lr_status cs = run_contracted(in, tuning, c, false, s);
         if (cs != LR_ERR_NOT_FOUND) return cs;
@@ -1029,6 +1069,7 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
     }
     if (narrow && narrow_mode(c->host_words[12]) == kNarrowNone) {      // (the flags, either way)
       kind0 = kRecKind16;
+      chased = false;
       LR_TRY(pack(kind0, true, nullptr));
     }
     hb = std::max<uint64_t>(1, c->host_words[1]);
@@ -1052,8 +1093,9 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
   InitParams ip = init_params(p);
   ip.err = err;
   ip.err_bits = found;
-  LR_TRY(launch_init(desc, ip, acc_heads ? acc : nullptr, kind0 == kRecKind8w ? wflags : nullptr, hA, ns,
-                     hB, s));
+  if (!chased)
+    LR_TRY(launch_init(desc, ip, acc_heads ? acc : nullptr, kind0 == kRecKind8w ? wflags : nullptr, hA, ns,
+                       hB, s));
   if (!in.ctx) { c->last_desc = desc; c->last_nlev = p.nlev; }
   if (p.spawn_cap) LR_TRY(cudaMemsetAsync(var + p.off_sctr, 0, p.spawn_zero, s));
   SpawnArgs spa;
@@ -1106,7 +1148,9 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
       LR_TRY(launch_heads(desc, l, p.nlev, bitmap, hin, (l == 0 && log0) ? (void *)in.succ : work_of(l),
                         kind, ns, hout, bcnt, err, p.base, p.hcap, s));
     prof.mark(PH_SELECT);
-    if (l == 0 && log0)
+    if (l == 0 && chased) {
+      // (queued before the wait)
+    } else if (l == 0 && log0)
       LR_TRY(launch_chase_log(desc, in.succ, work_of(1), ns, qctr, p.chase_grid, p.chase_block, err,
                               (uint32_t *)(var + p.off_log), (uint2 *)(var + p.off_hdr),
                               p.total_chunks, (uint32_t *)(fixed + p.off_logctr), s));

@@ -67,7 +67,8 @@ struct Ctx {
   bool direct_clean = false;
   uint32_t *host_words = nullptr;   // [0] device error bits, [1] head count, [2..3] tile-local
                                     // links, [4..7] sampled tile-local links and elements,
-                                    // [8..9] int64 scratch
+                                    // [8..9] int64 scratch, [4..15] first-pass sums, [16] token
+  uint32_t token = 0;               // the last one a call of this context waited for
   bool pending_status = false;
   const LevelDesc *last_desc = nullptr;   // level descriptors of the last ruling-set call
   int last_nlev = 0;

@@ -111,10 +111,20 @@ __device__ __forceinline__ void open_level(LevelDesc &e, uint64_t n1, uint32_t h
 
 // One warp: the descriptors; and with a single list (one terminal, and the
 // other successors are every id but the head's) its head and level 0's choice
-// of rulers, which otherwise takes five more launches.
-__global__ void __launch_bounds__(32)
+// of rulers, which otherwise takes five more launches.  A second warp copies
+// the sums to the host meanwhile (InitParams::publish).
+__global__ void __launch_bounds__(64)
 k_init(LevelDesc *desc, InitParams p, const unsigned long long *__restrict__ acc, const uint32_t *__restrict__ wflags,
        uint32_t *__restrict__ hlist0, uint32_t *__restrict__ ns, uint32_t *__restrict__ hnext) {
+  if (threadIdx.x >= 32) {
+    const int i = (int)threadIdx.x - 32;
+    if (!p.publish) return;
+    if (i < 6) reinterpret_cast<volatile unsigned long long *>(p.publish + 4)[i] = acc[i];
+    __threadfence_system();
+    __syncwarp();
+    if (i == 0) *reinterpret_cast<volatile uint32_t *>(p.publish + kHostToken) = p.token;
+    return;
+  }
   init_levels(desc, p, (int)threadIdx.x);
   __syncwarp();
   if (threadIdx.x != 0) return;
@@ -123,7 +133,11 @@ k_init(LevelDesc *desc, InitParams p, const unsigned long long *__restrict__ acc
   if (p.err_bits) record_error(p.err, p.err_bits);
   if (!acc || p.nlev < 2) return;
   const unsigned long long n = p.n0, h = n * (n - 1) / 2 - acc[1];
-  if (acc[0] != 1 || h >= n) return;
+  if (acc[0] != 1 || h >= n || (p.check_local && acc[2] * 2 >= n) ||
+      (p.publish && wflags && d.narrow == kNarrowNone)) {
+    if (p.publish) d.mode = kModeOff;
+    return;
+  }
   hlist0[0] = (uint32_t)h;
   d.h = 1;
   d.hsrc = kHeadsList;
@@ -141,7 +155,7 @@ k_init(LevelDesc *desc, InitParams p, const unsigned long long *__restrict__ acc
 
 cudaError_t launch_init(LevelDesc *desc, const InitParams &p, const unsigned long long *acc, const uint32_t *wflags,
                         uint32_t *hlist0, uint32_t *ns, uint32_t *hnext, cudaStream_t s) {
-  k_init<<<1, 32, 0, s>>>(desc, p, acc, wflags, hlist0, ns, hnext);
+  k_init<<<1, p.publish ? 64 : 32, 0, s>>>(desc, p, acc, wflags, hlist0, ns, hnext);
   count_launch();
   return cudaGetLastError();
 }

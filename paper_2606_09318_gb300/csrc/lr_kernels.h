@@ -27,7 +27,18 @@ struct InitParams {
   uint32_t base;                      // largest level >= 1 that the base case ranks
   uint32_t err_bits;                  // errors the host has found, recorded in *err
   uint32_t *err;
+  // The host goes on as if the input were one list that is not to be
+  // contracted (check_local: fewer than half its links stay in their tile) and
+  // whose weights fit its records: where that is not so, level 0 stays off.
+  // acc's words are copied to publish[4..15] (pinned), then token to
+  // publish[kHostToken], which the host waits for.
+  uint32_t *publish;
+  uint32_t token;
+  uint32_t check_local;
 };
+
+constexpr int kHostToken = 16;
+constexpr size_t kHostWordsBytes = 128;
 
 // Kernel launch counter (all streams).
 void count_launch(int k = 1);
