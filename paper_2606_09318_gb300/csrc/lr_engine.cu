@@ -959,8 +959,16 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
   // reads succ, and counts every tile on the way; a shorter list is packed
   // sooner than the wait for the sample takes.)
   const bool local_exact = count_local && (log0 || ((sums0 || sumsv) && in.n < kPackFirst));
-  if (count_local && !local_exact) {
-    LR_TRY(launch_local_sample(in.succ, (uint32_t)in.n, acc + 2, s));
+  // Most single instances are one list: its descriptors and level-0 chase are
+  // queued before the sums are read, and do nothing if the device finds it is
+  // not one (or that the sample says to contract it: then nor does the first
+  // pass).  The sums come by a pinned word that the host watches, while the
+  // chase runs.  (2^20 elements: the device sat idle for 13 of the call's 131
+  // us, and 9 more of 737 in the wait for the sample at 2^24.)
+  const bool guess = need_count && sums0 && !in.ws && !spawn0 && !ord0 && !prof.on;
+  const uint32_t ask_local = local_exact ? kLocalCounted : count_local && guess ? kLocalSampled : kLocalUnasked;
+  if (count_local && !local_exact) LR_TRY(launch_local_sample(in.succ, (uint32_t)in.n, acc + 2, s));
+  if (count_local && !local_exact && !guess) {
     LR_TRY(cudaMemcpyAsync(c->host_words + 4, acc + 2, 16, cudaMemcpyDeviceToHost, s));
     LR_TRY(cudaStreamSynchronize(s));
     uint64_t smp[2];
@@ -981,6 +989,7 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
     WeightScan scan;
     scan.flags = kind == kRecKind8w && in.rank_bytes == 8 ? wflags : nullptr;
     scan.unless_narrow = unless_narrow;
+    scan.unless_local = ask_local == kLocalSampled && !again ? acc : nullptr;
     unsigned long long *isums = again ? nullptr : reinterpret_cast<unsigned long long *>(bitmap);
     uint32_t *marks = again || sums0 ? nullptr : bitmap;
     if (ptrs && sums0b)
@@ -1005,11 +1014,6 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
   uint64_t one_head = 0;
   uint32_t one_term = 0;
   bool one_list = false;                       // the host has seen that level 0 is one list
-  // Most single instances are one list: its descriptors and level-0 chase are
-  // queued before the sums are read, and do nothing if the device finds it is
-  // not one.  The sums come by a pinned word that the host watches, while the
-  // chase runs (2^20 elements: the device sat idle for 13 of the call's 131 us).
-  const bool guess = need_count && sums0 && !in.ws && !spawn0 && !ord0 && !prof.on;
   bool chased = false;                         // and it was one
   if (guess) {
     const Plan g = make_plan(in.n, 1, u, rec16_0, in.rank_bytes, in.seed, grid, log0, false, false, spawn0, ord0, narrow);
@@ -1019,7 +1023,7 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
     InitParams ip = init_params(g);
     ip.publish = c->host_words;
     ip.token = ++c->token;
-    ip.check_local = local_exact;
+    ip.check_local = ask_local;
     uint32_t *ns = (uint32_t *)(v + g.off_ns);
     LR_TRY(launch_init(desc, ip, acc, kind0 == kRecKind8w ? wflags : nullptr, (uint32_t *)(v + g.off_hA), ns,
                        (uint32_t *)(v + g.off_hB), s));
@@ -1033,7 +1037,7 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
     // a single-instance pass counts terminals in its reduction, a batch adds
     // its instances' terminal counts, the other passes count zero bits of the
     // has-predecessor bitmap
-    uint64_t sums[6];                          // terminals, other successors, local links, (sample), flags,
+    unsigned long long sums[6];                // terminals, other successors, local links, (sample), flags,
                                                // a terminal
     const bool acc_read = log0 || sums0 || sumsv;
     if (acc_read && !guess)
@@ -1058,14 +1062,17 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
       if (one_list && !log0) extras = t0ws = false;    // one terminal, one total: added at the end
       chased = guess && one_list;
     }
-    if (local_exact) {
-      if (sums[2] * 2 >= in.n) {           // at least half the links stay in their tile
-        chased = false;
-        prof.cancel();
-        const lr_status cs = run_contracted(in, tuning, c, false, s);
-        if (cs != LR_ERR_NOT_FOUND) return cs;
-        prof.begin(s, (int64_t)in.n);          // not contracted after all: carry on
+    if (mostly_local(ask_local, sums, in.n)) {
+      chased = false;
+      prof.cancel();
+      const lr_status cs = run_contracted(in, tuning, c, false, s);
+      if (cs != LR_ERR_NOT_FOUND) return cs;
+      if (ask_local == kLocalSampled) {        // not contracted after all: nothing is packed yet
+        Inputs again = in;
+        again.no_contract = 1;
+        return run(again, tuning, s);
       }
+      prof.begin(s, (int64_t)in.n);            // the same: carry on
     }
     if (narrow && narrow_mode(c->host_words[12]) == kNarrowNone) {      // (the flags, either way)
       kind0 = kRecKind16;

@@ -133,7 +133,7 @@ k_init(LevelDesc *desc, InitParams p, const unsigned long long *__restrict__ acc
   if (p.err_bits) record_error(p.err, p.err_bits);
   if (!acc || p.nlev < 2) return;
   const unsigned long long n = p.n0, h = n * (n - 1) / 2 - acc[1];
-  if (acc[0] != 1 || h >= n || (p.check_local && acc[2] * 2 >= n) ||
+  if (acc[0] != 1 || h >= n || mostly_local(p.check_local, acc, n) ||
       (p.publish && wflags && d.narrow == kNarrowNone)) {
     if (p.publish) d.mode = kModeOff;
     return;
@@ -231,6 +231,7 @@ k_prep0(const uint32_t *__restrict__ succ, const void *__restrict__ weight, uint
         unsigned long long *__restrict__ sums, unsigned long long *__restrict__ local,
         WeightScan scan, LevelDesc *__restrict__ desc, InitParams ip) {
   if (scan.unless_narrow && narrow_mode(*scan.unless_narrow)) return;
+  if (scan.unless_local && mostly_local(kLocalSampled, scan.unless_local, n)) return;
   uint32_t wide = 0;
   if (desc && blockIdx.x == 0) init_levels(desc, ip, (int)threadIdx.x);
   unsigned long long sT = 0, sS = 0, sL = 0;

@@ -28,7 +28,7 @@ struct InitParams {
   uint32_t err_bits;                  // errors the host has found, recorded in *err
   uint32_t *err;
   // The host goes on as if the input were one list that is not to be
-  // contracted (check_local: fewer than half its links stay in their tile) and
+  // contracted (check_local: kLocalCounted or kLocalSampled) and
   // whose weights fit its records: where that is not so, level 0 stays off.
   // acc's words are copied to publish[4..15] (pinned), then token to
   // publish[kHostToken], which the host waits for.
@@ -38,6 +38,13 @@ struct InitParams {
 };
 
 constexpr int kHostToken = 16;
+
+// Whether at least half the links stay in their tile, from the first pass's
+// sums: counted over all n links, or over a sample, or not asked.
+enum : uint32_t { kLocalUnasked = 0, kLocalCounted = 1, kLocalSampled = 2 };
+__host__ __device__ inline bool mostly_local(uint32_t how, const unsigned long long *acc, unsigned long long n) {
+  return how != kLocalUnasked && acc[2] * 2 >= (how == kLocalCounted ? n : acc[3]);
+}
 constexpr size_t kHostWordsBytes = 128;
 
 // Kernel launch counter (all streams).
@@ -68,6 +75,8 @@ cudaError_t launch_init(LevelDesc *desc, const InitParams &p, const unsigned lon
 struct WeightScan {
   uint32_t *flags;
   const uint32_t *unless_narrow;
+  const unsigned long long *unless_local;   // launch_prep0: the sums, whose sample may show that the input will be
+                                            // contracted; the pass does nothing then (null: not asked)
 };
 
 constexpr int kSumTerminal = 5;

@@ -186,3 +186,20 @@ def test_errors_with_contraction():
     assert _status(inner.astype(np.uint32), tuning=ON, validate=True) == "LR_ERR_NOT_A_LIST"
     # the stream still works
     np.testing.assert_array_equal(rank(succ.astype(np.uint32), tuning=ON), oracle.rank(succ.astype(np.uint32)))
+
+
+@pytest.mark.parametrize("wt", [None, "i32", "i64"])
+@pytest.mark.parametrize("n", [(1 << 22) - 4096, (1 << 22) + 4096 * 3 + 17])
+def test_only_the_sampled_tiles_are_local(n, wt):
+    # every 16th tile of 4096 is one run of the list, the rest in random order:
+    # the sample says to contract, the tiles' heads then do not
+    ids = np.arange(n, dtype=np.uint32)
+    sampled = (ids >> 12) % 16 == 0
+    order = np.concatenate([ids[sampled], gen.rng(9970).permutation(ids[~sampled])])
+    succ = np.empty(n, np.uint32)
+    succ[order[:-1]] = order[1:]
+    succ[order[-1]] = order[-1]
+    w = None if wt is None else (gen.weights_i32 if wt == "i32" else gen.weights_i64)(n, 9971)
+    want = oracle.rank(succ, w, np.int32 if wt is None else np.int64)
+    got = lr.rank(dev(succ), None if w is None else dev(w))
+    np.testing.assert_array_equal(got.cpu().numpy(), want)
