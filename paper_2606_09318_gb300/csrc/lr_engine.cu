@@ -965,7 +965,7 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
   // pass).  The sums come by a pinned word that the host watches, while the
   // chase runs.  (2^20 elements: the device sat idle for 13 of the call's 131
   // us, and 9 more of 737 in the wait for the sample at 2^24.)
-  const bool guess = need_count && sums0 && !in.ws && !spawn0 && !ord0 && !prof.on;
+  const bool guess = need_count && (sums0 || sumsv) && !in.ws && !spawn0 && !ord0 && !prof.on;
   const uint32_t ask_local = local_exact ? kLocalCounted : count_local && guess ? kLocalSampled : kLocalUnasked;
   if (count_local && !local_exact) LR_TRY(launch_local_sample(in.succ, (uint32_t)in.n, acc + 2, s));
   if (count_local && !local_exact && !guess) {
@@ -1024,6 +1024,10 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
     ip.publish = c->host_words;
     ip.token = ++c->token;
     ip.check_local = ask_local;
+    if (sumsv) {
+      ip.heads = hcount;
+      LR_TRY(launch_count_heads(bitmap, (uint32_t)in.n, hcount, s));
+    }
     uint32_t *ns = (uint32_t *)(v + g.off_ns);
     LR_TRY(launch_init(desc, ip, acc, kind0 == kRecKind8w ? wflags : nullptr, (uint32_t *)(v + g.off_hA), ns,
                        (uint32_t *)(v + g.off_hB), s));
@@ -1042,7 +1046,7 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
     const bool acc_read = log0 || sums0 || sumsv;
     if (acc_read && !guess)
       LR_TRY(cudaMemcpyAsync(c->host_words + 4, acc, sizeof(sums), cudaMemcpyDeviceToHost, s));
-    if (log0 || sums0) {
+    if (log0 || sums0 || guess) {
     } else if (sums0b) {
       LR_TRY(launch_count_batch(reinterpret_cast<const unsigned long long *>(bitmap), in.k, hcount, s));
       LR_TRY(cudaMemcpyAsync(c->host_words + 1, hcount, 4, cudaMemcpyDeviceToHost, s));

@@ -120,6 +120,7 @@ k_init(LevelDesc *desc, InitParams p, const unsigned long long *__restrict__ acc
     const int i = (int)threadIdx.x - 32;
     if (!p.publish) return;
     if (i < 6) reinterpret_cast<volatile unsigned long long *>(p.publish + 4)[i] = acc[i];
+    if (i == 6 && p.heads) *reinterpret_cast<volatile uint32_t *>(p.publish + 1) = *p.heads;
     __threadfence_system();
     __syncwarp();
     if (i == 0) *reinterpret_cast<volatile uint32_t *>(p.publish + kHostToken) = p.token;
@@ -133,7 +134,7 @@ k_init(LevelDesc *desc, InitParams p, const unsigned long long *__restrict__ acc
   if (p.err_bits) record_error(p.err, p.err_bits);
   if (!acc || p.nlev < 2) return;
   const unsigned long long n = p.n0, h = n * (n - 1) / 2 - acc[1];
-  if (acc[0] != 1 || h >= n || mostly_local(p.check_local, acc, n) ||
+  if (acc[0] != 1 || h >= n || (p.heads && *p.heads != 1) || mostly_local(p.check_local, acc, n) ||
       (p.publish && wflags && d.narrow == kNarrowNone)) {
     if (p.publish) d.mode = kModeOff;
     return;

@@ -30,9 +30,11 @@ struct InitParams {
   // The host goes on as if the input were one list that is not to be
   // contracted (check_local: kLocalCounted or kLocalSampled) and
   // whose weights fit its records: where that is not so, level 0 stays off.
-  // acc's words are copied to publish[4..15] (pinned), then token to
+  // acc's words are copied to publish[4..15] (pinned) and the counted heads,
+  // if any (validation: one list has one), to publish[1], then token to
   // publish[kHostToken], which the host waits for.
   uint32_t *publish;
+  const uint32_t *heads;
   uint32_t token;
   uint32_t check_local;
 };
