@@ -965,7 +965,10 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
   // pass).  The sums come by a pinned word that the host watches, while the
   // chase runs.  (2^20 elements: the device sat idle for 13 of the call's 131
   // us, and 9 more of 737 in the wait for the sample at 2^24.)
-  const bool guess = need_count && (sums0 || sumsv) && !in.ws && !spawn0 && !ord0 && !prof.on;
+  // Likewise a batch, as one list per instance.
+  const bool guess_batch = sums0b && in.k <= kMaxOpenBatch && !ord_used;
+  const bool guess = need_count && (sums0 || sumsv || guess_batch) && !in.ws && !spawn0 && !prof.on;
+  const uint64_t guess_lists = guess_batch ? (uint64_t)in.k : 1;
   const uint32_t ask_local = local_exact ? kLocalCounted : count_local && guess ? kLocalSampled : kLocalUnasked;
   if (count_local && !local_exact) LR_TRY(launch_local_sample(in.succ, (uint32_t)in.n, acc + 2, s));
   if (count_local && !local_exact && !guess) {
@@ -1016,7 +1019,7 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
   bool one_list = false;                       // the host has seen that level 0 is one list
   bool chased = false;                         // and it was one
   if (guess) {
-    const Plan g = make_plan(in.n, 1, u, rec16_0, in.rank_bytes, in.seed, grid, log0, false, false, spawn0, ord0, narrow);
+    const Plan g = make_plan(in.n, guess_lists, u, rec16_0, in.rank_bytes, in.seed, grid, log0, false, false, spawn0, ord0, narrow);
     st = ensure_buffer(&c->var, &c->var_bytes, g.var_bytes, s);
     if (st != LR_OK) return st;
     char *v = (char *)c->var;
@@ -1029,8 +1032,13 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
       LR_TRY(launch_count_heads(bitmap, (uint32_t)in.n, hcount, s));
     }
     uint32_t *ns = (uint32_t *)(v + g.off_ns);
-    LR_TRY(launch_init(desc, ip, acc, kind0 == kRecKind8w ? wflags : nullptr, (uint32_t *)(v + g.off_hA), ns,
-                       (uint32_t *)(v + g.off_hB), s));
+    if (guess_batch)
+      LR_TRY(launch_open_batch(desc, ip, reinterpret_cast<const unsigned long long *>(bitmap), in.offsets, in.k,
+                               kind0 == kRecKind8w ? wflags : nullptr, work0, kind0, ns,
+                               (uint32_t *)(v + g.off_hB), s));
+    else
+      LR_TRY(launch_init(desc, ip, acc, kind0 == kRecKind8w ? wflags : nullptr, (uint32_t *)(v + g.off_hA), ns,
+                         (uint32_t *)(v + g.off_hB), s));
     LR_TRY(launch_chase(desc, 0, work0, kind0, v + g.off_work[1], ns, qctr, g.chase_grid, g.chase_block, err,
                         (int)u.xchg, nullptr, nullptr, nullptr, nullptr, s));
     st = wait_word(c->host_words + kHostToken, ip.token, s);
@@ -1054,7 +1062,7 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
       LR_TRY(launch_count_heads(bitmap, (uint32_t)in.n, hcount, s));
       LR_TRY(cudaMemcpyAsync(c->host_words + 1, hcount, 4, cudaMemcpyDeviceToHost, s));
     }
-    if (narrow && !acc_read) LR_TRY(cudaMemcpyAsync(c->host_words + 12, wflags, 4, cudaMemcpyDeviceToHost, s));
+    if (narrow && !acc_read && !guess) LR_TRY(cudaMemcpyAsync(c->host_words + 12, wflags, 4, cudaMemcpyDeviceToHost, s));
     if (!guess) LR_TRY(cudaStreamSynchronize(s));
     if (acc_read) {
       memcpy(sums, c->host_words + 4, sizeof(sums));
@@ -1065,6 +1073,8 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
       one_term = (uint32_t)sums[5];
       if (one_list && !log0) extras = t0ws = false;    // one terminal, one total: added at the end
       chased = guess && one_list;
+    } else if (guess) {
+      chased = c->host_words[2] != 0;
     }
     if (mostly_local(ask_local, sums, in.n)) {
       chased = false;
@@ -1083,7 +1093,7 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
       chased = false;
       LR_TRY(pack(kind0, true, nullptr));
     }
-    hb = std::max<uint64_t>(1, c->host_words[1]);
+    hb = chased ? guess_lists : std::max<uint64_t>(1, c->host_words[1]);
     p = make_plan(in.n, hb, u, rec16_0, in.rank_bytes, in.seed, grid, log0, extras, t0ws, spawn0, ord0, narrow);
   }
   if (!in.ws) {
@@ -1124,7 +1134,7 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
   if ((log0 || sums0) && !one_list) {
     if (late_bitmap) LR_TRY(cudaMemsetAsync(bitmap, 0, bitmap_bytes, s));
     LR_TRY(launch_bitmap0(desc, in.succ, (uint32_t)in.n, bitmap, err, in.validate, s));
-  } else if (sums0b)
+  } else if (sums0b && !chased)
     LR_TRY(launch_heads0_batch(desc, reinterpret_cast<unsigned long long *>(bitmap), in.offsets, in.k, hA,
                                p.hcap, work0, kind0, (uint32_t)in.n, bitmap, s));
 
@@ -1155,7 +1165,7 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
       }
     }
     const int kind = (l == 0 && log0) ? kRecKindSucc : l == 0 ? kind0 : kRecKind16;
-    if (l > 0 || !one_list)
+    if (l > 0 || !(one_list || chased))
       LR_TRY(launch_heads(desc, l, p.nlev, bitmap, hin, (l == 0 && log0) ? (void *)in.succ : work_of(l),
                         kind, ns, hout, bcnt, err, p.base, p.hcap, s));
     prof.mark(PH_SELECT);

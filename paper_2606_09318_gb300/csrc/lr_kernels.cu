@@ -1054,6 +1054,100 @@ k_heads_few(LevelDesc *desc, int lev, int nlev, const uint32_t *__restrict__ hli
   }
 }
 
+// A batch of one list per instance: what k_init, k_count_batch,
+// k_heads0_batch and the ruler selection do, in one CTA that needs no bitmap
+// and whose result the host reads while the chase runs (48 requests, 3 million
+// elements: the call 495 us with the seven launches and the wait, 449 with
+// this).  The first pass over the instances only looks, so that a batch of
+// another kind is left as it was found.
+template <class Rec>
+__global__ void __launch_bounds__(1024)
+k_open_batch(LevelDesc *desc, InitParams p, const unsigned long long *__restrict__ isums,
+             const int64_t *__restrict__ offsets, int32_t k, const uint32_t *__restrict__ wflags,
+             Rec *__restrict__ work, uint32_t *__restrict__ ns, uint32_t *__restrict__ hnext) {
+  __shared__ uint64_t sm[33];
+  init_levels(desc, p, (int)threadIdx.x);
+  const uint32_t n = p.n0;
+  const uint32_t narrow = std::is_same<Rec, Rec8w>::value && wflags ? narrow_mode(*wflags) : kNarrowNone;
+  // the head of instance j; false: none (empty), or (ok cleared) not one list
+  auto head_of = [&](int32_t j, bool &ok, uint64_t &terms, uint32_t &x) -> bool {
+    const int64_t b0 = offsets[j], b1 = offsets[j + 1];
+    const unsigned long long T = isums[2 * (size_t)j], S = isums[2 * (size_t)j + 1];
+    terms += T;
+    if (b0 < 0 || b1 < b0 || (uint64_t)b1 > n) { ok = false; return false; }
+    const uint64_t nj = (uint64_t)(b1 - b0), h = nj * (nj - 1) / 2 - S;
+    if (nj == 0) return false;
+    if (T != 1 || h >= nj) { ok = false; return false; }
+    x = (uint32_t)((uint64_t)b0 + h);
+    return true;
+  };
+  bool ok = !(std::is_same<Rec, Rec8w>::value && wflags && narrow == kNarrowNone);
+  uint64_t terms = 0, total;
+  uint32_t heads = 0;
+  for (int32_t j = (int32_t)threadIdx.x; j < k; j += (int32_t)blockDim.x) {
+    uint32_t x;
+    heads += head_of(j, ok, terms, x);
+  }
+  block_exclusive_scan(terms, sm, &total);
+  ok = __syncthreads_and(ok);
+  if (threadIdx.x == 32) {
+    volatile uint32_t *w = p.publish;
+    w[1] = total > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)total;
+    w[2] = ok;
+    w[12] = wflags ? *wflags : 0u;
+    __threadfence_system();
+    w[kHostToken] = p.token;
+  }
+  LevelDesc &m = desc[0];
+  if (!ok) {
+    if (threadIdx.x == 0) m.mode = kModeOff;
+    return;
+  }
+  Perm P;
+  P.init(n, p.seed[0]);
+  const uint32_t r = (uint32_t)(((uint64_t)n + p.f_inv[0] - 1) / p.f_inv[0]);
+  uint32_t nN = 0, nH = 0, nZ = 0;               // extra rulers, heads below, resolved so far
+  for (int32_t j0 = 0; j0 < k; j0 += (int32_t)blockDim.x) {
+    const int32_t j = j0 + (int32_t)threadIdx.x;
+    uint32_t x = 0, id = 0;
+    uint64_t w = 0, t = 0;
+    int c = -1;
+    bool fine = true;
+    if (j < k && head_of(j, fine, t, x)) c = classify_head<Rec, true>(x, P, r, narrow, work, &id, &w);
+    const bool isnew = c == kCatNew, ishead = isnew || c == kCatSampled;
+    const uint64_t at = block_exclusive_scan(((uint64_t)ishead << 32) | (isnew ? 1u : 0u), sm, &total);
+    const uint32_t posN = nN + (uint32_t)at, posH = nH + (uint32_t)(at >> 32);
+    if (ishead) hnext[posH] = isnew ? r + posN : id;      // (the lists hold k)
+    if (isnew) ns[posN] = x;
+    if (c == kCatSingle) st_rec(work + x, kZeroCid, (uint64_t)0 - w);
+    nZ += __syncthreads_count(c == kCatSingle);
+    nN += (uint32_t)total;
+    nH += (uint32_t)(total >> 32);
+  }
+  if (threadIdx.x == 0) {
+    m.narrow = narrow;
+    m.h = nH + nZ;
+    m.hsrc = kHeadsList;
+    m.k = nN;
+    m.visited = nZ;
+    m.picked = 1u;
+    open_level(desc[1], (uint64_t)r + nN, nH, p.nlev == 2, p.base);
+  }
+}
+
+cudaError_t launch_open_batch(LevelDesc *desc, const InitParams &p, const unsigned long long *isums,
+                              const int64_t *offsets, int32_t k, const uint32_t *wflags, void *work, int kind,
+                              uint32_t *ns, uint32_t *hnext, cudaStream_t s) {
+#define LR_OPEN(REC)                                                                                              \
+  k_open_batch<REC><<<1, 1024, 0, s>>>(desc, p, isums, offsets, k, wflags, reinterpret_cast<REC *>(work), ns, hnext)
+  if (kind == kRecKind8w) LR_OPEN(Rec8w);
+  else if (kind == kRecKind16) LR_OPEN(Rec16);
+  else LR_OPEN(Rec8);
+#undef LR_OPEN
+  count_launch();
+  return cudaGetLastError();
+}
+
 cudaError_t launch_heads(LevelDesc *desc, int lev, int nlev, const uint32_t *bitmap,
                          const uint32_t *hlist, void *work, int rec_kind, uint32_t *ns,
                          uint32_t *hnext, uint64_t *blockcnt, uint32_t *err, uint32_t cutoff,

@@ -105,6 +105,14 @@ cudaError_t launch_prep0_sums(const uint32_t *succ, const void *weight, int wtyp
                               const WeightScan &ws, uint32_t *err, const int64_t *offsets, int32_t k, unsigned long long *isums,
                               cudaStream_t s);
 cudaError_t launch_count_batch(const unsigned long long *isums, int32_t k, uint32_t *out, cudaStream_t s);
+// Batch that the host takes for one list per instance: the descriptors, the
+// heads and level 0's choice of rulers in one launch, and to p.publish the
+// number of lists ([1]), whether it is so ([2]; otherwise level 0 stays off and
+// the sums stay as they are) and *wflags ([12]), then the token.
+constexpr int32_t kMaxOpenBatch = 4096;
+cudaError_t launch_open_batch(LevelDesc *desc, const InitParams &p, const unsigned long long *isums,
+                              const int64_t *offsets, int32_t k, const uint32_t *wflags, void *work, int kind,
+                              uint32_t *ns, uint32_t *hnext, cudaStream_t s);
 cudaError_t launch_heads0_batch(LevelDesc *desc, unsigned long long *isums, const int64_t *offsets, int32_t k,
                                 uint32_t *hlist0, uint32_t hcap, const void *work, int kind, uint32_t n,
                                 uint32_t *bitmap, cudaStream_t s);

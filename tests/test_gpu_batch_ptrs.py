@@ -166,3 +166,28 @@ def test_instances_across_runs(wt, shift):
         with pytest.raises(lr.LRError) as e:
             lr.rank_batch(args[0], pad(bad), args[2])
         assert e.value.name == "LR_ERR_OUT_OF_RANGE"
+
+
+@pytest.mark.parametrize("k,mean", [(1, 600_000), (1024, 700), (1025, 700), (4096, 200), (4097, 200)])
+@pytest.mark.parametrize("odd", [None, "forest", "wide", "two terminals"])
+def test_one_list_per_instance_or_not(k, mean, odd):
+    # the head of every instance from its sums, with empty and one-element
+    # instances, and batches that turn out not to be of that kind
+    sizes = [mean] if k == 1 else [int(x) for x in gen.rng(9980 + k).integers(0, 2 * mean, size=k)]
+    if k > 1:
+        sizes[k // 2:k // 2 + 2] = [0, 1]
+    at = int(np.argmax(sizes))
+    succs = _instances(9981, sizes, forest_at=(at,) if odd == "forest" else ())
+    w = [x % 1000 for x in _weights("i64", sizes, 9982)]
+    if odd == "wide":
+        w[at][sizes[at] // 2] = 1 << 40
+    if odd == "two terminals":
+        succs[at][sizes[at] // 2] = sizes[at] // 2
+    want = np.concatenate([oracle.rank(s, w[j], np.int64) if len(s) else np.zeros(0, np.int64)
+                           for j, s in enumerate(succs)])
+    offs = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+    got = lr.rank_batch(dev(offs), dev(np.concatenate(succs)), dev(np.concatenate(w)))
+    np.testing.assert_array_equal(got.cpu().numpy(), want)
+    if k <= 1025:
+        outs = lr.rank_batch_ptrs([dev(s) for s in succs], [dev(x) for x in w])
+        np.testing.assert_array_equal(torch.cat(outs).cpu().numpy(), want)
