@@ -270,8 +270,9 @@ lr_status lr_rank_batch_outputs(const int64_t *offsets, const uint32_t *succ, co
 
 /*
  * End-to-end form with HOST buffers (pageable or pinned): copies succ and
- * weight to the device, ranks, copies rank back and waits.  Returns the
- * final status (argument or device error).
+ * weight to the device, ranks, copies rank back and waits.  Pinned buffers
+ * aligned to their elements may be read and written by the kernels in place
+ * of the copies.  Returns the final status (argument or device error).
  */
 lr_status lr_rank_host(const uint32_t *succ_host, const void *weight_host, int64_t n,
                        void *rank_host, const lr_opts *opts, lr_stream stream);

@@ -538,6 +538,17 @@ struct Profiler {
 enum { PH_PREP = 0, PH_SELECT, PH_CHASE0, PH_CHASE, PH_BASE, PH_FINAL };
 
 // ---------------------------------------------------------------- the run
+// Pinned host buffers, as the device sees them (or null): the inputs, of which
+// Inputs::succ and weight are then device memory to hold a copy where one is
+// needed, and where the ranks go; *ranks_out is set if they went there rather
+// than to Inputs::rank.
+struct HostBuffers {
+  const uint32_t *succ;
+  const void *weight;
+  void *rank;
+  bool *ranks_out;
+};
+
 struct Inputs {
   const uint32_t *succ;
   const void *weight;
@@ -564,6 +575,7 @@ struct Inputs {
   uint32_t *err_ext;             // record device errors here (and do not clear it)
   int no_contract;               // never contract (the contracted list itself)
   int builtin_tuning;            // ignore LR_TUNING and the autotuned table
+  HostBuffers h;
 };
 
 static lr_status map_device_bits(uint32_t bits) {
@@ -843,7 +855,8 @@ static lr_status run_contracted(const Inputs &in, const lr_tuning *tuning, Ctx *
   return finish_call(c, err, in.sync, s);
 }
 
-lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
+lr_status run(const Inputs &given, const lr_tuning *tuning, cudaStream_t s) {
+  Inputs in = given;
   const bool ptrs = in.sptr != nullptr;
   lr_status st = LR_OK;
   Ctx *c = in.ctx ? in.ctx : get_ctx(s, &st);
@@ -854,12 +867,24 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
     c->pending_status = false;
     return LR_OK;
   }
+  // Inputs in host memory: the base case and the first pass of the exchange
+  // form, which read them once, read them where they are; the other forms
+  // copy them first.
+  auto fetch = [&]() -> cudaError_t {
+    if (!in.h.succ) return cudaSuccess;
+    cudaError_t e = cudaMemcpyAsync((void *)in.succ, in.h.succ, 4 * in.n, cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess && in.wtype)
+      e = cudaMemcpyAsync((void *)in.weight, in.h.weight, (in.wtype == 1 ? 4 : 8) * in.n, cudaMemcpyHostToDevice, s);
+    in.h.succ = nullptr;
+    return e;
+  };
   const bool capturing = stream_capturing(s);
   const Tuning u = in.builtin_tuning ? resolve_tuning_builtin((int64_t)in.n, in.wtype != 0, false)
                                      : resolve_tuning(tuning, (int64_t)in.n, in.wtype != 0,
                                                       in.offsets != nullptr || ptrs);
   if (u.algo == LR_ALGO_WYLLIE && !ptrs) {
     if (in.term || in.prefix || in.incl) return LR_ERR_INVALID_ARGUMENT;   // default algorithm only
+    LR_TRY(fetch());
     return run_wyllie(in, c, s);
   }
   if (u.algo != LR_ALGO_SRS && u.algo != LR_ALGO_WYLLIE) return LR_ERR_INVALID_ARGUMENT;
@@ -882,6 +907,7 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
                             in.offsets == nullptr && !extras && in.ws == nullptr && in.ctx == nullptr &&
                             !capturing && in.max_lists <= 0 && in.n >= 16384 && in.n <= 0xFFFFFFFEull;
   if (contractible && u.contract == LR_CONTRACT_ON) {
+    LR_TRY(fetch());
     const lr_status cs = run_contracted(in, tuning, c, true, s);
     if (cs != LR_ERR_NOT_FOUND) return cs;
   }
@@ -919,8 +945,19 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
       if (st != LR_OK) return st;
       var = (char *)c->var;
     }
+    if (in.h.succ) {
+      in.succ = in.h.succ;
+      in.weight = in.h.weight;
+    }
+    if (in.h.rank) {
+      in.rank = in.h.rank;
+      *in.h.ranks_out = true;
+    }
     return run_base(in, p, checked, fixed, var, c, s);
   }
+  if (log0) LR_TRY(fetch());
+  // (the log form's last pass would hold every SM for the time of the link)
+  const bool ranks_to_host = in.h.rank && !log0;
   LevelDesc *desc = (LevelDesc *)(fixed + p.off_desc);
   uint32_t *err = in.err_ext ? in.err_ext : (uint32_t *)(fixed + p.off_err);
   uint32_t *hcount = (uint32_t *)(fixed + p.off_hcount);
@@ -970,13 +1007,15 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
   const bool guess = need_count && (sums0 || sumsv || guess_batch) && !in.ws && !spawn0 && !prof.on;
   const uint64_t guess_lists = guess_batch ? (uint64_t)in.k : 1;
   const uint32_t ask_local = local_exact ? kLocalCounted : count_local && guess ? kLocalSampled : kLocalUnasked;
-  if (count_local && !local_exact) LR_TRY(launch_local_sample(in.succ, (uint32_t)in.n, acc + 2, s));
+  if (count_local && !local_exact)
+    LR_TRY(launch_local_sample(in.h.succ ? in.h.succ : in.succ, (uint32_t)in.n, acc + 2, s));
   if (count_local && !local_exact && !guess) {
     LR_TRY(cudaMemcpyAsync(c->host_words + 4, acc + 2, 16, cudaMemcpyDeviceToHost, s));
     LR_TRY(cudaStreamSynchronize(s));
     uint64_t smp[2];
     memcpy(smp, c->host_words + 4, 16);
     if (smp[0] * 2 >= smp[1]) {                // at least half the sampled links stay in their tile
+      LR_TRY(fetch());
       prof.cancel();
       const lr_status cs = run_contracted(in, tuning, c, false, s);
       if (cs != LR_ERR_NOT_FOUND) return cs;
@@ -993,6 +1032,9 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
     scan.flags = kind == kRecKind8w && in.rank_bytes == 8 ? wflags : nullptr;
     scan.unless_narrow = unless_narrow;
     scan.unless_local = ask_local == kLocalSampled && !again ? acc : nullptr;
+    const bool host = in.h.succ && !again;
+    scan.succ_copy = host ? (uint32_t *)in.succ : nullptr;
+    scan.weight_copy = host ? (void *)in.weight : nullptr;
     unsigned long long *isums = again ? nullptr : reinterpret_cast<unsigned long long *>(bitmap);
     uint32_t *marks = again || sums0 ? nullptr : bitmap;
     if (ptrs && sums0b)
@@ -1003,7 +1045,7 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
     if (sums0b)
       return launch_prep0_sums(in.succ, in.weight, in.wtype, n, work0, kind, scan, err, in.offsets, in.k, isums, s);
     const bool sums = (sums0 || sumsv) && !again;
-    return launch_prep0(in.succ, in.weight, in.wtype, n, work0, kind, marks, err, in.validate && !sumsv, in.offsets,
+    return launch_prep0(host ? in.h.succ : in.succ, host ? in.h.weight : in.weight, in.wtype, n, work0, kind, marks, err, in.validate && !sumsv, in.offsets,
                         in.k, sums ? acc : nullptr, sums && local_exact ? acc + 2 : nullptr, scan, nullptr, nullptr, s);
   };
   int kind0 = narrow ? kRecKind8w : rec16_0 ? kRecKind16 : kRecKind8;
@@ -1079,6 +1121,7 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
     if (mostly_local(ask_local, sums, in.n)) {
       chased = false;
       prof.cancel();
+      if (ask_local == kLocalSampled) LR_TRY(fetch());
       const lr_status cs = run_contracted(in, tuning, c, false, s);
       if (cs != LR_ERR_NOT_FOUND) return cs;
       if (ask_local == kLocalSampled) {        // not contracted after all: nothing is packed yet
@@ -1139,7 +1182,7 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
                                p.hcap, work0, kind0, (uint32_t)in.n, bitmap, s));
 
   auto work_of = [&](int l) -> void * { return l == 0 ? work0 : (void *)(var + p.off_work[l]); };
-  auto R_of = [&](int l) -> void * { return l == 0 ? in.rank : (void *)(var + p.off_R[l]); };
+  auto R_of = [&](int l) -> void * { return l == 0 ? (ranks_to_host ? in.h.rank : in.rank) : (void *)(var + p.off_R[l]); };
   // terminal ids: T_l of every element of level l (the caller's array, or
   // workspace, at level 0), tid_l of every terminal of level l >= 1
   uint32_t *T0 = extras ? (in.term ? in.term : (uint32_t *)(var + p.off_T0)) : nullptr;
@@ -1218,19 +1261,20 @@ lr_status run(const Inputs &in, const lr_tuning *tuning, cudaStream_t s) {
       LR_TRY(launch_spawn_scatter(desc, 0, R_of(1), var + p.off_srraw, p.rank_bytes, spa.used,
                                   (uint32_t *)(var + p.off_supre), p.raw_cap, s));
       LR_TRY(launch_finalize(desc, 0, work0, kind0, var + p.off_srraw, R_of(0), p.rank_bytes, p.cap[0],
-                             err, nullptr, nullptr, nullptr, s));
+                             err, nullptr, nullptr, nullptr, s, ranks_to_host));
     } else
       LR_TRY(launch_finalize(desc, l, work_of(l), l > 0 ? (int)kRecKind16 : kind0, R_of(l + 1), R_of(l),
-                             p.rank_bytes, p.cap[l], err, T_of(l + 1), T_of(l), tid_of(l), s));
+                             p.rank_bytes, p.cap[l], err, T_of(l + 1), T_of(l), tid_of(l), s, l == 0 && ranks_to_host));
     if (l == 0 && both) {
       if (ptrs)
         LR_TRY(launch_finalize_ptrs(desc, work0, kRecKind16, R_of(1), in.rptr, p.rank_bytes, p.cap[0], in.offsets,
                                     in.k, err, s));
       else
         LR_TRY(launch_finalize(desc, 0, work0, kRecKind16, R_of(1), R_of(0), p.rank_bytes, p.cap[0], err, nullptr,
-                               nullptr, nullptr, s));
+                               nullptr, nullptr, s, ranks_to_host));
     }
   }
+  if (ranks_to_host) *in.h.ranks_out = true;
   if (outputs && !extras) {
     Perm P;                                    // the head is a ruler: its rank at level 1
     P.init((uint32_t)in.n, p.seed[0]);
@@ -1369,7 +1413,8 @@ static void set_outputs(Inputs &in, const lr_outputs *outs) {
 }
 
 static lr_status rank_ex_impl(const uint32_t *succ, const void *weight, int64_t n, void *rank,
-                              const lr_outputs *outs, const lr_opts *opts, lr_stream stream) {
+                              const lr_outputs *outs, const lr_opts *opts, lr_stream stream,
+                              const HostBuffers *host = nullptr) {
   lr_opts d;
   if (!opts) { lr_opts_default(&d); if (weight) { d.wtype = LR_I64; d.rtype = LR_I64; } opts = &d; }
   if (n < 0 || n > LR_MAX_N) return LR_ERR_INVALID_ARGUMENT;
@@ -1392,6 +1437,7 @@ static lr_status rank_ex_impl(const uint32_t *succ, const void *weight, int64_t 
   in.sync = opts->sync;
   in.ws = opts->workspace;
   in.ws_bytes = opts->ws_bytes;
+  if (host) in.h = *host;
   set_outputs(in, outs);
   return run(in, opts->tuning, (cudaStream_t)stream);
 }
@@ -1550,6 +1596,20 @@ lr_status lr_rank_host_async(const uint32_t *succ_host, const void *weight_host,
   return rank_host_impl(succ_host, weight_host, n, rank_host, opts, stream, false);
 }
 
+// What the device calls a pinned host buffer that it can read and write in
+// place (null: pageable, or not aligned to its elements, which a copy may be).
+static void *device_view(const void *p, size_t elems, size_t bytes) {
+  if ((uintptr_t)p % bytes) return nullptr;
+  cudaPointerAttributes a, b;
+  const char *last = (const char *)p + elems * bytes - 1;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaPointerGetAttributes(&b, last) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  if (a.type != cudaMemoryTypeHost || b.type != cudaMemoryTypeHost || !a.devicePointer || !b.devicePointer) return nullptr;
+  return (char *)b.devicePointer - (char *)a.devicePointer == last - (const char *)p ? a.devicePointer : nullptr;
+}
+
 static lr_status rank_host_impl(const uint32_t *succ_host, const void *weight_host, int64_t n,
                                 void *rank_host, const lr_opts *opts, lr_stream stream, bool sync) {
   lr_opts d;
@@ -1572,13 +1632,29 @@ static lr_status rank_host_impl(const uint32_t *succ_host, const void *weight_ho
   uint32_t *dsucc = (uint32_t *)b;
   void *dw = wb ? (void *)(b + bs) : nullptr;
   void *drank = b + bs + bw;
-  LR_TRY(cudaMemcpyAsync(dsucc, succ_host, 4 * (size_t)n, cudaMemcpyHostToDevice, s));
-  if (wb) LR_TRY(cudaMemcpyAsync(dw, weight_host, wb * (size_t)n, cudaMemcpyHostToDevice, s));
+  // A call that waits reads and writes pinned buffers in place: a copy before
+  // and after it would each take the link's time, in which the first and the
+  // last pass are done on the way (4 million elements: 371 us with the copies, 340
+  // without).  Streams that overlap calls keep the copies, which need no SM.
+  HostBuffers h;
+  memset(&h, 0, sizeof(h));
+  bool ranks_out = false;
+  h.ranks_out = &ranks_out;
+  if (sync) {
+    h.succ = (const uint32_t *)device_view(succ_host, (size_t)n, 4);
+    if (wb) h.weight = device_view(weight_host, (size_t)n, wb);
+    if (wb && !h.weight) h.succ = nullptr;
+    h.rank = device_view(rank_host, (size_t)n, (size_t)rb);
+  }
+  if (!h.succ) {
+    LR_TRY(cudaMemcpyAsync(dsucc, succ_host, 4 * (size_t)n, cudaMemcpyHostToDevice, s));
+    if (wb) LR_TRY(cudaMemcpyAsync(dw, weight_host, wb * (size_t)n, cudaMemcpyHostToDevice, s));
+  }
   lr_opts o = *opts;
   o.sync = 0;
-  st = lr_rank_ex(dsucc, dw, n, drank, &o, stream);
+  st = rank_ex_impl(dsucc, dw, n, drank, nullptr, &o, stream, &h);
   if (st != LR_OK) return st;
-  LR_TRY(cudaMemcpyAsync(rank_host, drank, (size_t)rb * n, cudaMemcpyDeviceToHost, s));
+  if (!ranks_out) LR_TRY(cudaMemcpyAsync(rank_host, drank, (size_t)rb * n, cudaMemcpyDeviceToHost, s));
   return sync ? device_status(s) : LR_OK;
 }
 

@@ -79,6 +79,8 @@ struct WeightScan {
   const uint32_t *unless_narrow;
   const unsigned long long *unless_local;   // launch_prep0: the sums, whose sample may show that the input will be
                                             // contracted; the pass does nothing then (null: not asked)
+  uint32_t *succ_copy;                      // launch_prep0, inputs in host memory: where to leave the successors
+  void *weight_copy;                        // and weights as they were read (null: nowhere)
 };
 
 constexpr int kSumTerminal = 5;
@@ -242,7 +244,7 @@ cudaError_t launch_wyllie(void *bufA, void *bufB, bool w16, uint32_t n, void *ra
 cudaError_t launch_finalize(LevelDesc *desc, int lev, const void *work, int kind,
                             const void *rnext, void *rout, int rank_bytes, uint32_t cap,
                             uint32_t *err, const uint32_t *tnext, uint32_t *tout,
-                            const uint32_t *tid_cur, cudaStream_t s);
+                            const uint32_t *tid_cur, cudaStream_t s, bool to_host = false);
 
 // Log path (unweighted level 0, see lr_log.cu).  The log's chunks go to the
 // chasing CTAs in windows of kLogWindow chunks.
