@@ -368,6 +368,25 @@ __device__ inline uint64_t block_exclusive_scan(uint64_t v, uint64_t *smem, uint
   return r;
 }
 
+// A kernel that may be launched before the one ahead of it in the stream has
+// ended (launch_after): wait for that one, then let the next one come.  Every
+// such kernel does this first, in all its threads, so that whatever came
+// before the one ahead has ended too.  The pointers given go through an empty
+// asm of their own behind the wait, so that no read through them can be moved
+// ahead of it; every other read has to depend on what those reads returned.
+template <class P>
+__device__ __forceinline__ void behind_wait(P &p) {
+  asm volatile("" : "+l"(p));
+}
+template <class... P>
+__device__ __forceinline__ void after_previous(P &...p) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  (behind_wait(p), ...);
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+// A kernel that is launched in the ordinary way, before one that is not.
+__device__ __forceinline__ void let_next_come() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // Add each v[k], summed over the CTA, to *out[k] (null: not wanted), with one
 // atomic per CTA and sum: one address serves an atomic in some 1.5 ns, so a
 // sum from every warp of a full grid would cost 15 us.  All threads call it.

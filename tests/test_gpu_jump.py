@@ -245,3 +245,30 @@ def test_validation_by_counts(n, wt):
     np.testing.assert_array_equal(r.cpu().numpy(), want_r)
     np.testing.assert_array_equal(t.cpu().numpy().view(np.uint32), want_t)
     np.testing.assert_array_equal(p.cpu().numpy(), want_p)
+
+
+def test_calls_back_to_back_on_two_streams():
+    # a kernel may start before the one ahead of it has ended: many calls of
+    # every kind, none waited for, each with its own inputs and outputs
+    kinds = []
+    for j, n in enumerate((20_000, 600_001, 1 << 20, 3_000_000)):
+        succ = gen.random_list(n, 9900 + j) if j != 1 else gen.forest(n, 9900 + j, n_long=3, long_len=n // 8,
+                                                                       mean_short=6)[0].astype(np.uint32)
+        w = gen.weights_i32(n, 9910 + j) if j % 2 else None
+        lists = int((succ == np.arange(n)).sum())
+        want = oracle.rank(succ, w, np.int64 if j % 2 else np.int32)
+        kinds.append((dev(succ), None if w is None else dev(w), lists, want))
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    torch.cuda.synchronize()
+    outs = []
+    for rnd in range(12):
+        for j, (succ, w, lists, want) in enumerate(kinds):
+            st = streams[(rnd + j) % 2]
+            with torch.cuda.stream(st):
+                mine = succ.clone()
+                out = lr.rank(mine, w, max_lists=lists if rnd % 3 else 0, sync=False, validate=rnd % 4 == 1)
+                mine.fill_(0)                       # the call has read them by then
+            outs.append((out, want))
+    torch.cuda.synchronize()
+    for out, want in outs:
+        np.testing.assert_array_equal(out.cpu().numpy(), want)
