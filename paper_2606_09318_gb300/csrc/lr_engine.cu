@@ -810,9 +810,9 @@ static lr_status run_contracted(const Inputs &in, const lr_tuning *tuning, Ctx *
   uint32_t *tpre = (uint32_t *)(b + off_tpre);
   uint16_t *tail16 = (uint16_t *)(b + off_tail);
   LR_TRY(launch_lc_solve(in.succ, in.weight, in.wtype, n, in.rank, in.rank_bytes, tail16, hb, wpre, tcnt,
-                         tpre, err, s));
-  LR_TRY(cudaMemcpyAsync(c->host_words + 1, tpre + nt, 4, cudaMemcpyDeviceToHost, s));
-  LR_TRY(cudaStreamSynchronize(s));
+                         tpre, err, c->host_words, ++c->token, s));
+  st = wait_word(c->host_words + kHostToken, c->token, s);
+  if (st != LR_OK) return st;
   const uint64_t m = c->host_words[1];
   if (!forced && m * 5 > (uint64_t)n * 3) { prof.cancel(); return LR_ERR_NOT_FOUND; }
   // the contracted list: successors, weights (int32 unweighted: at most one
