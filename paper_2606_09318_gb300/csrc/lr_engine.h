@@ -65,9 +65,9 @@ struct Ctx {
   void *direct = nullptr;           // run_base's words and predecessor marks: zero between calls
   size_t direct_bytes = 0;
   bool direct_clean = false;
-  uint32_t *host_words = nullptr;   // [0] device error bits, [1] head count, [2..3] tile-local
-                                    // links, [4..7] sampled tile-local links and elements,
-                                    // [8..9] int64 scratch, [4..15] first-pass sums, [16] token
+  uint32_t *host_words = nullptr;   // [0] device error bits, [1] list or node count, [2] a batch of one
+                                    // list per instance, [4..15] first-pass sums ([4..7] the sample,
+                                    // [8..9] an int64, [12] weight flags), [16] token
   uint32_t token = 0;               // the last one a call of this context waited for
   bool pending_status = false;
   const LevelDesc *last_desc = nullptr;   // level descriptors of the last ruling-set call
