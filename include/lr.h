@@ -294,10 +294,11 @@ lr_status lr_rank_host_async(const uint32_t *succ_host, const void *weight_host,
                              void *rank_host, const lr_opts *opts, lr_stream stream);
 
 /*
- * Bytes of workspace a call with these sizes needs when the caller passes
- * lr_opts.workspace.  k = 0 for lr_rank_ex.  Uses opts->max_lists as the
- * bound on the number of lists (0: assumes every element may be a head).
- * Host-only; needs no GPU.
+ * Bytes of workspace that serve any call of up to n_total elements when the
+ * caller passes lr_opts.workspace (a call itself may need less: fewer rulers
+ * are taken above some sizes).  k = 0 for lr_rank_ex.  Uses opts->max_lists
+ * as the bound on the number of lists (0: assumes every element may be a
+ * head).  Host-only; needs no GPU.
  */
 size_t lr_workspace_size(int64_t n_total, int32_t k, const lr_opts *opts);
 
@@ -541,8 +542,8 @@ void lr_autotune_clear(void);
  * submission still overlap this ranking), and the engine grows its own
  * buffers to the count.  depth: 2..4 (0 selects 2).  Device memory:
  * depth * max_n * (4 + weight bytes + rank bytes), plus
- * per ranking stream, when max_lists > 0, the most that lr_workspace_size
- * gives for any size up to max_n (the engine's own buffers otherwise).
+ * lr_workspace_size(max_n, 0, opts) per ranking stream when max_lists > 0
+ * (the engine's own buffers per ranking stream otherwise).
  *
  * Host buffers should be pinned (cudaHostAlloc / cudaHostRegister); pageable
  * buffers work but their copies block the submitting thread.  The caller

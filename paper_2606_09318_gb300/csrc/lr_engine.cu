@@ -97,7 +97,7 @@ constexpr uint32_t kBase0Max = 1u << 19;
 // Default ruler fraction below level 0: 1/4 where that already reaches the
 // base case (2^24, 10^6 rulers: 900 us a call at 1/4, 907 at 1/6, 912 at 1/8).
 static uint32_t default_f_inv(int64_t n, uint32_t f0_inv) {
-  return n / f0_inv <= (int64_t)kJumpMax * 4 ? 4 : 8;
+  return n / f0_inv <= 4ll * kJumpMax ? 4 : 8;
 }
 
 Tuning resolve_tuning_builtin(int64_t n, bool weighted, bool batch) {
@@ -1661,30 +1661,8 @@ static lr_status rank_host_impl(const uint32_t *succ_host, const void *weight_ho
 }  // extern "C"
 
 namespace lr {
-// The plan's size is not monotone in n: the default ruler fraction falls as n
-// grows.  Each fraction's largest size counts, and each power of two (tuned
-// entries are kept per power of two).
-size_t workspace_upto(int64_t n, const lr_opts *opts) {
-  size_t w = lr_workspace_size(n, 0, opts);
-  auto consider = [&](int64_t m) { if (m > 0 && m < n) w = std::max(w, lr_workspace_size(m, 0, opts)); };
-  for (int64_t m = 1; m < n; m *= 2) { consider(m - 1); consider(m); }
-  for (const F0Step &t : kF0Steps) consider(t.below - 1);
-  return w;
-}
-}  // namespace lr
-
-extern "C" {
-
-size_t lr_workspace_size(int64_t n_total, int32_t k, const lr_opts *opts) {
-  return lr_workspace_size_outputs(n_total, k, nullptr, opts);
-}
-
-size_t lr_workspace_size_outputs(int64_t n_total, int32_t k, const lr_outputs *outs,
-                                 const lr_opts *opts) {
-  lr_opts d;
-  if (!opts) { lr_opts_default(&d); opts = &d; }
-  if (n_total <= 0) return 0;
-  const Tuning u = resolve_tuning(opts->tuning, n_total, opts->wtype != LR_NONE, k > 0);
+// Bytes of workspace for a call of exactly this size.
+static size_t workspace_exact(int64_t n_total, int32_t k, const lr_outputs *outs, const lr_opts *opts, const Tuning &u) {
   // The chase grid depends on the device; size for a generous upper bound so
   // the answer needs no GPU: 256 SMs x 16 CTAs.
   if (u.algo == LR_ALGO_WYLLIE) {
@@ -1706,6 +1684,64 @@ size_t lr_workspace_size_outputs(int64_t n_total, int32_t k, const lr_outputs *o
                      extras && !outs->term, spawn0, ord0,
                      use_narrow(u, (uint64_t)n_total, opts->wtype != LR_NONE, spawn0, extras, true));
   return p.fixed_bytes + p.var_bytes;
+}
+
+// Sizes from which on a call may need less workspace than just below them:
+// with n growing, the need grows except where a rule on n gives fewer rulers,
+// fewer bytes an element or another form of level 0.  (Fewer rulers below
+// level 0: workspace_rulers_end; the log form's partition: log_geometry_step.
+// Powers of two: tuned entries are kept by them, and the partition's buckets
+// widen after them.)
+template <class F>
+static void workspace_steps(uint32_t base0, F &&step) {
+  for (const F0Step &t : kF0Steps) step(t.below);
+  step(1ll << 23);                               // default_f0_inv_batch
+  step(kOrdSpacingFrom);
+  step((int64_t)base0 + 1);                      // the base case: terminal ids make its records larger
+  step((int64_t)kLogAutoMin);                    // the log form at level 0, and its end
+  step((1ll << 30) + 1);
+  step(0x7FFFFF01ll);                            // 8-byte weighted records (room for cut segments) end
+  for (int b = 1; b < 33; ++b) { step(1ll << b); step((1ll << b) + 1); }
+}
+
+// The largest size with ruler fraction f0_inv for which default_f_inv takes
+// the larger share of rulers below level 0.
+static int64_t workspace_rulers_end(uint32_t f0_inv) { return (int64_t)f0_inv * (4ll * kJumpMax + 1) - 1; }
+}  // namespace lr
+
+extern "C" {
+
+size_t lr_workspace_size(int64_t n_total, int32_t k, const lr_opts *opts) {
+  return lr_workspace_size_outputs(n_total, k, nullptr, opts);
+}
+
+size_t lr_workspace_size_outputs(int64_t n_total, int32_t k, const lr_outputs *outs,
+                                 const lr_opts *opts) {
+  lr_opts d;
+  if (!opts) { lr_opts_default(&d); opts = &d; }
+  if (n_total <= 0) return 0;
+  const bool weighted = opts->wtype != LR_NONE;
+  const uint32_t base0 = resolve_tuning(opts->tuning, n_total, weighted, k > 0).base0;
+  // enough for every size up to n_total: for it, and for the last size of
+  // each stretch below it over which the need grows (at any ruler fraction an
+  // element takes 8 bytes at least and 64 at most, so an eighth of n_total
+  // never needs more than n_total)
+  size_t most = 0;
+  auto at = [&](int64_t m) {
+    const Tuning v = resolve_tuning(opts->tuning, m, weighted, k > 0);
+    most = std::max(most, workspace_exact(m, k, outs, opts, v));
+    return v.f0_inv;
+  };
+  auto consider = [&](int64_t m) {
+    if (m <= n_total / 8 || m > n_total) return;
+    const uint32_t f0 = at(m);
+    const int64_t rulers = workspace_rulers_end(f0), part = log_geometry_step(m);
+    if (rulers < m) at(rulers);
+    if (part > 0) at(part);
+  };
+  consider(n_total);
+  workspace_steps(base0, [&](int64_t from) { if (from <= n_total) consider(from - 1); });
+  return most;
 }
 
 lr_status lr_get_device_status(lr_stream stream) { return device_status((cudaStream_t)stream); }

@@ -88,9 +88,6 @@ bool tuned_lookup(int64_t n, bool weighted, bool batch, lr_tuning *out);
 Plan make_plan(uint64_t n, uint64_t h, const Tuning &u, bool rec16_0, int rank_bytes,
                uint64_t seed, int chase_grid, bool log0, bool term = false, bool t0ws = false,
                bool spawn0 = false, bool ord0 = false, bool narrow = false);
-// Workspace that serves a single instance of any size up to n (lr_workspace_size
-// is for one size).
-size_t workspace_upto(int64_t n, const lr_opts *opts);
 int chase_grid_for(const Tuning &u, bool rec16, bool log0, bool ord0, bool weighted);
 Ctx *get_ctx(cudaStream_t stream, lr_status *st);
 // Forget the context of a stream that is about to be destroyed (waits for

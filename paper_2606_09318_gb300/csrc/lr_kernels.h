@@ -265,6 +265,9 @@ struct LogGeom {
   uint32_t nw, sB, na, shiftA, gridA, claimA, capA, kb, claimB, capB, nbB;
 };
 LogGeom log_geometry(uint32_t n);
+// The largest size below n whose windows get more room each (0: none before
+// the last power of two): just above it the partition needs less.
+int64_t log_geometry_step(int64_t n);
 cudaError_t launch_finalize_log(LevelDesc *desc, const uint32_t *log, const uint2 *hdr, uint32_t total_chunks,
                                 const uint32_t *chunk_ctr, const void *r1, uint2 *pairsA, uint2 *pairsB,
                                 uint32_t *curA, uint32_t *curB, const LogGeom &g, uint32_t *rank, uint32_t *err,

@@ -679,6 +679,8 @@ static int part_resident_ctas() {
   return cached[dev];
 }
 
+constexpr uint32_t kLgClaimCtas = 2048;                     // CTAs of the second partition, over all A-buckets
+
 LogGeom log_geometry(uint32_t n) {
   LogGeom g;
   g.nw = (uint32_t)(((uint64_t)n + (1u << kLgWin) - 1) >> kLgWin);
@@ -692,11 +694,19 @@ LogGeom log_geometry(uint32_t n) {
   g.gridA = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(part_resident_ctas(), want));
   g.claimA = g.sB ? 32 : 8;
   g.capA = (1u << g.shiftA) + g.gridA * g.claimA;
-  g.kb = g.sB ? std::max<uint32_t>(1, 2048 / g.na) : 0;
+  g.kb = g.sB ? std::max<uint32_t>(1, kLgClaimCtas / g.na) : 0;
   g.claimB = 16;
   g.capB = g.sB ? (1u << kLgWin) + g.kb * g.claimB : 0;
   g.nbB = g.sB ? (g.na << g.sB) : 0;
   return g;
+}
+
+int64_t log_geometry_step(int64_t n) {
+  if (n > (1ll << 30)) return 0;                            // beyond the log form
+  const LogGeom g = log_geometry((uint32_t)n);
+  if (!g.sB) return 0;
+  const uint32_t na = kLgClaimCtas / (g.kb + 1);            // most A-buckets with one CTA more each
+  return na > 128 ? ((int64_t)na << g.sB) << kLgWin : 0;    // (more than 128: as wide as n's)
 }
 
 cudaError_t log_setup() {

@@ -150,7 +150,7 @@ extern "C" lr_status lr_pipeline_create(int64_t max_n, const lr_opts *opts, int3
   // With a bound on the lists the workspace is allocated here and no
   // submission allocates or waits; without one every submission counts its
   // lists first and the engine sizes its own buffers from the count.
-  p->ws_bytes = o.max_lists > 0 ? lr::workspace_upto(max_n, &o) : 0;
+  p->ws_bytes = o.max_lists > 0 ? lr_workspace_size(max_n, 0, &o) : 0;
 
   cudaError_t e = cudaStreamCreateWithFlags(&p->up, cudaStreamNonBlocking);
   for (int s = 0; s < p->ncomp && e == cudaSuccess; ++s) {
