@@ -25,6 +25,7 @@
 #include <type_traits>
 
 #include "lr_kernels.h"
+#include "lr_ordq.h"
 
 namespace lr {
 
@@ -1370,94 +1371,39 @@ cudaError_t launch_order(LevelDesc *desc, int lev, uint32_t cap, uint64_t *cnt, 
   return cudaGetLastError();
 }
 
-
-// Ordered queue: CTAs draw positions of the ruler sequence from one global
-// counter, kOrdChunk at a time, and hand them to their threads through a
-// shared-memory window, (end << 32) | next.  The lanes of a warp that ask
-// together take theirs with one atomic.  The group that brings the window
-// down to kOrdLow positions draws the next chunk, which waits in s_next; the
-// first group that runs past the window's end and finds it there makes it the
-// window.  A group that does not find it draws just what it lacks from the
-// global counter.  Nobody waits.
-//
-// The counter is one address, which serves one atomic in some 1.5 ns, so how
-// often it is asked can bound the chase.  With 32 positions a draw, fetched
-// only when the window had run out, and single draws until they came, a batch
-// of 7.5e7 unweighted elements took 1.51 ms, however many threads chased; now
-// 1.37 ms, and 1.06 with half as many threads again.  A CTA that starts with
-// one draw for all its threads saves 0.23 ms at any size, and once the
-// sequence has run out, nobody asks.
-constexpr uint32_t kOrdChunk = 128, kOrdLow = kOrdChunk / 2;
-static_assert(kOrdLow >= 32, "a chunk serves a warp and stays above the low mark");
-
+// A CTA's end of the ordered queue (lr_ordq.h), in shared memory.
 struct OrdQueue {
   unsigned long long win, next;    // the window; the chunk after it (0: not there)
   uint32_t out;                    // the sequence has run out
 };
 
-__device__ __forceinline__ unsigned long long ord_window(uint64_t from, uint64_t to) {
-  return ((unsigned long long)to << 32) | from;
-}
+struct OrdAccess {
+  OrdQueue &q;
+  uint32_t *counter;
+  __device__ __forceinline__ void exchange_window(unsigned long long w) const { atomicExch(&q.win, w); }
+  __device__ __forceinline__ unsigned long long window() const { return *(volatile unsigned long long *)&q.win; }
+  __device__ __forceinline__ unsigned long long exchange_next(unsigned long long w) const { return atomicExch(&q.next, w); }
+  __device__ __forceinline__ uint32_t draw(uint32_t c) const { return atomicAdd(counter, c); }
+  __device__ __forceinline__ bool out() const { return *(volatile uint32_t *)&q.out != 0u; }
+  __device__ __forceinline__ void set_out() const { *(volatile uint32_t *)&q.out = 1u; }
+};
 
-// Draw a chunk from the global counter; 0 when there is none.
-__device__ __forceinline__ unsigned long long ord_draw(OrdQueue &q, uint32_t *gq, uint64_t total, uint32_t *fresh) {
-  const uint32_t j = atomicAdd(gq, kOrdChunk);
-  if (j >= total) {
-    *(volatile uint32_t *)&q.out = 1u;
-    return 0ull;
-  }
-  *fresh = j;
-  // the chunk is this CTA's whatever its length: every position of it must be
-  // handed out, up to the end of the sequence
-  return ord_window(j, (uint64_t)j + kOrdChunk < total ? (uint64_t)j + kOrdChunk : total);
-}
-
-// Position for this lane (total or more: none left).  *fresh: set on the lane
-// that drew a chunk, to the chunk's first position.
-__device__ __forceinline__ uint64_t ord_take(OrdQueue &q, uint32_t *gq, uint64_t total, uint32_t *fresh) {
+// Position for this lane (total or more: none left); one request for all the
+// lanes that ask together.  *fresh: set on the lane that drew a chunk, to the
+// chunk's first position.
+__device__ __forceinline__ uint32_t ord_take(OrdQueue &q, uint32_t *gq, uint32_t total, uint32_t *fresh) {
   const uint32_t mask = __activemask();
   const uint32_t lane = threadIdx.x & 31u, leader = __ffs(mask) - 1;
   const uint32_t cnt = __popc(mask), mine = __popc(mask & ((1u << lane) - 1u));
-  unsigned long long w = 0;
-  if (lane == leader) w = atomicAdd(&q.win, (unsigned long long)cnt);
-  w = __shfl_sync(mask, w, leader);
-  const uint32_t next = (uint32_t)w, end = (uint32_t)(w >> 32);
-  const uint32_t have = next < end ? min(end - next, cnt) : 0u, lack = cnt - have;
-  uint64_t more = total;                       // where the lacking positions start
+  unsigned long long w = 0, more = 0;
   if (lane == leader) {
-    bool draw = next + kOrdLow < end && next + cnt + kOrdLow >= end;     // brings the window down to the mark
-    if (lack) {
-      const unsigned long long c = atomicExch(&q.next, 0ull);
-      if (c) {
-        const uint32_t from = (uint32_t)c, to = (uint32_t)(c >> 32), left = to - from;
-        more = from;
-        draw = left <= lack + kOrdLow;         // a short chunk starts below the mark
-        if (left > lack) {
-          // the window, unless another group has opened one since this one
-          // asked: then it goes back (whoever holds the chunk is the only one
-          // who could open a window)
-          const unsigned long long now = *(volatile unsigned long long *)&q.win;
-          const bool spent = (uint32_t)now >= (uint32_t)(now >> 32);
-          atomicExch(spent ? &q.win : &q.next, ord_window(from + lack, to));
-          draw = draw && spent;
-        }
-        if (left < lack) {                     // only the sequence's last chunk: the rest is past its end
-          *(volatile uint32_t *)&q.out = 1u;
-          draw = false;
-        }
-      } else if (!*(volatile uint32_t *)&q.out) {
-        const uint32_t j = atomicAdd(gq, lack);
-        more = j;
-        if (j >= total) *(volatile uint32_t *)&q.out = 1u;
-      }
-    }
-    if (draw && !*(volatile uint32_t *)&q.out) {
-      const unsigned long long c = ord_draw(q, gq, total, fresh);
-      if (c) atomicExch(&q.next, c);
-    }
+    w = atomicAdd(&q.win, (unsigned long long)cnt);
+    more = ord_ask(OrdAccess{q, gq}, w, cnt, total, fresh);
   }
-  more = __shfl_sync(mask, more, leader);
-  return mine < have ? (uint64_t)next + mine : more + (mine - have);
+  w = __shfl_sync(mask, w, leader);
+  const uint32_t have = ord_window_has(w, cnt);          // the same in every lane
+  if (have < cnt) more = __shfl_sync(mask, more, leader);
+  return ord_position(w, have, more, total, mine);
 }
 
 // ---------------------------------------------------------------- chase
@@ -1527,7 +1473,7 @@ k_chase(LevelDesc *__restrict__ desc, int lev, Rec *__restrict__ work, Rec16 *__
   const uint64_t R = (uint64_t)r + d.k;
   if (ord && threadIdx.x == 0) {               // the CTA's first window and chunk
     const uint32_t first = 2u * blockDim.x, j = atomicAdd(qctr, first);
-    s_q.win = j < R ? ord_window(j, min((uint64_t)j + first, R)) : 0ull;
+    s_q.win = j < R ? ord_window(j, (uint32_t)min((uint64_t)j + first, R)) : 0ull;
     s_q.next = 0ull;
     s_q.out = j >= R;
   }
@@ -1542,7 +1488,8 @@ k_chase(LevelDesc *__restrict__ desc, int lev, Rec *__restrict__ work, Rec16 *__
   auto take = [&]() -> uint64_t {
     if (ord) {
       uint32_t fresh = 0xFFFFFFFFu;              // first position of a chunk this thread drew
-      const uint64_t got = ord_take(s_q, qctr, R, &fresh);
+      uint32_t got;
+      do got = ord_take(s_q, qctr, (uint32_t)R, &fresh); while (got == kOrdAgain);
       if (const uint64_t j = fresh; fresh != 0xFFFFFFFFu && oa.pf_lead && j >= d.k) {
         // the CTA took the rulers from j on: bring the records of the
         // elements up to its next draw's first ruler, pf_lead elements ahead,
