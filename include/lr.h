@@ -84,7 +84,9 @@ typedef enum lr_dtype { LR_NONE = 0, LR_I32 = 1, LR_I64 = 2 } lr_dtype;
 typedef struct lr_tuning {
     uint32_t f0_inv;     /* 1/f at level 0 (default by n: 4 for the smallest     */
                          /* lists that take it to 96 from 2^29; a batch takes    */
-                         /* 16 from 2^23 and 12 from 2^24)                       */
+                         /* 16 from 2^23 and 12 from 2^24).  Another than the    */
+                         /* default keeps level 0 to the ruling set where the    */
+                         /* base case would rank it whole                        */
     uint32_t f_inv;      /* 1/f at levels >= 1 (default 4 or 8, by size)         */
     uint32_t cutoff;     /* largest level ranked by the base case when below     */
                          /* 12288; 12288 and more, and 0: the built-in bound     */
@@ -476,14 +478,15 @@ lr_status lr_server_stats_get(lr_server *s, lr_server_stats *out);
 void lr_server_destroy(lr_server *s);
 
 /*
- * Autotuner.  The best ruler fractions, base-case cutoff and chase block
- * depend on n, on the weights and on whether the input is a batch (small
- * lists are bound by the latency along one segment, large ones by the
- * random-access rate).  lr_autotune measures candidates on the current
- * device by coordinate descent from the built-in defaults (level-0 fraction
- * 1/f0, deeper fraction 1/f, cutoff, chase block, then f0 again), each the
- * fastest of a few timed calls on `stream`, and checks that the winner's
- * ranks equal the defaults' bit for bit (else LR_ERR_INTERNAL).
+ * Autotuner.  The best ruler fractions and chase block depend on n, on the
+ * weights and on whether the input is a batch (small lists are bound by the
+ * latency along one segment, large ones by the random-access rate).
+ * lr_autotune measures candidates on the current device by coordinate
+ * descent from the built-in defaults (level-0 fraction 1/f0, deeper fraction
+ * 1/f, chase block, then f0 again), each the fastest of a few timed calls on
+ * `stream`, and checks that the winner's ranks equal the defaults' bit for
+ * bit (else LR_ERR_INTERNAL).  Up to 2^19 elements, which the base case ranks
+ * whole, nothing is searched: the default call is timed.
  *
  * Inputs: the caller's device arrays (succ, weight, offsets as for
  * lr_rank_ex / lr_rank_batch_ex; offsets required when k > 0), or, with
@@ -493,17 +496,20 @@ void lr_server_destroy(lr_server *s);
  * as for the ranking call; workspace must be NULL; the call allocates and
  * frees its own scratch.  Synchronises `stream`.
  *
- * The winner is stored in a process-wide table keyed by (floor(log2 n),
- * weighted, batched) and written to *out (may be NULL).  Every later call
- * whose opts->tuning is NULL uses its key's entry (an explicit lr_tuning,
- * then LR_TUNING in the environment, take precedence).  The table is saved
- * and loaded as JSON; LR_TUNING_FILE names a file loaded on first use.
+ * The winner is written to *out (may be NULL) and stored in a process-wide
+ * table keyed by (floor(log2 n), weighted, batched), where zeros stand for
+ * the defaults of each size if nothing beat them.  Every later call whose
+ * opts->tuning is NULL uses its key's entry (an explicit lr_tuning, then
+ * LR_TUNING in the environment, take precedence), except for the entry's
+ * cutoff: bounds saved by earlier versions do not take the base case away.
+ * The table is saved and loaded as JSON; LR_TUNING_FILE names a file loaded
+ * on first use.
  */
 typedef struct lr_tune_entry {
     int32_t log2n;       /* floor(log2 n) of the tuned size                      */
     int32_t weighted;    /* 1: weighted                                          */
     int32_t batch;       /* 1: batched form (k > 0)                              */
-    lr_tuning tuning;    /* the winner                                           */
+    lr_tuning tuning;    /* the winner (zero fields: the defaults)               */
     float ms;            /* its time per call on the tuning input                */
 } lr_tune_entry;
 

@@ -122,12 +122,14 @@ Tuning resolve_tuning_builtin(int64_t n, bool weighted, bool batch) {
 
 Tuning resolve_tuning(const lr_tuning *t, int64_t n, bool weighted, bool batch) {
   Tuning u = resolve_tuning_builtin(n, weighted, batch);
+  const uint32_t f0_builtin = u.f0_inv;
   u.f_inv = 0;
   lr_tuning tt;
   if (tuned_lookup(n, weighted, batch, &tt)) {
     if (tt.f0_inv) u.f0_inv = tt.f0_inv;
     if (tt.f_inv) u.f_inv = tt.f_inv;
-    if (tt.cutoff) u.cutoff = tt.cutoff;
+    // (not its cutoff: entries saved before the base case jumped pointers hold
+    // bounds of 12288 and less, which would take it away from whole octaves)
     if (tt.chase_block) u.block = tt.chase_block;
     if (tt.chase_ctas) u.ctas = tt.chase_ctas;
   }
@@ -160,9 +162,10 @@ Tuning resolve_tuning(const lr_tuning *t, int64_t n, bool weighted, bool batch) 
   u.f_inv = u.f_inv ? std::max<uint32_t>(2, u.f_inv) : default_f_inv(n, u.f0_inv);
   u.cutoff = std::min<uint32_t>(std::max<uint32_t>(u.cutoff, 64), kMaxCutoff);
   if (u.block != 128 && u.block != 256 && u.block != 512) u.block = 256;
-  // what asks for the ruling set itself keeps level 0 to it
+  // what asks for the ruling set itself keeps level 0 to it; a caller's
+  // spacing does unless it is the default, as the autotuner hands it out
   const bool srs = u.cutoff < kMaxCutoff || u.spawn || u.chase0 != LR_CHASE0_AUTO || env_u32(env, "f0", 0) ||
-                   (t && t->f0_inv);
+                   (t && t->f0_inv && t->f0_inv != f0_builtin);
   u.base0 = srs ? u.cutoff : kBase0Max;
   u.base = u.cutoff >= kMaxCutoff ? kJumpMax : u.cutoff;
   return u;

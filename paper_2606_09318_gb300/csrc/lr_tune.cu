@@ -1,21 +1,22 @@
 // lr_tune.cu -- autotuner for the ruling-set recursion (lr_autotune*).
 //
-// The best ruler fraction, base-case cutoff and chase launch shape depend on
-// the list size, the weights and whether the input is a batch: small lists
-// are bound by the latency of one segment's dependent exchanges, large ones
-// by the random-access rate (see the level-0 chase).  lr_autotune measures
-// candidates on the device, by coordinate descent from the built-in
-// defaults:
+// The best ruler fractions and chase launch shape depend on the list size,
+// the weights and whether the input is a batch: small lists are bound by the
+// latency of one segment's dependent exchanges, large ones by the
+// random-access rate (see the level-0 chase).  lr_autotune measures
+// candidates on the device, by coordinate descent from the built-in defaults:
 //   1. level-0 ruler fraction 1/f0 in {4, 8, 16, 32, 64, 128},
 //   2. deeper fraction 1/f in {4, 8, 16},
-//   3. base-case cutoff in {4096, 8192, 12288},
-//   4. chase block 128 / 256 / 512 threads,
-//   5. level-0 fraction again next to the best,
+//   3. chase block 128 / 256 / 512 threads,
+//   4. level-0 fraction again next to the best,
 // each timed as the fastest of a few calls with CUDA events, and checks that
-// the winner's ranks equal the defaults' bit for bit.  The winner is kept in
-// a table keyed by (floor(log2 n), weighted, batched); calls that pass no
-// tuning use the entry of their key.  The table is saved and loaded as JSON
-// (lr_autotune_save / _load; LR_TUNING_FILE is loaded on first use).
+// the winner's ranks equal the defaults' bit for bit.  Sizes that the base
+// case ranks whole have nothing to search: the default call is timed.  The
+// winner is kept in a table keyed by (floor(log2 n), weighted, batched), as
+// zeros (the defaults of each size) where nothing beat the defaults; calls
+// that pass no tuning use the entry of their key.  The table is saved and
+// loaded as JSON (lr_autotune_save / _load; LR_TUNING_FILE is loaded on first
+// use).
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -263,8 +264,11 @@ extern "C" lr_status lr_autotune(const uint32_t *succ, const void *weight, const
     return e == cudaErrorMemoryAllocation ? LR_ERR_OUT_OF_MEMORY : LR_ERR_CUDA;
   }
 
-  // reference output with the built-in defaults (table entries ignored)
+  // reference output with the built-in defaults (table entries ignored; the
+  // default values, named, take the default call's route)
   const Tuning d = resolve_tuning_builtin(n_total, weighted, k > 0);
+  const bool search = n_total > (int64_t)d.base0;
+  bool better = false;
   lr_tuning best;
   memset(&best, 0, sizeof(best));
   best.f0_inv = d.f0_inv;
@@ -283,16 +287,17 @@ extern "C" lr_status lr_autotune(const uint32_t *succ, const void *weight, const
       lr_tuning c = best;
       c.*field = v;
       const float ms = R.time(c, reps);
-      if (ms < best_ms) { best_ms = ms; best = c; }
+      if (ms < best_ms) { best_ms = ms; best = c; better = true; }
     }
   };
-  if (st == LR_OK) {
+  if (st == LR_OK && search) {
     try_field(&lr_tuning::f0_inv, {4, 8, 16, 32, 64, 128});
     try_field(&lr_tuning::f_inv, {4, 8, 16});
-    try_field(&lr_tuning::cutoff, {4096, 8192, 12288});
     try_field(&lr_tuning::chase_block, {128, 256, 512});
     const uint32_t f0 = best.f0_inv;
     try_field(&lr_tuning::f0_inv, {std::max<uint32_t>(2, f0 * 2 / 3), f0 * 3 / 2});
+  }
+  if (st == LR_OK && better) {
     // the winner must rank exactly as the defaults do
     st = R.call(&best, rank);
     if (st == LR_OK) st = device_status(s);
@@ -315,7 +320,7 @@ extern "C" lr_status lr_autotune(const uint32_t *succ, const void *weight, const
   ent.log2n = log2_floor(n_total);
   ent.weighted = weighted ? 1 : 0;
   ent.batch = k > 0 ? 1 : 0;
-  ent.tuning = best;
+  if (better) ent.tuning = best;
   ent.ms = best_ms;
   {
     std::lock_guard<std::mutex> g(g_tmu);
