@@ -457,6 +457,13 @@ static bool inject_alloc_failure() {
   return v && v[0] == '1';
 }
 
+// The same with LR_INJECT_LAUNCH_FAIL=1 for the base case of an input: it
+// fails between its two launches, as if the second had been refused.
+static bool inject_launch_failure() {
+  const char *v = getenv("LR_INJECT_LAUNCH_FAIL");
+  return v && v[0] == '1';
+}
+
 lr_status ensure_buffer(void **buf, size_t *cur, size_t want, cudaStream_t s) {
   if (inject_alloc_failure()) return LR_ERR_OUT_OF_MEMORY;
   if (*cur >= want && *buf) return LR_OK;
@@ -700,6 +707,23 @@ static InitParams init_params(const Plan &p) {
   return ip;
 }
 
+// The words that run_base's two launches share, while a call uses them.  A call
+// that fails between the launches clears them itself, so that neither the next
+// call nor a graph captured before finds what it left.  A captured call has
+// not run: it leaves the context's note of them alone.
+struct OwnWords {
+  Ctx *ctx;                                    // null: not used (or captured)
+  size_t bytes;
+  cudaStream_t s;
+  void left_clean() {
+    if (ctx) ctx->direct_clean = true;
+    ctx = nullptr;
+  }
+  ~OwnWords() {
+    if (ctx) ctx->direct_clean = cudaMemsetAsync(ctx->direct, 0, bytes, s) == cudaSuccess;
+  }
+};
+
 // An input that the base case ranks as it is: one pass that packs the records,
 // then k_jump, which needs no heads.  From `checked` elements on (and for a
 // batch of separate buffers) two predecessors and a broken promise of
@@ -734,11 +758,12 @@ static lr_status run_base(const Inputs &in, const Plan &p, bool checked, char *f
   memset(&ji, 0, sizeof(ji));
   bool own = !in.ws && !in.ctx && !in.err_ext && !extras && n <= kBase0Max;
   const size_t own_bytes = 256 + kBase0Max / 8;
-  if (own && !c->direct) own = !stream_capturing(s) && ensure_buffer(&c->direct, &c->direct_bytes, own_bytes, s) == LR_OK;
+  const bool capturing = stream_capturing(s);
+  OwnWords words_used = {nullptr, own_bytes, s};
+  if (own && !c->direct) own = !capturing && ensure_buffer(&c->direct, &c->direct_bytes, own_bytes, s) == LR_OK;
   if (own) {
-    // new, or a call that failed on the way left them as they were
-    if (!c->direct_clean) LR_TRY(cudaMemsetAsync(c->direct, 0, own_bytes, s));
-    c->direct_clean = false;
+    if (!c->direct_clean) LR_TRY(cudaMemsetAsync(c->direct, 0, own_bytes, s));       // new
+    if (!capturing) words_used.ctx = c;
     uint32_t *words = (uint32_t *)c->direct;
     err = words;
     ji.count = words + 16;
@@ -764,6 +789,7 @@ static lr_status run_base(const Inputs &in, const Plan &p, bool checked, char *f
   }
   if (!in.ctx) { c->last_desc = desc; c->last_nlev = 1; }
   prof.mark(PH_PREP);
+  if (inject_launch_failure()) return LR_ERR_CUDA;
   if (checked && in.max_lists > 0) {
     ji.max_lists = (uint64_t)in.max_lists;
     ji.bitmap = bitmap;
@@ -772,7 +798,7 @@ static lr_status run_base(const Inputs &in, const Plan &p, bool checked, char *f
   ji.offsets = in.offsets;
   ji.k = in.k;
   LR_TRY(launch_jump(desc, 0, work, p.rec16_0, in.rank, p.rank_bytes, n, err, nullptr, nullptr, T0, &ji, s));
-  if (own) c->direct_clean = true;
+  words_used.left_clean();
   prof.mark(PH_BASE);
   if (extras)
     LR_TRY(launch_outputs(desc, bitmap, nullptr, n, T0, in.rank, in.prefix, p.rank_bytes, in.incl, in.weight,
