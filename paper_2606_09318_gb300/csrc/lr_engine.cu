@@ -457,10 +457,10 @@ static bool inject_alloc_failure() {
   return v && v[0] == '1';
 }
 
-// The same with LR_INJECT_LAUNCH_FAIL=1 for the base case of an input: it
-// fails between its two launches, as if the second had been refused.
+// In a debug build LR_INJECT_LAUNCH_FAIL=1 makes the base case of an input fail
+// between its two launches, as if the second had been refused.
 static bool inject_launch_failure() {
-  const char *v = getenv("LR_INJECT_LAUNCH_FAIL");
+  const char *v = kDebugChecks ? getenv("LR_INJECT_LAUNCH_FAIL") : nullptr;
   return v && v[0] == '1';
 }
 
@@ -728,8 +728,8 @@ struct OwnWords {
 // then k_jump, which needs no heads.  From `checked` elements on (and for a
 // batch of separate buffers) two predecessors and a broken promise of
 // max_lists are looked for, as the ruling set notices them there.
-static lr_status run_base(const Inputs &in, const Plan &p, bool checked, char *fixed, char *var, Ctx *c,
-                          cudaStream_t s) {
+static lr_status run_base(const Inputs &in, const Plan &p, bool checked, bool capturing, char *fixed, char *var,
+                          Ctx *c, cudaStream_t s) {
   const uint32_t n = (uint32_t)in.n;
   const bool extras = p.term, marks = checked || in.validate || in.prefix != nullptr;
   LevelDesc *desc = (LevelDesc *)(fixed + p.off_desc);
@@ -758,7 +758,6 @@ static lr_status run_base(const Inputs &in, const Plan &p, bool checked, char *f
   memset(&ji, 0, sizeof(ji));
   bool own = !in.ws && !in.ctx && !in.err_ext && !extras && n <= kBase0Max;
   const size_t own_bytes = 256 + kBase0Max / 8;
-  const bool capturing = stream_capturing(s);
   OwnWords words_used = {nullptr, own_bytes, s};
   if (own && !c->direct) own = !capturing && ensure_buffer(&c->direct, &c->direct_bytes, own_bytes, s) == LR_OK;
   if (own) {
@@ -982,7 +981,7 @@ lr_status run(const Inputs &given, const lr_tuning *tuning, cudaStream_t s) {
       in.rank = in.h.rank;
       *in.h.ranks_out = true;
     }
-    return run_base(in, p, checked, fixed, var, c, s);
+    return run_base(in, p, checked, capturing, fixed, var, c, s);
   }
   if (log0) LR_TRY(fetch());
   // (the log form's last pass would hold every SM for the time of the link)
