@@ -604,15 +604,19 @@ static lr_status map_device_bits(uint32_t bits) {
     if (e__ != cudaSuccess) return from_cuda(e__);     \
   } while (0)
 
-// Copy the call's device error word to the context's pinned status word;
-// with sync, wait and return the status it encodes.  err == nullptr: a kernel
-// has written the status word itself.
 // Wait for a kernel on stream s to write `token` to the pinned word *w.  The
 // stream's state is looked at now and then, so that the wait ends whatever
-// becomes of the kernel.
+// becomes of the kernel; and a caller that has asked for waits which give up
+// their core (cudaSetDeviceFlags: blocking, yield) gets one, for the stream.
 static lr_status wait_word(const uint32_t *w, uint32_t token, cudaStream_t s) {
+  bool asked = false;
   for (uint32_t spin = 1; __atomic_load_n(w, __ATOMIC_ACQUIRE) != token; ++spin) {
     if (spin % 4096 != 0) continue;
+    unsigned flags = 0;
+    if (!asked && cudaGetDeviceFlags(&flags) == cudaSuccess &&
+        (flags & (cudaDeviceScheduleYield | cudaDeviceScheduleBlockingSync)))
+      LR_TRY(cudaStreamSynchronize(s));
+    asked = true;
     const cudaError_t e = cudaStreamQuery(s);
     if (e == cudaErrorNotReady) continue;
     LR_TRY(e);
@@ -621,6 +625,9 @@ static lr_status wait_word(const uint32_t *w, uint32_t token, cudaStream_t s) {
   return LR_OK;
 }
 
+// Copy the call's device error word to the context's pinned status word;
+// with sync, wait and return the status it encodes.  err == nullptr: a kernel
+// has written the status word itself.
 static lr_status finish_call(Ctx *c, const uint32_t *err, int sync, cudaStream_t s) {
   if (err) LR_TRY(cudaMemcpyAsync(c->host_words, err, 4, cudaMemcpyDeviceToHost, s));
   c->pending_status = true;
