@@ -518,7 +518,13 @@ struct Profiler {
     mark(-1);
   }
   void mark(int phase) {
+    note(phase);
+    record(phase);
+  }
+  void note(int phase) {
     if (ranged && phase >= 0) nvtxMarkA(kPhaseNames[phase]);
+  }
+  void record(int phase) {
     if (!on) return;
     ProfMark m;
     m.phase = phase;
@@ -533,6 +539,11 @@ struct Profiler {
     call.launches = launch_count() - call.launches;
     std::lock_guard<std::mutex> g(g_mu);
     g_prof_pending.push_back(call);
+  }
+  // take back the marks from the k-th on (work that turned out not to be done)
+  void drop_from(size_t k) {
+    for (size_t i = k; i < call.marks.size(); ++i) cudaEventDestroy(call.marks[i].ev);
+    if (call.marks.size() > k) call.marks.resize(k);
   }
   // drop a call that turned out not to happen (its marks are not recorded)
   void cancel() {
@@ -1039,7 +1050,7 @@ lr_status run(const Inputs &given, const lr_tuning *tuning, cudaStream_t s) {
   // us, and 9 more of 737 in the wait for the sample at 2^24.)
   // Likewise a batch, as one list per instance.
   const bool guess_batch = sums0b && in.k <= kMaxOpenBatch && !ord_used;
-  const bool guess = need_count && (sums0 || sumsv || guess_batch) && !in.ws && !spawn0 && !prof.on;
+  const bool guess = need_count && (sums0 || sumsv || guess_batch) && !in.ws && !spawn0;
   const uint64_t guess_lists = guess_batch ? (uint64_t)in.k : 1;
   const uint32_t ask_local = local_exact ? kLocalCounted : count_local && guess ? kLocalSampled : kLocalUnasked;
   if (count_local && !local_exact)
@@ -1095,6 +1106,7 @@ lr_status run(const Inputs &given, const lr_tuning *tuning, cudaStream_t s) {
   uint32_t one_term = 0;
   bool one_list = false;                       // the host has seen that level 0 is one list
   bool chased = false;                         // and it was one
+  const size_t marks_before = prof.call.marks.size();
   if (guess) {
     const Plan g = make_plan(in.n, guess_lists, u, rec16_0, in.rank_bytes, in.seed, grid, log0, false, false, spawn0, ord0, narrow);
     st = ensure_buffer(&c->var, &c->var_bytes, g.var_bytes, s);
@@ -1116,8 +1128,10 @@ lr_status run(const Inputs &given, const lr_tuning *tuning, cudaStream_t s) {
     else
       LR_TRY(launch_init(desc, ip, acc, kind0 == kRecKind8w ? wflags : nullptr, (uint32_t *)(v + g.off_hA), ns,
                          (uint32_t *)(v + g.off_hB), s));
+    prof.record(PH_PREP);
     LR_TRY(launch_chase(desc, 0, work0, kind0, v + g.off_work[1], ns, qctr, g.chase_grid, g.chase_block, err,
                         (int)u.xchg, nullptr, nullptr, nullptr, nullptr, s));
+    prof.record(PH_CHASE0);
     st = wait_word(c->host_words + kHostToken, ip.token, s);
     if (st != LR_OK) return st;
   }
@@ -1182,7 +1196,11 @@ lr_status run(const Inputs &given, const lr_tuning *tuning, cudaStream_t s) {
     LR_TRY(cudaStreamSynchronize(s));     // nothing else may still write the caller's memory
     return LR_ERR_CAPACITY;               // the lists need more workspace than was given
   }
-  prof.mark(PH_PREP);
+  if (!chased) {
+    prof.drop_from(marks_before);
+    prof.record(PH_PREP);
+  }
+  prof.note(PH_PREP);
 
   uint32_t *hA = (uint32_t *)(var + p.off_hA);
   uint32_t *hB = (uint32_t *)(var + p.off_hB);
@@ -1246,7 +1264,9 @@ lr_status run(const Inputs &given, const lr_tuning *tuning, cudaStream_t s) {
     if (l > 0 || !(one_list || chased))
       LR_TRY(launch_heads(desc, l, p.nlev, bitmap, hin, (l == 0 && log0) ? (void *)in.succ : work_of(l),
                         kind, ns, hout, bcnt, err, p.base, p.hcap, s));
-    prof.mark(PH_SELECT);
+    const bool recorded = l == 0 && chased;
+    prof.note(PH_SELECT);
+    if (!recorded) prof.record(PH_SELECT);
     if (l == 0 && chased) {
       // (queued before the wait)
     } else if (l == 0 && log0)
@@ -1277,7 +1297,8 @@ lr_status run(const Inputs &given, const lr_tuning *tuning, cudaStream_t s) {
                             (int)u.xchg, nullptr, nullptr, nullptr, oa.ord ? &oa : nullptr, s));
     }
     if (l == 0) prof.call.log0 = log0;
-    prof.mark(l == 0 ? PH_CHASE0 : PH_CHASE);
+    prof.note(l == 0 ? PH_CHASE0 : PH_CHASE);
+    if (!recorded) prof.record(l == 0 ? PH_CHASE0 : PH_CHASE);
   }
   LR_TRY(launch_jump(desc, L, work_of(L), true, R_of(L), p.rank_bytes, p.cap[L], err, head_list(L),
                      tid_of(L), T_of(L), nullptr, s));
