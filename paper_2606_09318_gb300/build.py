@@ -21,7 +21,7 @@ LIB = os.path.join(OUT, "liblr.so")
 OUT_DEBUG = os.path.join(HERE, "_build_debug")
 LIB_DEBUG = os.path.join(OUT_DEBUG, "liblr_debug.so")
 SOURCES = ["lr_kernels.cu", "lr_log.cu", "lr_engine.cu", "lr_server.cu", "lr_noalloc.cu", "lr_probe.cu", "lr_pipeline.cu", "lr_wyllie.cu", "lr_tune.cu", "lr_contract.cu"]
-HEADERS = ["lr_device.cuh", "lr_kernels.h", "lr_engine.h", "lr_ordq.h"]
+HEADERS = ["lr_device.cuh", "lr_kernels.h", "lr_engine.h", "lr_ordq.h", "lr_hostview.h"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC,-O2", "--expt-relaxed-constexpr",
          "-I" + os.path.join(ROOT, "include"), "-I" + CSRC]

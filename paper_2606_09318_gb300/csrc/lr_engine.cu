@@ -11,6 +11,7 @@
 // on the device (each level's head scan writes the next level's size and
 // mode), so a call never waits for the device unless h has to be counted
 // first, and a call with a known bound can be captured in a CUDA graph.
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -27,6 +28,7 @@
 
 #include "lr.h"
 #include "lr_engine.h"
+#include "lr_hostview.h"
 #include "lr_kernels.h"
 
 namespace lr {
@@ -1652,18 +1654,40 @@ lr_status lr_rank_host_async(const uint32_t *succ_host, const void *weight_host,
   return rank_host_impl(succ_host, weight_host, n, rank_host, opts, stream, false);
 }
 
-// What the device calls a pinned host buffer that it can read and write in
-// place (null: pageable, or not aligned to its elements, which a copy may be).
-static void *device_view(const void *p, size_t elems, size_t bytes) {
-  if ((uintptr_t)p % bytes) return nullptr;
-  cudaPointerAttributes a, b;
-  const char *last = (const char *)p + elems * bytes - 1;
-  if (cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaPointerGetAttributes(&b, last) != cudaSuccess) {
+// The pinned piece of host memory around q (pinned_view).
+static bool pinned_piece(const void *q, PinnedPiece &piece) {
+  using Ask = CUresult (*)(void *, CUpointer_attribute, CUdeviceptr);
+  static const Ask ask = [] {
+    void *f = nullptr;
+    cudaDriverEntryPointQueryResult got;
+    if (cudaGetDriverEntryPointByVersion("cuPointerGetAttribute", &f, 12000, cudaEnableDefault, &got) != cudaSuccess) {
+      cudaGetLastError();
+      f = nullptr;
+    }
+    return reinterpret_cast<Ask>(f);
+  }();
+  cudaPointerAttributes a;
+  if (cudaPointerGetAttributes(&a, q) != cudaSuccess) {
     cudaGetLastError();
-    return nullptr;
+    return false;
   }
-  if (a.type != cudaMemoryTypeHost || b.type != cudaMemoryTypeHost || !a.devicePointer || !b.devicePointer) return nullptr;
-  return (char *)b.devicePointer - (char *)a.devicePointer == last - (const char *)p ? a.devicePointer : nullptr;
+  if (!ask || a.type != cudaMemoryTypeHost || !a.devicePointer) return false;
+  CUdeviceptr start = 0;
+  size_t size = 0;
+  const CUdeviceptr d = reinterpret_cast<CUdeviceptr>(a.devicePointer);
+  if (ask(&start, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, d) != CUDA_SUCCESS ||
+      ask(&size, CU_POINTER_ATTRIBUTE_RANGE_SIZE, d) != CUDA_SUCCESS || d < start || d - start >= size)
+    return false;
+  piece.device = a.devicePointer;
+  piece.left = size - (size_t)(d - start);
+  return true;
+}
+
+// What the device calls a host buffer that it can read and write in place
+// (null: not pinned throughout, or not aligned to its elements, which a copy
+// may be).
+static void *device_view(const void *p, size_t elems, size_t bytes) {
+  return (uintptr_t)p % bytes ? nullptr : pinned_view(p, elems * bytes, pinned_piece);
 }
 
 static lr_status rank_host_impl(const uint32_t *succ_host, const void *weight_host, int64_t n,
