@@ -2178,9 +2178,9 @@ __device__ __forceinline__ uint64_t jump_hash(uint32_t x, uint64_t seed) {
   return splitmix64(seed ^ ((uint64_t)x * 0xD1342543DE82EF95ull));
 }
 
-// Level 0 (JumpInput): heads are not needed; with a bound on the lists, those
-// of two or more elements are counted from the has-predecessor bitmap.  PTRS:
-// ranks go to one buffer per instance.
+// Level 0 (JumpInput): heads are not needed; with a bound on the lists, they
+// are counted from the has-predecessor bitmap, as many as the ruling set would
+// have to provide for.  PTRS: ranks go to one buffer per instance.
 template <class Rec, class RT, bool TERM, bool PTRS>
 __global__ void __launch_bounds__(kJumpThreads, kJumpCtasPerSm)
 k_jump(LevelDesc *__restrict__ desc, int lev, Rec *work, RT *__restrict__ rout, uint32_t *__restrict__ err,
@@ -2221,6 +2221,10 @@ k_jump(LevelDesc *__restrict__ desc, int lev, Rec *work, RT *__restrict__ rout, 
         else bad |= kErrInternal;              // never written by a prep or a chase
         if (heads) chk += jump_hash(s, d.seed);
         if (in.max_lists) lists += !((__ldcg(in.bitmap + (i >> 5)) >> (i & 31u)) & 1u);
+      } else if (in.max_lists && !((__ldcg(in.bitmap + (i >> 5)) >> (i & 31u)) & 1u)) {
+        Perm Q;                                // a list of one: the ruling set takes it for a
+        Q.init(n, d.seed);                     // list if it is a sampled ruler
+        lists += Q.fwd(i) < d.r;
       }
       if (heads) chk -= jump_hash(i, d.seed);
     }

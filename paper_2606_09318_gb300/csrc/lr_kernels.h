@@ -193,9 +193,9 @@ cudaError_t launch_chase(LevelDesc *desc, int lev, void *work, int kind, void *n
                          const OrdArgs *ord, cudaStream_t s);
 
 // What the base case needs to rank level 0 itself (all optional): the most
-// lists of two or more elements the caller promised (0: any number), counted
-// from the has-predecessor bitmap into *count (zeroed); one rank buffer per
-// instance.  With ticket (zeroed), the kernel ends the call: it copies the
+// lists the caller promised (0: any number), counted from the has-predecessor
+// bitmap into *count (zeroed; lists of one element as far as they are sampled
+// rulers, like the ruling set); one rank buffer per instance.  With ticket (zeroed), the kernel ends the call: it copies the
 // error bits to *status (host memory the device can write) and leaves the
 // error word, *count, *ticket and the bitmap (clear) at zero.
 struct JumpInput {
