@@ -76,10 +76,11 @@ typedef enum lr_dtype { LR_NONE = 0, LR_I32 = 1, LR_I64 = 2 } lr_dtype;
  * explicit lr_tuning takes precedence) overrides them for measurement, as comma-separated
  * key=value pairs: f0, f, cutoff, block, ctas (the fields below); xchg=0
  * (visits by load and store instead of an atomic exchange); log=0 / log=1
- * (force the level-0 form); algo, contract, spawn; ord (batches: 0 chases
- * by per-CTA slices of ruler ids, 1 takes level 0's rulers in element
- * order, 2, the default, every level; only levels whose records exceed L2); pf (the
- * element order's L2 prefetch lead in K elements, 0 off, 4 by default).
+ * (force the level-0 form); algo, contract, spawn; ord (batches, levels of
+ * more than 128 MiB of records: 0 chases by per-CTA slices of ruler ids, 1
+ * takes level 0's rulers in element order, 2, the default, every such
+ * level's); pf (the element order's L2 prefetch lead in K elements, 0 off, 4
+ * by default).
  */
 typedef struct lr_tuning {
     uint32_t f0_inv;     /* 1/f at level 0 (default by n: 4 for the smallest     */
@@ -92,8 +93,8 @@ typedef struct lr_tuning {
                          /* 12288; 12288 and more, and 0: the built-in bound     */
     uint32_t chase_block;/* threads per CTA of the chase kernel (default 256)    */
     uint32_t chase_ctas; /* CTAs per SM of the chase kernel (default: occupancy; */
-                         /* a batch's level 0, chased in element order, 1024    */
-                         /* threads per SM)                                      */
+                         /* a batch chased in element order, 1024 threads per    */
+                         /* SM when weighted, 1536 unweighted)                   */
     uint32_t algorithm;  /* LR_ALGO_SRS (0, default) or LR_ALGO_WYLLIE            */
     uint32_t contract;   /* tile-local contraction: 0 auto (default),            */
                          /* LR_CONTRACT_OFF or LR_CONTRACT_ON                     */
@@ -143,9 +144,10 @@ typedef struct lr_tuning {
  * default) lets the prep pass count the links that stay inside their tile
  * and contracts when at least half do, decided at the wait that counts the
  * lists; it applies to single-instance calls that count their lists anyway
- * (max_lists == 0, no workspace, not during capture, no extra outputs,
- * n >= 16384).  LR_CONTRACT_ON contracts without counting;
- * LR_CONTRACT_OFF never contracts.  Results are identical either way.
+ * (max_lists == 0, no workspace, not during capture, no extra outputs) and
+ * are too long for the base case (n > 2^19).  LR_CONTRACT_ON contracts such
+ * calls without counting, from n = 16384 on; LR_CONTRACT_OFF never contracts.
+ * Results are identical either way.
  */
 #define LR_CONTRACT_AUTO 0u
 #define LR_CONTRACT_OFF 1u

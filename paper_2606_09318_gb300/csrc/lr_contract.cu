@@ -100,7 +100,7 @@ struct LcMarks {
   uint32_t nlinks, nmarked;  // local links; marked elements
   uint32_t wflags;           // over the tile's local links: kWBig19 | kWNeg | kWBig20
 };
-// A tile whose local-link weights all lie in (-2^19, 2^19), or all in
+// A tile whose local-link weights all lie in [-2^19, 2^19), or all in
 // [0, 2^20), has every distance (at most kTile - 1 links) within 32 bits,
 // signed or unsigned: its prefix sums are taken modulo 2^32.
 constexpr uint32_t kWBig19 = 1u, kWNeg = 2u, kWBig20 = 4u;

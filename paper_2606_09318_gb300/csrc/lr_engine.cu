@@ -115,7 +115,7 @@ Tuning resolve_tuning_builtin(int64_t n, bool weighted, bool batch) {
   u.algo = LR_ALGO_SRS;
   u.contract = LR_CONTRACT_AUTO;
   u.spawn = 0;
-  u.ord = 2;              // batches: every level of 2^20 or more in element order
+  u.ord = 2;              // batches: every level of more than kOrdMinBytes in element order
   u.base0 = kBase0Max;
   u.base = kJumpMax;
   u.pf = 4;               // ... prefetching its records 4K elements ahead of each draw
@@ -193,6 +193,9 @@ static bool use_log0(const Tuning &u, uint64_t n, bool weighted, int rank_bytes,
 // to build it and half the threads (3.8 million weighted elements 249 us
 // without, 306 with it; 15 million unweighted 586 / 663; 22 million weighted,
 // 355 MB of records, 1237 / 1016).
+// (Deeper levels of a batch keep each instance's rulers together too, and are
+// chased in order by the same rule; LR_TUNING ord=1: level 0 only; ord=0: no
+// level.)
 constexpr uint64_t kOrdMinBytes = 128ull << 20;
 static bool use_ord0(const Tuning &u, uint64_t n, bool rec16, bool log0, bool spawn0, bool extras, bool multi) {
   return u.ord != 0 && multi && !log0 && !spawn0 && !extras && n <= 0x7FFFFFFFull &&
@@ -209,9 +212,6 @@ constexpr int kOrdCtasWeighted = 4, kOrdCtasUnweighted = 6;
 // Below this size the packing pass counts the links that stay in their tiles
 // itself, instead of a sample and a wait of its own before it.
 constexpr uint64_t kPackFirst = 1ull << 22;
-// (Deeper levels of a batch keep each instance's rulers together too, and are
-// chased in order by the same rule; LR_TUNING ord=1: level 0 only; ord=0: no
-// level.)
 
 int chase_grid_for(const Tuning &u, bool rec16, bool log0, bool ord0, bool weighted) {
   int per = u.ctas ? (int)u.ctas : (log0 ? chase_log_occupancy((int)u.block) : chase_occupancy(rec16, (int)u.block));

@@ -2172,7 +2172,7 @@ struct JumpState<Rec16> {
 
 // A level below the first holds every element once among the successors of
 // its non-terminals and its heads, or some element has two predecessors.
-// Both sides are compared as sums of this hash (jump_check in LevelDesc,
+// Both sides are compared as sums of this hash (check in LevelDesc,
 // examined by the propagation that reads the level's ranks).
 __device__ __forceinline__ uint64_t jump_hash(uint32_t x, uint64_t seed) {
   return splitmix64(seed ^ ((uint64_t)x * 0xD1342543DE82EF95ull));
